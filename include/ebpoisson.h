@@ -176,8 +176,8 @@ typedef struct {
   double tol;        /* stop when max|r| <= tol * max|b| (Sec. 3.3.2), default 1e-10 */
   int max_cycles;    /* cap on V-cycles in total, default 100 */
   int nu1, nu2;      /* red-black Gauss-Seidel sweeps before / after the coarse correction;
-                        -1 (the default) = by dimension: 2 in 2D, 6 in 3D, the fastest
-                        to 1e-10 on the rod-plane and pin-plane workloads */
+                        -1 (the default) = by dimension: 2 in 2D, 3 in 3D, the fastest
+                        on the rod-plane and pin-plane workloads */
   int precision;     /* EB_PREC_FP64: FP64 V-cycles; EB_PREC_MIXED: FP32 V-cycles inside FP64 defect correction */
   int inner_cycles;  /* FP32 V-cycles per FP64 outer iteration (mixed), default 2 */
   int bottom_sweeps; /* relaxation sweeps on the coarsest level, default 64 */
@@ -199,12 +199,12 @@ typedef struct {
   double kernel_ms; /* device time of the persistent solve kernel(s) of this call, from CUDA
                        events on the stream they ran on; 0 on the multi-launch paths */
   int bottom;       /* how the coarsest level was solved: EB_BOTTOM_* */
-  int levels;       /* multigrid levels of the V-cycle */
-  int sweep_levels; /* levels relaxed by tile-streamed sweeps (FP32 3D levels of at least 2^25 cells,
+  int levels;       /* multigrid levels of the V-cycle, algebraic ones included */
+  int sweep_levels; /* levels relaxed by tile-streamed sweeps: only on request, by the environment
+                       variable EBP_SWEEP_MIN_CELLS=n at set-up (FP32 3D levels of at least n cells,
                        x extent a multiple of 16, y and z multiples of 4: both colours in one pass
-                       over the level, tiles staged in shared memory by TMA); the others use one
-                       pass per colour.  The environment variable EBP_SWEEP=0 turns them off,
-                       EBP_SWEEP_MIN_CELLS=n moves the threshold, EBP_SWEEP_RESTRICT=1 also
+                       over the level, tiles staged in shared memory by TMA); all others use one
+                       pass per colour.  EBP_SWEEP=0 turns them off, EBP_SWEEP_RESTRICT=1 also
                        restricts these levels by a tile-streamed residual + restriction pass */
 } eb_solve_info;
 
@@ -212,8 +212,9 @@ typedef struct {
  * or by relaxation; which one applies follows from the coarsest level's size):
  * an exact FP64 inverse for at most 256 unknowns, applied inside one CTA; an
  * FP32 Gauss-Jordan inverse for at most 1024 unknowns, applied by the whole
- * grid; BiCGStab over the whole grid when coarsening stopped above 4096 cells;
- * else red-black relaxation sweeps inside one CTA (also the bottom of the
+ * grid; above that, algebraic levels (cells joined two by two per axis) down
+ * to at most 16 cells, those solved by BiCGStab when the geometric coarsening
+ * stopped above 4096 cells, else by relaxation sweeps (also the bottom of the
  * per-phase launch paths). */
 enum { EB_BOTTOM_RELAX = 1, EB_BOTTOM_INV64 = 2, EB_BOTTOM_INV32 = 3, EB_BOTTOM_KRYLOV = 4 };
 

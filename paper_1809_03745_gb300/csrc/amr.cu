@@ -593,11 +593,11 @@ extern "C" eb_status eb_amr_setup_levels(const eb_geom_desc* desc, int n_levels,
   oc.inner_cycles = 1;
   oc.nu1 = oc.nu2 = 3;
   oc.bottom_sweeps = std::min(oc.bottom_sweeps, 32);
-  st = eb_poisson_setup(A->lv[0].G, &oc, stream, &A->lv[0].P);
+  st = poisson_setup(A->lv[0].G, &oc, false, &A->lv[0].P);
   A->lv[0].P0 = A->lv[0].P;
   for (int l = 1; l < L && st == EB_OK; ++l) {
-    st = eb_poisson_setup(A->lv[l].G, &A->o, stream, &A->lv[l].P);
-    if (st == EB_OK) st = eb_poisson_setup(A->lv[l].G0, &oc, stream, &A->lv[l].P0);
+    st = poisson_setup(A->lv[l].G, &A->o, false, &A->lv[l].P);
+    if (st == EB_OK) st = poisson_setup(A->lv[l].G0, &oc, false, &A->lv[l].P0);
   }
   if (st != EB_OK) return amr_fail(A, st);
   if (cudaStreamSynchronize(s) != cudaSuccess) return amr_fail(A, cuda_fail(cudaGetLastError(), "amr setup"));

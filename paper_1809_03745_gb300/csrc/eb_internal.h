@@ -32,6 +32,7 @@ struct DevLevel {
   long long nnz = 0;
   int* eb_q = nullptr;          // finest level: cut-record index of each EB-list cell
   long long n_eb = 0;
+  double* sdiag = nullptr;      // [2 nirr] shift part of diag (algebraic levels)
   std::vector<void*> allocs;
 };
 
@@ -124,6 +125,7 @@ eb_status batch_prepare(eb_poisson* P, const double* rhs, const double* sigma, c
 eb_status batch_step(eb_poisson* const* P, int n, const double* const* rhs, const double* const* sigma,
                      double* const* phi, bool fresh, bool copy_out, int max_iters, cudaStream_t s,
                      double* kernel_ms);
+eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, bool kry, eb_poisson** out);
 void batch_info(eb_poisson* Q, eb_solve_info* inf);
 eb_status batch_copy_out(eb_poisson* P, double* phi, cudaStream_t s);
 long long poisson_device_bytes(const eb_poisson* P);

@@ -1,4 +1,7 @@
-// persistent.cuh -- the whole solve in one cooperative launch.
+// persistent.cuh -- the whole solve in one cooperative launch, in the plain
+// cell layout: hierarchies with tile-streamed levels (on request); every
+// other solve runs the colour-split form of rbsolve.cuh, which shares the
+// barrier, the controls and the set-up kernels here.
 //
 // Multigrid phases (arXiv:1809.03745, Sec. 3.3.2) run as grid-stride loops
 // separated by a software grid barrier; levels small enough for one CTA run
@@ -84,6 +87,8 @@ struct SolveCtl {
   int* out;                   // [0] status, [1] outer iterations, [2] V-cycles, [3] norm slot of the final residual
   unsigned long long* trace;  // [1 + TRMAX]: count, then (code << 48 | ns) per phase of the first V-cycle
   int max_iters;              // outer iterations allowed in this launch (0: no limit); status 7 when reached
+  int kry;    // 1: Krylov acceleration of the corrections (rbsolve.cuh)
+  int fresh;  // 1: a solve starts with this launch, 0: one is resumed
 };
 
 __device__ __forceinline__ unsigned long long now_ns() {
@@ -838,13 +843,10 @@ __device__ bool ph_smooth(const Op<T>& o, int nu, const Ctx& c, int l) {
 // pass over the level, and the black cut cells.  Within each of the four
 // groups no cell reads another's new value except through the colour order,
 // as in the colour passes.
-// SW: the kernel carries the tile-streamed passes (an instantiation without
-// them keeps their out-of-line calls, and the registers those cost around
-// the call sites, out of every other solve).
-template <class T, bool SW>
+template <class T>
 __device__ bool ph_smooth_grid(const Hier<T>& H, int l, int nu, const Ctx& c) {
   const Op<T>& o = H.op[l];
-  if (!SW || !H.sw[l].on || c.local || c.gsize < 2) return ph_smooth(o, nu, c, l);
+  if (!H.sw[l].on || c.local || c.gsize < 2) return ph_smooth(o, nu, c, l);
   const long long rr = 2 * o.nirr_red, rn = 2 * o.nirr;
   for (int s = 0; s < nu; ++s) {
     if (rr > 0) {
@@ -1113,16 +1115,16 @@ __device__ bool ph_bicgstab_grid(const Hier<T>& H, const Ctx& c) {
   return true;
 }
 
-template <class T, bool SW>
+template <class T>
 __device__ bool vcycle_dev(const Hier<T>& H, const Op<T>* lop, const Ctx& G) {
   for (int l = 0; l < H.lc; ++l) {
     const Op<T>& o = H.op[l];
-    if (!ph_smooth_grid<T, SW>(H, l, H.nu1, G)) return false;
+    if (!ph_smooth_grid<T>(H, l, H.nu1, G)) return false;
     if (o.nirr) {
       ph_rows(o, 0, 2 * o.nirr, 1, G);
       if (!G.sync((l << 4) | 5)) return false;
     }
-    if (SW && H.sw[l].on && H.sw[l].rs && G.gsize >= 2 && o.n[0] == 2 * H.op[l + 1].n[0] && o.n[1] == 2 * H.op[l + 1].n[1] &&
+    if (H.sw[l].on && H.sw[l].rs && G.gsize >= 2 && o.n[0] == 2 * H.op[l + 1].n[0] && o.n[1] == 2 * H.op[l + 1].n[1] &&
         o.n[2] == 2 * H.op[l + 1].n[2]) {
       if (!ph_restrict3d(H, l, G)) return false;
     } else {
@@ -1145,7 +1147,7 @@ __device__ bool vcycle_dev(const Hier<T>& H, const Op<T>* lop, const Ctx& G) {
   for (int l = H.lc - 1; l >= 0; --l) {
     ph_prolong(H.op[l], H.op[l + 1], G);
     if (!G.sync((l << 4) | 7)) return false;
-    if (!ph_smooth_grid<T, SW>(H, l, H.nu2, G)) return false;
+    if (!ph_smooth_grid<T>(H, l, H.nu2, G)) return false;
   }
   return true;
 }
@@ -1202,21 +1204,7 @@ __device__ __forceinline__ void stage_words(unsigned char* dst, const void* src,
   for (long long i = threadIdx.x; i < words; i += blockDim.x) d[i] = s[i];
 }
 
-// The V-cycle as the FP64 solve calls it: out of line, which keeps ptxas
-// from spilling the FP64 V-cycle's registers into the outer loop (1276 bytes
-// of spills inlined, 92 out of line); the FP32 V-cycle stays inline (64
-// bytes inlined, 92 out of line).
-template <class T, bool SW>
-__device__ __noinline__ bool vcycle_dev_ool(const Hier<T>& H, const Op<T>* lop, const Ctx& G) {
-  return vcycle_dev<T, SW>(H, lop, G);
-}
-template <class T, bool SW>
-__device__ __forceinline__ bool vcycle_call(const Hier<T>& H, const Op<T>* lop, const Ctx& G) {
-  if constexpr (sizeof(T) == 8) return vcycle_dev_ool<T, SW>(H, lop, G);
-  else return vcycle_dev<T, SW>(H, lop, G);
-}
-
-template <class T, bool SW>
+template <class T>
 __device__ __forceinline__ void solve_group(const Hier<T>* __restrict__ Hg, const Op<double>* __restrict__ Fg,
                                             const SolveCtl& ctl, const Barrier& B, int gcta, int gsize) {
   __shared__ Hier<T> H;
@@ -1312,7 +1300,7 @@ __device__ __forceinline__ void solve_group(const Hier<T>* __restrict__ Hg, cons
         Gk.tr = ctl.trace;
         if (gcta == 0 && threadIdx.x == 0) ctl.trace[1 + tn++] = ((unsigned long long)0xfff << 48) | (now_ns() & 0xffffffffffffULL);
       }
-      ok = vcycle_call<T, SW>(H, lop, Gk);
+      ok = vcycle_dev<T>(H, lop, Gk);
     }
     if (ok && ctl.mixed) {
       ph_update64(F, H.op[0], G);
@@ -1335,10 +1323,10 @@ __device__ __forceinline__ void solve_group(const Hier<T>* __restrict__ Hg, cons
   }
 }
 
-template <class T, bool SW>
+template <class T>
 __global__ void __launch_bounds__(PT, 1) k_solve(const Hier<T>* __restrict__ Hg, const Op<double>* __restrict__ Fg,
                                                  SolveCtl ctl, Barrier B) {
-  solve_group<T, SW>(Hg, Fg, ctl, B, (int)blockIdx.x, (int)gridDim.x);
+  solve_group<T>(Hg, Fg, ctl, B, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // one instance of a batched solve: its hierarchy, fine operator, controls,
@@ -1354,11 +1342,11 @@ struct BatchItem {
 
 // Many independent solves in one cooperative launch: each CTA finds its
 // instance and runs the solve with the instance's own group barrier.
-template <class T, bool SW>
+template <class T>
 __global__ void __launch_bounds__(PT, 1) k_solve_batch(const BatchItem<T>* __restrict__ items,
                                                        const int* __restrict__ cta_item) {
   const BatchItem<T>& it = items[cta_item[blockIdx.x]];
-  solve_group<T, SW>(it.H, it.F, it.ctl, it.B, (int)blockIdx.x - it.start, it.size);
+  solve_group<T>(it.H, it.F, it.ctl, it.B, (int)blockIdx.x - it.start, it.size);
 }
 
 // Setup of the tile-streamed passes: one CTA per (tile, plane).  Entry
@@ -1528,8 +1516,8 @@ __global__ void k_convert(const S* a, T* b, long long n) {
   if (i < n) b[(i % m) * m + i / m] = (T)a[i];
 }
 
-template <class T>
-__global__ void k_from_float(const float* a, T* b, long long n) {
+template <class T, class S>
+__global__ void k_from(const S* a, T* b, long long n) {
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) b[i] = (T)a[i];
 }

@@ -1,0 +1,1584 @@
+// rbsolve.cuh -- the persistent solve on colour-split levels.
+//
+// Multigrid (arXiv:1809.03745, Sec. 3.3.2) with every level stored split by
+// the red-black colouring: the red cells of an x row lie next to each other,
+// then, in a second half, the black ones.  What that buys on a GB300:
+//   * a colour pass reads only the other colour's values and its own
+//     right-hand side and writes only its own values, four cells of the colour
+//     per 16-byte access, where the plain layout moves both colours' lines for
+//     each pass (256^3 FP32: 100 MB per pass instead of 218 MB);
+//   * a pass writes a third buffer, which then takes the place of the colour's
+//     old one.  The sparse rows of the colour's cut cells, whose stencils may
+//     reach cells of their own colour, therefore read the values of before the
+//     pass, in the same phase as the regular cells: one grid barrier per
+//     colour instead of two, with the same values;
+//   * the four (2D: two) red cells under four neighbouring coarse cells lie at
+//     the same four positions as those, so restriction and prolongation are
+//     vector passes too.  After a black pass the residual of a regular black
+//     cell is zero (its equation was just solved), so restriction forms the
+//     red ones only.
+// The correction of each V-cycle joins a Krylov space (rb_kry_coeff): a few
+// modes that the coarse grids represent badly (a pin thinner than a coarse
+// cell, a rough interface) no longer set the rate, so three sweeps per leg do
+// in 3D what six did.  Measured on a GB300, solves to 1e-13 of max|b|, against
+// the plain layout without any of this: pin-plane 256^3 134 -> 40 ms (24
+// V-cycles of 6+6 sweeps -> 16 of 3+3), 384^3 334 -> 95 ms; rod-plane 1024^2
+// 10.2 -> 8.4 ms; 632 x 488, whose 79 x 61 bottom was BiCGStab over the grid
+// and is now algebraic levels, 62 -> 7.5 ms; 512^2 in FP64 20.7 -> 12.5 ms.
+// The phases are functions out of line: inlined into one kernel, ptxas spilled
+// 4.8 KB of them and took minutes.  The grid barrier, the bounded waits and the
+// trace are those of persistent.cuh.
+#pragma once
+
+#include "persistent.cuh"
+
+namespace ebp {
+
+constexpr int RMAX = 28;  // levels, the algebraic ones included
+constexpr int KH = 4;     // Krylov slots: the new direction and the three before it
+constexpr int KDOT = 2 * KH;  // sums per pass: (r, q), (q, q), then (q, q_i) and (r, q_i)
+struct KryState;
+
+// split flags: the cell flags of eb_common.cuh and, per cell,
+constexpr unsigned R_SPC = 8;       // a child has a sparse row (its right-hand side comes from the special list)
+constexpr unsigned R_LIN0 = 16;     // phase p: every coarse cell of the linear interpolation has an unknown (R_LIN0 << p)
+constexpr unsigned R_NOHOME0 = 64;  // phase p: the coarse cell above has no unknown (R_NOHOME0 << p)
+constexpr unsigned R_BASE = 0x07070707u;
+
+template <class T>
+struct RLev {
+  FastDiv dq, dn1;  // nq, n[1]
+  int D, n[3];
+  int hx;   // cells of one colour per x row, rounded up to 4 (entries past the row have flags 0)
+  int nq;   // groups of four of them
+  int nqt;  // groups per colour
+  int H;    // entries per colour
+  int two;  // both phases
+  int dense;  // the level has regular cells
+  int full;   // x rows fill their groups (n[0] a multiple of 8)
+  T dge[2];   // diagonal count of a cell at the low / high x wall and nowhere else
+  T ide[2][2];  // and its reciprocal with the shift, [side][phase]
+  int p1o, p1n;  // the entries of a dielectric half that are stored (the slabs that hold the phase)
+  T wr[6], w3[6], lh[2], idg[2], ceps[2], h2e[2];
+  // per phase three halves: after s sweeps red is x[p][2s % 3], black
+  // x[p][(2s + 1) % 3], and the third is written next
+  T* x[2][3];
+  T* b[2][2];  // [phase][colour]
+  const uint8_t* f[2];
+  // sparse rows of cells and phases with an unknown, red first
+  int nr, nr0;
+  int staged;            // entries in T in this CTA's shared memory
+  const int2* re;        // first and last entry
+  const unsigned* rs;    // the row's own cell: phase << 31 | colour * H + position
+  const unsigned* col;   // entries' cells, encoded alike
+  const void *val, *diag, *dinv;  // double, or T when staged; dinv = 1 / diag
+  // coarse cells (of the next level) with a child that has a sparse row, and
+  // per such cell the rows of its children (slot child + 2^D * phase, -1: none)
+  int nsp;
+  const int *sp, *sprow;
+};
+
+template <class T>
+struct RHier {
+  int nlev, lc;     // levels; the first one inside CTA 0
+  int nu1[RMAX], nu2[RMAX], bsweeps;  // sweeps per level, and on the last one
+  int bot;          // 0 relaxation, 1 inverse (in CTA 0 when local, else over the grid)
+  int bm;           // order of the inverse
+  const T* binv;    // [bm][bm] row-major, slots as bslot
+  const unsigned* bslot;  // slot -> phase << 31 | colour * H + position; ~0u: no unknown
+  int smem;         // levels lc.. in CTA 0's shared memory
+  RLev<T> L[RMAX];
+  // byte offsets into shared memory of levels lc..
+  int off_x[RMAX][2][3], off_b[RMAX][2][2], off_f[RMAX][2], off_re[RMAX], off_rs[RMAX], off_col[RMAX], off_val[RMAX],
+      off_dg[RMAX], off_di[RMAX], off_sp[RMAX], off_spr[RMAX], nnz[RMAX];
+  int srows[RMAX];  // rows staged too
+  // finest level in FP64: natural cell of every sparse row, entries' natural
+  // columns and values, the rows' diagonals
+  const int *rnat, *ncol;
+  const double *rval, *rdiag;
+  // Krylov directions of the finest level, [slot][phase][colour]: z and q = A z
+  T *kz[KH][2][2], *kq[KH][2][2];
+  double* kpart;       // [chunk][KDOT] partial sums
+  int kcs, kch, krows;  // groups per chunk, chunks, sparse rows per chunk
+  KryState* kst;
+};
+
+struct RCtx {
+  int i0, st;        // this thread's first item and the stride over items
+  int g0, gst;       // groups of 8 lanes, counted from the other end
+  bool local;
+  Barrier B;
+  unsigned* epoch;
+  unsigned long long* tr;
+  unsigned* tn;
+  int gcta, gsize;
+  __device__ __forceinline__ bool sync(int code) const {
+    bool ok = true;
+    if (local) __syncthreads();
+    else ok = grid_sync(B, epoch, gsize);
+    if (tr && gcta == 0 && threadIdx.x == 0 && *tn < TRMAX) {
+      tr[1 + *tn] = ((unsigned long long)code << 48) | (now_ns() & 0xffffffffffffULL);
+      *tn += 1;
+    }
+    return ok;
+  }
+};
+
+template <class T>
+__device__ __forceinline__ void st4(T* p, const T v[4]) {
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+    reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
+  }
+}
+template <class T>
+__device__ __forceinline__ void ld2(const T* p, T& a, T& b) {
+  if constexpr (sizeof(T) == 4) {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    a = q.x;
+    b = q.y;
+  } else {
+    const double2 q = *reinterpret_cast<const double2*>(p);
+    a = q.x;
+    b = q.y;
+  }
+}
+
+// a group of four cells of one colour: x row (j, k), positions q0 .. q0 + 3,
+// cells i = 2 q + s
+struct QPos {
+  int t, j, k, q0, s;
+};
+template <class T>
+__device__ __forceinline__ QPos quad_pos(const RLev<T>& L, int t, int colour) {
+  QPos g;
+  const unsigned row = fdiv((unsigned)t, L.dq);
+  const unsigned kq = fdiv(row, L.dn1);
+  g.t = t;
+  g.j = (int)(row - kq * (unsigned)L.n[1]);
+  g.k = (int)kq;
+  g.q0 = 4 * (t - (int)row * L.nq);
+  g.s = (g.j + g.k + colour) & 1;
+  return g;
+}
+// bytes 0xff where the cell is regular and of phase p
+__device__ __forceinline__ unsigned regular_mask(unsigned w, int p) {
+  return __vcmpeq4(w & R_BASE, p ? 0x02020202u : 0x01010101u);
+}
+
+// the other colour's values around a group: row centre, y and z neighbours,
+// and the one x neighbour outside the group
+template <class T>
+struct QNb {
+  T c[4], ym[4], yp[4], zm[4], zp[4], xs;
+};
+template <class T>
+__device__ __forceinline__ void quad_load(const RLev<T>& L, const QPos& g, const T* xn, QNb<T>& v) {
+  const T* c = xn + 4 * (long long)g.t;
+  const int sy = L.hx, sz = L.hx * L.n[1];
+  ld4(c, v.c);
+  v.xs = T(0);
+  if (g.s == 0) {
+    if (g.q0 > 0) v.xs = c[-1];
+  } else if (2 * g.q0 + 8 < L.n[0]) {
+    v.xs = c[4];
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) v.ym[e] = v.yp[e] = v.zm[e] = v.zp[e] = T(0);
+  if (g.j > 0) ld4(c - sy, v.ym);
+  if (g.j < L.n[1] - 1) ld4(c + sy, v.yp);
+  if (L.D == 3) {
+    if (g.k > 0) ld4(c - sz, v.zm);
+    if (g.k < L.n[2] - 1) ld4(c + sz, v.zp);
+  }
+}
+// per lane the neighbour sum and the diagonal count (open faces, 3 w per wall
+// face of weight w) of the implicit stencil; walls as in mg_kernels.cuh
+template <class T>
+__device__ __forceinline__ void quad_sums(const RLev<T>& L, const QPos& g, QNb<T>& v, T sum[4], T dg[4]) {
+  T d0 = T(2 * L.D);
+  if (g.j == 0) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v.ym[e] = L.w3[2] * v.yp[e];
+    d0 += T(3) * L.wr[2] - T(1);
+  }
+  if (g.j == L.n[1] - 1) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v.yp[e] = L.w3[3] * v.ym[e];
+    d0 += T(3) * L.wr[3] - T(1);
+  }
+  if (L.D == 3) {
+    if (g.k == 0) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v.zm[e] = L.w3[4] * v.zp[e];
+      d0 += T(3) * L.wr[4] - T(1);
+    }
+    if (g.k == L.n[2] - 1) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v.zp[e] = L.w3[5] * v.zm[e];
+      d0 += T(3) * L.wr[5] - T(1);
+    }
+  }
+  const int last = L.n[0] - 1 - 2 * g.q0 - g.s;  // twice the lane of the row's last cell, if even
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    T l = g.s ? v.c[e] : (e ? v.c[e ? e - 1 : 0] : v.xs);
+    T r = g.s ? (e < 3 ? v.c[e < 3 ? e + 1 : 3] : v.xs) : v.c[e];
+    T d = d0;
+    if (e == 0 && g.s == 0 && g.q0 == 0) {
+      l = L.w3[0] * r;
+      d += T(3) * L.wr[0] - T(1);
+    }
+    if (last == 2 * e) {
+      r = L.w3[1] * l;
+      d += T(3) * L.wr[1] - T(1);
+    }
+    sum[e] = ((l + r) + (v.ym[e] + v.yp[e])) + (v.zm[e] + v.zp[e]);
+    dg[e] = d;
+  }
+}
+// The same for a group away from the y and z walls in a full row, in a third
+// of the instructions: the group may touch one x wall, with its first lane
+// (s = 0) or its last one (s = 1), whose diagonal count is `de`.
+template <class T>
+__device__ __forceinline__ bool quad_inner(const RLev<T>& L, const QPos& g) {
+  return L.full && (unsigned)(g.j - 1) < (unsigned)(L.n[1] - 2) && (L.D == 2 || (unsigned)(g.k - 1) < (unsigned)(L.n[2] - 2));
+}
+template <class T>
+__device__ __forceinline__ void quad_load_in(const RLev<T>& L, const QPos& g, const T* xn, QNb<T>& v, bool& edge) {
+  const T* c = xn + 4 * g.t;
+  edge = g.s ? g.q0 + 4 == L.hx : g.q0 == 0;
+  ld4(c, v.c);
+  v.xs = c[edge ? 0 : (g.s ? 4 : -1)];
+  ld4(c - L.hx, v.ym);
+  ld4(c + L.hx, v.yp);
+  if (L.D == 3) {
+    const int sz = L.hx * L.n[1];
+    ld4(c - sz, v.zm);
+    ld4(c + sz, v.zp);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v.zm[e] = v.zp[e] = T(0);
+  }
+}
+template <class T>
+__device__ __forceinline__ void quad_sums_in(const RLev<T>& L, const QPos& g, const QNb<T>& v, bool edge, T sum[4]) {
+  const T ce = g.s ? v.c[3] : v.c[0];
+  const T xs = edge ? L.w3[g.s] * ce : v.xs;
+  const T o = xs + ce, a = v.c[0] + v.c[1], b = v.c[1] + v.c[2], d = v.c[2] + v.c[3];
+  const T h[4] = {g.s ? a : o, g.s ? b : a, g.s ? d : b, g.s ? o : d};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) sum[e] = (h[e] + (v.ym[e] + v.yp[e])) + (v.zm[e] + v.zp[e]);
+}
+
+template <class T>
+__device__ __forceinline__ T quad_inv(const RLev<T>& L, int p, T dg) {
+  return dg == T(2 * L.D) ? L.idg[p] : rcp_rn(dg + L.lh[p]);
+}
+
+// writes the lanes of `m` (byte masks) of a group
+template <class T>
+__device__ __forceinline__ void quad_store(T* dst, unsigned m, const T v[4]) {
+  if (m == 0xffffffffu) {
+    st4(dst, v);
+    return;
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if ((m >> (8 * e)) & 1u) dst[e] = v[e];
+}
+
+// one group of one phase: relaxed values written
+template <class T>
+__device__ __forceinline__ void quad_relax(const RLev<T>& L, const QPos& g, int p, unsigned m, QNb<T>& v, const T bb[4],
+                                           T* dst) {
+  T sum[4], dg[4], o[4];
+  quad_sums(L, g, v, sum, dg);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) o[e] = (L.h2e[p] * bb[e] + sum[e]) * quad_inv(L, p, dg[e]);
+  quad_store(dst + 4 * (long long)g.t, m, o);
+}
+
+template <class T>
+__device__ __forceinline__ void quad_relax_in(const RLev<T>& L, const QPos& g, int p, unsigned m, const QNb<T>& v,
+                                              bool edge, const T bb[4], T* dst) {
+  T sum[4], o[4];
+  quad_sums_in(L, g, v, edge, sum);
+  const T inv = L.idg[p], ie = edge ? L.ide[g.s][p] : inv;
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    o[e] = (L.h2e[p] * bb[e] + sum[e]) * (e == 0 ? (g.s ? inv : ie) : (e == 3 ? (g.s ? ie : inv) : inv));
+  quad_store(dst + 4 * (long long)g.t, m, o);
+}
+
+// buffers of a level after s sweeps
+__device__ __forceinline__ int rb_red(int s) { return (2 * s) % 3; }
+__device__ __forceinline__ int rb_black(int s) { return (2 * s + 1) % 3; }
+
+// the regular cells of one colour in sweep s (zero: the iterate is zero
+// before the sweep and not read)
+template <class T>
+__device__ __noinline__ void rb_dense(const RLev<T>& __restrict__ L, int colour, int s, bool zero, const RCtx& c) {
+  const int in = colour ? rb_red(s + 1) : rb_black(s);
+  const int out = colour ? rb_black(s + 1) : rb_red(s + 1);
+  const unsigned* fw = reinterpret_cast<const unsigned*>(L.f[colour]);
+  if (zero && colour == 0) {
+    for (int t = c.i0; t < L.nqt; t += c.st) {
+      const unsigned w = fw[t];
+      for (int p = 0; p < 2; ++p) {
+        const unsigned m = regular_mask(w, p);
+        if (!m) continue;
+        QPos g = quad_pos(L, t, 0);
+        QNb<T> v;
+        T bb[4], sum[4], dg[4], o[4];
+        ld4(L.b[p][0] + 4 * (long long)t, bb);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v.c[e] = v.ym[e] = v.yp[e] = v.zm[e] = v.zp[e] = T(0);
+        v.xs = T(0);
+        quad_sums(L, g, v, sum, dg);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[e] = L.h2e[p] * bb[e] * quad_inv(L, p, dg[e]);
+        quad_store(L.x[p][out] + 4 * (long long)t, m, o);
+      }
+    }
+    return;
+  }
+  // U groups per thread with all their loads issued first; the flags of the
+  // next ones are loaded one iteration ahead
+  constexpr int U = sizeof(T) == 4 ? 2 : 1;
+  unsigned wn[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) wn[u] = c.i0 + u * c.st < L.nqt ? fw[c.i0 + u * c.st] : 0u;
+  for (int t0 = c.i0; t0 < L.nqt; t0 += U * c.st) {
+    unsigned w[U], m[U];
+    int pp[U];
+    QPos g[U];
+    QNb<T> v[U];
+    T bb[U][4];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      w[u] = wn[u];
+      const int tn = t0 + (U + u) * c.st;
+      wn[u] = tn < L.nqt ? fw[tn] : 0u;
+    }
+    bool ed[U], in4[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      m[u] = regular_mask(w[u], 0);
+      pp[u] = m[u] ? 0 : 1;
+      if (!m[u]) m[u] = regular_mask(w[u], 1);
+      in4[u] = false;
+      if (!m[u]) continue;
+      g[u] = quad_pos(L, t0 + u * c.st, colour);
+      in4[u] = quad_inner(L, g[u]);
+      if (in4[u]) {
+        quad_load_in(L, g[u], L.x[pp[u]][in], v[u], ed[u]);
+        ld4(L.b[pp[u]][colour] + 4 * g[u].t, bb[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (!m[u]) continue;
+      if (in4[u]) {
+        quad_relax_in(L, g[u], pp[u], m[u], v[u], ed[u], bb[u], L.x[pp[u]][out]);
+      } else {
+        quad_load(L, g[u], L.x[pp[u]][in], v[u]);
+        ld4(L.b[pp[u]][colour] + 4 * (long long)g[u].t, bb[u]);
+        quad_relax(L, g[u], pp[u], m[u], v[u], bb[u], L.x[pp[u]][out]);
+      }
+      if (pp[u] == 0 && m[u] != 0xffffffffu && L.two) {  // lanes of the other phase
+        const unsigned m1 = regular_mask(w[u], 1);
+        if (m1) {
+          quad_load(L, g[u], L.x[1][in], v[u]);
+          ld4(L.b[1][colour] + 4 * (long long)g[u].t, bb[u]);
+          quad_relax(L, g[u], 1, m1, v[u], bb[u], L.x[1][out]);
+        }
+      }
+    }
+  }
+}
+
+// a value by its encoded cell (phase << 31 | colour * H + position)
+template <class T>
+struct Gather {
+  const T *r0, *b0, *r1, *b1;
+  unsigned H;
+  __device__ __forceinline__ T operator()(unsigned cl) const {
+    const unsigned s = cl & 0x7fffffffu;
+    const bool blk = s >= H;
+    const T* p = (cl >> 31) ? (blk ? b1 : r1) : (blk ? b0 : r0);
+    return p[blk ? s - H : s];
+  }
+};
+template <class T>
+__device__ __forceinline__ Gather<T> rb_gather(const RLev<T>& L, int red, int black) {
+  return Gather<T>{L.x[0][red], L.x[0][black], L.x[1][red], L.x[1][black], (unsigned)L.H};
+}
+template <class T>
+__device__ __forceinline__ T* rb_rhs(const RLev<T>& L, unsigned cl, unsigned& pos) {
+  const unsigned s = cl & 0x7fffffffu;
+  const int colour = s >= (unsigned)L.H;
+  pos = colour ? s - (unsigned)L.H : s;
+  return L.b[cl >> 31][colour];
+}
+
+// off-diagonal sum of a row by one thread, entries eight at a time
+template <class T, class V>
+__device__ __forceinline__ V row_sum1(const RLev<T>& L, int2 re, const Gather<T>& x, unsigned lim) {
+  V s = V(0);
+  const V* val = (const V*)L.val;
+  for (int e = re.x; e < re.y; e += 8) {
+    unsigned cl[8];
+    V a[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      cl[k] = 0xffffffffu;
+      a[k] = V(0);
+      if (e + k < re.y) {
+        cl[k] = L.col[e + k];
+        a[k] = val[e + k];
+      }
+    }
+    T xv[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) xv[k] = (e + k < re.y && (cl[k] & 0x7fffffffu) < lim) ? x(cl[k]) : T(0);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += a[k] * (V)xv[k];
+  }
+  return s;
+}
+
+// a lane's part (entries g, g + 8, ...) of the sum by a group of 8 lanes, all
+// loads of up to 48 entries of the row in flight at once
+template <class T, class V>
+__device__ __forceinline__ V row_sum8(const unsigned* __restrict__ col, const V* __restrict__ val, int2 re, int g,
+                                      const Gather<T>& x, unsigned lim) {
+  constexpr int RU = 6;
+  V s = V(0);
+  for (int e = re.x + g; e < re.y; e += 8 * RU) {
+    unsigned cl[RU];
+    V a[RU];
+    T xv[RU];
+#pragma unroll
+    for (int k = 0; k < RU; ++k) {
+      cl[k] = 0x7fffffffu;
+      a[k] = V(0);
+      if (e + 8 * k < re.y) {
+        cl[k] = col[e + 8 * k];
+        a[k] = val[e + 8 * k];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < RU; ++k) xv[k] = e + 8 * k < re.y && (cl[k] & 0x7fffffffu) < lim ? x(cl[k]) : T(0);
+#pragma unroll
+    for (int k = 0; k < RU; ++k) s += a[k] * (V)xv[k];
+  }
+  return s;
+}
+
+// The sparse rows of one colour in sweep s: the new values from the current
+// iterate, into the buffer the colour's regular cells are written to.  On
+// grid levels a group of 8 lanes takes a row (a row is a chain of dependent
+// loads, so rows in flight matter, not lanes per row), counted from the other
+// end of the grid than the regular cells so that small levels use different
+// warps for the two; the sum is in a fixed lane order.  Inside CTA 0 a thread
+// takes a row.
+template <class T, class V>
+__device__ __noinline__ void rb_rows_v(const RLev<T>& __restrict__ L, int colour, int s, bool zero, const RCtx& c) {
+  const int r0 = colour ? L.nr0 : 0, r1 = colour ? L.nr : L.nr0;
+  const int ired = colour ? rb_red(s + 1) : rb_red(s), iblk = rb_black(s);
+  const int out = colour ? rb_black(s + 1) : rb_red(s + 1);
+  const Gather<T> x = rb_gather(L, ired, iblk);
+  // zero: entries whose cells are still zero (all of them in the red pass, the black ones in the black pass)
+  const unsigned lim = zero ? (colour ? (unsigned)L.H : 0u) : 0x80000000u;
+  const V* dgp = (const V*)L.dinv;
+  if (c.local) {
+    for (int r = r0 + (int)threadIdx.x; r < r1; r += blockDim.x) {
+      const unsigned cl = L.rs[r];
+      unsigned pos;
+      const T* b = rb_rhs(L, cl, pos);
+      const V v = (V)b[pos] - (lim ? row_sum1<T, V>(L, L.re[r], x, lim) : V(0));
+      L.x[cl >> 31][out][pos] = (T)(v * dgp[r]);
+    }
+    return;
+  }
+  const int g = threadIdx.x & 7;
+  const unsigned gmask = 0xffu << (threadIdx.x & 24);
+  const V* val = (const V*)L.val;
+  const int rend = r0 + ((r1 - r0 + c.gst - 1) / c.gst) * c.gst;  // every lane of a warp runs the same trips
+  for (int r = r0 + c.g0; r < rend; r += c.gst) {
+    const bool live = r < r1;
+    const int2 re = live ? L.re[r] : make_int2(0, 0);
+    const unsigned cl = live ? L.rs[r] : 0u;
+    const V d = live ? dgp[r] : V(0);
+    unsigned pos = 0;
+    V bc = V(0), sum = V(0);
+    if (live) {
+      const T* b = rb_rhs(L, cl, pos);
+      bc = (V)b[pos];
+      if (lim) sum = row_sum8<T, V>(L.col, val, re, g, x, lim);
+    }
+    for (int off = 4; off > 0; off >>= 1) sum += __shfl_xor_sync(gmask, sum, off);
+    if (live && g == 0) L.x[cl >> 31][out][pos] = (T)((bc - sum) * d);
+  }
+}
+
+// one colour of sweep s
+template <class T>
+__device__ __forceinline__ void rb_pass(const RLev<T>& L, int colour, int s, bool zero, const RCtx& c) {
+  const int n = colour ? L.nr - L.nr0 : L.nr0;
+  if (n) {
+    if (L.staged) rb_rows_v<T, T>(L, colour, s, zero, c);
+    else rb_rows_v<T, double>(L, colour, s, zero, c);
+  }
+  if (L.dense) rb_dense(L, colour, s, zero, c);
+}
+
+// sweeps s0 .. s1 - 1 of level l; zero: the first one starts from a zero
+// iterate, which is not read
+template <class T>
+__device__ __noinline__ bool rb_smooth(const RLev<T>& L, int s0, int s1, bool zero, const RCtx& c, int l) {
+  for (int s = s0; s < s1; ++s)
+    for (int colour = 0; colour < 2; ++colour) {
+      rb_pass(L, colour, s, zero && s == s0, c);
+      if (!c.sync((l << 4) | (colour ? 3 : 1))) return false;
+    }
+  return true;
+}
+
+// zero iterate (V-cycles without pre-smoothing)
+template <class T>
+__device__ __noinline__ bool rb_zero(const RLev<T>& __restrict__ L, const RCtx& c, int l) {
+  const T z[4] = {T(0), T(0), T(0), T(0)};
+  for (int t = c.i0; t < L.nqt; t += c.st) {
+    const unsigned w = reinterpret_cast<const unsigned*>(L.f[0])[t] | reinterpret_cast<const unsigned*>(L.f[1])[t];
+    for (int p = 0; p < 2; ++p)
+      if (w & (p ? 0x02020202u : 0x01010101u)) {
+        st4(L.x[p][rb_red(0)] + 4 * (long long)t, z);
+        st4(L.x[p][rb_black(0)] + 4 * (long long)t, z);
+      }
+  }
+  return c.sync((l << 4) | 12);
+}
+
+// residual of a single regular cell (a child of a special coarse cell)
+template <class T>
+__device__ __noinline__ T cell_res(const RLev<T>& L, int p, int i, int j, int k, int red, int black) {
+  const int colour = (i + j + k) & 1;
+  const long long pos = (i >> 1) + (long long)L.hx * (j + (long long)L.n[1] * k);
+  const T* xn = L.x[p][colour ? red : black];
+  const T xc = L.x[p][colour ? black : red][pos];
+  const int I[3] = {i, j, k};
+  T sum = T(0), dg = T(0);
+  for (int a = 0; a < L.D; ++a) {
+    // in the other colour's half the x neighbours are at (i -+ 1) >> 1, the others a row or a plane away
+    const long long lo = a == 0 ? pos - (i >> 1) + ((i - 1) >> 1) : pos - (a == 1 ? L.hx : (long long)L.hx * L.n[1]);
+    const long long hi = a == 0 ? pos - (i >> 1) + ((i + 1) >> 1) : pos + (a == 1 ? L.hx : (long long)L.hx * L.n[1]);
+    if (I[a] > 0) {
+      sum += xn[lo];
+      dg += T(1);
+    } else {
+      sum += L.w3[2 * a] * xn[hi];
+      dg += T(3) * L.wr[2 * a];
+    }
+    if (I[a] < L.n[a] - 1) {
+      sum += xn[hi];
+      dg += T(1);
+    } else {
+      sum += L.w3[2 * a + 1] * xn[lo];
+      dg += T(3) * L.wr[2 * a + 1];
+    }
+  }
+  return L.b[p][colour][pos] - L.ceps[p] * ((dg + L.lh[p]) * xc - sum);
+}
+
+// The special coarse cells: a group of 8 lanes each, a lane per child (2D: and
+// phase) for the regular children and all lanes together for each child's row.
+template <class T, class V>
+__device__ __noinline__ void rb_restrict_special(const RLev<T>& __restrict__ F, const RLev<T>& __restrict__ C, int s,
+                                                 bool full, const RCtx& c) {
+  const int red = rb_red(s), black = rb_black(s);
+  const Gather<T> x = rb_gather(F, red, black);
+  const int lane = threadIdx.x & 7, nch = 1 << F.D;
+  const int shift = threadIdx.x & 24;
+  const unsigned gmask = 0xffu << shift;
+  const T scale = T(1) / T(nch);
+  const V* dgp = (const V*)F.diag;
+  const V* val = (const V*)F.val;
+  const int nend = ((F.nsp + c.gst - 1) / c.gst) * c.gst;
+  for (int q = c.g0; q < nend; q += c.gst) {
+    const bool live = q < F.nsp;
+    const unsigned cc = live ? (unsigned)F.sp[q] : 0u;
+    const int I = (int)(cc % (unsigned)C.n[0]), rowc = (int)(cc / (unsigned)C.n[0]);
+    const int J = rowc % C.n[1], K = rowc / C.n[1];
+    V acc[2] = {V(0), V(0)};
+    if (live)
+      for (int h = 0; h < (F.D == 3 ? 2 : 1); ++h) {
+        const int slot = lane + 8 * h, ch = slot & (nch - 1), p = slot >> F.D;
+        if (F.D == 3 && h && !F.two) break;  // the dielectric's slots
+        const int r = F.sprow[(long long)q * 2 * nch + slot];
+        int2 re = make_int2(0, 0);
+        unsigned cl = 0;
+        V d = V(0);
+        if (r >= 0) {
+          re = F.re[r];
+          cl = F.rs[r];
+          d = dgp[r];
+        } else if (!p || F.two) {
+          const int i = 2 * I + (ch & 1), j = 2 * J + ((ch >> 1) & 1), k = F.D == 3 ? 2 * K + (ch >> 2) : 0;
+          if (i < F.n[0] && j < F.n[1] && k < F.n[2] && (full || !((i + j + k) & 1))) {
+            const long long pos = (i >> 1) + (long long)F.hx * (j + (long long)F.n[1] * k);
+            if ((F.f[(i + j + k) & 1][pos] & 7u) == (1u << p)) acc[p] += (V)cell_res(F, p, i, j, k, red, black);
+          }
+        }
+        unsigned rows = (__ballot_sync(gmask, r >= 0) >> shift) & 0xffu;
+        while (rows) {
+          const int src = __ffs(rows) - 1;
+          rows &= rows - 1;
+          const int2 e = make_int2(__shfl_sync(gmask, re.x, src, 8), __shfl_sync(gmask, re.y, src, 8));
+          const V part = row_sum8<T, V>(F.col, val, e, lane, x, 0x80000000u);
+          // the group's parts are summed with everything else below
+          const int ps = F.D == 3 ? h : src >> 2;
+          if (ps) acc[1] -= part;
+          else acc[0] -= part;
+        }
+        if (r >= 0) {
+          unsigned pos;
+          const T* b = rb_rhs(F, cl, pos);
+          const V v = (V)b[pos] - d * (V)x(cl);
+          if (p) acc[1] += v;
+          else acc[0] += v;
+        }
+      }
+    for (int off = 4; off > 0; off >>= 1)
+      for (int p = 0; p < 2; ++p) acc[p] += __shfl_xor_sync(gmask, acc[p], off);
+    if (live && lane == 0) {
+      const int colour = (I + J + K) & 1;
+      const long long pos = (I >> 1) + (long long)C.hx * (J + (long long)C.n[1] * K);
+      const unsigned fl = C.f[colour][pos];
+      if (fl & 1u) C.b[0][colour][pos] = (T)acc[0] * scale;
+      if (fl & 2u) C.b[1][colour][pos] = (T)acc[1] * scale;
+    }
+  }
+}
+
+// Residual of F after s sweeps, averaged over the children into C's
+// right-hand side: four coarse cells per item, whose children of one colour
+// are the groups at the same position of the fine rows.  full: black
+// residuals too (no sweep has solved them).
+template <class T>
+__device__ __noinline__ void rb_restrict(const RLev<T>& __restrict__ F, const RLev<T>& __restrict__ C, int s, bool full, const RCtx& c) {
+  if (F.nsp) {
+    if (F.staged) rb_restrict_special<T, T>(F, C, s, full, c);
+    else rb_restrict_special<T, double>(F, C, s, full, c);
+  }
+  if (!F.dense) return;
+  const int rows = C.n[1] * C.n[2], items = rows * F.nq;
+  const T scale = T(1) / T(1 << F.D);
+  const unsigned* fr = reinterpret_cast<const unsigned*>(F.f[0]);
+  const T *xr = F.x[0][rb_red(s)], *xb = F.x[0][rb_black(s)];
+  for (int it = c.i0; it < items; it += c.st) {
+    const unsigned rc = fdiv((unsigned)it, F.dq);
+    const int g = it - (int)rc * F.nq;
+    const unsigned K = fdiv(rc, C.dn1);
+    const int J = (int)(rc - K * (unsigned)C.n[1]);
+    // coarse flags: cells 4g, 4g + 2 of one colour, 4g + 1, 4g + 3 of the other
+    const int ce = (J + (int)K) & 1;
+    const long long cp = (long long)rc * C.hx + 2 * g;
+    const unsigned short fe = *reinterpret_cast<const unsigned short*>(C.f[ce] + cp);
+    const unsigned short fo = *reinterpret_cast<const unsigned short*>(C.f[ce ^ 1] + cp);
+    if (!((fe | fo) & 0x0303u)) continue;
+    const int t00 = (2 * J + (F.D == 3 ? F.n[1] * 2 * (int)K : 0)) * F.nq + g;
+    bool inner = F.full && !full && J > 0 && 2 * J + 2 < F.n[1] && (F.D == 2 || ((int)K > 0 && 2 * (int)K + 2 < F.n[2]));
+    if (inner) {
+      unsigned all = fr[t00] ^ 0x01010101u;
+      all |= fr[t00 + F.nq] ^ 0x01010101u;
+      if (F.D == 3) all |= (fr[t00 + F.nq * F.n[1]] ^ 0x01010101u) | (fr[t00 + F.nq * (F.n[1] + 1)] ^ 0x01010101u);
+      inner = !(all & R_BASE);
+    }
+    for (int p = 0; p <= F.two; ++p) {
+      const unsigned pm = 0x0101u << p;
+      if (!((fe | fo) & pm)) continue;
+      T acc[4] = {T(0), T(0), T(0), T(0)};
+      if (inner && p == 0) {
+        // all children regular gas away from the y and z walls: two rows' loads at a time
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          if (hh && F.D == 2) continue;
+          QNb<T> v[2];
+          T bb[2][4], xo[2][4];
+          bool ed[2];
+          QPos q[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int t = t00 + u * F.nq + hh * F.nq * F.n[1];
+            q[u] = QPos{t, 2 * J + u, F.D == 3 ? 2 * (int)K + hh : 0, 4 * g, (u + hh) & 1};
+            quad_load_in(F, q[u], xb, v[u], ed[u]);
+            ld4(xr + 4 * t, xo[u]);
+            ld4(F.b[0][0] + 4 * t, bb[u]);
+          }
+          const T d = T(2 * F.D) + F.lh[0];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            T sum[4];
+            quad_sums_in(F, q[u], v[u], ed[u], sum);
+            const T de = ed[u] ? F.dge[q[u].s] + F.lh[0] : d;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const T de4 = e == 0 ? (q[u].s ? d : de) : (e == 3 ? (q[u].s ? de : d) : d);
+              acc[e] += bb[u][e] - F.ceps[0] * (de4 * xo[u][e] - sum[e]);
+            }
+          }
+        }
+      } else
+      for (int h = 0; h < (F.D == 3 ? 4 : 2); ++h) {
+        const int j = 2 * J + (h & 1), k = F.D == 3 ? 2 * (int)K + (h >> 1) : 0;
+        if (j >= F.n[1] || k >= F.n[2]) continue;
+        const int t = (j + F.n[1] * k) * F.nq + g;
+        for (int colour = 0; colour <= (full ? 1 : 0); ++colour) {
+          const unsigned m = regular_mask(reinterpret_cast<const unsigned*>(F.f[colour])[t], p);
+          if (!m) continue;
+          const QPos q{t, j, k, 4 * g, (j + k + colour) & 1};
+          QNb<T> v;
+          T bb[4], xo[4], sum[4], dg[4];
+          quad_load(F, q, F.x[p][colour ? rb_red(s) : rb_black(s)], v);
+          ld4(F.x[p][colour ? rb_black(s) : rb_red(s)] + 4 * (long long)t, xo);
+          ld4(F.b[p][colour] + 4 * (long long)t, bb);
+          quad_sums(F, q, v, sum, dg);
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if ((m >> (8 * e)) & 1u) acc[e] += bb[e] - F.ceps[p] * ((dg[e] + F.lh[p]) * xo[e] - sum[e]);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const unsigned f = ((e & 1) ? fo : fe) >> (8 * (e >> 1));
+        if (((f >> p) & 1u) && !(f & R_SPC)) C.b[p][(e & 1) ? ce ^ 1 : ce][cp + (e >> 1)] = acc[e] * scale;
+      }
+    }
+  }
+}
+
+// x += P e: (bi/tri)linear where every coarse cell of the interpolation has an
+// unknown of the phase, the value of the cell above elsewhere (0 where that
+// one has none).  An item is the eight cells of one position of a fine row,
+// both colours; sF, sC: the sweeps done on the two levels.
+template <class T>
+__device__ __noinline__ void rb_prolong(const RLev<T>& __restrict__ F, const RLev<T>& __restrict__ C, int sF, int sC, const RCtx& c) {
+  const int cr = rb_red(sC), cb = rb_black(sC);
+  const unsigned *f0 = reinterpret_cast<const unsigned*>(F.f[0]), *f1 = reinterpret_cast<const unsigned*>(F.f[1]);
+  unsigned n0 = c.i0 < F.nqt ? f0[c.i0] : 0u, n1 = c.i0 < F.nqt ? f1[c.i0] : 0u;  // flags one item ahead
+  for (int t = c.i0; t < F.nqt; t += c.st) {
+    const unsigned w0 = n0, w1 = n1;
+    if (t + c.st < F.nqt) {
+      n0 = f0[t + c.st];
+      n1 = f1[t + c.st];
+    }
+    if (!((w0 | w1) & 0x03030303u)) continue;
+    const QPos g = quad_pos(F, t, 0);  // red cells at i = 2 q + s
+    const unsigned we = g.s ? w1 : w0, wo = g.s ? w0 : w1;  // flags of the even and the odd cells
+    const int J = g.j >> 1, K = g.k >> 1;
+    const int J2 = min(max(J + ((g.j & 1) ? 1 : -1), 0), C.n[1] - 1);
+    const int K2 = min(max(K + ((g.k & 1) ? 1 : -1), 0), C.n[2] - 1);
+    for (int p = 0; p <= F.two; ++p) {
+      const unsigned pm = 0x01010101u << p;
+      if (!((w0 | w1) & pm)) continue;
+      T cs[6] = {T(0), T(0), T(0), T(0), T(0), T(0)}, home[4] = {T(0), T(0), T(0), T(0)};
+      T *xe = F.x[p][g.s ? rb_black(sF) : rb_red(sF)] + 4 * (long long)t;
+      T *xo = F.x[p][g.s ? rb_red(sF) : rb_black(sF)] + 4 * (long long)t;
+      T ve[4], vo[4], a[4][6];
+      ld4(xe, ve);
+      ld4(xo, vo);
+      // a neighbour outside the grid is replaced by the cell itself: no lane
+      // that is interpolated linearly uses it, and every load goes out at once
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (h >= 2 && F.D == 2) continue;
+        const int j = (h & 1) ? J2 : J, k = (h & 2) ? K2 : K;
+        const int par = (j + k) & 1;  // colour of the coarse cells at even I
+        const T* ae = C.x[p][par ? cb : cr];
+        const T* ao = C.x[p][par ? cr : cb];
+        const int cp = C.hx * (j + C.n[1] * k) + (g.q0 >> 1);
+        ld2(ae + cp, a[h][1], a[h][3]);
+        ld2(ao + cp, a[h][2], a[h][4]);
+        a[h][0] = ao[g.q0 > 0 ? cp - 1 : cp];
+        a[h][5] = ae[g.q0 + 4 < C.n[0] ? cp + 2 : cp];
+      }
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (h >= 2 && F.D == 2) continue;
+        const T wgt = ((h & 1) ? T(0.25) : T(0.75)) * (F.D == 3 ? ((h & 2) ? T(0.25) : T(0.75)) : T(1));
+#pragma unroll
+        for (int e = 0; e < 6; ++e) cs[e] += wgt * a[h][e];
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) home[e] = a[0][e + 1];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const unsigned a = we >> (8 * e), b = wo >> (8 * e);
+        const T le = T(0.75) * cs[e + 1] + T(0.25) * cs[e], lo = T(0.75) * cs[e + 1] + T(0.25) * cs[e + 2];
+        const T he = (a & (R_NOHOME0 << p)) ? T(0) : home[e], ho = (b & (R_NOHOME0 << p)) ? T(0) : home[e];
+        if ((a >> p) & 1u) ve[e] += (a & (R_LIN0 << p)) ? le : he;
+        if ((b >> p) & 1u) vo[e] += (b & (R_LIN0 << p)) ? lo : ho;
+      }
+      st4(xe, ve);
+      st4(xo, vo);
+    }
+  }
+}
+
+// x = binv b on the bottom level: a warp per row, lanes over the columns
+template <class T>
+__device__ __noinline__ void rb_inverse(const RHier<T>& __restrict__ H, const RLev<T>& __restrict__ L, const RCtx& c) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int w0 = c.local ? (int)(threadIdx.x >> 5) : (int)(threadIdx.x >> 5) * c.gsize + c.gcta;
+  const int ws = c.local ? nw : nw * c.gsize;
+  for (int i = w0; i < H.bm; i += ws) {
+    const unsigned si = H.bslot[i];
+    if (si == 0xffffffffu) continue;
+    const T* row = H.binv + (long long)i * H.bm;
+    T acc = T(0);
+    for (int j = lane; j < H.bm; j += 32) {
+      const unsigned sj = H.bslot[j];
+      if (sj == 0xffffffffu) continue;
+      unsigned pos;
+      const T* b = rb_rhs(L, sj, pos);
+      acc += row[j] * b[pos];
+    }
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    if (lane == 0) {
+      const unsigned s = si & 0x7fffffffu;
+      const int colour = s >= (unsigned)L.H;
+      L.x[si >> 31][colour ? rb_black(0) : rb_red(0)][colour ? s - (unsigned)L.H : s] = acc;
+    }
+  }
+}
+
+// BiCGStab on a bottom level of at most 32 rows by one warp, a lane per row,
+// from zero until |r| <= 1e-4 |b| (2-norms) or 16 iterations; vectors in
+// registers, matrix-vector products through the level's own arrays.
+template <class T, class V>
+__device__ __noinline__ void rb_bicgstab_v(const RLev<T>& L) {
+  const int lane = threadIdx.x & 31;
+  const bool live = lane < L.nr;
+  const unsigned cl = live ? L.rs[lane] : 0u;
+  const int2 re = live ? L.re[lane] : make_int2(0, 0);
+  const T d = live ? (T)((const V*)L.diag)[lane] : T(1);
+  unsigned pos;
+  const T* bp = rb_rhs(L, cl, pos);
+  const bool blk = (cl & 0x7fffffffu) >= (unsigned)L.H;
+  T* slot = L.x[cl >> 31][blk ? rb_black(0) : rb_red(0)] + pos;
+  const Gather<T> x = rb_gather(L, rb_red(0), rb_black(0));
+  auto dot = [](T a, T b) {
+    T v = a * b;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  auto mul = [&](T y) {
+    __syncwarp();
+    if (live) *slot = y;
+    __syncwarp();
+    return live ? (T)(d * y + (T)row_sum1<T, V>(L, re, x, 0x80000000u)) : T(0);
+  };
+  const T b = live ? *bp : T(0);
+  T r = b, pv = T(0), v = T(0), sol = T(0);
+  const T r0 = b, bb = dot(b, b);
+  T rho = T(1), alpha = T(1), omega = T(1);
+  for (int it = 0; it < 16 && bb > T(0); ++it) {
+    const T rho1 = dot(r0, r);
+    if (rho1 == T(0) || omega == T(0)) break;
+    pv = r + (rho1 / rho) * (alpha / omega) * (pv - omega * v);
+    rho = rho1;
+    // diagonal scaling: the cells' coefficients differ by the permittivities and cut fractions
+    const T ph = pv / d;
+    v = mul(ph);
+    const T rv = dot(r0, v);
+    if (rv == T(0)) break;
+    alpha = rho / rv;
+    const T sv = r - alpha * v;
+    const T sh = sv / d;
+    const T t = mul(sh);
+    const T tt = dot(t, t);
+    omega = tt > T(0) ? dot(t, sv) / tt : T(0);
+    sol += alpha * ph + omega * sh;
+    r = sv - omega * t;
+    if (dot(r, r) <= T(1e-8) * bb) break;
+  }
+  __syncwarp();
+  if (live) *slot = sol;
+}
+
+// sweeps done on a level when its correction is taken up by the finer one
+template <class T>
+__device__ __forceinline__ int rb_done(const RHier<T>& H, int l) {
+  return l < H.nlev - 1 ? H.nu1[l] + H.nu2[l] : (H.bot ? 0 : H.bsweeps);
+}
+
+// level L (index l) down to N, the next one, and back up
+template <class T>
+__device__ __noinline__ bool rb_down(const RHier<T>& H, const RLev<T>& L, const RLev<T>& N, int l, const RCtx& c) {
+  const int nu = H.nu1[l];
+  if (nu == 0) {
+    if (!rb_zero(L, c, l)) return false;
+  } else if (!rb_smooth(L, 0, nu, true, c, l)) {
+    return false;
+  }
+  rb_restrict(L, N, nu, nu == 0, c);
+  return c.sync((l << 4) | 6);
+}
+template <class T>
+__device__ __noinline__ bool rb_up(const RHier<T>& H, const RLev<T>& L, const RLev<T>& N, int l, const RCtx& c) {
+  const int nu = H.nu1[l];
+  rb_prolong(L, N, nu, rb_done(H, l + 1), c);
+  if (!c.sync((l << 4) | 7)) return false;
+  return rb_smooth(L, nu, nu + H.nu2[l], false, c, l);
+}
+
+__device__ __forceinline__ void copy_words(void* dst, const void* src, long long bytes) {
+  const int* s = (const int*)src;
+  int* d = (int*)dst;
+  for (long long i = threadIdx.x; i < bytes / 4; i += blockDim.x) d[i] = s[i];
+}
+
+// levels lc.. inside CTA 0; g: level lc as the grid sees it
+template <class T>
+__device__ __noinline__ void rb_coarse(const RHier<T>& H, const RLev<T>& g, const RCtx& c) {
+  const int lc = H.lc;
+  if (H.smem) {
+    const RLev<T>& s = H.L[lc];
+    for (int p = 0; p <= s.two; ++p) {
+      const int o = p ? s.p1o : 0, n = p ? s.p1n : s.H;
+      for (int q = 0; q < 2; ++q) copy_words(s.b[p][q] + o, g.b[p][q] + o, (long long)n * sizeof(T));
+    }
+    __syncthreads();
+  }
+  for (int l = lc; l < H.nlev - 1; ++l) rb_down(H, H.L[l], H.L[l + 1], l, c);
+  const RLev<T>& B = H.L[H.nlev - 1];
+  if (H.bot == 0) {
+    rb_smooth(B, 0, H.bsweeps, true, c, H.nlev - 1);
+  } else {
+    if (H.bot == 1) rb_inverse(H, B, c);
+    else if (threadIdx.x < 32) {
+      if (B.staged) rb_bicgstab_v<T, T>(B);
+      else rb_bicgstab_v<T, double>(B);
+    }
+    c.sync(((H.nlev - 1) << 4) | 9);
+  }
+  for (int l = H.nlev - 2; l >= lc; --l) rb_up(H, H.L[l], H.L[l + 1], l, c);
+  if (H.smem) {
+    const RLev<T>& s = H.L[lc];
+    const int d = rb_done(H, lc);
+    for (int p = 0; p <= s.two; ++p) {
+      const int o = p ? s.p1o : 0, n = p ? s.p1n : s.H;
+      copy_words(g.x[p][rb_red(d)] + o, s.x[p][rb_red(d)] + o, (long long)n * sizeof(T));
+      copy_words(g.x[p][rb_black(d)] + o, s.x[p][rb_black(d)] + o, (long long)n * sizeof(T));
+    }
+  }
+}
+
+// one V-cycle from zero: level 0's right-hand side in its b, the result in
+// its x after rb_done(H, 0) sweeps; gl: level lc as the grid sees it (in CTA
+// 0 the entry H.L[lc] points into shared memory)
+template <class T>
+__device__ __noinline__ bool rb_vcycle(const RHier<T>& H, const RLev<T>& gl, const RCtx& G) {
+  for (int l = 0; l < H.lc; ++l)
+    if (!rb_down(H, H.L[l], l + 1 == H.lc ? gl : H.L[l + 1], l, G)) return false;
+  if (H.bot == 1 && !H.smem) {  // the inverse applied by the whole grid
+    rb_inverse(H, gl, G);
+    if (!G.sync(((H.nlev - 1) << 4) | 9)) return false;
+  } else {
+    if (G.gcta == 0) {
+      RCtx L = G;
+      L.local = true;
+      L.i0 = (int)threadIdx.x;
+      L.st = (int)blockDim.x;
+      L.g0 = (int)(threadIdx.x >> 3);
+      L.gst = (int)(blockDim.x >> 3);
+      rb_coarse(H, gl, L);
+    }
+    if (!G.sync((15 << 4) | 8)) return false;
+  }
+  for (int l = H.lc - 1; l >= 0; --l)
+    if (!rb_up(H, H.L[l], l + 1 == H.lc ? gl : H.L[l + 1], l, G)) return false;
+  return true;
+}
+
+// ------------------------------------------------------------ the FP64 outer loop
+
+// max over non-negative doubles by their bit patterns (NaN passed over, as fmax does)
+__device__ __forceinline__ void bits_max(unsigned long long& m, double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  if (b > m && b <= 0x7ff0000000000000ull) m = b;
+}
+
+// FP64 residual of the finest level into level 0's right-hand side (rounded
+// to T) and its max norm; eight cells of an x row per item, seven FP64
+// operations each (GB300 issues about two FP64 operations per clock and SM,
+// which bounds the pass from 256^2 cells up).
+template <class T>
+__device__ __noinline__ bool rb_resid64(const RHier<T>& __restrict__ H, const RLev<T>& __restrict__ L, const Op<double>& __restrict__ F, unsigned long long* norm,
+                           const RCtx& G) {
+  unsigned long long mx = 0ull;
+  {
+    const int g = threadIdx.x & 7;
+    const unsigned gmask = 0xffu << (threadIdx.x & 24);
+    const int rend = ((L.nr + G.gst - 1) / G.gst) * G.gst;
+    for (int r = G.g0; r < rend; r += G.gst) {
+      const bool live = r < L.nr;
+      const int2 re = live ? L.re[r] : make_int2(0, 0);
+      const unsigned cl = live ? L.rs[r] : 0u;
+      const int p = (int)(cl >> 31);
+      double s = 0.0, bc = 0.0, xc = 0.0, d = 0.0;
+      if (live) {
+        const int c = H.rnat[r];
+        d = H.rdiag[r];
+        bc = F.b[p][c];
+        xc = F.x[p][c];
+        for (int e = re.x + g; e < re.y; e += 32) {
+          unsigned ce[4];
+          double a[4], xv[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            ce[k] = 0u;
+            a[k] = 0.0;
+            if (e + 8 * k < re.y) {
+              ce[k] = (unsigned)H.ncol[e + 8 * k];
+              a[k] = H.rval[e + 8 * k];
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < 4; ++k) xv[k] = e + 8 * k < re.y ? F.x[ce[k] >> 30][ce[k] & 0x3fffffffu] : 0.0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) s += a[k] * xv[k];
+        }
+      }
+      for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(gmask, s, off);
+      if (live && g == 0) {
+        const double v = (bc - s) - d * xc;
+        unsigned pos;
+        T* b = rb_rhs(L, cl, pos);
+        b[pos] = (T)v;
+        bits_max(mx, v);
+      }
+    }
+  }
+  const int n0 = F.n[0], n1 = F.n[1], n2 = F.D == 3 ? F.n[2] : 1;
+  const long long sy = n0, sz = (long long)n0 * n1;
+  for (int t = G.i0; t < L.nqt; t += G.st) {
+    const unsigned w0 = reinterpret_cast<const unsigned*>(L.f[0])[t], w1 = reinterpret_cast<const unsigned*>(L.f[1])[t];
+    if (!((w0 | w1) & 0x03030303u)) continue;
+    const QPos g = quad_pos(L, t, 0);
+    const unsigned we = g.s ? w1 : w0, wo = g.s ? w0 : w1;
+    const long long nb = ((long long)g.j + (long long)n1 * g.k) * n0 + 2 * g.q0;
+    for (int p = 0; p <= L.two; ++p) {
+      const unsigned me = regular_mask(we, p), mo = regular_mask(wo, p);
+      if (!(me | mo)) continue;
+      const double* x = F.x[p] + nb;
+      double c[8], s[8];
+      ld4(x, c);
+      ld4(x + 4, c + 4);
+      const double xl = g.q0 > 0 ? x[-1] : F.w3[0] * c[1];
+      const double xr = 2 * g.q0 + 8 < n0 ? x[8] : F.w3[1] * c[6];
+      double d0 = (double)(2 * F.D) + F.lh[p];
+      double dl = d0, dr = d0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s[e] = (e ? c[e ? e - 1 : 0] : xl) + (e < 7 ? c[e < 7 ? e + 1 : 7] : xr);
+      double wd = 0.0;
+      for (int a = 1; a < F.D; ++a) {
+        const long long st = a == 1 ? sy : sz;
+        const int i = a == 1 ? g.j : g.k, n = a == 1 ? n1 : n2;
+        double u[8], v[8];
+        if (i > 0) {
+          ld4(x - st, u);
+          ld4(x - st + 4, u + 4);
+        }
+        if (i < n - 1) {
+          ld4(x + st, v);
+          ld4(x + st + 4, v + 4);
+        }
+        if (i == 0) {
+          wd += 3.0 * F.wr[2 * a] - 1.0;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) u[e] = F.w3[2 * a] * v[e];
+        }
+        if (i == n - 1) {
+          wd += 3.0 * F.wr[2 * a + 1] - 1.0;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[e] = F.w3[2 * a + 1] * u[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] += u[e] + v[e];
+      }
+      if (wd != 0.0) d0 += wd;
+      dl = g.q0 > 0 ? d0 : d0 + 3.0 * F.wr[0] - 1.0;
+      dr = 2 * g.q0 + 8 < n0 ? d0 : d0 + 3.0 * F.wr[1] - 1.0;
+      double bb[8];
+      ld4(F.b[p] + nb, bb);
+      ld4(F.b[p] + nb + 4, bb + 4);
+      T oe[4], oo[4];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const double dg = e == 0 ? dl : (e == 7 ? dr : d0);
+        const double r = bb[e] - F.ceps[p] * (dg * c[e] - s[e]);
+        if (e & 1) oo[e >> 1] = (T)r;
+        else oe[e >> 1] = (T)r;
+        if (((e & 1) ? mo : me) >> (8 * (e >> 1)) & 1u) bits_max(mx, r);
+      }
+      quad_store(L.b[p][g.s] + 4 * (long long)t, me, oe);
+      quad_store(L.b[p][g.s ^ 1] + 4 * (long long)t, mo, oo);
+    }
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
+    mx = o > mx ? o : mx;
+  }
+  if ((threadIdx.x & 31) == 0 && mx) atomicMax(norm, mx);
+  return G.sync((14 << 4) | 11);
+}
+
+// Krylov pass 1: q = A z of the V-cycle's result z (level 0 after sZ sweeps)
+// into slot `slot`, and the partial sums of (r, q), (q, q) and, for the m
+// directions before it, (q, q_i) and (r, q_i).  The sums' chunks depend on the level alone, not
+// on the CTAs that take them, so a solve's results do not depend on its group.
+template <class T>
+__device__ __noinline__ void rb_kry1(const RHier<T>& __restrict__ H, const RLev<T>& __restrict__ L, int sZ, int slot, int m, const RCtx& G, T (*red)[KDOT]) {
+  const int ir = rb_red(sZ), ib = rb_black(sZ);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int os[KH];
+#pragma unroll
+  for (int i = 0; i < KH - 1; ++i) os[i] = (slot + KH - 1 - i) % KH;
+  const Gather<T> x = rb_gather(L, ir, ib);
+  for (int ch = G.gcta; ch < H.kch; ch += G.gsize) {
+    T acc[KDOT];
+#pragma unroll
+    for (int d = 0; d < KDOT; ++d) acc[d] = T(0);
+    // the chunk's share of the sparse rows, a group of 8 lanes each
+    {
+      const int g = threadIdx.x & 7;
+      const unsigned gmask = 0xffu << (threadIdx.x & 24);
+      const int r1 = min((ch + 1) * H.krows, L.nr), ng = (int)(blockDim.x >> 3);
+      for (int r0 = ch * H.krows; r0 < r1; r0 += ng) {
+        const int r = r0 + (int)(threadIdx.x >> 3);
+        const bool live = r < r1;
+        const int2 re = live ? L.re[r] : make_int2(0, 0);
+        const unsigned cl = live ? L.rs[r] : 0u;
+        double s = row_sum8<T, double>(L.col, H.rval, re, g, x, 0x80000000u);
+        for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(gmask, s, off);
+        if (live && g == 0) {
+          unsigned pos;
+          const T* b = rb_rhs(L, cl, pos);
+          const int colour = (cl & 0x7fffffffu) >= (unsigned)L.H, p = (int)(cl >> 31);
+          const T q = (T)(s + H.rdiag[r] * (double)x(cl));
+          H.kq[slot][p][colour][pos] = q;
+          const T rv = b[pos];
+          acc[0] += rv * q;
+          acc[1] += q * q;
+#pragma unroll
+          for (int i = 0; i < KH - 1; ++i)
+            if (i < m) {
+              const T qi = H.kq[os[i]][p][colour][pos];
+              acc[2 + i] += q * qi;
+              acc[KH + 1 + i] += rv * qi;
+            }
+        }
+      }
+    }
+    const int t1 = min((ch + 1) * H.kcs, L.nqt);
+    for (int t = ch * H.kcs + (int)threadIdx.x; t < t1; t += (int)blockDim.x) {
+      const unsigned w[2] = {reinterpret_cast<const unsigned*>(L.f[0])[t], reinterpret_cast<const unsigned*>(L.f[1])[t]};
+      for (int p = 0; p <= L.two; ++p)
+#pragma unroll
+        for (int colour = 0; colour < 2; ++colour) {
+          const unsigned mk = regular_mask(w[colour], p);
+          if (!mk) continue;
+          const QPos g = quad_pos(L, t, colour);
+          QNb<T> v;
+          T xo[4], sum[4], dg[4], q[4], rr[4];
+          T qi[KH - 1][4];
+          const bool in = quad_inner(L, g);
+          bool ed = false;
+          if (in) quad_load_in(L, g, L.x[p][colour ? ir : ib], v, ed);
+          ld4(L.x[p][colour ? ib : ir] + 4 * (long long)t, xo);
+          ld4(L.b[p][colour] + 4 * (long long)t, rr);
+#pragma unroll
+          for (int i = 0; i < KH - 1; ++i)
+            if (i < m) ld4(H.kq[os[i]][p][colour] + 4 * (long long)t, qi[i]);
+          if (in) {
+            quad_sums_in(L, g, v, ed, sum);
+            const T d = T(2 * L.D), de = ed ? L.dge[g.s] : d;
+            dg[0] = g.s ? d : de;
+            dg[1] = dg[2] = d;
+            dg[3] = g.s ? de : d;
+          } else {
+            quad_load(L, g, L.x[p][colour ? ir : ib], v);
+            quad_sums(L, g, v, sum, dg);
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            q[e] = L.ceps[p] * ((dg[e] + L.lh[p]) * xo[e] - sum[e]);
+            if (!((mk >> (8 * e)) & 1u)) continue;
+            acc[0] += rr[e] * q[e];
+            acc[1] += q[e] * q[e];
+#pragma unroll
+            for (int i = 0; i < KH - 1; ++i)
+              if (i < m) {
+                acc[2 + i] += q[e] * qi[i][e];
+                acc[KH + 1 + i] += rr[e] * qi[i][e];
+              }
+          }
+          quad_store(H.kq[slot][p][colour] + 4 * (long long)t, mk, q);
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < KDOT; ++d) {
+      T a = acc[d];
+      for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+      if (lane == 0) red[wid][d] = a;
+    }
+    __syncthreads();
+    if (threadIdx.x < KDOT) {
+      double t = 0.0;
+      for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += (double)red[k][threadIdx.x];
+      H.kpart[(long long)ch * KDOT + threadIdx.x] = t;
+    }
+    __syncthreads();
+  }
+}
+
+// The directions kept: in shared memory, and in global memory between the
+// launches of a resumed solve.
+struct KryState {
+  int count, next;   // directions kept, slot of the next one
+  double g[KH][KH];  // (q_i, q_j) by slot
+};
+
+// The sums of pass 1 in a fixed order, then the step: the combination of the
+// new and the kept directions that minimises |r - sum c q| (2-norm), by the
+// normal equations.  The directions stay as they were formed, q = A z each:
+// made orthogonal one after the other (as in GCR), their FP32 rounding errors
+// pass from one to the next and grow, since successive corrections are nearly
+// parallel, until the step no longer belongs to the residual (seen from
+// 1e-10 of max|b| on).  c[i]: direction i before the new one, c[KH - 1]: the new one.
+__device__ __forceinline__ void rb_kry_coeff(const double* part, int nch, int m, KryState& K, double* dots, double* c) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (wid < KDOT) {
+    double s = 0.0;
+    for (int k = lane; k < nch; k += 32) s += __ldcg(part + (long long)k * KDOT + wid);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) dots[wid] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int nw = K.next;
+    int sl[KH];
+    double A[KH][KH], b[KH], x[KH];
+    sl[0] = nw;
+    b[0] = dots[0];
+    K.g[nw][nw] = dots[1];
+    for (int i = 0; i < m; ++i) {
+      sl[1 + i] = (nw + KH - 1 - i) % KH;
+      b[1 + i] = dots[KH + 1 + i];
+      K.g[nw][sl[1 + i]] = K.g[sl[1 + i]][nw] = dots[2 + i];
+    }
+    // Cholesky factor, newest first; a direction that depends on the ones before it is left out
+    int use[KH], nu = 0;
+    for (int i = 0; i <= m; ++i) {
+      const double d = K.g[sl[i]][sl[i]];
+      double t[KH], p = d;
+      for (int k = 0; k < nu; ++k) {
+        double v = K.g[sl[i]][sl[use[k]]];
+        for (int q = 0; q < k; ++q) v -= t[q] * A[k][q];
+        t[k] = v / A[k][k];
+        p -= t[k] * t[k];
+      }
+      if (!(p > 1e-6 * d)) continue;
+      for (int k = 0; k < nu; ++k) A[nu][k] = t[k];
+      A[nu][nu] = sqrt(p);
+      use[nu++] = i;
+    }
+    for (int i = 0; i < KH; ++i) c[i] = 0.0;
+    bool fin = nu > 0 && use[0] == 0;
+    for (int k = 0; k < nu; ++k) {
+      double v = b[use[k]];
+      for (int q = 0; q < k; ++q) v -= A[k][q] * x[q];
+      x[k] = v / A[k][k];
+    }
+    for (int k = nu - 1; k >= 0; --k) {
+      double v = x[k];
+      for (int q = k + 1; q < nu; ++q) v -= A[q][k] * x[q];
+      x[k] = v / A[k][k];
+      fin = fin && fabs(x[k]) < 1e3;
+    }
+    for (int k = 0; k < nu && fin; ++k) c[use[k] ? use[k] - 1 : KH - 1] = x[k];
+    if (!fin) c[KH - 1] = 1.0;  // the plain correction
+    K.count = min(m + 1, KH - 1);
+    K.next = (nw + 1) % KH;
+  }
+  __syncthreads();
+}
+
+// Krylov pass 2: phi += sum c z in FP64, z kept in slot `slot`, and r -= sum
+// c q where another V-cycle follows before the next FP64 residual.  slot < 0:
+// the plain correction, phi += z.
+template <class T>
+__device__ __noinline__ void rb_kry2(const RHier<T>& __restrict__ H, const RLev<T>& __restrict__ L,
+                                     const Op<double>& __restrict__ F, int sZ, int slot, int m,
+                                     const double* __restrict__ c, bool upd_r, const RCtx& G) {
+  const int ir = rb_red(sZ), ib = rb_black(sZ);
+  const int n0 = F.n[0], n1 = F.n[1];
+  double cc[KH - 1];
+  int os[KH - 1];
+#pragma unroll
+  for (int i = 0; i < KH - 1; ++i) {
+    cc[i] = i < m ? c[i] : 0.0;
+    os[i] = (slot + KH - 1 - i) % KH;
+  }
+  const double cn = slot < 0 ? 1.0 : c[KH - 1];
+  for (int t = G.i0; t < L.nqt; t += G.st) {
+    const unsigned w[2] = {reinterpret_cast<const unsigned*>(L.f[0])[t], reinterpret_cast<const unsigned*>(L.f[1])[t]};
+    if (!((w[0] | w[1]) & 0x03030303u)) continue;
+    const QPos g = quad_pos(L, t, 0);
+    const long long o4 = 4 * (long long)t;
+    for (int p = 0; p <= L.two; ++p) {
+      if (!((w[0] | w[1]) & (0x01010101u << p))) continue;
+      double* ph = F.x[p] + ((long long)g.j + (long long)n1 * g.k) * n0 + 2 * g.q0;
+      double f[8];
+      ld4(ph, f);
+      ld4(ph + 4, f + 4);
+#pragma unroll
+      for (int colour = 0; colour < 2; ++colour) {
+        T z[4], s[4];
+        ld4(L.x[p][colour ? ib : ir] + o4, z);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (!((w[colour] >> (8 * e + p)) & 1u)) z[e] = T(0);
+          s[e] = (T)cn * z[e];
+        }
+        if (slot >= 0) {
+          st4(H.kz[slot][p][colour] + o4, z);
+#pragma unroll
+          for (int i = 0; i < KH - 1; ++i) {
+            if (i >= m) continue;
+            T zi[4];
+            ld4(H.kz[os[i]][p][colour] + o4, zi);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[e] += (T)cc[i] * zi[e];
+          }
+          if (upd_r) {
+            T r[4], q[4];
+            ld4(L.b[p][colour] + o4, r);
+            ld4(H.kq[slot][p][colour] + o4, q);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) r[e] -= (T)cn * q[e];
+#pragma unroll
+            for (int i = 0; i < KH - 1; ++i) {
+              if (i >= m) continue;
+              ld4(H.kq[os[i]][p][colour] + o4, q);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) r[e] -= (T)cc[i] * q[e];
+            }
+            st4(L.b[p][colour] + o4, r);
+          }
+        }
+        const int odd = g.s ^ colour;  // red cells are the even ones where s = 0
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (odd) f[2 * e + 1] += (double)s[e];
+          else f[2 * e] += (double)s[e];
+        }
+      }
+      st4(ph, f);
+      st4(ph + 4, f + 4);
+    }
+  }
+}
+
+template <class T>
+__device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, const Op<double>* __restrict__ Fg,
+                                               const SolveCtl& ctl, const Barrier& B, int gcta, int gsize) {
+  __shared__ RHier<T> H;
+  __shared__ RLev<T> gl;
+  __shared__ Op<double> F;
+  __shared__ unsigned epoch, tn;
+  __shared__ T red[PT / 32][KDOT];
+  __shared__ double dots[KDOT], coef[KH];
+  __shared__ KryState K;
+  extern __shared__ __align__(128) unsigned char dyn[];
+  copy_words(&H, Hg, sizeof(RHier<T>));
+  copy_words(&F, Fg, sizeof(Op<double>));
+  copy_words(&gl, &Hg->L[Hg->lc], sizeof(RLev<T>));
+  if (threadIdx.x == 0) {
+    epoch = 0u;
+    tn = 0u;
+  }
+  copy_words(&K, Hg->kst, sizeof(KryState));
+  __syncthreads();
+  if (threadIdx.x == 0 && ctl.fresh) K.count = K.next = 0;
+  if (gcta == 0 && H.smem) {
+    // levels lc.. into shared memory: flags, rows (entries in T) and special lists, constant over the launch
+    for (int l = H.lc; l < H.nlev; ++l) {
+      const RLev<T>& g = Hg->L[l];
+      for (int q = 0; q < 2; ++q) copy_words(dyn + H.off_f[l][q], g.f[q], g.H);
+      if (g.nr && H.srows[l]) {
+        copy_words(dyn + H.off_re[l], g.re, 8ll * g.nr);
+        copy_words(dyn + H.off_rs[l], g.rs, 4ll * g.nr);
+        copy_words(dyn + H.off_col[l], g.col, 4ll * H.nnz[l]);
+        T* v = (T*)(dyn + H.off_val[l]);
+        T* d = (T*)(dyn + H.off_dg[l]);
+        for (int i = threadIdx.x; i < H.nnz[l]; i += blockDim.x) v[i] = (T)((const double*)g.val)[i];
+        T* di = (T*)(dyn + H.off_di[l]);
+        for (int i = threadIdx.x; i < g.nr; i += blockDim.x) {
+          d[i] = (T)((const double*)g.diag)[i];
+          di[i] = (T)((const double*)g.dinv)[i];
+        }
+        copy_words(dyn + H.off_sp[l], g.sp, 4ll * g.nsp);
+        copy_words(dyn + H.off_spr[l], g.sprow, 4ll * g.nsp * (2 << g.D));
+      }
+    }
+    if ((int)threadIdx.x >= H.lc && (int)threadIdx.x < H.nlev) {
+      const int l = threadIdx.x;
+      RLev<T>& v = H.L[l];
+      for (int p = 0; p <= v.two; ++p) {
+        for (int k = 0; k < 3; ++k) v.x[p][k] = (T*)(dyn + H.off_x[l][p][k]);
+        for (int k = 0; k < 2; ++k) v.b[p][k] = (T*)(dyn + H.off_b[l][p][k]);
+      }
+      for (int k = 0; k < 2; ++k) v.f[k] = dyn + H.off_f[l][k];
+      if (v.nr && H.srows[l]) {
+        v.re = (const int2*)(dyn + H.off_re[l]);
+        v.rs = (const unsigned*)(dyn + H.off_rs[l]);
+        v.col = (const unsigned*)(dyn + H.off_col[l]);
+        v.val = dyn + H.off_val[l];
+        v.diag = dyn + H.off_dg[l];
+        v.dinv = dyn + H.off_di[l];
+        v.sp = (const int*)(dyn + H.off_sp[l]);
+        v.sprow = (const int*)(dyn + H.off_spr[l]);
+        v.staged = 1;
+      }
+    }
+  }
+  __syncthreads();
+  RCtx G;
+  const int wi = (int)(threadIdx.x >> 5) * gsize + gcta;  // warps interleaved over the CTAs
+  G.i0 = wi * 32 + (int)(threadIdx.x & 31);
+  G.st = gsize * (int)blockDim.x;
+  G.gst = gsize * (int)(blockDim.x >> 3);
+  G.g0 = G.gst - 1 - (wi * 4 + (int)((threadIdx.x >> 3) & 3));
+  G.local = false;
+  G.B = B;
+  G.epoch = &epoch;
+  G.tr = nullptr;
+  G.tn = &tn;
+  G.gcta = gcta;
+  G.gsize = gsize;
+  // the finest level as the grid sees it (level 0 may be the first one inside CTA 0)
+  const RLev<T>& L0 = H.lc == 0 ? gl : H.L[0];
+  const int sZ = rb_done(H, 0);
+  const double bn = *ctl.bnorm;
+  int it = 0, cycles = 0, status = 0;
+  double r0 = 0.0, r = 0.0;
+  if (bn == 0.0) {  // b = 0: the solution is 0
+    for (long long cc = G.i0; cc < F.ncell; cc += G.st) {
+      F.x[0][cc] = 0.0;
+      if (F.x[1]) F.x[1][cc] = 0.0;
+    }
+  }
+  for (; bn != 0.0;) {
+    if (!rb_resid64(H, L0, F, ctl.norms + it, G)) {
+      status = 5;
+      break;
+    }
+    r = load_norm(ctl.norms + it);
+    if (it == 0) r0 = r;
+    if (r <= ctl.tol * bn) break;
+    if (cycles + ctl.inner > ctl.max_cycles || !(r == r) || r > 1e6 * r0) {
+      status = 3;
+      break;
+    }
+    if (ctl.max_iters && it >= ctl.max_iters) {  // resumable: stop at a V-cycle boundary
+      status = 7;
+      break;
+    }
+    bool ok = true;
+    for (int k = 0; k < ctl.inner && ok; ++k) {
+      RCtx Gk = G;
+      if (it == 0 && k == 0 && ctl.trace) {  // trace the first V-cycle
+        Gk.tr = ctl.trace;
+        if (gcta == 0 && threadIdx.x == 0) ctl.trace[1 + tn++] = ((unsigned long long)0xfff << 48) | (now_ns() & 0xffffffffffffULL);
+      }
+      ok = rb_vcycle(H, gl, Gk);
+      if (!ok) break;
+      if (ctl.kry) {
+        const int slot = K.next, m = K.count;
+        rb_kry1(H, L0, sZ, slot, m, Gk, red);
+        ok = Gk.sync((14 << 4) | 14);
+        if (!ok) break;
+        rb_kry_coeff(H.kpart, H.kch, m, K, dots, coef);
+        rb_kry2(H, L0, F, sZ, slot, m, coef, k + 1 < ctl.inner, Gk);
+      } else {
+        rb_kry2(H, L0, F, sZ, -1, 0, coef, false, Gk);
+      }
+      ok = Gk.sync((14 << 4) | 12);
+    }
+    if (!ok) {
+      status = 5;
+      break;
+    }
+    cycles += ctl.inner;
+    ++it;
+  }
+  if (gcta == 0 && threadIdx.x == 0) {
+    if (ctl.trace) ctl.trace[0] = tn;
+    ctl.norms[ctl.max_cycles + 1] = (unsigned long long)__double_as_longlong(r);  // final residual max
+    ctl.out[0] = status;
+    ctl.out[1] = it;
+    ctl.out[2] = cycles;
+    ctl.out[3] = it;
+    *H.kst = K;
+  }
+}
+
+template <class T>
+__global__ void __launch_bounds__(PT, 1) k_rb_solve(const RHier<T>* __restrict__ Hg, const Op<double>* __restrict__ Fg,
+                                                    SolveCtl ctl, Barrier B) {
+  rb_solve_group<T>(Hg, Fg, ctl, B, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// many independent solves in one cooperative launch (see BatchItem)
+template <class T>
+struct RBatchItem {
+  const RHier<T>* H;
+  const Op<double>* F;
+  SolveCtl ctl;
+  Barrier B;
+  int start, size;
+};
+template <class T>
+__global__ void __launch_bounds__(PT, 1) k_rb_batch(const RBatchItem<T>* __restrict__ items,
+                                                    const int* __restrict__ cta_item) {
+  const RBatchItem<T>& it = items[cta_item[blockIdx.x]];
+  rb_solve_group<T>(it.H, it.F, it.ctl, it.B, (int)blockIdx.x - it.start, it.size);
+}
+
+// single phases of the finest level in the persistent kernel's grid shape, to
+// time them: 0 a colour pass, 1 the residual + restriction, 6 the prolongation
+template <class T>
+__global__ void __launch_bounds__(PT, 1) k_rb_phase(const RHier<T>* __restrict__ Hg, int kernel, int colour) {
+  __shared__ RLev<T> L, N;
+  copy_words(&L, &Hg->L[0], sizeof(RLev<T>));
+  if (Hg->nlev > 1) copy_words(&N, &Hg->L[1], sizeof(RLev<T>));
+  __syncthreads();
+  RCtx G{};
+  const int gsize = (int)gridDim.x, wi = (int)(threadIdx.x >> 5) * gsize + (int)blockIdx.x;
+  G.i0 = wi * 32 + (int)(threadIdx.x & 31);
+  G.st = gsize * (int)blockDim.x;
+  G.gst = gsize * (int)(blockDim.x >> 3);
+  G.g0 = G.gst - 1 - (wi * 4 + (int)((threadIdx.x >> 3) & 3));
+  G.gsize = gsize;
+  G.gcta = (int)blockIdx.x;
+  if (kernel == 0) rb_dense(L, colour, 1, false, G);
+  else if (kernel == 1) rb_restrict(L, N, 1, false, G);
+  else rb_prolong(L, N, 1, rb_done(*Hg, 1), G);
+}
+}  // namespace ebp

@@ -16,6 +16,7 @@
 
 #include "eb_internal.h"
 #include "persistent.cuh"
+#include "rbsetup.cuh"
 
 // ----------------------------------------------------------------- errors
 
@@ -310,6 +311,12 @@ struct eb_poisson {
   int sweep_ns = 0;              // ring slots
   int sweep_first = -1;          // the finest of them
   std::vector<int*> sweep_ticks;  // their ticket counters (4 ints per level)
+  bool rb = false;                // the colour-split persistent solve (rbsolve.cuh)
+  bool resumed = false;           // the next batched launch continues a solve
+  bool kry = true;                // its Krylov acceleration (off inside an outer Krylov method)
+  std::vector<DevLevel> alg;      // algebraic levels below the geometric ones
+  unsigned char* pool = nullptr;  // rest of the last block taken by pool_alloc
+  size_t pool_left = 0;
   int smem_bytes = 0;  // dynamic shared memory of the persistent kernel
   cudaEvent_t kev[2] = {nullptr, nullptr};  // bracket the persistent kernel
   double kernel_ms = 0.0;                   // its device time in the last call
@@ -354,9 +361,9 @@ static void set_stencil_terms(Op<T>& o, const Grid& g) {
   }
 }
 
+// A level's operator without vectors.
 template <class T>
-static Op<T> make_op(const DevLevel& L, std::vector<void*>& owner, long long* bytes, eb_status* st, int nphase,
-                     T* x0 = nullptr, T* b0 = nullptr, T* x1 = nullptr, T* b1 = nullptr) {
+static Op<T> make_terms(const DevLevel& L) {
   Op<T> o;
   std::memset(&o, 0, sizeof(o));
   o.D = L.g.D;
@@ -367,13 +374,6 @@ static Op<T> make_op(const DevLevel& L, std::vector<void*>& owner, long long* by
   o.dq = make_fastdiv((unsigned)std::max(1, L.g.n[0] / 4));
   o.ncell = L.g.ncell;
   set_stencil_terms(o, L.g);
-  size_t n = (size_t)L.g.ncell;
-  o.x[0] = x0 ? x0 : (T*)dev_alloc(owner, n * sizeof(T), bytes, st);
-  o.b[0] = b0 ? b0 : (T*)dev_alloc(owner, n * sizeof(T), bytes, st);
-  if (nphase == 2) {
-    o.x[1] = x1 ? x1 : (T*)dev_alloc(owner, n * sizeof(T), bytes, st);
-    o.b[1] = b1 ? b1 : (T*)dev_alloc(owner, n * sizeof(T), bytes, st);
-  }
   o.flags = L.flags;
   o.irr_cell = L.irr_cell;
   o.irr_of_cell = L.irr_of_cell;
@@ -381,7 +381,6 @@ static Op<T> make_op(const DevLevel& L, std::vector<void*>& owner, long long* by
   o.col = L.col;
   o.val = L.val;
   o.diag = L.diag;
-  o.tmp = (T*)dev_alloc(owner, sizeof(T) * std::max<long long>(2 * L.nirr, 1), bytes, st);
   o.nirr = L.nirr;
   o.nirr_red = L.nirr_red;
   for (int p = 0; p < 2; ++p) {
@@ -389,6 +388,21 @@ static Op<T> make_op(const DevLevel& L, std::vector<void*>& owner, long long* by
     o.ceps[p] = (T)(e / h2);
     o.h2e[p] = (T)(h2 / e);
   }
+  return o;
+}
+
+template <class T>
+static Op<T> make_op(const DevLevel& L, std::vector<void*>& owner, long long* bytes, eb_status* st, int nphase,
+                     T* x0 = nullptr, T* b0 = nullptr, T* x1 = nullptr, T* b1 = nullptr) {
+  Op<T> o = make_terms<T>(L);
+  size_t n = (size_t)L.g.ncell;
+  o.x[0] = x0 ? x0 : (T*)dev_alloc(owner, n * sizeof(T), bytes, st);
+  o.b[0] = b0 ? b0 : (T*)dev_alloc(owner, n * sizeof(T), bytes, st);
+  if (nphase == 2) {
+    o.x[1] = x1 ? x1 : (T*)dev_alloc(owner, n * sizeof(T), bytes, st);
+    o.b[1] = b1 ? b1 : (T*)dev_alloc(owner, n * sizeof(T), bytes, st);
+  }
+  o.tmp = (T*)dev_alloc(owner, sizeof(T) * std::max<long long>(2 * L.nirr, 1), bytes, st);
   if (*st == EB_OK) {
     cudaMemset(o.x[0], 0, n * sizeof(T));
     cudaMemset(o.b[0], 0, n * sizeof(T));
@@ -520,12 +534,10 @@ static bool tmap3(CUtensorMap* m, CUtensorMapDataType type, int esize, const voi
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Levels of at least 2^25 cells (about 322^3) relax by tile-streamed sweeps:
-// measured on a GB300 at 384^3 a streamed sweep takes 0.39 ms against 0.53 ms
-// for the two colour passes, at 256^3 0.19 ms against 0.17 ms.  The streamed
-// residual + restriction is slower than the block restriction at both sizes
-// (0.36 / 0.31 ms, 0.19 / 0.10 ms) and is used only on request
-// (EBP_SWEEP_RESTRICT=1).
+// Tile-streamed sweeps run on request alone (EBP_SWEEP_MIN_CELLS=n: levels of
+// at least n cells).  Measured on a GB300 at 384^3 a streamed sweep of the plain
+// layout takes 0.39 ms; two passes over the colour-split layout of rbsolve.cuh
+// take 0.18 ms.
 static constexpr long long SW_MIN_CELLS = 1LL << 25;
 
 // Items of a level cut into z-chunks of zc planes: tile t = it % ntiles,
@@ -585,7 +597,7 @@ static eb_status setup_sweeps(eb_poisson* P, std::vector<Op<T>>& ops, Hier<T>& H
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, P->G->device);
   const int workers = std::max(1, nsm - 1);
-  long long min_cells = SW_MIN_CELLS;  // EBP_SWEEP_MIN_CELLS lowers it (tests run small grids through the path)
+  long long min_cells = SW_MIN_CELLS;
   if (const char* env = std::getenv("EBP_SWEEP_MIN_CELLS")) min_cells = std::max(1LL, std::atoll(env));
   int restrict_streamed = 0;
   if (const char* env = std::getenv("EBP_SWEEP_RESTRICT")) restrict_streamed = std::atoi(env) != 0;
@@ -679,6 +691,78 @@ static void sweep_reset(eb_poisson* P, cudaStream_t s) {
   for (int* t : P->sweep_ticks) cudaMemsetAsync(t, 0, 4 * sizeof(int), s);
 }
 
+// Dense inverse of the coarsest operator `ob` with m slots: FP64 Gauss-Jordan
+// up to 256 (stored transposed on request), FP32 up to 1024 (row-major).  *bm
+// stays 0 when there is none (too large, singular, or no room).
+template <class T>
+static eb_status bottom_inverse(eb_poisson* P, const Op<T>& ob, int m, bool transposed, const T** inv, int* bm) {
+  eb_status st = EB_OK;
+  if (m <= 256) {
+    std::vector<void*> tmp;
+    double* M = (double*)dev_alloc(tmp, sizeof(double) * m * m, nullptr, &st);
+    double* Mi = (double*)dev_alloc(tmp, sizeof(double) * m * m, nullptr, &st);
+    int* stat = (int*)dev_alloc(tmp, sizeof(int), nullptr, &st);
+    T* binv = (T*)dev_alloc(P->allocs, sizeof(T) * m * m, &P->bytes, &st);
+    if (st == EB_OK) {
+      const DevLevel& Lb = P->G->L[P->nlev - 1];
+      double h2 = Lb.g.h * Lb.g.h;
+      cudaMemsetAsync(stat, 0, sizeof(int), P->s);
+      cudaMemsetAsync(M, 0, sizeof(double) * m * m, P->s);
+      k_bottom_matrix<T><<<blocks(m), 256, 0, P->s>>>(ob, Lb.g.eps[0] / h2, Lb.g.eps[1] / h2, m, M);
+      k_gauss_jordan<<<1, 1024, 0, P->s>>>(M, Mi, m, stat);
+      if (transposed) k_convert<T><<<blocks((long long)m * m), 256, 0, P->s>>>(Mi, binv, (long long)m * m);
+      else k_from<T><<<blocks((long long)m * m), 256, 0, P->s>>>(Mi, binv, (long long)m * m);
+      int hs = 0;
+      cudaError_t e = cudaMemcpyAsync(&hs, stat, sizeof(int), cudaMemcpyDeviceToHost, P->s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(P->s);
+      if (e != cudaSuccess) st = cuda_fail(e, "bottom inverse");
+      if (st == EB_OK && hs == 0) {
+        *bm = m;
+        *inv = binv;
+      }
+    }
+    for (void* p : tmp) cudaFree(p);
+  } else if (m <= 1024) {
+    // larger bottoms: FP32 Gauss-Jordan with partial pivoting, one pivot step
+    // per pair of launches (an approximate inverse is enough for a bottom
+    // solve inside the V-cycle; a failed pivot keeps the relaxation bottom)
+    std::vector<void*> tmp;
+    double* M = (double*)dev_alloc(tmp, sizeof(double) * m * m, nullptr, &st);
+    float* Af = (float*)dev_alloc(tmp, sizeof(float) * m * m, nullptr, &st);
+    float* Ai = (float*)dev_alloc(tmp, sizeof(float) * m * m, nullptr, &st);
+    int* stat = (int*)dev_alloc(tmp, sizeof(int), nullptr, &st);
+    T* binv = st == EB_OK ? (T*)dev_alloc(P->allocs, sizeof(T) * m * m, &P->bytes, &st) : nullptr;
+    if (st == EB_OK) {
+      const DevLevel& Lb = P->G->L[P->nlev - 1];
+      double h2 = Lb.g.h * Lb.g.h;
+      long long mm = (long long)m * m;
+      cudaMemsetAsync(stat, 0, sizeof(int), P->s);
+      cudaMemsetAsync(M, 0, sizeof(double) * m * m, P->s);
+      k_bottom_matrix<T><<<blocks(m), 256, 0, P->s>>>(ob, Lb.g.eps[0] / h2, Lb.g.eps[1] / h2, m, M);
+      k_to_float<<<blocks(mm), 256, 0, P->s>>>(M, Af, mm);
+      k_identity<<<blocks(mm), 256, 0, P->s>>>(Ai, m);
+      const int eb = (int)(((long long)m * 32 + 255) / 256);
+      for (int k = 0; k < m; ++k) {
+        k_gj_pivot<<<1, 1024, 0, P->s>>>(Af, Ai, m, k, stat);
+        k_gj_elim<<<eb, 256, 0, P->s>>>(Af, Ai, m, k, stat);
+      }
+      k_from<T><<<blocks(mm), 256, 0, P->s>>>(Ai, binv, mm);  // row-major for ph_bottom_grid
+      int hs = 0;
+      cudaError_t e = cudaMemcpyAsync(&hs, stat, sizeof(int), cudaMemcpyDeviceToHost, P->s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(P->s);
+      if (e != cudaSuccess) st = cuda_fail(e, "bottom inverse");
+      if (st == EB_OK && hs == 0) {
+        *bm = m;
+        *inv = binv;
+      }
+    }
+    for (void* p : tmp) cudaFree(p);
+    st = st == EB_ERR_OOM ? EB_OK : st;  // no room for the inverse: relaxation bottom
+    if (st == EB_OK && *bm == 0) cudaGetLastError();
+  }
+  return st;
+}
+
 template <class T>
 static eb_status build_hier(eb_poisson* P, std::vector<Op<T>>& ops) {
   Hier<T> H;
@@ -763,71 +847,8 @@ static eb_status build_hier(eb_poisson* P, std::vector<Op<T>>& ops) {
     H.smem_bytes = (int)off;
   }
   for (int l = 0; l < P->nlev; ++l) H.op[l] = ops[l];
-  eb_status st = EB_OK;
-  // dense inverse of the coarsest operator (FP64 Gauss-Jordan on the device)
-  if (m <= 256) {
-    std::vector<void*> tmp;
-    double* M = (double*)dev_alloc(tmp, sizeof(double) * m * m, nullptr, &st);
-    double* Mi = (double*)dev_alloc(tmp, sizeof(double) * m * m, nullptr, &st);
-    int* stat = (int*)dev_alloc(tmp, sizeof(int), nullptr, &st);
-    T* binv = (T*)dev_alloc(P->allocs, sizeof(T) * m * m, &P->bytes, &st);
-    if (st == EB_OK) {
-      const DevLevel& Lb = P->G->L[P->nlev - 1];
-      double h2 = Lb.g.h * Lb.g.h;
-      cudaMemsetAsync(stat, 0, sizeof(int), P->s);
-      cudaMemsetAsync(M, 0, sizeof(double) * m * m, P->s);
-      k_bottom_matrix<T><<<blocks(m), 256, 0, P->s>>>(ob, Lb.g.eps[0] / h2, Lb.g.eps[1] / h2, m, M);
-      k_gauss_jordan<<<1, 1024, 0, P->s>>>(M, Mi, m, stat);
-      k_convert<T><<<blocks((long long)m * m), 256, 0, P->s>>>(Mi, binv, (long long)m * m);
-      int hs = 0;
-      cudaError_t e = cudaMemcpyAsync(&hs, stat, sizeof(int), cudaMemcpyDeviceToHost, P->s);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(P->s);
-      if (e != cudaSuccess) st = cuda_fail(e, "bottom inverse");
-      if (st == EB_OK && hs == 0) {
-        H.bm = m;
-        H.binv = binv;
-      }
-    }
-    for (void* p : tmp) cudaFree(p);
-  } else if (m <= 1024) {
-    // larger bottoms: FP32 Gauss-Jordan with partial pivoting, one pivot step
-    // per pair of launches (an approximate inverse is enough for a bottom
-    // solve inside the V-cycle; a failed pivot keeps the relaxation bottom)
-    std::vector<void*> tmp;
-    double* M = (double*)dev_alloc(tmp, sizeof(double) * m * m, nullptr, &st);
-    float* Af = (float*)dev_alloc(tmp, sizeof(float) * m * m, nullptr, &st);
-    float* Ai = (float*)dev_alloc(tmp, sizeof(float) * m * m, nullptr, &st);
-    int* stat = (int*)dev_alloc(tmp, sizeof(int), nullptr, &st);
-    T* binv = st == EB_OK ? (T*)dev_alloc(P->allocs, sizeof(T) * m * m, &P->bytes, &st) : nullptr;
-    if (st == EB_OK) {
-      const DevLevel& Lb = P->G->L[P->nlev - 1];
-      double h2 = Lb.g.h * Lb.g.h;
-      long long mm = (long long)m * m;
-      cudaMemsetAsync(stat, 0, sizeof(int), P->s);
-      cudaMemsetAsync(M, 0, sizeof(double) * m * m, P->s);
-      k_bottom_matrix<T><<<blocks(m), 256, 0, P->s>>>(ob, Lb.g.eps[0] / h2, Lb.g.eps[1] / h2, m, M);
-      k_to_float<<<blocks(mm), 256, 0, P->s>>>(M, Af, mm);
-      k_identity<<<blocks(mm), 256, 0, P->s>>>(Ai, m);
-      const int eb = (int)(((long long)m * 32 + 255) / 256);
-      for (int k = 0; k < m; ++k) {
-        k_gj_pivot<<<1, 1024, 0, P->s>>>(Af, Ai, m, k, stat);
-        k_gj_elim<<<eb, 256, 0, P->s>>>(Af, Ai, m, k, stat);
-      }
-      k_from_float<T><<<blocks(mm), 256, 0, P->s>>>(Ai, binv, mm);  // row-major for ph_bottom_grid
-      int hs = 0;
-      cudaError_t e = cudaMemcpyAsync(&hs, stat, sizeof(int), cudaMemcpyDeviceToHost, P->s);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(P->s);
-      if (e != cudaSuccess) st = cuda_fail(e, "bottom inverse");
-      if (st == EB_OK && hs == 0) {
-        H.bm = m;
-        H.binv = binv;
-        H.gbot = 1;
-      }
-    }
-    for (void* p : tmp) cudaFree(p);
-    st = st == EB_ERR_OOM ? EB_OK : st;  // no room for the inverse: relaxation bottom
-    if (st == EB_OK && H.bm == 0) cudaGetLastError();
-  }
+  eb_status st = bottom_inverse<T>(P, ob, m, m <= 256, &H.binv, &H.bm);
+  if (H.bm > 256) H.gbot = 1;
   if (st != EB_OK) return st;
   if (krylov_bottom && H.bm == 0) {
     H.kry = (T*)dev_alloc(P->allocs, sizeof(T) * 12 * (size_t)ob.ncell, &P->bytes, &st);
@@ -857,17 +878,339 @@ static eb_status build_hier(eb_poisson* P, std::vector<Op<T>>& ops) {
   return st;
 }
 
-// The persistent kernels in two builds: with the tile-streamed passes (FP32
-// hierarchies that have streamed levels) and without them, so that every
-// other solve runs the lean build.
-static const void* solve_kernel(bool mixed, bool sw) {
-  if (!mixed) return (const void*)k_solve<double, false>;
-  return sw ? (const void*)k_solve<float, true> : (const void*)k_solve<float, false>;
+// ------------------------------------------------- colour-split hierarchy (rbsolve.cuh)
+
+// Part of a block of device memory owned by the handle: a set-up takes dozens
+// of small arrays, and a cudaMalloc each would cost more than filling them.
+static void* pool_alloc(eb_poisson* P, size_t bytes, eb_status* st) {
+  bytes = (bytes + 255) / 256 * 256;
+  if (bytes > P->pool_left) {
+    if (bytes >= (1u << 20)) return dev_alloc(P->allocs, bytes, &P->bytes, st);
+    P->pool = (unsigned char*)dev_alloc(P->allocs, 1u << 20, &P->bytes, st);
+    P->pool_left = P->pool ? 1u << 20 : 0;
+    if (!P->pool) return nullptr;
+  }
+  void* p = P->pool;
+  P->pool += bytes;
+  P->pool_left -= bytes;
+  return p;
 }
-static const void* batch_kernel(bool mixed, bool sw) {
-  if (!mixed) return (const void*)k_solve_batch<double, false>;
-  return sw ? (const void*)k_solve_batch<float, true> : (const void*)k_solve_batch<float, false>;
+
+static SplitDim split_dim(const DevLevel& L) {
+  SplitDim d;
+  d.n0 = L.g.n[0];
+  d.n1 = L.g.n[1];
+  d.n2 = L.g.D == 3 ? L.g.n[2] : 1;
+  d.hx = ((d.n0 + 1) / 2 + 3) / 4 * 4;
+  d.H = d.hx * d.n1 * d.n2;
+  return d;
 }
+
+// Coarsest cells of the algebraic levels: few enough that a handful of
+// sweeps, or BiCGStab by one warp (32 rows), solves them.
+static constexpr long long ALG_MIN_CELLS = 16;
+static constexpr int ALG_BOTTOM_SWEEPS = 8;
+static constexpr int ALG_SWEEPS = 2;
+
+// Levels of at most LOCAL_CELLS cells run inside CTA 0, out of RB_SMEM_CAP
+// bytes of its shared memory.  Every CTA of the launch gives up that much of
+// its L1, and with it loads in flight on the large levels.
+static constexpr long long LOCAL_CELLS = 1024;
+static constexpr int RB_SMEM_CAP = 72 * 1024;
+
+template <class T>
+static eb_status setup_rb(eb_poisson* P, int smem_cap) {
+  smem_cap = std::min(smem_cap, RB_SMEM_CAP);
+  const eb_geom* G = P->G;
+  cudaStream_t s = P->s;
+  eb_status st = EB_OK;
+  std::vector<RHier<T>> hold(1);
+  RHier<T>& H = hold[0];
+  std::memset(&H, 0, sizeof(H));
+  H.bsweeps = P->o.bottom_sweeps;
+  const DevLevel& Lb = G->L.back();
+  const int m = (int)std::min<long long>(G->n_phase * Lb.g.ncell, 1 << 20);
+  bool grid_bottom = false;
+  P->bottom = EB_BOTTOM_RELAX;
+  if (m <= 1024) {
+    const T* inv = nullptr;
+    int bm = 0;
+    const Op<T> ob = make_terms<T>(Lb);
+    st = bottom_inverse<T>(P, ob, m, false, &inv, &bm);
+    if (st != EB_OK) return st;
+    if (bm) {
+      H.bot = 1;
+      H.bm = bm;
+      H.binv = inv;
+      grid_bottom = bm > 256;
+      P->bottom = grid_bottom ? EB_BOTTOM_INV32 : EB_BOTTOM_INV64;
+    }
+  } else {
+    // algebraic levels down to a few cells
+    while ((P->alg.empty() ? Lb : P->alg.back()).g.ncell > ALG_MIN_CELLS && (int)(G->L.size() + P->alg.size()) < RMAX) {
+      DevLevel C;
+      st = build_alg_level(P->alg.empty() ? Lb : P->alg.back(), C, &P->bytes, s);
+      if (st != EB_OK) {
+        free_level(C);
+        return st;
+      }
+      P->alg.push_back(C);
+    }
+    if (Lb.g.ncell > 4096) {
+      P->bottom = EB_BOTTOM_KRYLOV;
+      H.bot = 2;
+    } else {
+      H.bsweeps = std::min(H.bsweeps, ALG_BOTTOM_SWEEPS);
+    }
+  }
+  std::vector<const DevLevel*> lev;
+  for (const DevLevel& L : G->L) lev.push_back(&L);
+  for (const DevLevel& L : P->alg) lev.push_back(&L);
+  const int nl = (int)lev.size();
+  H.nlev = nl;
+  for (int l = 0; l < nl; ++l) {
+    // the caller's schedule down to the coarsest grid; that one and the
+    // algebraic levels are its bottom solve, which needs sweeps on both sides
+    const bool bottom = !P->alg.empty() && l >= (int)G->L.size() - 1;
+    H.nu1[l] = bottom ? ALG_SWEEPS : P->o.nu1;
+    H.nu2[l] = bottom ? ALG_SWEEPS : P->o.nu2;
+  }
+  // the dielectric's slabs (rows in 2D, planes in 3D): its vectors are stored for these alone
+  const int D = G->L[0].g.D;
+  int lohi[2] = {0x7fffffff, -1};
+  int* d_cnt = (int*)pool_alloc(P, sizeof(int) * (4 * RMAX + 2), &st);
+  if (st != EB_OK) return st;
+  cudaMemsetAsync(d_cnt, 0, sizeof(int) * 4 * RMAX, s);
+  const bool two = G->n_phase == 2;
+  if (two) {
+    int* d_lohi = d_cnt + 4 * RMAX;
+    cudaError_t e = cudaMemcpyAsync(d_lohi, lohi, sizeof(lohi), cudaMemcpyHostToDevice, s);
+    k_phase1_rows<<<blocks(G->L[0].g.ncell), 256, 0, s>>>(G->L[0].flags, G->L[0].g.ncell, G->L[0].g.n[0], d_lohi);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(lohi, d_lohi, sizeof(lohi), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_fail(e, "dielectric extent");
+  }
+  const int per = D == 3 ? G->L[0].g.n[1] : 1;
+  int sa = lohi[1] >= 0 ? lohi[0] / per : 0, sb = lohi[1] >= 0 ? lohi[1] / per : 0;
+  struct Band {
+    int row0, rows;
+  };
+  std::vector<Band> band(nl);
+  for (int l = 0; l < nl; ++l) {
+    const Grid& g = lev[l]->g;
+    const int ns = D == 3 ? g.n[2] : g.n[1], rps = D == 3 ? g.n[1] : 1;
+    if (l > 0) {
+      sa /= 2;
+      sb /= 2;
+    }
+    sa = std::max(0, sa - 1);
+    sb = std::min(ns - 1, sb + 1);
+    band[l] = {sa * rps, (sb - sa + 1) * rps};
+  }
+  // one half of a vector (both colours have the same extent): the pointer is
+  // to entry 0 of the half even where only the band is stored
+  auto half = [&](int l, int p, const SplitDim& d) -> T* {
+    const size_t skip = p ? (size_t)band[l].row0 * d.hx : 0;
+    const size_t n = p ? (size_t)band[l].rows * d.hx : (size_t)d.H;
+    T* q = (T*)pool_alloc(P, n * sizeof(T), &st);
+    if (!q) return nullptr;
+    cudaMemsetAsync(q, 0, n * sizeof(T), s);
+    return q - skip;
+  };
+  std::vector<SplitDim> dim(nl);
+  for (int l = 0; l < nl && st == EB_OK; ++l) {
+    const DevLevel& L = *lev[l];
+    const SplitDim d = dim[l] = split_dim(L);
+    RLev<T>& R = H.L[l];
+    const Op<T> o = make_terms<T>(L);
+    R.D = D;
+    for (int k = 0; k < 3; ++k) R.n[k] = k < D ? L.g.n[k] : 1;
+    R.hx = d.hx;
+    R.nq = d.hx / 4;
+    R.H = d.H;
+    R.nqt = d.H / 4;
+    R.dq = make_fastdiv((unsigned)R.nq);
+    R.dn1 = make_fastdiv((unsigned)R.n[1]);
+    R.two = two ? 1 : 0;
+    R.full = R.n[0] % 8 == 0;
+    for (int k = 0; k < 2; ++k) {
+      R.dge[k] = T(2 * D - 1) + T(3) * o.wr[k];
+      for (int p = 0; p < 2; ++p) R.ide[k][p] = T(1) / (R.dge[k] + o.lh[p]);
+    }
+    R.p1o = band[l].row0 * d.hx;
+    R.p1n = band[l].rows * d.hx;
+    for (int k = 0; k < 6; ++k) {
+      R.wr[k] = o.wr[k];
+      R.w3[k] = o.w3[k];
+    }
+    for (int p = 0; p < 2; ++p) {
+      R.lh[p] = o.lh[p];
+      R.idg[p] = o.idg[p];
+      R.ceps[p] = o.ceps[p];
+      R.h2e[p] = o.h2e[p];
+    }
+    for (int p = 0; p <= R.two; ++p) {
+      for (int k = 0; k < 3; ++k) R.x[p][k] = half(l, p, d);
+      for (int k = 0; k < 2; ++k) R.b[p][k] = half(l, p, d);
+    }
+    uint8_t* f = (uint8_t*)pool_alloc(P, 2 * (size_t)d.H, &st);
+    const long long nr = 2 * L.nirr, nnz = L.nnz, n = L.g.ncell;
+    int2* re = (int2*)pool_alloc(P, sizeof(int2) * std::max<long long>(nr, 1), &st);
+    unsigned* rs = (unsigned*)pool_alloc(P, sizeof(unsigned) * std::max<long long>(nr, 1), &st);
+    double* dg = (double*)pool_alloc(P, sizeof(double) * std::max<long long>(nr, 1), &st);
+    double* di = (double*)pool_alloc(P, sizeof(double) * std::max<long long>(nr, 1), &st);
+    int* rnat = (int*)pool_alloc(P, sizeof(int) * std::max<long long>(nr, 1), &st);
+    int* inv = (int*)pool_alloc(P, sizeof(int) * std::max<long long>(nr, 1), &st);
+    unsigned* col = (unsigned*)pool_alloc(P, sizeof(unsigned) * std::max<long long>(nnz, 1), &st);
+    const bool last = l == nl - 1;
+    const size_t nsp = last ? 1 : std::max<long long>(L.nirr, 1);
+    int* sp = (int*)pool_alloc(P, sizeof(int) * nsp, &st);
+    int* spr = (int*)pool_alloc(P, sizeof(int) * nsp * (2 << D), &st);
+    if (st != EB_OK) return st;
+    int* cnt = d_cnt + 4 * l;
+    cudaMemsetAsync(f, 0, 2 * (size_t)d.H, s);
+    const DevLevel* Lf = l > 0 ? lev[l - 1] : nullptr;
+    const DevLevel* Lc = last ? nullptr : lev[l + 1];
+    const int one[3] = {1, 1, 1};
+    const int *fn = Lf ? Lf->g.n : one, *cn = Lc ? Lc->g.n : one;
+    const int f2 = D == 3 ? fn[2] : 1, c2 = D == 3 ? cn[2] : 1;
+    k_split_flags<<<blocks(n), 256, 0, s>>>(D, d, L.flags, Lf ? Lf->flags : nullptr, fn[0], fn[1], f2,
+                                            Lc ? Lc->flags : nullptr, cn[0], cn[1], c2, f, cnt + 3);
+    if (nr) {
+      k_split_rows<<<1, 1024, 0, s>>>(d, L.flags, L.irr_cell, (int)L.nirr, (int)L.nirr_red, L.row_ptr, L.diag, re, rs,
+                                      dg, di, rnat, inv, cnt);
+      if (nnz) k_split_cols<<<blocks(nnz), 256, 0, s>>>(d, L.col, nnz, col);
+      if (Lc)
+        k_split_special<<<blocks(Lc->g.ncell), 256, 0, s>>>(D, L.flags, d.n0, d.n1, d.n2, L.irr_of_cell, inv, cn[0],
+                                                            cn[1], c2, sp, spr, cnt);
+    }
+    R.f[0] = f;
+    R.f[1] = f + d.H;
+    R.re = re;
+    R.rs = rs;
+    R.col = col;
+    R.val = L.val;
+    R.diag = dg;
+    R.dinv = di;
+    R.sp = sp;
+    R.sprow = spr;
+    H.nnz[l] = (int)nnz;
+    if (l == 0) {
+      H.rnat = rnat;
+      H.ncol = L.col;
+      H.rval = L.val;
+      H.rdiag = dg;
+    }
+  }
+  if (H.bot == 1) {
+    const int lb = nl - 1;
+    unsigned* bs = (unsigned*)pool_alloc(P, sizeof(unsigned) * H.bm, &st);
+    if (st == EB_OK)
+      k_split_slots<<<blocks(H.bm), 256, 0, s>>>(dim[lb], Lb.flags, H.bm, (int)Lb.g.ncell, bs);
+    H.bslot = bs;
+  }
+  // Krylov directions and the chunks of their sums: chunks of the finest
+  // level's groups alone, about two per CTA of a whole GPU on large levels
+  const RLev<T>& R0 = H.L[0];
+  H.kcs = ((R0.nqt + 303) / 304 + PT - 1) / PT * PT;
+  H.kch = (R0.nqt + H.kcs - 1) / H.kcs;
+  if (P->kry) {
+    for (int i = 0; i < KH && st == EB_OK; ++i)
+      for (int p = 0; p <= R0.two; ++p)
+        for (int c = 0; c < 2; ++c) {
+          H.kz[i][p][c] = half(0, p, dim[0]);
+          H.kq[i][p][c] = half(0, p, dim[0]);
+        }
+    H.kpart = (double*)pool_alloc(P, sizeof(double) * KDOT * (size_t)H.kch, &st);
+  }
+  H.kst = (KryState*)pool_alloc(P, sizeof(KryState), &st);
+  if (st != EB_OK) return st;
+  cudaMemsetAsync(H.kst, 0, sizeof(KryState), s);
+  int cnt[4 * RMAX];
+  cudaError_t e = cudaMemcpyAsync(cnt, d_cnt, sizeof(cnt), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "split set-up");
+  for (int l = 0; l < nl; ++l) {
+    H.L[l].nr = cnt[4 * l];
+    H.L[l].nr0 = cnt[4 * l + 1];
+    H.L[l].nsp = l < nl - 1 ? cnt[4 * l + 2] : 0;
+    H.L[l].dense = cnt[4 * l + 3];
+  }
+  H.krows = (H.L[0].nr + H.kch - 1) / H.kch;
+  if (H.bot == 2 && H.L[nl - 1].nr > 32) H.bot = 0, H.bsweeps = std::min(H.bsweeps, ALG_BOTTOM_SWEEPS);
+  // the small levels inside CTA 0, on shared-memory copies when their vectors
+  // fit; their rows join them while there is room
+  auto layout = [&](int l0) {
+    long long off = 0;
+    auto take = [&](long long bytes) {
+      const long long o = off;
+      off += (bytes + 15) / 16 * 16;
+      return (int)o;
+    };
+    for (int l = l0; l < nl; ++l) {
+      const RLev<T>& R = H.L[l];
+      const long long hb = (long long)R.H * (long long)sizeof(T);
+      for (int p = 0; p <= R.two; ++p) {
+        for (int k = 0; k < 3; ++k) H.off_x[l][p][k] = take(hb);
+        for (int k = 0; k < 2; ++k) H.off_b[l][p][k] = take(hb);
+      }
+      for (int k = 0; k < 2; ++k) H.off_f[l][k] = take(R.H);
+    }
+    return off;
+  };
+  H.lc = nl - 1;
+  for (int l = 0; l < nl; ++l)
+    if (lev[l]->g.ncell <= LOCAL_CELLS) {
+      H.lc = std::min(l, nl - 1);
+      break;
+    }
+  if (grid_bottom) H.lc = nl - 1;
+  while (H.lc < nl - 1 && layout(H.lc) > smem_cap) ++H.lc;
+  long long off = layout(H.lc);
+  H.smem = off <= smem_cap && !grid_bottom ? 1 : 0;
+  if (H.smem) {
+    for (int l = H.lc; l < nl; ++l) {
+      const RLev<T>& R = H.L[l];
+      if (!R.nr) continue;
+      auto al = [](long long b) { return (b + 15) / 16 * 16; };
+      const long long b[8] = {al(8ll * R.nr), al(4ll * R.nr), al(4ll * H.nnz[l]), al((long long)sizeof(T) * H.nnz[l]),
+                              al((long long)sizeof(T) * R.nr), al((long long)sizeof(T) * R.nr), al(4ll * R.nsp),
+                              al(4ll * R.nsp * (2 << D))};
+      long long need = 0;
+      for (long long v : b) need += v;
+      if (off + need > smem_cap) continue;
+      int* dst[8] = {&H.off_re[l], &H.off_rs[l], &H.off_col[l], &H.off_val[l],
+                     &H.off_dg[l], &H.off_di[l], &H.off_sp[l],  &H.off_spr[l]};
+      for (int k = 0; k < 8; ++k) {
+        *dst[k] = (int)off;
+        off += b[k];
+      }
+      H.srows[l] = 1;
+    }
+  }
+  P->smem_bytes = H.smem ? (int)off : 0;
+  P->bm = H.bm;
+  P->d_hier = pool_alloc(P, sizeof(RHier<T>), &st);
+  if (st != EB_OK) return st;
+  e = cudaMemcpyAsync(P->d_hier, &H, sizeof(RHier<T>), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  return e == cudaSuccess ? EB_OK : cuda_fail(e, "hierarchy upload");
+}
+
+// The persistent kernels: the colour-split ones, and for hierarchies with
+// tile-streamed levels (on request) the plain-layout ones.
+static const void* solve_kernel(const eb_poisson* P) {
+  if (!P->rb) return (const void*)k_solve<float>;
+  return P->o.precision == EB_PREC_MIXED ? (const void*)k_rb_solve<float> : (const void*)k_rb_solve<double>;
+}
+static const void* batch_kernel(const eb_poisson* P) {
+  if (!P->rb) return (const void*)k_solve_batch<float>;
+  return P->o.precision == EB_PREC_MIXED ? (const void*)k_rb_batch<float> : (const void*)k_rb_batch<double>;
+}
+
+// shared memory left for a kernel's static part (the hierarchy's description)
+static constexpr int STATIC_SMEM = 20 * 1024;
 
 static eb_status setup_persistent(eb_poisson* P) {
   int dev = P->G->device, coop = 0, nsm = 0;
@@ -875,7 +1218,11 @@ static eb_status setup_persistent(eb_poisson* P) {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   eb_status st = EB_OK;
   bool mixed = P->o.precision == EB_PREC_MIXED;
-  st = mixed ? build_hier<float>(P, P->op32) : build_hier<double>(P, P->op64);
+  int smax = 0;
+  cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  smax -= STATIC_SMEM;
+  if (P->rb) st = mixed ? setup_rb<float>(P, smax) : setup_rb<double>(P, smax);
+  else if (P->o.launch_mode == 0 && mixed) st = build_hier<float>(P, P->op32);  // tile-streamed levels
   if (st != EB_OK) return st;
   P->d_fine = (Op<double>*)dev_alloc(P->allocs, sizeof(Op<double>), &P->bytes, &st);
   P->d_bar = (unsigned*)dev_alloc(P->allocs, 4 * sizeof(unsigned), &P->bytes, &st);
@@ -889,14 +1236,12 @@ static eb_status setup_persistent(eb_poisson* P) {
   if (e == cudaSuccess) e = cudaMallocHost(&P->h_out, 4 * sizeof(int));
   if (e != cudaSuccess) return cuda_fail(e, "persistent setup");
   if (!coop || P->o.launch_mode != 0) return EB_OK;  // per-phase kernels
-  int per_sm = 0, smax = 0;
-  const bool sw = P->sweep_levels > 0;
-  const void* fn = solve_kernel(mixed, sw);
+  if (!P->rb && !P->sweep_levels) return EB_OK;
+  int per_sm = 0;
+  const void* fn = solve_kernel(P);
   // the attribute is per kernel, shared by every handle: allow the device maximum once
-  cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  smax -= 16 * 1024;  // headroom for the kernel's static shared memory
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(batch_kernel(mixed, sw), cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(batch_kernel(P), cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
   if (e == cudaSuccess && P->sweep_levels)
     e = cudaFuncSetAttribute((const void*)k_sweep_phase<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
   if (e == cudaSuccess && P->sweep_levels)
@@ -905,7 +1250,9 @@ static eb_status setup_persistent(eb_poisson* P) {
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, PT, P->smem_bytes);
   if (e != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
-    return EB_OK;
+    if (!P->rb) return EB_OK;
+    set_error("the persistent kernel does not fit the device");
+    return EB_ERR_UNSUPPORTED;
   }
   // CTAs per SM of the persistent kernel: fewer CTAs make the grid barrier
   // cheaper, more hide memory latency on the largest levels
@@ -939,27 +1286,16 @@ static eb_status solve_persistent(eb_poisson* P, double* r, int* iters, int* cyc
   ctl.trace = P->d_stamps;
   ctl.max_iters = 0;
   Barrier B{P->d_bar, (int*)(P->d_bar + 2)};
-  void* args[4];
+  ctl.kry = P->kry ? 1 : 0;
+  ctl.fresh = 1;
+  if (P->rb && !ctl.kry) ctl.inner = 1;
   cudaError_t e = kernel_events(P);
   if (e != cudaSuccess) return cuda_fail(e, "event");
   cudaEventRecord(P->kev[0], s);
-  if (ctl.mixed) {
-    const Hier<float>* H = (const Hier<float>*)P->d_hier;
-    const Op<double>* F = P->d_fine;
-    args[0] = (void*)&H;
-    args[1] = (void*)&F;
-    args[2] = (void*)&ctl;
-    args[3] = (void*)&B;
-    e = cudaLaunchCooperativeKernel(solve_kernel(true, P->sweep_levels > 0), dim3(P->grid), dim3(PT), args, dyn, s);
-  } else {
-    const Hier<double>* H = (const Hier<double>*)P->d_hier;
-    const Op<double>* F = P->d_fine;
-    args[0] = (void*)&H;
-    args[1] = (void*)&F;
-    args[2] = (void*)&ctl;
-    args[3] = (void*)&B;
-    e = cudaLaunchCooperativeKernel(solve_kernel(false, false), dim3(P->grid), dim3(PT), args, dyn, s);
-  }
+  const void* H = P->d_hier;
+  const Op<double>* F = P->d_fine;
+  void* args[4] = {(void*)&H, (void*)&F, (void*)&ctl, (void*)&B};
+  e = cudaLaunchCooperativeKernel(solve_kernel(P), dim3(P->grid), dim3(PT), args, dyn, s);
   counted();
   cudaEventRecord(P->kev[1], s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(P->h_out, P->d_out, 4 * sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -980,7 +1316,25 @@ static eb_status solve_persistent(eb_poisson* P, double* r, int* iters, int* cyc
   return EB_OK;
 }
 
+// Whether the environment asks for tile-streamed sweeps (EBP_SWEEP_MIN_CELLS=n)
+// and the finest level takes them.
+static bool sweeps_requested(const eb_poisson* P) {
+  const char* env = std::getenv("EBP_SWEEP_MIN_CELLS");
+  if (!env || P->o.precision != EB_PREC_MIXED || P->nlev < 2) return false;
+  if (const char* off = std::getenv("EBP_SWEEP"))
+    if (std::atoi(off) == 0) return false;
+  const Grid& g = P->G->L[0].g;
+  return g.D == 3 && g.ncell >= std::max(1LL, std::atoll(env)) && g.ncell > 4096 && g.n[0] % 16 == 0 && g.n[1] % 4 == 0 &&
+         g.n[2] % 4 == 0;
+}
+
 extern "C" eb_status eb_poisson_setup(const eb_geom* G, const eb_solver_opts* opts, void* stream, eb_poisson** out) {
+  return poisson_setup(G, opts, true, out);
+}
+
+// kry: Krylov acceleration of the V-cycles (a handle whose V-cycles precondition
+// an outer Krylov method goes without, and without its memory)
+eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, bool kry, eb_poisson** out) {
   if (!G || !out) {
     set_error("null argument");
     return EB_ERR_INVALID;
@@ -991,7 +1345,7 @@ extern "C" eb_status eb_poisson_setup(const eb_geom* G, const eb_solver_opts* op
   if (opts) P->o = *opts;
   else eb_solver_opts_default(&P->o);
   eb_solver_opts& o = P->o;
-  const int nu_auto = G->L[0].g.D == 3 ? 6 : 2;
+  const int nu_auto = G->L[0].g.D == 3 ? 3 : 2;
   if (o.nu1 == -1) o.nu1 = nu_auto;
   if (o.nu2 == -1) o.nu2 = nu_auto;
   if (!(o.tol > 0.0) || o.max_cycles < 1 || o.nu1 < 0 || o.nu2 < 0 || o.inner_cycles < 1 || o.bottom_sweeps < 1 ||
@@ -1014,7 +1368,13 @@ extern "C" eb_status eb_poisson_setup(const eb_geom* G, const eb_solver_opts* op
   }
   // finest FP64 operator over the solver's own phi and b
   P->op64.push_back(make_op<double>(F, P->allocs, &P->bytes, &st, np, P->phi64, P->b64, P->phi64 + n0, P->b64 + n0));
-  if (o.precision == EB_PREC_FP64) {
+  int coop = 0;
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, G->device);
+  P->rb = coop && o.launch_mode == 0 && !sweeps_requested(P);
+  P->kry = kry;
+  if (P->rb) {
+    // the colour-split hierarchy has vectors of its own
+  } else if (o.precision == EB_PREC_FP64) {
     for (int l = 1; l < P->nlev; ++l) P->op64.push_back(make_op<double>(G->L[l], P->allocs, &P->bytes, &st, np));
   } else {
     for (int l = 0; l < P->nlev; ++l) P->op32.push_back(make_op<float>(G->L[l], P->allocs, &P->bytes, &st, np));
@@ -1038,7 +1398,6 @@ extern "C" eb_status eb_poisson_setup(const eb_geom* G, const eb_solver_opts* op
     if (e == cudaSuccess) e = cudaGraphInstantiate(&P->gexec, P->graph, 0);
     if (e != cudaSuccess) st = cuda_fail(e, "graph capture");
   }
-  (void)stream;
   if (st != EB_OK) {
     eb_poisson_destroy(P);
     return st;
@@ -1059,6 +1418,7 @@ extern "C" void eb_poisson_destroy(eb_poisson* P) {
   if (P->h_norm) cudaFreeHost(P->h_norm);
   if (P->h_out) cudaFreeHost(P->h_out);
   for (void* p : P->allocs) cudaFree(p);
+  for (DevLevel& L : P->alg) free_level(L);
   delete P;
 }
 
@@ -1194,7 +1554,7 @@ extern "C" eb_status eb_poisson_solve(eb_poisson* P, const double* d_rhs, const 
     inf.bnorm = b;
     inf.rel_res = b > 0.0 ? r / b : 0.0;
     inf.bottom = P->bottom;
-    inf.levels = P->nlev;
+    inf.levels = P->nlev + (int)P->alg.size();
     inf.sweep_levels = P->sweep_levels;
     if (info) *info = inf;
     return st;
@@ -1294,7 +1654,7 @@ static std::vector<int> split_ctas(const std::vector<long long>& cells, int tota
   return size;
 }
 
-template <class T>
+template <class Item>
 static eb_status launch_batch_t(eb_poisson* const* P, int n, int max_iters, int grid_total, int smem, cudaStream_t s,
                                 double* kernel_ms) {
   std::vector<long long> cells(n);
@@ -1304,13 +1664,13 @@ static eb_status launch_batch_t(eb_poisson* const* P, int n, int max_iters, int 
   std::vector<int> mins(n);
   for (int i = 0; i < n; ++i) mins[i] = P[i]->sweep_levels ? 2 : 1;
   std::vector<int> size = split_ctas(cells, grid_total, std::max(2, nsm), mins);
-  std::vector<BatchItem<T>> items(n);
+  std::vector<Item> items(n);
   std::vector<int> cta_item;
   int start = 0;
   for (int i = 0; i < n; ++i) {
     eb_poisson* Q = P[i];
-    BatchItem<T>& it = items[i];
-    it.H = (const Hier<T>*)Q->d_hier;
+    Item& it = items[i];
+    it.H = (decltype(it.H))Q->d_hier;
     it.F = Q->d_fine;
     SolveCtl& c = it.ctl;
     c.tol = Q->o.tol;
@@ -1322,6 +1682,10 @@ static eb_status launch_batch_t(eb_poisson* const* P, int n, int max_iters, int 
     c.out = Q->d_out;
     c.trace = Q->d_stamps;
     c.max_iters = max_iters;
+    c.kry = Q->kry ? 1 : 0;
+    if (Q->rb && !c.kry) c.inner = 1;
+    c.fresh = Q->resumed ? 0 : 1;
+    Q->resumed = true;
     it.B = Barrier{Q->d_bar, (int*)(Q->d_bar + 2)};
     it.start = start;
     it.size = size[i];
@@ -1330,21 +1694,18 @@ static eb_status launch_batch_t(eb_poisson* const* P, int n, int max_iters, int 
     cudaMemsetAsync(Q->d_bar, 0, 4 * sizeof(unsigned), s);
     cudaMemsetAsync(Q->d_norms, 0, sizeof(unsigned long long) * (Q->o.max_cycles + 2), s);
   }
-  BatchItem<T>* d_items = nullptr;
+  Item* d_items = nullptr;
   int* d_cta = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&d_items, sizeof(BatchItem<T>) * n, s);
+  cudaError_t e = cudaMallocAsync((void**)&d_items, sizeof(Item) * n, s);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&d_cta, sizeof(int) * cta_item.size(), s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_items, items.data(), sizeof(BatchItem<T>) * n, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d_items, items.data(), sizeof(Item) * n, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_cta, cta_item.data(), sizeof(int) * cta_item.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = kernel_events(P[0]);
   if (e == cudaSuccess) {
     void* args[2] = {(void*)&d_items, (void*)&d_cta};
     cudaEventRecord(P[0]->kev[0], s);
-    bool sw = false;
-    for (int i = 0; i < n; ++i) sw = sw || P[i]->sweep_levels > 0;
-    e = cudaLaunchCooperativeKernel(batch_kernel(std::is_same<T, float>::value, sw), dim3(start), dim3(PT), args,
-                                    (size_t)smem, s);
+    e = cudaLaunchCooperativeKernel(batch_kernel(P[0]), dim3(start), dim3(PT), args, (size_t)smem, s);
     cudaEventRecord(P[0]->kev[1], s);
     counted();
   }
@@ -1366,6 +1727,7 @@ eb_status batch_prepare(eb_poisson* P, const double* rhs, const double* sigma, c
   cudaMemsetAsync(P->d_norm + 1, 0, sizeof(unsigned long long), s);
   eb_status st = launch_rhs64(P->G, rhs, sigma, P->b64, (double*)(P->d_norm + 1), s);
   if (st != EB_OK) return st;
+  P->resumed = false;
   k_copy_masked<<<blocks(F.g.ncell), 256, 0, s>>>(F.flags, F.g.ncell, phi, P->phi64);
   counted(2);
   return EB_OK;
@@ -1436,27 +1798,32 @@ eb_status batch_step(eb_poisson* const* P, int n, const double* const* rhs, cons
   int nsm = 0, per_sm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, P[0]->G->device);
   cudaError_t e = cudaSuccess;
-  bool sw = false;
-  for (int i = 0; i < n; ++i) sw = sw || P[i]->sweep_levels > 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel(mixed, sw), PT, smem);
-  if (e != cudaSuccess || per_sm < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "batch occupancy");
-  int total = nsm * std::min(per_sm, 1);
   if (fresh)
     for (int i = 0; i < n; ++i) {
       eb_status st = batch_prepare(P[i], rhs[i], sigma ? sigma[i] : nullptr, phi[i], s);
       if (st != EB_OK) return st;
     }
+  // one kernel per launch: the colour-split instances, then any with tile-streamed levels
+  std::vector<eb_poisson*> order(P, P + n);
+  std::stable_partition(order.begin(), order.end(), [](const eb_poisson* Q) { return Q->rb; });
   // as many instances per launch as their minimum CTA counts allow
   for (int b0 = 0, m = 0; b0 < n; b0 += m) {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel(order[b0]), PT, smem);
+    if (e != cudaSuccess || per_sm < 1)
+      return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "batch occupancy");
+    const int total = nsm;
     int need = 0;
-    for (m = 0; b0 + m < n; ++m) {
-      const int c = P[b0 + m]->sweep_levels ? 2 : 1;
+    for (m = 0; b0 + m < n && order[b0 + m]->rb == order[b0]->rb; ++m) {
+      const int c = order[b0 + m]->sweep_levels ? 2 : 1;
       if (need + c > total) break;
       need += c;
     }
     if (m == 0) m = 1;  // (total >= 2 on every device with a persistent kernel)
-    eb_status st = mixed ? launch_batch_t<float>(P + b0, m, max_iters, total, smem, s, kernel_ms)
-                         : launch_batch_t<double>(P + b0, m, max_iters, total, smem, s, kernel_ms);
+    eb_poisson* const* Q = order.data() + b0;
+    eb_status st;
+    if (!Q[0]->rb) st = launch_batch_t<BatchItem<float>>(Q, m, max_iters, total, smem, s, kernel_ms);
+    else if (mixed) st = launch_batch_t<RBatchItem<float>>(Q, m, max_iters, total, smem, s, kernel_ms);
+    else st = launch_batch_t<RBatchItem<double>>(Q, m, max_iters, total, smem, s, kernel_ms);
     if (st != EB_OK) return st;
   }
   for (int i = 0; i < n; ++i) {
@@ -1487,7 +1854,7 @@ void batch_info(eb_poisson* Q, eb_solve_info* inf) {
   inf->bnorm = b;
   inf->rel_res = b > 0.0 ? r / b : 0.0;
   inf->bottom = Q->bottom;
-  inf->levels = Q->nlev;
+  inf->levels = Q->nlev + (int)Q->alg.size();
   inf->sweep_levels = Q->sweep_levels;
 }
 
@@ -1664,7 +2031,10 @@ extern "C" eb_status eb_poisson_profile(eb_poisson* P, int kernel, int reps, dou
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, P->G->device);
   const int grid = P->persistent ? P->grid : nsm;
   auto launch = [&](int i) {
-    if (kernel == 0) {
+    if (P->rb) {
+      if (mixed) k_rb_phase<float><<<grid, PT, 0, s>>>((const RHier<float>*)P->d_hier, kernel, i & 1);
+      else k_rb_phase<double><<<grid, PT, 0, s>>>((const RHier<double>*)P->d_hier, kernel, i & 1);
+    } else if (kernel == 0) {
       if (mixed) k_dense_phase<float><<<grid, PT, 0, s>>>(P->op32[0], i & 1);
       else k_dense_phase<double><<<grid, PT, 0, s>>>(P->op64[0], i & 1);
     } else if (kernel == 1) {
