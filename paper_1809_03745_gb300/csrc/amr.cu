@@ -126,7 +126,7 @@ __global__ void k_cf_flux(const CFFace* faces, long long nface, const double* pc
 
 // fine rows of one CF side (one face per fine cell within a side)
 __global__ void k_cf_fine_apply(const CFFace* faces, long long t0, long long t1, const double* fl, double hf,
-                                double* rf) {
+                                double* rf) {  // hf < 0: the fluxes' share of A phi instead of b - A phi
   long long t = t0 + (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= t1) return;
   const CFFace& f = faces[t];
@@ -136,7 +136,7 @@ __global__ void k_cf_fine_apply(const CFFace* faces, long long t0, long long t1,
 // coarse rows next to the box: take the coarse face flux out, put minus the
 // mean fine flux in
 __global__ void k_cf_coarse_apply(const CFCoarse* cf, long long n, const double* fl, const double* pc, long long ncc,
-                                  double hc, int D, double* rc) {
+                                  double hc, int D, double sgn, double* rc) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   const CFCoarse& c = cf[t];
@@ -148,7 +148,7 @@ __global__ void k_cf_coarse_apply(const CFCoarse* cf, long long n, const double*
   }
   double fsum = 0.0;
   for (int k = 0; k < c.nfine; ++k) fsum += fl[c.fine[k]];
-  rc[c.ccell] += -own - fsum / (hc * (double)(1 << (D - 1)));
+  rc[c.ccell] += sgn * (-own - fsum / (hc * (double)(1 << (D - 1))));
 }
 
 __global__ void k_zero_under(BoxIdx B, double* rc, long long ncc) {
@@ -181,33 +181,20 @@ __global__ void k_restrict_under(BoxIdx B, const uint8_t* fflags, const double* 
   }
 }
 
-// phi_c += e_c outside the box; phi_f += e_c of the parent where the fine cell has the phase
-__global__ void k_add_coarse(BoxIdx B, const double* ec, double* pc, long long ncc) {
-  long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncc) return;
-  int I[3];
-  ijk3(B.nc, c, I);
-  if (under_box(B, I)) return;
-  pc[c] += ec[c];
-  pc[ncc + c] += ec[ncc + c];
-}
+// pf = e_c of the parent where the fine cell has the phase
 __global__ void k_prolong_const(BoxIdx B, const uint8_t* fflags, const double* ec, double* pf, long long ncc,
                                 long long nff) {
   long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= nff) return;
+  const unsigned fl = fflags[f];
+  if (!(fl & 3u)) return;
   int F[3];
   ijk3(B.nf, f, F);
   int I[3] = {0, 0, 0};
   for (int a = 0; a < B.D; ++a) I[a] = B.lo[a] + F[a] / 2;
   long long c = lin3(B.nc, I);
   for (int p = 0; p < 2; ++p)
-    if ((fflags[f] >> p) & 1) pf[p * nff + f] += ec[p * ncc + c];
-}
-__global__ void k_axpy_masked(const uint8_t* flags, long long n, const double* x, double* y) {
-  long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n) return;
-  for (int p = 0; p < 2; ++p)
-    if ((flags[c] >> p) & 1) y[p * n + c] += x[p * n + c];
+    if ((fl >> p) & 1) pf[p * nff + f] = ec[p * ncc + c];
 }
 __global__ void k_absmax2(const uint8_t* flags, long long n, const double* v, unsigned long long* out) {
   long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -219,124 +206,185 @@ __global__ void k_absmax2(const uint8_t* flags, long long n, const double* v, un
   if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
 
-// Composite vectors: coarse [2][ncc] (entries under the box and without an
-// unknown ignored) and fine [2][nff].  Partial sums per block, added on the
-// host in block order, so every dot product is deterministic.
-constexpr int DOT_BLOCKS = 512;
-__global__ void k_cv_dot(BoxIdx B, const uint8_t* flags, long long n, int coarse, const double* a, const double* b,
-                         double* part) {
-  __shared__ double sh[TBA];
-  double acc = 0.0;
-  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-    if (coarse) {
-      int I[3];
-      ijk3(B.nc, c, I);
-      if (under_box(B, I)) continue;
-    }
-    for (int p = 0; p < 2; ++p)
-      if ((flags[c] >> p) & 1) acc += a[p * n + c] * b[p * n + c];
-  }
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s2 = blockDim.x / 2; s2 > 0; s2 >>= 1) {
-    if ((int)threadIdx.x < s2) sh[threadIdx.x] += sh[threadIdx.x + s2];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-}
-// Dot products of w with m vectors at once (m <= CV_MAXV): per block the m
-// partial sums, part[i * gridDim.x + block]; the caller adds the blocks in
-// order (deterministic).  Coarse entries under the box are skipped.
+// Composite vectors: one [2][n] array per level.  The entries that count are
+// those of a level's own unknowns: `own` holds its flags with the cells under
+// the next finer box cleared.  Entries without them (and all of the second
+// phase's, where a group of four cells has none of it) are neither read nor
+// written.  Sums go block by block into `part`, and one block adds those in a
+// fixed order, so every dot product is deterministic.
+constexpr int DOT_BLOCKS = 608;
 constexpr int CV_MAXV = 14;
 struct CVPtrs {
   const double* v[CV_MAXV];
   double a[CV_MAXV];
 };
-__global__ void k_cv_mdot(BoxIdx B, const uint8_t* flags, long long n, int coarse, int m, CVPtrs V, const double* w,
-                          double* part) {
-  __shared__ double sh[CV_MAXV][TBA / 32];
-  double acc[CV_MAXV];
-#pragma unroll
-  for (int i = 0; i < CV_MAXV; ++i) acc[i] = 0.0;
-  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-    if (coarse) {
-      int I[3];
-      ijk3(B.nc, c, I);
-      if (under_box(B, I)) continue;
-    }
-    const unsigned f = flags[c];
-    for (int p = 0; p < 2; ++p) {
-      if (!((f >> p) & 1u)) continue;
-      const double wv = w[p * n + c];
-#pragma unroll
-      for (int i = 0; i < CV_MAXV; ++i)
-        if (i < m) acc[i] += V.v[i][p * n + c] * wv;
-    }
+__global__ void k_own_flags(BoxIdx B, const uint8_t* flags, long long n, int coarse, uint8_t* own) {
+  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n) return;
+  unsigned f = flags[c] & 3u;
+  if (f && coarse) {
+    int I[3];
+    ijk3(B.nc, c, I);
+    if (under_box(B, I)) f = 0;
   }
+  own[c] = (uint8_t)f;
+}
+__device__ __forceinline__ void ldq(const double* p, double v[4]) {
+  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = b.x;
+  v[3] = b.y;
+}
+__device__ __forceinline__ void stq(double* p, const double v[4]) {
+  reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
+  reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
+}
+// the lanes of a group of four cells that carry phase p, as bits
+__device__ __forceinline__ unsigned lanes4(unsigned w, int p) {
+  const unsigned b = (w >> p) & 0x01010101u;
+  return (b & 1u) | ((b >> 7) & 2u) | ((b >> 14) & 4u) | ((b >> 21) & 8u);
+}
+template <int NS>
+__device__ __forceinline__ void block_sums(double (&acc)[NS], int m, double* part) {
+  __shared__ double sh[NS][TBA / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-  for (int i = 0; i < CV_MAXV; ++i) {
+  for (int i = 0; i < NS; ++i) {
+    if (i >= m) continue;
     double a = acc[i];
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if (lane == 0) sh[i][wid] = a;
   }
   __syncthreads();
-  if (threadIdx.x < m) {
+  if ((int)threadIdx.x < m) {
     double t = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += sh[threadIdx.x][k];
+    for (int k = 0; k < TBA / 32; ++k) t += sh[threadIdx.x][k];
     part[threadIdx.x * gridDim.x + blockIdx.x] = t;
   }
 }
-// w -= sum_i a_i v_i on the entries with an unknown (others 0), and from the
-// same pass the per-block partial sums of the new w . w over the entries a
-// dot product counts (the caller adds the blocks in order: deterministic)
-__global__ void k_cv_maxpy_norm(BoxIdx B, const uint8_t* flags, long long n, int coarse, int m, CVPtrs V, double* w,
-                                double* part) {
-  __shared__ double sh[TBA];
-  double acc = 0.0;
-  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-    bool counted = true;
-    if (coarse) {
-      int I[3];
-      ijk3(B.nc, c, I);
-      counted = !under_box(B, I);
-    }
-    const unsigned f = flags[c];
-    for (int p = 0; p < 2; ++p) {
-      if (!((f >> p) & 1u)) {
-        w[p * n + c] = 0.0;
-        continue;
-      }
-      double t = w[p * n + c];
+// (v_i, w) for i < m; *go = 0 skips the pass
+template <int MAXM>
+__global__ void __launch_bounds__(TBA) k_cv_mdot(const uint8_t* __restrict__ own, long long n, int m, CVPtrs V,
+                                                 const double* __restrict__ w, const int* go, double* part) {
+  if (go && !*go) return;
+  double acc[MAXM];
 #pragma unroll
-      for (int i = 0; i < CV_MAXV; ++i)
-        if (i < m) t -= V.a[i] * V.v[i][p * n + c];
-      w[p * n + c] = t;
-      if (counted) acc += t * t;
+  for (int i = 0; i < MAXM; ++i) acc[i] = 0.0;
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; 4 * q < n; q += (long long)gridDim.x * blockDim.x) {
+    const unsigned f = reinterpret_cast<const unsigned*>(own)[q];
+    for (int p = 0; p < 2; ++p) {
+      const unsigned ln = lanes4(f, p);
+      if (!ln) continue;
+      const long long c = p * n + 4 * q;
+      double wv[4];
+      ldq(w + c, wv);
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (!((ln >> e) & 1u)) wv[e] = 0.0;
+#pragma unroll
+      for (int i = 0; i < MAXM; ++i) {
+        if (i >= m) continue;
+        double v[4];
+        ldq(V.v[i] + c, v);
+        if (ln != 15u) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (!((ln >> e) & 1u)) v[e] = 0.0;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[i] += v[e] * wv[e];
+      }
     }
   }
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s2 = blockDim.x / 2; s2 > 0; s2 >>= 1) {
-    if ((int)threadIdx.x < s2) sh[threadIdx.x] += sh[threadIdx.x + s2];
-    __syncthreads();
+  block_sums<MAXM>(acc, m, part);
+}
+// w -= sum_i h_i v_i, and the block sums of the new (w, w); *go = 0 skips the pass
+__global__ void __launch_bounds__(TBA) k_cv_maxpy_norm(const uint8_t* __restrict__ own, long long n, int m, CVPtrs V,
+                                                       const double* __restrict__ h, double* __restrict__ w,
+                                                       const int* go, double* part) {
+  if (go && !*go) return;
+  double acc[1] = {0.0};
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; 4 * q < n; q += (long long)gridDim.x * blockDim.x) {
+    const unsigned f = reinterpret_cast<const unsigned*>(own)[q];
+    for (int p = 0; p < 2; ++p) {
+      const unsigned ln = lanes4(f, p);
+      if (!ln) continue;
+      const long long c = p * n + 4 * q;
+      double t[4], t0[4];
+      ldq(w + c, t);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) t0[e] = t[e];
+      for (int i = 0; i < m; ++i) {
+        double v[4];
+        ldq(V.v[i] + c, v);
+        const double a = h[i];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) t[e] -= a * v[e];
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (!((ln >> e) & 1u)) t[e] = t0[e];
+        else acc[0] += t[e] * t[e];
+      }
+      stq(w + c, t);
+    }
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+  block_sums<1>(acc, 1, part);
 }
-
-// y = a x + b y on the entries with an unknown
-__global__ void k_cv_axpby(const uint8_t* flags, long long n, double a, const double* x, double b, double* y) {
-  long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n) return;
-  for (int p = 0; p < 2; ++p)
-    if ((flags[c] >> p) & 1) y[p * n + c] = a * x[p * n + c] + b * y[p * n + c];
-    else y[p * n + c] = 0.0;
+// one block: the m sums over nlev levels' blocks, a warp each, in a fixed
+// order; what follows from them (the Gram-Schmidt step's numbers) on thread 0:
+//   0  out[0..m) = the sums (3: if *go)
+//   1  out[0] = the new norm after the first pass; *go = the second one is
+//      needed (the norm fell below 1/sqrt(2) of the old one, sqrt(in[m0]),
+//      the criterion of Daniel, Gragg, Kaufman and Stewart)
+//   2  out[0] = the norm after the second pass, if it ran (4: the norm)
+__global__ void k_cv_finish(const double* part, int nlev, long long lstride, int m, int what, const double* in, int m0,
+                            int* go, double* out) {
+  if ((what == 2 || what == 3) && !*go) return;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (wid >= m) return;
+  double s = 0.0;
+  for (int l = 0; l < nlev; ++l)
+    for (int k = lane; k < DOT_BLOCKS; k += 32) s += part[l * lstride + (long long)wid * DOT_BLOCKS + k];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane) return;
+  if (what == 0 || what == 3) {
+    out[wid] = s;
+    return;
+  }
+  const double w1 = sqrt(fmax(s, 0.0));
+  out[0] = w1;
+  if (what == 1) *go = w1 < sqrt(fmax(in[m0], 0.0)) * 0.70710678118654752440 ? 1 : 0;
 }
-// w = b - r (the operator applied to the vector whose residual r was formed)
-__global__ void k_cv_sub(const uint8_t* flags, long long n, const double* b, const double* r, double* w) {
-  long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// w *= 1 / *norm (left alone when it is not positive)
+__global__ void k_cv_scale(const uint8_t* __restrict__ own, long long n, const double* norm, double* __restrict__ w) {
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (4 * q >= n) return;
+  const double a = *norm;
+  if (!(a > 0.0)) return;
+  const double s = 1.0 / a;
+  const unsigned f = reinterpret_cast<const unsigned*>(own)[q];
+  for (int p = 0; p < 2; ++p) {
+    if (!lanes4(f, p)) continue;
+    double t[4];
+    ldq(w + p * n + 4 * q, t);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) t[e] *= s;
+    stq(w + p * n + 4 * q, t);
+  }
+}
+// x += sum_i a_i z_i on a level's unknowns (x: the caller's array)
+__global__ void k_cv_update(const uint8_t* __restrict__ flags, long long n, int m, CVPtrs Z, double* __restrict__ x) {
+  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n) return;
-  for (int p = 0; p < 2; ++p) w[p * n + c] = ((flags[c] >> p) & 1) ? b[p * n + c] - r[p * n + c] : 0.0;
+  const unsigned f = flags[c];
+  for (int p = 0; p < 2; ++p) {
+    if (!((f >> p) & 1u)) continue;
+    double t = x[p * n + c];
+    for (int i = 0; i < m; ++i) t += Z.a[i] * Z.v[i][p * n + c];
+    x[p * n + c] = t;
+  }
 }
 
 }  // namespace
@@ -358,8 +406,9 @@ struct AmrLevel {
   long long n = 0;
   double h = 0.0;
   const uint8_t* flags = nullptr;  // finest-level flags of G (owned by G)
+  uint8_t* own = nullptr;          // the same without the cells under the next box
   double *pc = nullptr;            // phi with the cells under the next box replaced by the finer means
-  double *r = nullptr, *b0 = nullptr, *e = nullptr, *kap = nullptr;
+  double *r = nullptr, *b0 = nullptr, *kap = nullptr;
 };
 
 // The coupling of levels l-1 (coarse) and l (fine), stored at index l
@@ -384,8 +433,11 @@ struct eb_amr {
   unsigned long long* d_norm = nullptr;
   // FGMRES work space (allocated at the first solve)
   std::vector<CVec> V, Z;
-  CVec bvec, tmp;
-  double* d_part = nullptr;
+  double* d_part = nullptr;  // block sums
+  double* d_h = nullptr;     // Gram-Schmidt numbers of the current step
+  int* d_go = nullptr;
+  double* h_h = nullptr;     // their copy (pinned)
+  std::vector<cudaEvent_t> ev;  // pairs around the V-cycles of a solve
   std::vector<void*> allocs;
   long long bytes = 0;
   // persistent solve launches of the last composite solve, coarse [0] and
@@ -416,6 +468,8 @@ extern "C" void eb_amr_destroy(eb_amr* A) {
     eb_geom_destroy(v.G);
   }
   for (void* p : A->allocs) cudaFree(p);
+  for (cudaEvent_t e : A->ev) cudaEventDestroy(e);
+  if (A->h_h) cudaFreeHost(A->h_h);
   delete A;
 }
 
@@ -568,11 +622,16 @@ extern "C" eb_status eb_amr_setup_levels(const eb_geom_desc* desc, int n_levels,
     if (l > 0) v.kap = (double*)alloc(b2);
     v.r = (double*)alloc(b2);
     v.b0 = (double*)alloc(b2);
-    v.e = (double*)alloc(b2);
+    v.own = (uint8_t*)alloc(v.n);
   }
   A->d_status = (int*)alloc(sizeof(int));
   A->d_norm = (unsigned long long*)alloc(sizeof(unsigned long long) * 2);
   if (st != EB_OK) return amr_fail(A, st);
+  for (int l = 0; l < L; ++l) {
+    AmrLevel& v = A->lv[l];
+    k_own_flags<<<nb(v.n), TBA, 0, s>>>(A->pr[l + 1 < L ? l + 1 : l].B, v.flags, v.n, l < L - 1, v.own);
+    if (v.pc) cudaMemsetAsync(v.pc, 0, sizeof(double) * 2 * v.n, s);
+  }
   for (int l = 1; l < L && st == EB_OK; ++l) {
     AmrPair& P = A->pr[l];
     st = build_cf(A->lv[l].G, A->lv[l - 1].G, P.cfb, P.faces, P.cfaces, A->d_status, s);
@@ -593,11 +652,11 @@ extern "C" eb_status eb_amr_setup_levels(const eb_geom_desc* desc, int n_levels,
   oc.inner_cycles = 1;
   oc.nu1 = oc.nu2 = 3;
   oc.bottom_sweeps = std::min(oc.bottom_sweeps, 32);
-  st = poisson_setup(A->lv[0].G, &oc, false, &A->lv[0].P);
+  st = poisson_setup(A->lv[0].G, &oc, PS_PLAIN, &A->lv[0].P);
   A->lv[0].P0 = A->lv[0].P;
   for (int l = 1; l < L && st == EB_OK; ++l) {
-    st = poisson_setup(A->lv[l].G, &A->o, false, &A->lv[l].P);
-    if (st == EB_OK) st = poisson_setup(A->lv[l].G0, &oc, false, &A->lv[l].P0);
+    st = poisson_setup(A->lv[l].G, &A->o, PS_OPERATOR, &A->lv[l].P);
+    if (st == EB_OK) st = poisson_setup(A->lv[l].G0, &oc, PS_PLAIN, &A->lv[l].P0);
   }
   if (st != EB_OK) return amr_fail(A, st);
   if (cudaStreamSynchronize(s) != cudaSuccess) return amr_fail(A, cuda_fail(cudaGetLastError(), "amr setup"));
@@ -659,24 +718,36 @@ static eb_status amr_rhs(eb_amr* A, const double* const* rhs, const double* cons
   return st;
 }
 
-// composite residual into lv[l].r: every level's values under the next finer
-// box are first replaced by the finer level's means, finest first
-static eb_status amr_resid(eb_amr* A, const double* const* phi, cudaStream_t s) {
+// The composite operator on levels >= lmin.  phi's values under a finer box
+// are first replaced by the finer level's means, finest first: in place
+// (copy = false), or in lv[l].pc.  out[l] = b[l] - A phi, or A phi where b is
+// null (entries without an unknown left alone).  Rows under a box come out
+// 0, except on a level whose out is the remainder of a correction (zero =
+// false), where restrict_down sets them.
+static eb_status amr_apply(eb_amr* A, const double* const* b, double* const* phi, double* const* out, int lmin,
+                           bool copy, bool zero, cudaStream_t s) {
   const int L = A->L;
+  const double sgn = b ? 1.0 : -1.0;
   const double* val[AMR_MAXL];
   val[L - 1] = phi[L - 1];
   for (int l = L - 2; l >= 0; --l) {
     AmrLevel &c = A->lv[l], &f = A->lv[l + 1];
-    cudaMemcpyAsync(c.pc, phi[l], 2 * c.n * sizeof(double), cudaMemcpyDeviceToDevice, s);
-    k_avg_down<<<nb(box_cells(A->pr[l + 1].B)), TBA, 0, s>>>(A->pr[l + 1].B, c.flags, f.flags, f.kap, val[l + 1],
-                                                            c.pc, c.n, f.n);
+    val[l] = phi[l];
+    if (l < lmin) continue;  // read outside its box alone
+    double* pc = phi[l];
+    if (copy) {
+      pc = c.pc;
+      cudaMemcpyAsync(pc, phi[l], 2 * c.n * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    }
+    k_avg_down<<<nb(box_cells(A->pr[l + 1].B)), TBA, 0, s>>>(A->pr[l + 1].B, c.flags, f.flags, f.kap, val[l + 1], pc,
+                                                            c.n, f.n);
     note_launch();
-    val[l] = c.pc;
+    val[l] = pc;
   }
   eb_status st = EB_OK;
-  for (int l = 0; l < L && st == EB_OK; ++l) st = poisson_residual_view(A->lv[l].P, A->lv[l].b0, val[l], A->lv[l].r, s);
+  for (int l = lmin; l < L && st == EB_OK; ++l) st = poisson_apply(A->lv[l].P, b ? b[l] : nullptr, val[l], sgn, out[l], s);
   if (st != EB_OK) return st;
-  for (int l = 1; l < L; ++l) {
+  for (int l = std::max(1, lmin); l < L; ++l) {
     const AmrPair& P = A->pr[l];
     AmrLevel &c = A->lv[l - 1], &f = A->lv[l];
     if (!P.nface) continue;
@@ -684,18 +755,30 @@ static eb_status amr_resid(eb_amr* A, const double* const* phi, cudaStream_t s) 
     note_launch();
     for (int sd = 0; sd < P.cfb.nside; ++sd) {
       long long t0 = P.cfb.off[sd], t1 = P.cfb.off[sd + 1];
-      k_cf_fine_apply<<<nb(t1 - t0), TBA, 0, s>>>(P.faces, t0, t1, P.fl, f.h, f.r);
+      k_cf_fine_apply<<<nb(t1 - t0), TBA, 0, s>>>(P.faces, t0, t1, P.fl, sgn * f.h, out[l]);
       note_launch();
     }
-    k_cf_coarse_apply<<<nb(P.ncface), TBA, 0, s>>>(P.cfaces, P.ncface, P.fl, val[l - 1], c.n, c.h, A->D, c.r);
+    if (l - 1 < lmin) continue;
+    k_cf_coarse_apply<<<nb(P.ncface), TBA, 0, s>>>(P.cfaces, P.ncface, P.fl, val[l - 1], c.n, c.h, A->D, sgn, out[l - 1]);
     note_launch();
   }
-  for (int l = 1; l < L; ++l) {
-    k_zero_under<<<nb(box_cells(A->pr[l].B)), TBA, 0, s>>>(A->pr[l].B, A->lv[l - 1].r, A->lv[l - 1].n);
+  for (int l = std::max(1, lmin + 1); l < L && zero; ++l) {
+    k_zero_under<<<nb(box_cells(A->pr[l].B)), TBA, 0, s>>>(A->pr[l].B, out[l - 1], A->lv[l - 1].n);
     note_launch();
   }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? EB_OK : cuda_fail(e, "composite residual");
+}
+
+// composite residual of the data in lv[l].b0 into lv[l].r
+static eb_status amr_resid(eb_amr* A, double* const* phi, bool copy, cudaStream_t s) {
+  const double* b[AMR_MAXL];
+  double* r[AMR_MAXL];
+  for (int l = 0; l < A->L; ++l) {
+    b[l] = A->lv[l].b0;
+    r[l] = A->lv[l].r;
+  }
+  return amr_apply(A, b, phi, r, 0, copy, true, s);
 }
 
 static eb_status amr_norm(eb_amr* A, cudaStream_t s, double* out) {
@@ -727,7 +810,8 @@ extern "C" eb_status eb_amr_residual_levels(eb_amr* A, const double* const* d_rh
   }
   cudaStream_t s = (cudaStream_t)stream;
   eb_status st = amr_rhs(A, d_rhs, d_sig, s);
-  if (st == EB_OK) st = amr_resid(A, d_phi, s);
+  for (int l = 0; l < A->L; ++l) cudaMemsetAsync(A->lv[l].r, 0, 2 * A->lv[l].n * sizeof(double), s);
+  if (st == EB_OK) st = amr_resid(A, const_cast<double* const*>(d_phi), true, s);  // copies: d_phi is only read
   if (st != EB_OK) return st;
   for (int l = 0; l < A->L; ++l)
     cudaMemcpyAsync(d_r[l], A->lv[l].r, 2 * A->lv[l].n * sizeof(double), cudaMemcpyDeviceToDevice, s);
@@ -749,183 +833,135 @@ extern "C" eb_status eb_amr_residual(eb_amr* A, const double* d_rhs_c, const dou
   return eb_amr_residual_levels(A, rhs, sig, phi, r, stream);
 }
 
-// level l's cells under the next finer box are skipped by the dot products
-static const BoxIdx& dot_box(const eb_amr* A, int l) { return A->pr[l + 1 < A->L ? l + 1 : l].B; }
-
-static double cv_dot(eb_amr* A, const CVec& a, const CVec& b, cudaStream_t s) {
-  const int L = A->L;
-  for (int l = 0; l < L; ++l) {
-    const AmrLevel& v = A->lv[l];
-    k_cv_dot<<<DOT_BLOCKS, TBA, 0, s>>>(dot_box(A, l), v.flags, v.n, l < L - 1, a.v[l], b.v[l],
-                                        A->d_part + l * DOT_BLOCKS);
-    note_launch();
-  }
-  std::vector<double> h(L * DOT_BLOCKS);
-  cudaMemcpyAsync(h.data(), A->d_part, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, s);
-  cudaStreamSynchronize(s);
-  double t = 0.0;
-  for (int i = 0; i < L * DOT_BLOCKS; ++i) t += h[i];
-  return t;
+static CVPtrs cv_ptrs(const std::vector<CVec>& V, int l, int m) {
+  CVPtrs p{};
+  for (int i = 0; i < m; ++i) p.v[i] = V[i].v[l];
+  return p;
 }
-static void cv_axpby(eb_amr* A, double a, const CVec& x, double b, const CVec& y, cudaStream_t s) {
+static constexpr long long CV_PART = (long long)CV_MAXV * DOT_BLOCKS;  // block sums per level
+
+// the sums of m vectors V[0..m) (and w itself when self) with w into d_h[0..)
+static void cv_mdot(eb_amr* A, int m, const CVec& w, bool self, const int* go, double* out, cudaStream_t s) {
+  const int k = m + (self ? 1 : 0);
   for (int l = 0; l < A->L; ++l) {
-    k_cv_axpby<<<nb(A->lv[l].n), TBA, 0, s>>>(A->lv[l].flags, A->lv[l].n, a, x.v[l], b, y.v[l]);
-    note_launch();
-  }
-}
-static void cv_copy(eb_amr* A, const CVec& x, const CVec& y, cudaStream_t s) {
-  for (int l = 0; l < A->L; ++l)
-    cudaMemcpyAsync(y.v[l], x.v[l], 2 * A->lv[l].n * sizeof(double), cudaMemcpyDeviceToDevice, s);
-}
-
-// h[i] = (V[i], w) for i < m, all levels, one launch per level and one sync;
-// with `self` also h[m] = (w, w), from the same pass over w
-static void cv_mdot(eb_amr* A, int m, const CVec& w, double* h, cudaStream_t s, bool self = false) {
-  const int L = A->L;
-  CVPtrs p[AMR_MAXL] = {};
-  for (int l = 0; l < L; ++l) {
-    for (int i = 0; i < m; ++i) p[l].v[i] = A->V[i].v[l];
-    if (self) p[l].v[m] = w.v[l];
-  }
-  if (self) ++m;
-  for (int l = 0; l < L; ++l) {
     const AmrLevel& v = A->lv[l];
-    k_cv_mdot<<<DOT_BLOCKS, TBA, 0, s>>>(dot_box(A, l), v.flags, v.n, l < L - 1, m, p[l], w.v[l],
-                                         A->d_part + l * CV_MAXV * DOT_BLOCKS);
+    CVPtrs p = cv_ptrs(A->V, l, m);
+    if (self) p.v[m] = w.v[l];
+    double* part = A->d_part + l * CV_PART;
+    // fewer accumulators leave registers for more loads in flight
+    if (k <= 4) k_cv_mdot<4><<<DOT_BLOCKS, TBA, 0, s>>>(v.own, v.n, k, p, w.v[l], go, part);
+    else if (k <= 8) k_cv_mdot<8><<<DOT_BLOCKS, TBA, 0, s>>>(v.own, v.n, k, p, w.v[l], go, part);
+    else k_cv_mdot<CV_MAXV><<<DOT_BLOCKS, TBA, 0, s>>>(v.own, v.n, k, p, w.v[l], go, part);
     note_launch();
   }
-  std::vector<double> hp(L * CV_MAXV * DOT_BLOCKS);
-  cudaMemcpyAsync(hp.data(), A->d_part, sizeof(double) * hp.size(), cudaMemcpyDeviceToHost, s);
-  cudaStreamSynchronize(s);
-  for (int i = 0; i < m; ++i) {
-    double t = 0.0;
-    for (int l = 0; l < L; ++l)
-      for (int b = 0; b < DOT_BLOCKS; ++b) t += hp[l * CV_MAXV * DOT_BLOCKS + i * DOT_BLOCKS + b];
-    h[i] = t;
-  }
+  k_cv_finish<<<1, 32 * CV_MAXV, 0, s>>>(A->d_part, A->L, CV_PART, k, go ? 3 : 0, nullptr, 0, A->d_go, out);
+  note_launch();
 }
-// w -= sum_{i < m} h[i] V[i], returning the new (w, w) from the same pass
-static double cv_maxpy_norm(eb_amr* A, int m, const double* h, const CVec& w, cudaStream_t s) {
-  const int L = A->L;
-  for (int l = 0; l < L; ++l) {
-    CVPtrs p{};
-    for (int i = 0; i < m; ++i) {
-      p.v[i] = A->V[i].v[l];
-      p.a[i] = h[i];
-    }
+static void cv_maxpy_norm(eb_amr* A, int m, const double* h, const CVec& w, const int* go, int what, const double* in,
+                          double* out, cudaStream_t s) {
+  for (int l = 0; l < A->L; ++l) {
     const AmrLevel& v = A->lv[l];
-    k_cv_maxpy_norm<<<DOT_BLOCKS, TBA, 0, s>>>(dot_box(A, l), v.flags, v.n, l < L - 1, m, p, w.v[l],
-                                               A->d_part + l * DOT_BLOCKS);
+    k_cv_maxpy_norm<<<DOT_BLOCKS, TBA, 0, s>>>(v.own, v.n, m, cv_ptrs(A->V, l, m), h, w.v[l], go, A->d_part + l * CV_PART);
     note_launch();
   }
-  std::vector<double> hp(L * DOT_BLOCKS);
-  cudaMemcpyAsync(hp.data(), A->d_part, sizeof(double) * hp.size(), cudaMemcpyDeviceToHost, s);
-  cudaStreamSynchronize(s);
-  double t = 0.0;
-  for (int i = 0; i < L * DOT_BLOCKS; ++i) t += hp[i];
-  return t;
+  k_cv_finish<<<1, 32, 0, s>>>(A->d_part, A->L, CV_PART, 1, what, in, m, A->d_go, out);
+  note_launch();
 }
-
-// accuracy asked of the multigrid corrections inside one FAC step: loose
-// enough that each stops after its first V-cycle
-constexpr double FAC_TOL = 3e-1;
+static void cv_scale(eb_amr* A, const double* norm, const CVec& w, cudaStream_t s) {
+  for (int l = 0; l < A->L; ++l) {
+    const AmrLevel& v = A->lv[l];
+    k_cv_scale<<<nb((v.n + 3) / 4), TBA, 0, s>>>(v.own, v.n, norm, w.v[l]);
+    note_launch();
+  }
+}
 
 // w[l] for l = L-2 .. lmin: cells under the next finer box take the mean of
 // that level's children (finest first, so every level sees the whole remainder)
-static void restrict_down(eb_amr* A, const CVec& w, int lmin, cudaStream_t s) {
+static void restrict_down(eb_amr* A, double* const* w, int lmin, cudaStream_t s) {
   for (int l = A->L - 2; l >= lmin; --l) {
     const AmrLevel &c = A->lv[l], &f = A->lv[l + 1];
-    k_zero_under<<<nb(box_cells(A->pr[l + 1].B)), TBA, 0, s>>>(A->pr[l + 1].B, w.v[l], c.n);
-    note_launch();
-    k_restrict_under<<<nb(box_cells(A->pr[l + 1].B)), TBA, 0, s>>>(A->pr[l + 1].B, f.flags, w.v[l + 1], w.v[l], c.n,
-                                                                   f.n);
+    k_restrict_under<<<nb(box_cells(A->pr[l + 1].B)), TBA, 0, s>>>(A->pr[l + 1].B, f.flags, w[l + 1], w[l], c.n, f.n);
     note_launch();
   }
+}
+
+// events around the next V-cycle of a solve
+static cudaEvent_t* next_events(eb_amr* A, size_t* used) {
+  while (A->ev.size() < *used + 2) {
+    cudaEvent_t e = nullptr;
+    if (cudaEventCreate(&e) != cudaSuccess) return nullptr;
+    A->ev.push_back(e);
+  }
+  *used += 2;
+  return A->ev.data() + *used - 2;
 }
 
 // z = M^-1 v: one multiplicative FAC sweep from zero, coarse to fine: a
-// correction of level 0 over the domain (the finer parts of v restricted
-// under the boxes), added constant per parent on level 1; then on every finer
-// level a correction of what remains there (zero Dirichlet CF sides), the
-// remainder of the still finer levels restricted under its box, added to the
-// level and constant per parent on the next.  Uses lv[].r / e and tmp.
-static eb_status fac_apply(eb_amr* A, const CVec& v, const CVec& z, int* cycles, cudaStream_t s) {
-  const double tol = FAC_TOL;
+// V-cycle on level 0 over the domain (the finer parts of v restricted under
+// the boxes, into v's entries there, which nothing else reads), constant per
+// parent on level 1; then on every finer level a V-cycle on what remains there,
+// v - A z (zero Dirichlet CF sides; the remainder of the still finer levels,
+// where z is still zero, restricted under its box), added to the level and
+// constant per parent on the next.  (Passing the whole of z on instead of the
+// level's own correction stalls with four levels.)  Only the levels that a
+// correction needs are applied, and A z is subtracted from v in the same
+// pass.  Uses lv[].r for the remainders and lv[].pc for inner corrections.
+static eb_status fac_apply(eb_amr* A, const CVec& v, const CVec& z, int* cycles, size_t* used, cudaStream_t s) {
   const int L = A->L;
-  cv_copy(A, v, A->tmp, s);
-  restrict_down(A, A->tmp, 0, s);
-  int cyc = 0, outer = 0;
-  double kms = 0.0;
-  eb_status st = poisson_solve_b(A->lv[0].P, A->tmp.v[0], A->lv[0].e, tol, &cyc, s, &outer, &kms);
-  *cycles += cyc;
-  amr_count(A, 0, cyc, outer, kms);
-  if (st != EB_OK) return st;
-  for (int l = 0; l < L; ++l) cudaMemsetAsync(z.v[l], 0, 2 * A->lv[l].n * sizeof(double), s);
-  for (int l = 0; l < L; ++l) {
-    if (l > 0) {
-      // what remains on levels l and finer: v - A z, restricted into level l
-      st = amr_resid(A, z.v, s);
-      if (st != EB_OK) return st;
-      for (int k = l; k < L; ++k) {
-        const AmrLevel& q = A->lv[k];
-        k_cv_sub<<<nb(q.n), TBA, 0, s>>>(q.flags, q.n, A->bvec.v[k], q.r, A->tmp.v[k]);  // (A z)_k
-        note_launch();
-        k_cv_axpby<<<nb(q.n), TBA, 0, s>>>(q.flags, q.n, 1.0, v.v[k], -1.0, A->tmp.v[k]);  // v_k - (A z)_k
-        note_launch();
-      }
-      restrict_down(A, A->tmp, l, s);
-      st = poisson_solve_b(A->lv[l].P0, A->tmp.v[l], A->lv[l].e, tol, &cyc, s, &outer, &kms);
-      *cycles += cyc;
-      amr_count(A, 1, cyc, outer, kms);
-      if (st != EB_OK) return st;
-    }
-    const AmrLevel& c = A->lv[l];
-    if (l < L - 1) {
-      const AmrLevel& f = A->lv[l + 1];
-      k_add_coarse<<<nb(c.n), TBA, 0, s>>>(A->pr[l + 1].B, c.e, z.v[l], c.n);
-      note_launch();
-      k_prolong_const<<<nb(f.n), TBA, 0, s>>>(A->pr[l + 1].B, f.flags, c.e, z.v[l + 1], c.n, f.n);
-      note_launch();
-    } else {
-      k_axpy_masked<<<nb(c.n), TBA, 0, s>>>(c.flags, c.n, c.e, z.v[l]);
-      note_launch();
-    }
-  }
-  return EB_OK;
-}
-
-// w = A z (homogeneous operator) = b - r(z)
-static eb_status op_apply(eb_amr* A, const CVec& z, const CVec& w, cudaStream_t s) {
-  eb_status st = amr_resid(A, z.v, s);
-  if (st != EB_OK) return st;
-  for (int l = 0; l < A->L; ++l) {
-    const AmrLevel& q = A->lv[l];
-    k_cv_sub<<<nb(q.n), TBA, 0, s>>>(q.flags, q.n, A->bvec.v[l], q.r, w.v[l]);
+  double* rem[AMR_MAXL];
+  for (int l = 0; l < L; ++l) rem[l] = A->lv[l].r;
+  restrict_down(A, v.v, 0, s);
+  for (int l = 2; l < L; ++l) cudaMemsetAsync(z.v[l], 0, 2 * A->lv[l].n * sizeof(double), s);
+  eb_status st = poisson_vcycle(A->lv[0].P, v.v[0], z.v[0], false, next_events(A, used), s);
+  const double* e = z.v[0];
+  for (int l = 1; l < L && st == EB_OK; ++l) {
+    const AmrLevel& f = A->lv[l];
+    k_prolong_const<<<nb(f.n), TBA, 0, s>>>(A->pr[l].B, f.flags, e, z.v[l], A->lv[l - 1].n, f.n);
     note_launch();
-    if (l < A->L - 1) {
-      k_zero_under<<<nb(box_cells(A->pr[l + 1].B)), TBA, 0, s>>>(A->pr[l + 1].B, w.v[l], q.n);
+    st = amr_apply(A, v.v, z.v, rem, l, false, false, s);
+    if (st != EB_OK) break;
+    restrict_down(A, rem, l, s);
+    if (l == L - 1) {
+      st = poisson_vcycle(f.P0, rem[l], z.v[l], true, next_events(A, used), s);
+    } else {
+      st = poisson_vcycle(f.P0, rem[l], f.pc, false, next_events(A, used), s);
+      CVPtrs p{};
+      p.v[0] = f.pc;
+      p.a[0] = 1.0;
+      k_cv_update<<<nb(f.n), TBA, 0, s>>>(f.own, f.n, 1, p, z.v[l]);
       note_launch();
+      e = f.pc;
     }
   }
-  return EB_OK;
+  *cycles += L;
+  return st;
 }
 
 static constexpr int GM = 12;  // FGMRES restart length
+// d_h: the first pass's sums, the second one's, the new norm, and the flag
+static constexpr int H2 = CV_MAXV, HN = 2 * CV_MAXV, HGO = HN + 2, HLEN = HGO + 2;
 
 static eb_status amr_workspace(eb_amr* A) {
   if (!A->V.empty()) return EB_OK;
   eb_status st = EB_OK;
   auto vec = [&]() {
     CVec v;
-    for (int l = 0; l < A->L; ++l)
+    for (int l = 0; l < A->L; ++l) {
       v.v[l] = (double*)dev_alloc(A->allocs, 2 * A->lv[l].n * sizeof(double), &A->bytes, &st);
+      if (v.v[l]) cudaMemset(v.v[l], 0, 2 * A->lv[l].n * sizeof(double));
+    }
     return v;
   };
   for (int i = 0; i <= GM; ++i) A->V.push_back(vec());
   for (int i = 0; i < GM; ++i) A->Z.push_back(vec());
-  A->bvec = vec();
-  A->tmp = vec();
-  A->d_part = (double*)dev_alloc(A->allocs, A->L * CV_MAXV * DOT_BLOCKS * sizeof(double), &A->bytes, &st);
+  A->d_part = (double*)dev_alloc(A->allocs, A->L * CV_PART * sizeof(double), &A->bytes, &st);
+  A->d_h = (double*)dev_alloc(A->allocs, HLEN * sizeof(double), &A->bytes, &st);
+  A->d_go = (int*)(A->d_h + HGO);
+  if (st == EB_OK && !A->h_h) {
+    cudaError_t e = cudaMallocHost(&A->h_h, HLEN * sizeof(double));
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) st = cuda_fail(e, "composite work space");
+  }
   if (st != EB_OK) {
     A->V.clear();
     A->Z.clear();
@@ -947,31 +983,24 @@ extern "C" eb_status eb_amr_solve_levels(eb_amr* A, const double* const* d_rhs, 
   const long long launches0 = launch_total();
   eb_status st = amr_workspace(A);
   if (st != EB_OK) return st;
+  for (int l = 0; l < L; ++l) poisson_vcycle_begin(A->lv[l].P0, s);
   // b: the composite residual at phi = 0
-  CVec zero;
-  for (int l = 0; l < L; ++l) {
-    zero.v[l] = A->lv[l].e;
-    cudaMemsetAsync(A->lv[l].e, 0, 2 * A->lv[l].n * sizeof(double), s);
-  }
+  for (int l = 0; l < L; ++l) cudaMemsetAsync(A->Z[0].v[l], 0, 2 * A->lv[l].n * sizeof(double), s);
   st = amr_rhs(A, d_rhs, d_sig, s);
-  if (st == EB_OK) st = amr_resid(A, zero.v, s);
+  if (st == EB_OK) st = amr_resid(A, A->Z[0].v, false, s);
   double bn = 0.0, r = 0.0;
   if (st == EB_OK) st = amr_norm(A, s, &bn);
   if (st != EB_OK) return st;
-  CVec res, x;
-  for (int l = 0; l < L; ++l) {
-    res.v[l] = A->lv[l].r;
-    x.v[l] = d_phi[l];
-  }
-  cv_copy(A, res, A->bvec, s);
   int it = 0, cycles = 0;
+  size_t used = 0;  // events
   const int max_it = std::max(1, A->o.max_cycles);
   // restarted FGMRES, right-preconditioned by one FAC sweep (Sec. 3.3.2's
   // multigrid as the inner solver of every correction)
   st = EB_ERR_NOT_CONVERGED;
   while (it < max_it) {
-    eb_status s2 = amr_resid(A, x.v, s);
+    eb_status s2 = amr_resid(A, d_phi, false, s);
     if (s2 == EB_OK) s2 = amr_norm(A, s, &r);
+    for (int l = 0; l < L && s2 == EB_OK && it > 0; ++l) s2 = poisson_vcycle_error(A->lv[l].P0, s);
     if (s2 != EB_OK) {
       st = s2;
       break;
@@ -982,17 +1011,17 @@ extern "C" eb_status eb_amr_solve_levels(eb_amr* A, const double* const* d_rhs, 
     }
     if (!(r == r) || r > 1e6 * bn) break;
     // v0 = r / |r|_2
-    cv_copy(A, res, A->V[0], s);
-    for (int l = 0; l < L - 1; ++l) {
-      k_zero_under<<<nb(box_cells(A->pr[l + 1].B)), TBA, 0, s>>>(A->pr[l + 1].B, A->V[0].v[l], A->lv[l].n);
-      note_launch();
-    }
-    double beta = std::sqrt(cv_dot(A, A->V[0], A->V[0], s));
+    for (int l = 0; l < L; ++l)
+      cudaMemcpyAsync(A->V[0].v[l], A->lv[l].r, 2 * A->lv[l].n * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    cv_maxpy_norm(A, 0, nullptr, A->V[0], nullptr, 4, nullptr, A->d_h + HN, s);
+    cv_scale(A, A->d_h + HN, A->V[0], s);
+    cudaMemcpyAsync(A->h_h, A->d_h, HLEN * sizeof(double), cudaMemcpyDeviceToHost, s);
+    cudaStreamSynchronize(s);
+    const double beta = A->h_h[HN];
     if (!(beta > 0.0)) {
       st = EB_OK;
       break;
     }
-    cv_axpby(A, 0.0, A->V[0], 1.0 / beta, A->V[0], s);
     // this cycle's target in the 2-norm estimate: the reduction the max norm
     // still needs, with a factor 1/2 of margin
     const double target = 0.5 * (A->o.tol * bn / r) * beta;
@@ -1002,26 +1031,29 @@ extern "C" eb_status eb_amr_solve_levels(eb_amr* A, const double* const* d_rhs, 
     g[0] = beta;
     int k = 0;
     for (; k < GM && it < max_it; ++k, ++it) {
-      s2 = fac_apply(A, A->V[k], A->Z[k], &cycles, s);
-      if (s2 == EB_OK) s2 = op_apply(A, A->Z[k], A->V[k + 1], s);
+      const CVec& w = A->V[k + 1];
+      s2 = fac_apply(A, A->V[k], A->Z[k], &cycles, &used, s);
+      if (s2 == EB_OK) s2 = amr_apply(A, nullptr, A->Z[k].v, w.v, 0, false, true, s);
       if (s2 != EB_OK) break;
       // classical Gram-Schmidt, all k + 1 projections in one pass, repeated
-      // only when the pass removed most of w (the criterion of Daniel, Gragg,
-      // Kaufman and Stewart: the new norm below 1/sqrt(2) of the old one,
-      // where cancellation may have left w short of orthogonal)
-      for (int i = 0; i <= k; ++i) H[i][k] = 0.0;
-      double hp[CV_MAXV];
-      cv_mdot(A, k + 1, A->V[k + 1], hp, s, true);  // (V_i, w) and (w, w)
-      const double w0 = std::sqrt(std::max(hp[k + 1], 0.0));
-      double w1 = std::sqrt(std::max(cv_maxpy_norm(A, k + 1, hp, A->V[k + 1], s), 0.0));
-      for (int i = 0; i <= k; ++i) H[i][k] += hp[i];
-      if (w1 < w0 / std::sqrt(2.0)) {
-        cv_mdot(A, k + 1, A->V[k + 1], hp, s);
-        w1 = std::sqrt(std::max(cv_maxpy_norm(A, k + 1, hp, A->V[k + 1], s), 0.0));
-        for (int i = 0; i <= k; ++i) H[i][k] += hp[i];
+      // only when the pass removed most of w (cancellation may then have left
+      // it short of orthogonal).  The sums, the decision and the norm stay on
+      // the device; the host reads the step's column of H once.
+      cv_mdot(A, k + 1, w, true, nullptr, A->d_h, s);
+      cv_maxpy_norm(A, k + 1, A->d_h, w, nullptr, 1, A->d_h, A->d_h + HN, s);
+      cv_mdot(A, k + 1, w, false, A->d_go, A->d_h + H2, s);
+      cv_maxpy_norm(A, k + 1, A->d_h + H2, w, A->d_go, 2, nullptr, A->d_h + HN, s);
+      cv_scale(A, A->d_h + HN, w, s);
+      cudaError_t e = cudaMemcpyAsync(A->h_h, A->d_h, HLEN * sizeof(double), cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) {
+        s2 = cuda_fail(e, "composite step");
+        break;
       }
-      H[k + 1][k] = w1;
-      if (H[k + 1][k] > 0.0) cv_axpby(A, 0.0, A->V[k + 1], 1.0 / H[k + 1][k], A->V[k + 1], s);
+      int go = 0;
+      std::memcpy(&go, A->h_h + HGO, sizeof(go));
+      for (int i = 0; i <= k; ++i) H[i][k] = A->h_h[i] + (go ? A->h_h[H2 + i] : 0.0);
+      H[k + 1][k] = A->h_h[HN];
       for (int i = 0; i < k; ++i) {  // earlier rotations
         double t = cs[i] * H[i][k] + sn[i] * H[i + 1][k];
         H[i + 1][k] = -sn[i] * H[i][k] + cs[i] * H[i + 1][k];
@@ -1052,7 +1084,12 @@ extern "C" eb_status eb_amr_solve_levels(eb_amr* A, const double* const* d_rhs, 
       for (int j = i + 1; j < k; ++j) t -= H[i][j] * y[j];
       y[i] = H[i][i] != 0.0 ? t / H[i][i] : 0.0;
     }
-    for (int i = 0; i < k; ++i) cv_axpby(A, y[i], A->Z[i], 1.0, x, s);
+    for (int l = 0; l < L; ++l) {
+      CVPtrs p = cv_ptrs(A->Z, l, k);
+      for (int i = 0; i < k; ++i) p.a[i] = y[i];
+      k_cv_update<<<nb(A->lv[l].n), TBA, 0, s>>>(A->lv[l].flags, A->lv[l].n, k, p, d_phi[l]);
+      note_launch();
+    }
   }
   // report every level's phi under the next finer box as the finer means (finest first)
   if (st == EB_OK || st == EB_ERR_NOT_CONVERGED) {
@@ -1064,8 +1101,17 @@ extern "C" eb_status eb_amr_solve_levels(eb_amr* A, const double* const* d_rhs, 
     }
     if (st == EB_ERR_NOT_CONVERGED) set_error("composite iteration cap reached");
   }
+  for (int l = 0; l < L && it > 0 && (st == EB_OK || st == EB_ERR_NOT_CONVERGED); ++l) {
+    const eb_status s2 = poisson_vcycle_error(A->lv[l].P0, s);
+    if (s2 != EB_OK) st = s2;
+  }
   cudaError_t e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess && st == EB_OK) st = cuda_fail(e, "composite solve");
+  if (e != cudaSuccess && (st == EB_OK || st == EB_ERR_NOT_CONVERGED)) st = cuda_fail(e, "composite solve");
+  for (size_t i = 0; i + 1 < used; i += 2) {  // a sweep's V-cycles in order of level
+    float ms = 0.0f;
+    if (cudaEventElapsedTime(&ms, A->ev[i], A->ev[i + 1]) == cudaSuccess) amr_count(A, (i / 2) % L ? 1 : 0, 1, 1, ms);
+  }
+  cudaGetLastError();
   inf.status = st;
   inf.outer_iters = it;
   inf.vcycles = cycles;

@@ -125,11 +125,18 @@ eb_status batch_prepare(eb_poisson* P, const double* rhs, const double* sigma, c
 eb_status batch_step(eb_poisson* const* P, int n, const double* const* rhs, const double* const* sigma,
                      double* const* phi, bool fresh, bool copy_out, int max_iters, cudaStream_t s,
                      double* kernel_ms);
-eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, bool kry, eb_poisson** out);
+// what a handle is for: solves, V-cycles that precondition an outer Krylov
+// method (no acceleration of their own), or applying the operator alone
+enum { PS_SOLVE = 0, PS_PLAIN = 1, PS_OPERATOR = 2 };
+eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, int use, eb_poisson** out);
 void batch_info(eb_poisson* Q, eb_solve_info* inf);
 eb_status batch_copy_out(eb_poisson* P, double* phi, cudaStream_t s);
 long long poisson_device_bytes(const eb_poisson* P);
 eb_status poisson_solve_b(eb_poisson* P, const double* d_b, double* d_x, double tol, int* cycles, cudaStream_t user,
                           int* outer = nullptr, double* kernel_ms = nullptr);
+eb_status poisson_vcycle(eb_poisson* P, const double* b, double* x, bool add, cudaEvent_t* ev, cudaStream_t s);
+void poisson_vcycle_begin(eb_poisson* P, cudaStream_t s);
+eb_status poisson_vcycle_error(eb_poisson* P, cudaStream_t s);
+eb_status poisson_apply(eb_poisson* P, const double* d_b, const double* d_phi, double sgn, double* d_r, cudaStream_t s);
 eb_status poisson_rhs(eb_poisson* P, const double* d_rhs, const double* d_sigma, double* d_b, cudaStream_t s);
 eb_status poisson_residual_view(eb_poisson* P, const double* d_b, const double* d_phi, double* d_r, cudaStream_t s);

@@ -1395,29 +1395,16 @@ __device__ __noinline__ void rb_kry2(const RHier<T>& __restrict__ H, const RLev<
   }
 }
 
+// The start of a launch: the hierarchy's description into shared memory, and in
+// CTA 0 the levels it keeps there (their flags, rows with entries in T and
+// special lists, constant over the launch).  gl: level lc as the grid sees it.
 template <class T>
-__device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, const Op<double>* __restrict__ Fg,
-                                               const SolveCtl& ctl, const Barrier& B, int gcta, int gsize) {
-  __shared__ RHier<T> H;
-  __shared__ RLev<T> gl;
-  __shared__ Op<double> F;
-  __shared__ unsigned epoch, tn;
-  __shared__ T red[PT / 32][KDOT];
-  __shared__ double dots[KDOT], coef[KH];
-  __shared__ KryState K;
-  extern __shared__ __align__(128) unsigned char dyn[];
+__device__ __noinline__ void rb_begin(const RHier<T>* __restrict__ Hg, RHier<T>& H, RLev<T>& gl, unsigned char* dyn,
+                                      int gcta) {
   copy_words(&H, Hg, sizeof(RHier<T>));
-  copy_words(&F, Fg, sizeof(Op<double>));
   copy_words(&gl, &Hg->L[Hg->lc], sizeof(RLev<T>));
-  if (threadIdx.x == 0) {
-    epoch = 0u;
-    tn = 0u;
-  }
-  copy_words(&K, Hg->kst, sizeof(KryState));
   __syncthreads();
-  if (threadIdx.x == 0 && ctl.fresh) K.count = K.next = 0;
   if (gcta == 0 && H.smem) {
-    // levels lc.. into shared memory: flags, rows (entries in T) and special lists, constant over the launch
     for (int l = H.lc; l < H.nlev; ++l) {
       const RLev<T>& g = Hg->L[l];
       for (int q = 0; q < 2; ++q) copy_words(dyn + H.off_f[l][q], g.f[q], g.H);
@@ -1459,6 +1446,8 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
     }
   }
   __syncthreads();
+}
+__device__ __forceinline__ RCtx rb_grid(const Barrier& B, unsigned* epoch, unsigned* tn, int gcta, int gsize) {
   RCtx G;
   const int wi = (int)(threadIdx.x >> 5) * gsize + gcta;  // warps interleaved over the CTAs
   G.i0 = wi * 32 + (int)(threadIdx.x & 31);
@@ -1467,11 +1456,35 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
   G.g0 = G.gst - 1 - (wi * 4 + (int)((threadIdx.x >> 3) & 3));
   G.local = false;
   G.B = B;
-  G.epoch = &epoch;
+  G.epoch = epoch;
   G.tr = nullptr;
-  G.tn = &tn;
+  G.tn = tn;
   G.gcta = gcta;
   G.gsize = gsize;
+  return G;
+}
+
+template <class T>
+__device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, const Op<double>* __restrict__ Fg,
+                                               const SolveCtl& ctl, const Barrier& B, int gcta, int gsize) {
+  __shared__ RHier<T> H;
+  __shared__ RLev<T> gl;
+  __shared__ Op<double> F;
+  __shared__ unsigned epoch, tn;
+  __shared__ T red[PT / 32][KDOT];
+  __shared__ double dots[KDOT], coef[KH];
+  __shared__ KryState K;
+  extern __shared__ __align__(128) unsigned char dyn[];
+  copy_words(&F, Fg, sizeof(Op<double>));
+  if (threadIdx.x == 0) {
+    epoch = 0u;
+    tn = 0u;
+  }
+  copy_words(&K, Hg->kst, sizeof(KryState));
+  rb_begin(Hg, H, gl, dyn, gcta);
+  if (threadIdx.x == 0 && ctl.fresh) K.count = K.next = 0;
+  __syncthreads();
+  const RCtx G = rb_grid(B, &epoch, &tn, gcta, gsize);
   // the finest level as the grid sees it (level 0 may be the first one inside CTA 0)
   const RLev<T>& L0 = H.lc == 0 ? gl : H.L[0];
   const int sZ = rb_done(H, 0);
@@ -1545,6 +1558,66 @@ __global__ void __launch_bounds__(PT, 1) k_rb_solve(const RHier<T>* __restrict__
   rb_solve_group<T>(Hg, Fg, ctl, B, (int)blockIdx.x, (int)gridDim.x);
 }
 
+// One V-cycle as a preconditioner: x = M b, or x += M b, on FP64 vectors in
+// the plain layout (entries without an unknown are left alone).
+template <class T>
+__global__ void __launch_bounds__(PT, 1) k_rb_vcycle(const RHier<T>* __restrict__ Hg, long long ncell,
+                                                     const double* __restrict__ b, double* __restrict__ x, int add,
+                                                     Barrier B) {
+  __shared__ RHier<T> H;
+  __shared__ RLev<T> gl;
+  __shared__ unsigned epoch, tn;
+  extern __shared__ __align__(128) unsigned char dyn[];
+  if (threadIdx.x == 0) {
+    epoch = 0u;
+    tn = 0u;
+  }
+  rb_begin(Hg, H, gl, dyn, (int)blockIdx.x);
+  const RCtx G = rb_grid(B, &epoch, &tn, (int)blockIdx.x, (int)gridDim.x);
+  const RLev<T>& L = H.lc == 0 ? gl : H.L[0];
+  for (int t = G.i0; t < L.nqt; t += G.st) {
+    const unsigned w0 = reinterpret_cast<const unsigned*>(L.f[0])[t], w1 = reinterpret_cast<const unsigned*>(L.f[1])[t];
+    const QPos g = quad_pos(L, t, 0);
+    for (int p = 0; p <= L.two; ++p) {
+      if (!((w0 | w1) & (0x01010101u << p))) continue;
+      const double* src = b + p * ncell + ((long long)g.j + (long long)L.n[1] * g.k) * L.n[0] + 2 * g.q0;
+      double v[8];
+      ld4(src, v);
+      ld4(src + 4, v + 4);
+      const T e[4] = {(T)v[0], (T)v[2], (T)v[4], (T)v[6]}, o[4] = {(T)v[1], (T)v[3], (T)v[5], (T)v[7]};
+      st4(L.b[p][g.s] + 4 * (long long)t, e);
+      st4(L.b[p][g.s ^ 1] + 4 * (long long)t, o);
+    }
+  }
+  if (!G.sync(0) || !rb_vcycle(H, gl, G)) return;
+  const int d = rb_done(H, 0), ir = rb_red(d), ib = rb_black(d);
+  for (int t = G.i0; t < L.nqt; t += G.st) {
+    const unsigned w[2] = {reinterpret_cast<const unsigned*>(L.f[0])[t], reinterpret_cast<const unsigned*>(L.f[1])[t]};
+    const QPos g = quad_pos(L, t, 0);
+    for (int p = 0; p <= L.two; ++p) {
+      if (!((w[0] | w[1]) & (0x01010101u << p))) continue;
+      double* dst = x + p * ncell + ((long long)g.j + (long long)L.n[1] * g.k) * L.n[0] + 2 * g.q0;
+      double v[8];
+      ld4(dst, v);
+      ld4(dst + 4, v + 4);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        T z[4];
+        ld4(L.x[p][c ? ib : ir] + 4 * (long long)t, z);
+        const int odd = g.s ^ c;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (!((w[c] >> (8 * e + p)) & 1u)) continue;
+          double& q = odd ? v[2 * e + 1] : v[2 * e];
+          q = (add ? q : 0.0) + (double)z[e];
+        }
+      }
+      st4(dst, v);
+      st4(dst + 4, v + 4);
+    }
+  }
+}
+
 // many independent solves in one cooperative launch (see BatchItem)
 template <class T>
 struct RBatchItem {
@@ -1569,14 +1642,7 @@ __global__ void __launch_bounds__(PT, 1) k_rb_phase(const RHier<T>* __restrict__
   copy_words(&L, &Hg->L[0], sizeof(RLev<T>));
   if (Hg->nlev > 1) copy_words(&N, &Hg->L[1], sizeof(RLev<T>));
   __syncthreads();
-  RCtx G{};
-  const int gsize = (int)gridDim.x, wi = (int)(threadIdx.x >> 5) * gsize + (int)blockIdx.x;
-  G.i0 = wi * 32 + (int)(threadIdx.x & 31);
-  G.st = gsize * (int)blockDim.x;
-  G.gst = gsize * (int)(blockDim.x >> 3);
-  G.g0 = G.gst - 1 - (wi * 4 + (int)((threadIdx.x >> 3) & 3));
-  G.gsize = gsize;
-  G.gcta = (int)blockIdx.x;
+  const RCtx G = rb_grid(Barrier{}, nullptr, nullptr, (int)blockIdx.x, (int)gridDim.x);
   if (kernel == 0) rb_dense(L, colour, 1, false, G);
   else if (kernel == 1) rb_restrict(L, N, 1, false, G);
   else rb_prolong(L, N, 1, rb_done(*Hg, 1), G);

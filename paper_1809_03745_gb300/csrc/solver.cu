@@ -372,6 +372,7 @@ static Op<T> make_terms(const DevLevel& L) {
   o.dn1 = make_fastdiv((unsigned)L.g.n[1]);
   o.dhx = make_fastdiv((unsigned)((L.g.n[0] + 1) / 2));
   o.dq = make_fastdiv((unsigned)std::max(1, L.g.n[0] / 4));
+  o.d8 = make_fastdiv((unsigned)std::max(1, L.g.n[0] / 8));
   o.ncell = L.g.ncell;
   set_stencil_terms(o, L.g);
   o.flags = L.flags;
@@ -1242,6 +1243,9 @@ static eb_status setup_persistent(eb_poisson* P) {
   // the attribute is per kernel, shared by every handle: allow the device maximum once
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(batch_kernel(P), cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
+  if (e == cudaSuccess && P->rb)
+    e = cudaFuncSetAttribute(mixed ? (const void*)k_rb_vcycle<float> : (const void*)k_rb_vcycle<double>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
   if (e == cudaSuccess && P->sweep_levels)
     e = cudaFuncSetAttribute((const void*)k_sweep_phase<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
   if (e == cudaSuccess && P->sweep_levels)
@@ -1329,12 +1333,10 @@ static bool sweeps_requested(const eb_poisson* P) {
 }
 
 extern "C" eb_status eb_poisson_setup(const eb_geom* G, const eb_solver_opts* opts, void* stream, eb_poisson** out) {
-  return poisson_setup(G, opts, true, out);
+  return poisson_setup(G, opts, PS_SOLVE, out);
 }
 
-// kry: Krylov acceleration of the V-cycles (a handle whose V-cycles precondition
-// an outer Krylov method goes without, and without its memory)
-eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, bool kry, eb_poisson** out) {
+eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, int use, eb_poisson** out) {
   if (!G || !out) {
     set_error("null argument");
     return EB_ERR_INVALID;
@@ -1370,9 +1372,9 @@ eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, bool kry, 
   P->op64.push_back(make_op<double>(F, P->allocs, &P->bytes, &st, np, P->phi64, P->b64, P->phi64 + n0, P->b64 + n0));
   int coop = 0;
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, G->device);
-  P->rb = coop && o.launch_mode == 0 && !sweeps_requested(P);
-  P->kry = kry;
-  if (P->rb) {
+  P->rb = coop && o.launch_mode == 0 && (use != PS_SOLVE || !sweeps_requested(P));
+  P->kry = use == PS_SOLVE;
+  if (P->rb || use == PS_OPERATOR) {
     // the colour-split hierarchy has vectors of its own
   } else if (o.precision == EB_PREC_FP64) {
     for (int l = 1; l < P->nlev; ++l) P->op64.push_back(make_op<double>(G->L[l], P->allocs, &P->bytes, &st, np));
@@ -1386,8 +1388,8 @@ eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, bool kry, 
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) st = cuda_fail(e, "solver setup");
   }
-  if (st == EB_OK) st = setup_persistent(P);
-  if (st == EB_OK && o.launch_mode != 2 && !P->persistent) {
+  if (st == EB_OK && use != PS_OPERATOR) st = setup_persistent(P);
+  if (st == EB_OK && o.launch_mode != 2 && !P->persistent && use != PS_OPERATOR) {
     cudaError_t e = cudaStreamBeginCapture(P->s, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       g_count = &P->per_iter;
@@ -1447,13 +1449,150 @@ static eb_status read_norms(eb_poisson* P, double* r, double* b) {
   return EB_OK;
 }
 
-__global__ void k_resid_field(Op<double> o, double* r) {
-  long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= o.ncell) return;
-  uint8_t f = o.flags[c];
-  int I[3];
-  ijk(o, c, I);
-  for (int p = 0; p < 2; ++p) r[p * o.ncell + c] = ((f >> p) & 1) ? cell_residual(o, c, p, I) : 0.0;
+// r = sgn (b - A x) on the finest level in the plain layout (b null: b = 0), in
+// two independent kernels: the regular cells, eight of an x row per thread
+// with seven FP64 operations each (GB300's FP64 pipe bounds it), and the
+// sparse rows, a group of 8 lanes each.  256^3: 0.30 ms, against 0.75 ms for
+// a thread per cell and a row pass before it.  zero: entries without an
+// unknown are written as 0, else left alone.
+// AL: x, b and r are 16-byte aligned (a caller's pointers need not be).
+template <bool AL>
+__device__ __forceinline__ void ldd4(const double* p, double v[4]) {
+  if constexpr (AL) {
+    ld4(p, v);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = p[e];
+  }
+}
+template <bool AL>
+__global__ void __launch_bounds__(128) k_apply_regular(Op<double> o, double sgn, double* __restrict__ r, int zero) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (8 * t >= o.ncell) return;
+  const long long c0 = 8 * t;
+  const uint2 fw = *reinterpret_cast<const uint2*>(o.flags + c0);
+  const unsigned row = fdiv((unsigned)(c0 >> 3), o.d8);
+  const unsigned kq = fdiv(row, o.dn1);
+  const int i0 = 8 * (int)((unsigned)(c0 >> 3) - row * (unsigned)(o.n[0] >> 3));
+  const int I[3] = {i0, (int)(row - kq * (unsigned)o.n[1]), (int)kq};
+  for (int p = 0; p < 2; ++p) {
+    double* rp = r + p * o.ncell + c0;
+    const unsigned ml = regular_mask(fw.x, p), mh = regular_mask(fw.y, p);
+    const unsigned al = (fw.x >> p) & 0x01010101u, ah = (fw.y >> p) & 0x01010101u;  // unknowns
+    double out[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) out[e] = 0.0;
+    if (ml | mh) {
+      const double* x = o.x[p] + c0;
+      double c[8], s[8];
+      ldd4<AL>(x, c);
+      ldd4<AL>(x + 4, c + 4);
+      const bool wl = i0 == 0, wh = i0 + 8 == o.n[0];
+      const double xl = wl ? o.w3[0] * c[1] : x[-1], xr = wh ? o.w3[1] * c[6] : x[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s[e] = (e ? c[e ? e - 1 : 0] : xl) + (e < 7 ? c[e < 7 ? e + 1 : 7] : xr);
+      double d0 = (double)(2 * o.D) + o.lh[p];
+      long long st = o.n[0];
+      for (int a = 1; a < o.D; ++a, st *= o.n[1]) {
+        double u[8], v[8];
+        const bool lo = I[a] > 0, hi = I[a] < o.n[a] - 1;
+        if (lo) {
+          ldd4<AL>(x - st, u);
+          ldd4<AL>(x - st + 4, u + 4);
+        }
+        if (hi) {
+          ldd4<AL>(x + st, v);
+          ldd4<AL>(x + st + 4, v + 4);
+        }
+        if (!lo) {
+          d0 += 3.0 * o.wr[2 * a] - 1.0;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) u[e] = o.w3[2 * a] * v[e];
+        }
+        if (!hi) {
+          d0 += 3.0 * o.wr[2 * a + 1] - 1.0;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[e] = o.w3[2 * a + 1] * u[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] += u[e] + v[e];
+      }
+      const double dl = wl ? d0 + 3.0 * o.wr[0] - 1.0 : d0, dr = wh ? d0 + 3.0 * o.wr[1] - 1.0 : d0;
+      double bb[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) bb[e] = 0.0;
+      if (o.b[p]) {
+        ldd4<AL>(o.b[p] + c0, bb);
+        ldd4<AL>(o.b[p] + c0 + 4, bb + 4);
+      }
+      const double cs = -sgn * o.ceps[p];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const double dg = e == 0 ? dl : (e == 7 ? dr : d0);
+        out[e] = cs * (dg * c[e] - s[e]) + sgn * bb[e];
+      }
+    }
+    // regular cells, and zeros where there is no unknown; the rows' cells are theirs
+    const unsigned kl = ml | (zero ? __vcmpeq4(al, 0u) : 0u), kh = mh | (zero ? __vcmpeq4(ah, 0u) : 0u);
+    if (zero && (ml != 0xffffffffu || mh != 0xffffffffu)) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (!((((e < 4 ? al : ah) >> (8 * (e & 3))) & 1u))) out[e] = 0.0;
+    }
+    if constexpr (AL) {
+      quad_store(rp, kl, out);
+      quad_store(rp + 4, kh, out + 4);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if ((e < 4 ? kl : kh) >> (8 * (e & 3)) & 1u) rp[e] = out[e];
+    }
+  }
+}
+__global__ void __launch_bounds__(256) k_apply_rows(Op<double> o, double sgn, double* __restrict__ r) {
+  const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  if (row >= 2 * o.nirr) return;  // whole groups leave together
+  const int g = threadIdx.x & 7;
+  const unsigned gmask = 0xffu << (threadIdx.x & 24);
+  const double d = o.diag[row];
+  if (d == 0.0) return;
+  const int e0 = o.row_ptr[row], e1 = o.row_ptr[row + 1];
+  const int cell = o.irr_cell[row >> 1], p = (int)(row & 1);
+  double s = 0.0;
+  for (int e = e0 + g; e < e1; e += 32) {
+    unsigned cl[4];
+    double a[4], xv[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      cl[k] = 0u;
+      a[k] = 0.0;
+      if (e + 8 * k < e1) {
+        cl[k] = (unsigned)o.col[e + 8 * k];
+        a[k] = o.val[e + 8 * k];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) xv[k] = e + 8 * k < e1 ? o.x[cl[k] >> 30][cl[k] & 0x3fffffffu] : 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s += a[k] * xv[k];
+  }
+  for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(gmask, s, off);
+  if (g == 0) r[p * o.ncell + cell] = sgn * (((o.b[p] ? o.b[p][cell] : 0.0) - s) - d * o.x[p][cell]);
+}
+static eb_status launch_apply(Op<double> o, const double* b, const double* x, double sgn, double* r, bool zero,
+                              cudaStream_t s) {
+  const long long n = o.ncell;
+  o.x[0] = const_cast<double*>(x);
+  o.x[1] = const_cast<double*>(x) + n;
+  o.b[0] = const_cast<double*>(b);
+  o.b[1] = b ? const_cast<double*>(b) + n : nullptr;
+  const bool al = !(((unsigned long long)b | (unsigned long long)x | (unsigned long long)r) & 15ull);
+  if (al) k_apply_regular<true><<<blocks(n / 8, 128), 128, 0, s>>>(o, sgn, r, zero ? 1 : 0);
+  else k_apply_regular<false><<<blocks(n / 8, 128), 128, 0, s>>>(o, sgn, r, zero ? 1 : 0);
+  if (o.nirr) k_apply_rows<<<blocks(16 * o.nirr), 256, 0, s>>>(o, sgn, r);
+  counted(o.nirr ? 2 : 1);
+  cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? EB_OK : cuda_fail(e, "residual");
 }
 
 // b (FP64 [2][n_cells]) of the finest level for the given data: kappa rhs
@@ -1463,23 +1602,14 @@ eb_status poisson_rhs(eb_poisson* P, const double* d_rhs, const double* d_sigma,
   return launch_rhs64(P->G, d_rhs, d_sigma, d_b, (double*)(P->d_norm + 1), s);
 }
 
-// r = b - A phi on the finest level for a b formed by poisson_rhs; phi is
-// read as given (its entries without an unknown must be finite), the sparse
-// rows use the handle's row scratch; enqueued on s, no sync.
+// r = b - A phi on the finest level for a b formed by poisson_rhs; enqueued
+// on s, no sync.
 eb_status poisson_residual_view(eb_poisson* P, const double* d_b, const double* d_phi, double* d_r, cudaStream_t s) {
-  Op<double> o = P->op64[0];
-  const long long n = o.ncell;
-  o.x[0] = const_cast<double*>(d_phi);
-  o.b[0] = const_cast<double*>(d_b);
-  if (o.x[1]) {
-    o.x[1] = const_cast<double*>(d_phi) + n;
-    o.b[1] = const_cast<double*>(d_b) + n;
-  }
-  if (o.nirr) k_rows<double><<<blocks(2 * o.nirr), 256, 0, s>>>(o, 0, 2 * o.nirr, 1);
-  k_resid_field<<<blocks(n), 256, 0, s>>>(o, d_r);
-  counted(o.nirr ? 2 : 1);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? EB_OK : cuda_fail(e, "residual");
+  return launch_apply(P->op64[0], d_b, d_phi, 1.0, d_r, true, s);
+}
+// r = sgn (b - A phi), b = 0 when null; entries of r without an unknown are left alone
+eb_status poisson_apply(eb_poisson* P, const double* d_b, const double* d_phi, double sgn, double* d_r, cudaStream_t s) {
+  return launch_apply(P->op64[0], d_b, d_phi, sgn, d_r, false, s);
 }
 
 extern "C" eb_status eb_poisson_residual(eb_poisson* P, const double* d_rhs, const double* d_sigma,
@@ -1496,12 +1626,10 @@ extern "C" eb_status eb_poisson_residual(eb_poisson* P, const double* d_rhs, con
   eb_status st = launch_rhs64(P->G, d_rhs, d_sigma, P->b64, (double*)(P->d_norm + 1), P->s);
   if (st != EB_OK) return st;
   k_copy_masked<<<blocks(n), 256, 0, P->s>>>(F.flags, n, d_phi, P->phi64);
-  const Op<double>& o = P->op64[0];
-  if (o.nirr) k_rows<double><<<blocks(2 * o.nirr), 256, 0, P->s>>>(o, 0, 2 * o.nirr, 1);
-  k_resid_field<<<blocks(n), 256, 0, P->s>>>(o, d_r);
-  counted(o.nirr ? 3 : 2);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaStreamSynchronize(P->s);
+  counted();
+  st = launch_apply(P->op64[0], P->b64, P->phi64, 1.0, d_r, true, P->s);
+  if (st != EB_OK) return st;
+  cudaError_t e = cudaStreamSynchronize(P->s);
   join_out(P, user);
   return e == cudaSuccess ? EB_OK : cuda_fail(e, "residual");
 }
@@ -1776,6 +1904,41 @@ eb_status poisson_solve_b(eb_poisson* P, const double* d_b, double* d_x, double 
   if (outer) *outer = iters;
   if (kernel_ms) *kernel_ms = P->kernel_ms;
   return st;
+}
+
+// x = M b (add: x += M b) with one V-cycle of a handle without Krylov
+// acceleration, FP64 vectors [2][ncell] in the plain layout; enqueued on s, no
+// sync.  ev: two events recorded around the kernel (may be null).  A wait that
+// gives up leaves its mark in the handle's error word, which poisson_vcycle_begin
+// clears and poisson_vcycle_error reads.
+eb_status poisson_vcycle(eb_poisson* P, const double* b, double* x, bool add, cudaEvent_t* ev, cudaStream_t s) {
+  if (!P->persistent || !P->rb) {
+    set_error("correction solves need the persistent path");
+    return EB_ERR_UNSUPPORTED;
+  }
+  const bool mixed = P->o.precision == EB_PREC_MIXED;
+  const void* fn = mixed ? (const void*)k_rb_vcycle<float> : (const void*)k_rb_vcycle<double>;
+  cudaMemsetAsync(P->d_bar, 0, 2 * sizeof(unsigned), s);
+  const void* H = P->d_hier;
+  long long n = P->G->L[0].g.ncell;
+  int ad = add ? 1 : 0;
+  Barrier B{P->d_bar, (int*)(P->d_bar + 2)};
+  void* args[6] = {(void*)&H, (void*)&n, (void*)&b, (void*)&x, (void*)&ad, (void*)&B};
+  if (ev) cudaEventRecord(ev[0], s);
+  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(P->grid), dim3(PT), args, (size_t)P->smem_bytes, s);
+  if (ev) cudaEventRecord(ev[1], s);
+  counted();
+  return e == cudaSuccess ? EB_OK : cuda_fail(e, "V-cycle");
+}
+void poisson_vcycle_begin(eb_poisson* P, cudaStream_t s) { cudaMemsetAsync(P->d_bar, 0, 4 * sizeof(unsigned), s); }
+eb_status poisson_vcycle_error(eb_poisson* P, cudaStream_t s) {
+  unsigned bar[4] = {0, 0, 0, 0};
+  cudaError_t e = cudaMemcpyAsync(bar, P->d_bar, sizeof(bar), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return cuda_fail(e, "V-cycle");
+  if (!bar[2]) return EB_OK;
+  set_error("a grid barrier wait gave up");
+  return EB_ERR_TIMEOUT;
 }
 
 // One cooperative launch over instances that share precision and device.
@@ -2208,8 +2371,7 @@ extern "C" eb_status eb_poisson_residual_noalloc(const eb_geom* G, const double*
   eb_status st = na_scratch(&base);
   if (st != EB_OK) return st;
   double* b = base;                       // [2][n] right-hand side
-  double* tmp = base + 2 * NA_MAX_CELLS;  // [nrow] sparse-row residuals
-  double* bnorm = tmp + NA_MAX_ROWS;      // max|b| (not returned)
+  double* bnorm = base + 2 * NA_MAX_CELLS + NA_MAX_ROWS;  // max|b| (not returned)
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaMemsetAsync(bnorm, 0, sizeof(double), s);
   if (e != cudaSuccess) return cuda_fail(e, "scratch clear");
@@ -2224,12 +2386,9 @@ extern "C" eb_status eb_poisson_residual_noalloc(const eb_geom* G, const double*
   o.dn1 = make_fastdiv((unsigned)F.g.n[1]);
   o.dhx = make_fastdiv((unsigned)((F.g.n[0] + 1) / 2));
   o.dq = make_fastdiv((unsigned)std::max(1, F.g.n[0] / 4));
+  o.d8 = make_fastdiv((unsigned)std::max(1, F.g.n[0] / 8));
   o.ncell = n;
   set_stencil_terms(o, F.g);
-  o.x[0] = const_cast<double*>(d_phi);
-  o.x[1] = const_cast<double*>(d_phi) + n;
-  o.b[0] = b;
-  o.b[1] = b + n;
   o.flags = F.flags;
   o.irr_cell = F.irr_cell;
   o.irr_of_cell = F.irr_of_cell;
@@ -2237,7 +2396,6 @@ extern "C" eb_status eb_poisson_residual_noalloc(const eb_geom* G, const double*
   o.col = F.col;
   o.val = F.val;
   o.diag = F.diag;
-  o.tmp = tmp;
   o.nirr = F.nirr;
   o.nirr_red = F.nirr_red;
   for (int p = 0; p < 2; ++p) {
@@ -2245,9 +2403,8 @@ extern "C" eb_status eb_poisson_residual_noalloc(const eb_geom* G, const double*
     o.ceps[p] = F.g.eps[p] / h2;
     o.h2e[p] = h2 / F.g.eps[p];
   }
-  if (nrow) k_rows<double><<<blocks(nrow), 256, 0, s>>>(o, 0, nrow, 1);
-  k_resid_field<<<blocks(n), 256, 0, s>>>(o, d_r);
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  st = launch_apply(o, b, d_phi, 1.0, d_r, true, s);
+  if (st != EB_OK) return st;
+  e = cudaStreamSynchronize(s);
   return e == cudaSuccess ? EB_OK : cuda_fail(e, "allocation-free residual");
 }
