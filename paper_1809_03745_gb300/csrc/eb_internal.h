@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -49,6 +50,9 @@ struct eb_geom {
   long long stencil_counts[3] = {0, 0, 0};
   long long bytes = 0;
   int* d_status = nullptr;
+  // scratch of eb_tag_cells, taken at its first call and kept
+  mutable std::mutex scratch_lock;
+  mutable void* scratch = nullptr;
 };
 
 namespace ebp {

@@ -243,6 +243,7 @@ extern "C" eb_status eb_geom_build(const eb_geom_desc* d, void* stream, eb_geom*
 extern "C" void eb_geom_destroy(eb_geom* G) {
   if (!G) return;
   for (auto& L : G->L) free_level(L);
+  if (G->scratch) cudaFree(G->scratch);
   delete G;
 }
 

@@ -3,19 +3,19 @@
 //
 // The tracer is T = |E| / max |E|; a cell is tagged for refinement when
 // |grad T| dx / T > eps1 or T > eps2 and for coarsening when
-// |grad T| dx / T < eps3 and T < eps4.  Three passes over the grid: the first
-// writes |E| per cell into a scratch array and takes its maximum (order-free
-// atomicMax on the bit pattern of a non-negative double), the second divides
-// by the maximum in place, the third reads T at the cell and its axis
-// neighbours, forms the gradient by centred or one-sided differences in
-// index units (dx cancels), the tag byte, and the bounding box and count of
-// the marked cells (warp reductions, then one atomic per warp).  FP64 is slow
-// on this part, so every square root and division is taken once per cell
-// (reading the neighbours' T instead of recomputing them costs 8 bytes each,
-// mostly from L1).  Every product and sum is written with round-to-nearest
-// intrinsics (this unit is also compiled without FMA contraction) and sqrt
-// and division are correctly rounded, so the tags are a function of E alone
-// and match a plain FP64 evaluation in the same order.
+// |grad T| dx / T < eps3 and T < eps4, with centred or one-sided differences
+// in index units (dx cancels).  The tags are a function of E alone: every
+// product and sum is written with round-to-nearest intrinsics (this unit is
+// also compiled without FMA contraction), sqrt and division are correctly
+// rounded, and they match a plain FP64 evaluation in the same order.
+//
+// FP64 is slow on this part (two operations per clock and SM), and a tag is
+// four comparisons, so almost no cell needs it.  The first pass writes |E| in
+// FP32 and takes max |E|^2 in FP64 (order-free atomicMax on the bit pattern;
+// the square root is monotone, so its root is max |E|).  The second evaluates
+// the tests in FP32 with a bound on their error, and where a threshold lies
+// within it, or a value outside FP32's range, in FP64 from E as above.
+// 256^3: 0.25 ms, against 1.9 ms for three passes in FP64.
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -33,7 +33,7 @@ constexpr int TBT = 256;
 int nbt(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + TBT - 1) / TBT, 152LL * 16)); }
 
 struct TagOut {
-  unsigned long long emax;  // bit pattern of max |E|
+  unsigned long long emax;  // bit pattern of max |E|^2
   unsigned long long count;
   int lo[3], hi[3];  // hi inclusive while reducing
 };
@@ -46,10 +46,9 @@ struct TagView {
   const double* E;  // [D][2][ncell]
 };
 
-// largest field magnitude over the phases with an unknown (0 where covered)
-__device__ __forceinline__ double cell_mag(const TagView& v, long long c) {
-  const unsigned f = v.flags[c];
-  double mag = 0.0;
+// largest squared field magnitude over the phases with an unknown (0 where covered)
+__device__ __forceinline__ double cell_mag2(const TagView& v, unsigned f, long long c) {
+  double m = 0.0;
   for (int p = 0; p < 2; ++p) {
     if (!((f >> p) & 1u)) continue;  // a phase without an unknown is never selected: skip its reads
     const double e0 = v.E[(long long)p * v.ncell + c];
@@ -58,63 +57,96 @@ __device__ __forceinline__ double cell_mag(const TagView& v, long long c) {
       const double e = v.E[((long long)a * 2 + p) * v.ncell + c];
       m2 = __dadd_rn(m2, __dmul_rn(e, e));
     }
-    const double m = sqrt(m2);
-    if (m > mag) mag = m;
+    if (m2 > m) m = m2;
   }
-  return mag;
+  return m;
 }
 
-__global__ void k_emag(TagView v, double* T, TagOut* out) {
-  double m = 0.0;
+__global__ void __launch_bounds__(TBT) k_emag(TagView v, float* __restrict__ M, TagOut* out) {
+  unsigned long long m = 0ull;
   for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < v.ncell;
        c += (long long)gridDim.x * blockDim.x) {
-    const double mc = cell_mag(v, c);
-    T[c] = mc;
-    m = fmax(m, mc);
+    const double m2 = cell_mag2(v, v.flags[c], c);
+    M[c] = sqrtf((float)m2);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(m2);
+    m = b > m ? b : m;
   }
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(&out->emax, (unsigned long long)__double_as_longlong(m));
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long b = __shfl_xor_sync(0xffffffffu, m, o);
+    m = b > m ? b : m;
+  }
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(&out->emax, m);
 }
 
-__global__ void k_tnorm(long long n, double* T, const TagOut* out) {
-  const double emax = __longlong_as_double((long long)out->emax);
-  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x)
-    T[c] = emax > 0.0 ? T[c] / emax : 0.0;
+// T of a cell in FP64
+__device__ __forceinline__ double tracer(const TagView& v, long long c, double emax) {
+  return emax > 0.0 ? sqrt(cell_mag2(v, v.flags[c], c)) / emax : 0.0;
+}
+// the tag of a cell in FP64 (bit 0 refine, bit 1 coarsen)
+template <int D>
+__device__ __noinline__ unsigned tag_exact(const TagView& v, long long c, const int I[3], double emax, double eps1,
+                                           double eps2, double eps3, double eps4) {
+  const long long stride[3] = {1, v.n[0], (long long)v.n[0] * v.n[1]};
+  const double T = tracer(v, c, emax);
+  double s2 = 0.0;
+  for (int a = 0; a < D; ++a) {
+    const bool hp = I[a] + 1 < v.n[a] && (v.flags[c + stride[a]] & 3u);
+    const bool hm = I[a] > 0 && (v.flags[c - stride[a]] & 3u);
+    const double Tp = hp ? tracer(v, c + stride[a], emax) : 0.0;
+    const double Tm = hm ? tracer(v, c - stride[a], emax) : 0.0;
+    const double d = hp && hm ? __dmul_rn(__dsub_rn(Tp, Tm), 0.5) : hp ? __dsub_rn(Tp, T)
+                                                                  : hm ? __dsub_rn(T, Tm) : 0.0;
+    s2 = __dadd_rn(s2, __dmul_rn(d, d));
+  }
+  const double g = sqrt(s2);
+  const double ratio = T > 0.0 ? g / T : (g > 0.0 ? INFINITY : 0.0);
+  return (ratio > eps1 || T > eps2 ? 1u : 0u) | (ratio < eps3 && T < eps4 ? 2u : 0u);
 }
 
 template <int D>
-__global__ void k_tag(TagView v, const double* __restrict__ Tt, double eps1, double eps2, double eps3, double eps4,
-                      int keep, int klo0, int klo1, int klo2, int khi0, int khi1, int khi2, uint8_t* tags,
-                      TagOut* out) {
+__global__ void __launch_bounds__(TBT) k_tag(TagView v, const float* __restrict__ M, double eps1, double eps2,
+                                             double eps3, double eps4, int keep, int klo0, int klo1, int klo2,
+                                             int khi0, int khi1, int khi2, uint8_t* tags, TagOut* out) {
   const int klo[3] = {klo0, klo1, klo2}, khi[3] = {khi0, khi1, khi2};
   int mlo[3] = {INT_MAX, INT_MAX, INT_MAX}, mhi[3] = {-1, -1, -1};
   unsigned cnt = 0;
-  const long long stride[3] = {1, v.n[0], (long long)v.n[0] * v.n[1]};
+  const double emax = sqrt(__longlong_as_double((long long)out->emax));
+  const float inv = (float)(1.0 / emax);
+  // FP32 decides where the magnitudes are far from its ends
+  const bool fast = emax > 1e-12 && emax < 1e12;
+  const float e1 = (float)eps1, e2 = (float)eps2, e3 = (float)eps3, e4 = (float)eps4;
+  const int stride[3] = {1, v.n[0], v.n[0] * v.n[1]};
   for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < v.ncell;
        c += (long long)gridDim.x * blockDim.x) {
-    const unsigned r = (unsigned)(c / v.n[0]);
-    const int I[3] = {(int)(c - (long long)r * v.n[0]), (int)(r % (unsigned)v.n[1]), (int)(r / (unsigned)v.n[1])};
-    uint8_t t = 0;
+    const unsigned cu = (unsigned)c, r = cu / (unsigned)v.n[0];
+    const int I[3] = {(int)(cu - r * (unsigned)v.n[0]), (int)(r % (unsigned)v.n[1]), (int)(r / (unsigned)v.n[1])};
+    unsigned t = 0;
     if (v.flags[c] & 3u) {
-      const double T = Tt[c];
-      double s2 = 0.0;
+      const float m = M[c];
+      float s2 = 0.0f, sum = 0.0f;
+      bool small = !(m > 1e-15f);
 #pragma unroll
       for (int a = 0; a < D; ++a) {
         const bool hp = I[a] + 1 < v.n[a] && (v.flags[c + stride[a]] & 3u);
         const bool hm = I[a] > 0 && (v.flags[c - stride[a]] & 3u);
-        const double Tp = hp ? Tt[c + stride[a]] : 0.0;
-        const double Tm = hm ? Tt[c - stride[a]] : 0.0;
-        const double d = hp && hm ? __dmul_rn(__dsub_rn(Tp, Tm), 0.5) : hp ? __dsub_rn(Tp, T)
-                                                                      : hm ? __dsub_rn(T, Tm) : 0.0;
-        s2 = __dadd_rn(s2, __dmul_rn(d, d));
+        const float mp = hp ? M[c + stride[a]] : 0.0f, mm = hm ? M[c - stride[a]] : 0.0f;
+        const float d = hp && hm ? 0.5f * (mp - mm) : hp ? mp - m : hm ? m - mm : 0.0f;
+        s2 += d * d;
+        sum += mp + mm + m;
+        small = small || (hp && !(mp > 1e-15f)) || (hm && !(mm > 1e-15f));
       }
-      const double g = sqrt(s2);
-      const double ratio = T > 0.0 ? g / T : (g > 0.0 ? INFINITY : 0.0);
-      const bool refine = ratio > eps1 || T > eps2;
-      const bool coarsen = ratio < eps3 && T < eps4;
-      t = (refine ? 1 : 0) | (coarsen ? 2 : 0);
-      bool marked = refine;
-      if (!marked && keep && !coarsen) {
+      const float T = m * inv, ratio = sqrtf(s2) / m;
+      // a magnitude is off by less than 2^-22 of itself, a difference by 2^-22
+      // of the sum of its two, so the ratio by 2^-22 (sum / m + ratio) with
+      // room for the rounding of the tests themselves
+      const float er = 1e-6f * (sum / m + ratio), et = 1e-6f * T;
+      const bool sure = fast && !small && sum < 1e18f && fabsf(ratio - e1) > er + 1e-6f * fabsf(e1) &&
+                        fabsf(ratio - e3) > er + 1e-6f * fabsf(e3) && fabsf(T - e2) > et + 1e-6f * fabsf(e2) &&
+                        fabsf(T - e4) > et + 1e-6f * fabsf(e4);
+      if (sure) t = (ratio > e1 || T > e2 ? 1u : 0u) | (ratio < e3 && T < e4 ? 2u : 0u);
+      else t = tag_exact<D>(v, c, I, emax, eps1, eps2, eps3, eps4);
+      bool marked = t & 1u;
+      if (!marked && keep && !(t & 2u)) {
         marked = true;
 #pragma unroll
         for (int a = 0; a < D; ++a) marked = marked && I[a] >= klo[a] && I[a] < khi[a];
@@ -128,7 +160,7 @@ __global__ void k_tag(TagView v, const double* __restrict__ Tt, double eps1, dou
         }
       }
     }
-    if (tags) tags[c] = t;
+    if (tags) tags[c] = (uint8_t)t;
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -184,18 +216,22 @@ extern "C" eb_status eb_tag_cells(const eb_geom* G, const double* d_E, const dou
     init.lo[a] = INT_MAX;
     init.hi[a] = -1;
   }
-  // one allocation: the result words, then T [ncell] (16-byte aligned)
+  // one block: the result words, then |E| in FP32.  The geometry keeps it for
+  // the next call; a call that finds it in use by another thread takes its own.
   const size_t head = (sizeof(TagOut) + 255) / 256 * 256;
-  char* d_buf = nullptr;
-  cudaError_t e = cudaMalloc(&d_buf, head + sizeof(double) * (size_t)v.ncell);
+  std::unique_lock<std::mutex> lock(G->scratch_lock, std::try_to_lock);
+  const bool kept = lock.owns_lock();
+  char* d_buf = kept ? (char*)G->scratch : nullptr;
+  cudaError_t e = cudaSuccess;
+  if (!d_buf) e = cudaMalloc(&d_buf, head + sizeof(float) * (size_t)v.ncell);
   if (e != cudaSuccess) return cuda_fail(e, "tag scratch");
+  if (kept) G->scratch = d_buf;
   TagOut* d_out = (TagOut*)d_buf;
-  double* d_T = (double*)(d_buf + head);
+  float* d_M = (float*)(d_buf + head);
   e = cudaMemcpyAsync(d_out, &init, sizeof(init), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) {
-    k_emag<<<nbt(v.ncell), TBT, 0, s>>>(v, d_T, d_out);
-    k_tnorm<<<nbt(v.ncell), TBT, 0, s>>>(v.ncell, d_T, d_out);
-    note_launch(2);
+    k_emag<<<nbt(v.ncell), TBT, 0, s>>>(v, d_M, d_out);
+    note_launch();
     const int keep = keep_lo ? 1 : 0;
     int klo[3] = {0, 0, 0}, khi[3] = {0, 0, 0};
     if (keep)
@@ -204,10 +240,10 @@ extern "C" eb_status eb_tag_cells(const eb_geom* G, const double* d_E, const dou
         khi[a] = keep_hi[a];
       }
     if (v.D == 2)
-      k_tag<2><<<nbt(v.ncell), TBT, 0, s>>>(v, d_T, eps[0], eps[1], eps[2], eps[3], keep, klo[0], klo[1], klo[2],
+      k_tag<2><<<nbt(v.ncell), TBT, 0, s>>>(v, d_M, eps[0], eps[1], eps[2], eps[3], keep, klo[0], klo[1], klo[2],
                                             khi[0], khi[1], khi[2], d_tags, d_out);
     else
-      k_tag<3><<<nbt(v.ncell), TBT, 0, s>>>(v, d_T, eps[0], eps[1], eps[2], eps[3], keep, klo[0], klo[1], klo[2],
+      k_tag<3><<<nbt(v.ncell), TBT, 0, s>>>(v, d_M, eps[0], eps[1], eps[2], eps[3], keep, klo[0], klo[1], klo[2],
                                             khi[0], khi[1], khi[2], d_tags, d_out);
     note_launch();
     e = cudaGetLastError();
@@ -215,7 +251,7 @@ extern "C" eb_status eb_tag_cells(const eb_geom* G, const double* d_E, const dou
   TagOut res;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&res, d_out, sizeof(res), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(d_buf);
+  if (!kept) cudaFree(d_buf);
   if (e != cudaSuccess) return cuda_fail(e, "refinement tags");
   *n_marked = (long long)res.count;
   for (int a = 0; a < 3; ++a) {
@@ -223,8 +259,9 @@ extern "C" eb_status eb_tag_cells(const eb_geom* G, const double* d_E, const dou
     bbox_hi[a] = res.count ? res.hi[a] + 1 : 0;
   }
   if (e_max) {
-    unsigned long long b = res.emax;
-    std::memcpy(e_max, &b, sizeof(double));
+    double m2 = 0.0;
+    std::memcpy(&m2, &res.emax, sizeof(double));
+    *e_max = std::sqrt(m2);
   }
   return EB_OK;
 }
