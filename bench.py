@@ -40,7 +40,7 @@ REF_STEP_SIDE = 24   # reference-arm steps: 24^3 + 12^3, a few seconds each
 C2_SIDE = 1024
 
 
-KERNEL_SOURCES = ("persistent.cuh", "sweep3d.cuh", "mg_kernels.cuh", "eb_common.cuh", "solver.cu")
+KERNEL_SOURCES = ("rbsolve.cuh", "rbsetup.cuh", "persistent.cuh", "sweep3d.cuh", "mg_kernels.cuh", "eb_common.cuh", "solver.cu")
 
 
 def kernel_sources_sha256(read=None) -> str:
@@ -218,29 +218,25 @@ def solve_bytes(ncell, dim, mixed, vcycles, outer, sweeps=4, launches=1):
 
 
 def kernels_at_scale(dev, E, W, n=384):
-    """The finest-level FP32 smoother (one tile-streamed sweep, both colours;
-    and one classic colour pass for comparison) and the fused residual +
-    restriction on a 3D pin-plane grid far larger than L2 (at 384^3 a sweep
-    touches ~0.7 GB), each launched on its own."""
+    """The finest-level FP32 phases (one colour of the smoother, the fused
+    residual + restriction, the prolongation) on a 3D pin-plane grid far larger
+    than L2 (at 384^3 a sweep touches ~0.7 GB), each launched on its own."""
     import torch
     g = E.Geometry(W.pin_plane_3d(n), device=dev)
     P = E.Poisson(g, precision="mixed", tol=1e-10, max_cycles=1)
-    sws, swb = P.profile(4, reps=20)
     sms, sb = P.profile(0, reps=40)
-    rms, rb = P.profile(5, reps=20)
-    rcms, rcb = P.profile(1, reps=20)
+    rms, rb = P.profile(1, reps=20)
+    pms, pb = P.profile(6, reps=20)
     peaks = _peaks()
     hbm = peaks["hbm_gbs"] if peaks else 6800.0
     out = {"workload": f"3D pin-plane {n}^3 with dielectric disk, FP32 finest level", "cells": n ** 3,
-           "sweep_ms": sws, "sweep_bytes": swb, "sweep_gbs": swb / sws / 1e6, "smooth_frac": swb / sws / 1e6 / hbm,
-           "sweep_note": "one red-black sweep, both colours in one tile-streamed (TMA) pass: read x, b, flags, write x",
            "smooth_colour_ms": sms, "smooth_colour_bytes": sb, "smooth_colour_gbs": sb / sms / 1e6,
-           "smooth_colour_frac": sb / sms / 1e6 / hbm,
+           "smooth_frac": sb / sms / 1e6 / hbm,
+           "smooth_note": "one colour on the colour-split level: read the other colour, b, flags, write the colour",
            "resid_restrict_ms": rms, "resid_restrict_bytes": rb, "resid_restrict_gbs": rb / rms / 1e6,
            "resid_restrict_frac": rb / rms / 1e6 / hbm,
-           "resid_restrict_note": "tile-streamed (TMA) residual + restriction: read x, b, flags, write coarse b, x",
-           "resid_restrict_blocks_ms": rcms, "resid_restrict_blocks_gbs": rcb / rcms / 1e6,
-           "resid_restrict_blocks_frac": rcb / rcms / 1e6 / hbm, "peak": hbm}
+           "prolong_ms": pms, "prolong_bytes": pb, "prolong_gbs": pb / pms / 1e6,
+           "prolong_frac": pb / pms / 1e6 / hbm, "peak": hbm}
     del P, g
     torch.cuda.empty_cache()
     return out
@@ -387,7 +383,7 @@ def run_gpu(args):
     ms = job_time(sum(ms_steps) / len(ms_steps))
     value = throughput(ncell, world, ms)
     infos = [r[0] for r in res]
-    # the dominant kernel: the persistent multigrid solve k_solve<float>, launched
+    # the dominant kernel: the persistent V-cycle k_rb_vcycle<float>, launched
     # for every coarse (256^3) and fine (128^3) correction; device time from CUDA
     # events on the stream it runs on, summed over its launches in a step
     kst = res[-1][1]
@@ -471,8 +467,8 @@ def run_gpu(args):
                    "l2": "inputs larger than L2 (134 MB per FP64 coarse field); 256 MB buffer written between steps",
                    "parallelism": f"{world} independent solves (one per GPU)"},
         "gpu_launches": int(statistics.median(i["kernel_launches"] for i in infos)),
-        "roofline": {"bound": "hbm", "kernel": "k_solve<float> (persistent multigrid: the FAC corrections' "
-                                               "FP32 V-cycles with FP64 defect correction)",
+        "roofline": {"bound": "hbm", "kernel": "k_rb_vcycle<float> (persistent multigrid: the FAC corrections' "
+                                               "FP32 V-cycles on colour-split levels)",
                      "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                      "traffic": traffic, "peak_source": "measured" if peaks else "fallback",
                      "ms_per_launch": k_ms / max(k_launch, 1), "bytes_per_launch": k_bytes / max(k_launch, 1),

@@ -133,7 +133,7 @@ def c4(count=64):
 
 
 TRACE_KIND = {1: "red", 2: "rows", 3: "black", 4: "write", 5: "resrows", 6: "restrict", 7: "prolong",
-              8: "coarseend", 9: "bottom", 12: "update", 13: "sweep"}
+              8: "coarseend", 9: "bottom", 12: "update", 13: "sweep", 14: "krylov"}
 
 
 def trace(workload, n=None, precision="mixed"):
@@ -193,11 +193,11 @@ def kernels_once(n, reps):
     on its own (eb_poisson_profile kernels 4, 0, 5, 1)."""
     P = E.Poisson(E.Geometry(W.pin_plane_3d(n)), precision="mixed", tol=1e-10, max_cycles=1)
     names = {4: "streamed sweep", 0: "colour pass", 5: "streamed residual + restriction",
-             1: "block residual + restriction", 6: "block prolongation"}
+             1: "residual + restriction", 6: "prolongation"}
     for k in (4, 0, 5, 1, 6):
         try:
             ms, by = P.profile(k, reps=reps)
-        except E.EBError as exc:  # no streamed level below 2^25 cells
+        except E.EBError as exc:  # streamed levels are built on request only
             print(json.dumps({"kernel": names[k], "n": n, "skipped": str(exc)}), flush=True)
             continue
         print(json.dumps({"kernel": names[k], "n": n, "ms": ms, "gbs": by / ms / 1e6}), flush=True)

@@ -340,7 +340,7 @@ __global__ void k_split_flags(int D, SplitDim d, const uint8_t* flags, const uin
 // one CTA: the rows of cells and phases with an unknown, in order (red first)
 __global__ void k_split_rows(SplitDim d, const uint8_t* flags, const int* irr_cell, int nirr, int nirr_red,
                              const int* row_ptr, const double* diag, int2* re, unsigned* rs, double* dg, double* di, int* rnat,
-                             int* inv, int* counts) {
+                             int* counts) {
   int at = 0, red = 0;
   for (int base = 0; base < 2 * nirr; base += (int)blockDim.x) {
     const int r = base + (int)threadIdx.x;
@@ -353,7 +353,6 @@ __global__ void k_split_rows(SplitDim d, const uint8_t* flags, const int* irr_ce
     int tot, totr;
     const int k = block_rank(v, &tot);
     block_rank(v && (r >> 1) < nirr_red, &totr);
-    if (r < 2 * nirr) inv[r] = v ? at + k : -1;
     if (v) {
       re[at + k] = make_int2(row_ptr[r], row_ptr[r + 1]);
       rs[at + k] = ((unsigned)(r & 1) << 31) | split_index(d, (unsigned)c);
@@ -375,32 +374,141 @@ __global__ void k_split_cols(SplitDim d, const int* col, long long nnz, unsigned
   const unsigned cl = (unsigned)col[e];
   out[e] = ((cl >> 30) << 31) | split_index(d, cl & 0x3fffffffu);
 }
-// coarse cells with a child that has a row, and their children's rows; the
-// order of the list does not matter (each entry writes its own cell)
-__global__ void k_split_special(int D, const uint8_t* fl, int f0, int f1, int f2, const int* irr_of_cell,
-                                const int* inv, int c0, int c1, int c2, int* sp, int* sprow, int* counts) {
+// Restriction rows: for every unknown of the coarse grid whose cell has a
+// child with a sparse row, the mean of its children's residuals as one row
+// over the fine level, the children's rows one after the other.  all: black
+// regular children too (without a sweep their residuals are not zero).  The
+// order of the rows does not matter (each writes its own unknown).
+// The groups that a pass takes from a list (rb_dense_list): counted into
+// n[colour], and written to out[colour] where that is given.
+__global__ void k_split_list(int D, SplitDim d, const uint8_t* f, int* n, unsigned* out0, unsigned* out1) {
+  const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x), colour = blockIdx.y, nq = d.hx / 4;
+  if (t >= d.H / 4) return;
+  const unsigned w = reinterpret_cast<const unsigned*>(f + (long long)colour * d.H)[t];
+  const unsigned m0 = regular_mask(w, 0), m1 = regular_mask(w, 1);
+  if (!(m0 | m1)) return;
+  QPos g;
+  const int row = t / nq;
+  g.t = t;
+  g.j = row % d.n1;
+  g.k = row / d.n1;
+  g.q0 = 4 * (t - row * nq);
+  const bool inner = inner_group(D, d.n0, d.n1, d.n2, g);
+  unsigned* out = colour ? out1 : out0;
+  for (unsigned p = 0; p < 2; ++p) {
+    if (!(p ? m1 : m0) || (inner && !(p && m0))) continue;
+    const int i = atomicAdd(n + colour, 1);
+    if (out) out[i] = (unsigned)t | p << 31;
+  }
+}
+struct RestrictView {
+  AlgView f;
+  SplitDim fd, cd;
+  const uint8_t* cf;
+  int c0, c1, c2, all;
+};
+__device__ __forceinline__ bool child_cell(const RestrictView& v, int C, int ch, int c[3], long long& cell) {
+  const int i = C % v.c0, j = C / v.c0 % v.c1, k = C / (v.c0 * v.c1);
+  c[0] = 2 * i + (ch & 1);
+  c[1] = 2 * j + ((ch >> 1) & 1);
+  c[2] = v.f.D == 3 ? 2 * k + (ch >> 2) : 0;
+  cell = (long long)c[0] + (long long)v.f.n[0] * (c[1] + (long long)v.f.n[1] * c[2]);
+  return c[0] < v.f.n[0] && c[1] < v.f.n[1] && c[2] < v.f.n[2];
+}
+__global__ void k_restrict_count(RestrictView v, int2* list, int* len, int* counts) {
   const int C = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (C >= c0 * c1 * c2) return;
-  const int i = C % c0, j = C / c0 % c1, k = C / (c0 * c1), nch = 1 << D;
+  if (C >= v.c0 * v.c1 * v.c2) return;
   bool any = false;
-  for (int ch = 0; ch < nch; ++ch) {
-    const int a = 2 * i + (ch & 1), b = 2 * j + ((ch >> 1) & 1), e = D == 3 ? 2 * k + (ch >> 2) : 0;
-    if (a < f0 && b < f1 && e < f2 && (fl[(long long)a + (long long)f0 * (b + (long long)f1 * e)] & F_IRR)) any = true;
-  }
+  int c[3];
+  long long cell;
+  for (int ch = 0; ch < (1 << v.f.D); ++ch)
+    if (child_cell(v, C, ch, c, cell) && (v.f.flags[cell] & F_IRR)) any = true;
   if (!any) return;
-  const int q = atomicAdd(counts + 2, 1);
-  sp[q] = C;
-  for (int ch = 0; ch < nch; ++ch) {
-    const int a = 2 * i + (ch & 1), b = 2 * j + ((ch >> 1) & 1), e = D == 3 ? 2 * k + (ch >> 2) : 0;
-    int r[2] = {-1, -1};
-    if (a < f0 && b < f1 && e < f2) {
-      const long long c = (long long)a + (long long)f0 * (b + (long long)f1 * e);
-      if (fl[c] & F_IRR)
-        for (int p = 0; p < 2; ++p) r[p] = inv[2ll * irr_of_cell[c] + p];
+  for (int p = 0; p < 2; ++p) {
+    if (!((v.cf[C] >> p) & 1)) continue;
+    int n = 0;
+    for (int ch = 0; ch < (1 << v.f.D); ++ch) {
+      if (!child_cell(v, C, ch, c, cell) || !((v.f.flags[cell] >> p) & 1)) continue;
+      if (v.f.flags[cell] & F_IRR) {
+        const long long r = 2ll * v.f.irr_of_cell[cell] + p;
+        if (v.f.diag[r] != 0.0) n += v.f.row_ptr[r + 1] - v.f.row_ptr[r] + 1;
+      } else if (v.all || !((c[0] + c[1] + c[2]) & 1)) {
+        n += 1 + 2 * v.f.D;
+      }
     }
-    sprow[(long long)q * 2 * nch + ch] = r[0];
-    sprow[(long long)q * 2 * nch + nch + ch] = r[1];
+    const int q = atomicAdd(counts + 2, 1);
+    list[q] = make_int2(C, p);
+    len[q] = n;
   }
+}
+// one CTA: exclusive sums of len[0..*n) in place, the total to *total
+__global__ void k_restrict_scan(int* len, const int* n, int* total) {
+  __shared__ int sh[1024];
+  int run = 0;
+  for (int base = 0; base < *n; base += 1024) {
+    const int i = base + (int)threadIdx.x;
+    const int v = i < *n ? len[i] : 0;
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    for (int o = 1; o < 1024; o <<= 1) {
+      const int y = (int)threadIdx.x >= o ? sh[threadIdx.x - o] : 0;
+      __syncthreads();
+      sh[threadIdx.x] += y;
+      __syncthreads();
+    }
+    if (i < *n) len[i] = run + sh[threadIdx.x] - v;
+    run += sh[1023];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *total = run;
+}
+__global__ void k_restrict_fill(RestrictView v, const int2* list, const int* start, const int* n, int4* sd,
+                                unsigned* scol, double* sval) {
+  const int q = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (q >= *n) return;
+  const int C = list[q].x, p = list[q].y;
+  const double sc = 1.0 / (double)(1 << v.f.D);
+  int at = start[q];
+  unsigned mask = 0u;
+  for (int ch = 0; ch < (1 << v.f.D); ++ch) {
+    int c[3];
+    long long cell;
+    if (!child_cell(v, C, ch, c, cell) || !((v.f.flags[cell] >> p) & 1)) continue;
+    const unsigned self = ((unsigned)p << 31) | split_index(v.fd, (unsigned)cell);
+    if (v.f.flags[cell] & F_IRR) {
+      const long long r = 2ll * v.f.irr_of_cell[cell] + p;
+      if (v.f.diag[r] == 0.0) continue;
+      mask |= 1u << ch;
+      scol[at] = self;
+      sval[at++] = sc * v.f.diag[r];
+      for (int e = v.f.row_ptr[r]; e < v.f.row_ptr[r + 1]; ++e) {
+        const unsigned cl = (unsigned)v.f.col[e];
+        scol[at] = ((cl >> 30) << 31) | split_index(v.fd, cl & 0x3fffffffu);
+        sval[at++] = sc * v.f.val[e];
+      }
+    } else if (v.all || !((c[0] + c[1] + c[2]) & 1)) {
+      mask |= 1u << ch;
+      const int me = at++;
+      double dg = v.f.lam[p] / v.f.ce[p];
+      long long st = 1;
+      for (int a = 0; a < v.f.D; ++a) {
+        for (int s = 0; s < 2; ++s) {
+          const bool open = s ? c[a] < v.f.n[a] - 1 : c[a] > 0;
+          const double w = v.f.w[2 * a + s];
+          const long long nb = cell + ((s == 1) == open ? st : -st);
+          scol[at] = ((unsigned)p << 31) | split_index(v.fd, (unsigned)nb);
+          sval[at++] = -sc * v.f.ce[p] * (open ? 1.0 : w / 3.0);
+          dg += open ? 1.0 : 3.0 * w;
+        }
+        st *= v.f.n[a];
+      }
+      scol[me] = self;
+      sval[me] = sc * v.f.ce[p] * dg;
+    }
+  }
+  const int i = C % v.c0, j = C / v.c0 % v.c1, k = C / (v.c0 * v.c1);
+  const int base = i + v.fd.hx * (2 * j + v.f.n[1] * 2 * k);
+  sd[q] = make_int4(start[q], (at - start[q]) | (int)(mask << 16) | (p << 24), base, (int)split_index(v.cd, (unsigned)C));
 }
 // first and last x row that holds a dielectric unknown
 __global__ void k_phase1_rows(const uint8_t* flags, long long ncell, int n0, int* lohi) {

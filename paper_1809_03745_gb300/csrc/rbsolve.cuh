@@ -56,6 +56,7 @@ struct RLev {
   int two;  // both phases
   int dense;  // the level has regular cells
   int full;   // x rows fill their groups (n[0] a multiple of 8)
+  int wide;   // at least two cells along every axis
   T dge[2];   // diagonal count of a cell at the low / high x wall and nowhere else
   T ide[2][2];  // and its reciprocal with the shift, [side][phase]
   int p1o, p1n;  // the entries of a dielectric half that are stored (the slabs that hold the phase)
@@ -65,17 +66,25 @@ struct RLev {
   T* x[2][3];
   T* b[2][2];  // [phase][colour]
   const uint8_t* f[2];
+  // groups per colour that a pass does not find on the common path (group | phase << 31), see rb_dense
+  const unsigned* gl[2];
+  int ngl[2];
   // sparse rows of cells and phases with an unknown, red first
   int nr, nr0;
   int staged;            // entries in T in this CTA's shared memory
   const int2* re;        // first and last entry
   const unsigned* rs;    // the row's own cell: phase << 31 | colour * H + position
   const unsigned* col;   // entries' cells, encoded alike
-  const void *val, *diag, *dinv;  // double, or T when staged; dinv = 1 / diag
-  // coarse cells (of the next level) with a child that has a sparse row, and
-  // per such cell the rows of its children (slot child + 2^D * phase, -1: none)
+  const void *val, *dinv;  // double, or T when staged; dinv = 1 / diagonal
+  // restriction rows: per unknown of the next level whose cell has a child
+  // with a sparse row, the mean of its children's residuals as one row over
+  // this level (first entry; entries | children mask << 16 | phase << 24;
+  // position of child 0; the unknown as colour * H + position)
   int nsp;
-  const int *sp, *sprow;
+  int sstaged;
+  const int4* sd;
+  const unsigned* scol;
+  const void* sval;  // double, or T when staged
 };
 
 template <class T>
@@ -87,11 +96,11 @@ struct RHier {
   const T* binv;    // [bm][bm] row-major, slots as bslot
   const unsigned* bslot;  // slot -> phase << 31 | colour * H + position; ~0u: no unknown
   int smem;         // levels lc.. in CTA 0's shared memory
-  RLev<T> L[RMAX];
+  RLev<T> L[RMAX + 1];  // L[RMAX]: level lc as the whole group sees it
   // byte offsets into shared memory of levels lc..
   int off_x[RMAX][2][3], off_b[RMAX][2][2], off_f[RMAX][2], off_re[RMAX], off_rs[RMAX], off_col[RMAX], off_val[RMAX],
-      off_dg[RMAX], off_di[RMAX], off_sp[RMAX], off_spr[RMAX], nnz[RMAX];
-  int srows[RMAX];  // rows staged too
+      off_di[RMAX], off_sd[RMAX], off_sc[RMAX], off_sv[RMAX], nnz[RMAX], snnz[RMAX];
+  int srows[RMAX];  // 1: rows staged too, 2: restriction rows
   // finest level in FP64: natural cell of every sparse row, entries' natural
   // columns and values, the rows' diagonals
   const int *rnat, *ncol;
@@ -103,15 +112,22 @@ struct RHier {
   KryState* kst;
 };
 
+// What a phase runs on: the whole group of CTAs, or CTA 0 alone.  Kept in
+// shared memory; what differs between threads is worked out where it is used.
 struct RCtx {
-  int i0, st;        // this thread's first item and the stride over items
-  int g0, gst;       // groups of 8 lanes, counted from the other end
+  int st, gst;  // strides over items and over groups of 8 lanes
   bool local;
+  int gcta, gsize;
   Barrier B;
   unsigned* epoch;
   unsigned long long* tr;
   unsigned* tn;
-  int gcta, gsize;
+  __device__ __forceinline__ int wi() const { return (int)(threadIdx.x >> 5) * gsize + gcta; }  // warps interleaved over the CTAs
+  __device__ __forceinline__ int i0() const { return local ? (int)threadIdx.x : wi() * 32 + (int)(threadIdx.x & 31); }
+  // groups of 8 lanes are counted from the other end
+  __device__ __forceinline__ int g0() const {
+    return local ? (int)(threadIdx.x >> 3) : gst - 1 - (wi() * 4 + (int)((threadIdx.x >> 3) & 3));
+  }
   __device__ __forceinline__ bool sync(int code) const {
     bool ok = true;
     if (local) __syncthreads();
@@ -123,6 +139,32 @@ struct RCtx {
     return ok;
   }
 };
+
+// The state of a launch.  The phases are functions out of line that find it
+// here and take a few integers: ptxas gives a function the registers that its
+// callers leave, and with descriptions, contexts and loop state held in the
+// callers' registers the phases spilled in their loops (a tenth of all
+// instructions; a solve of 1024^2 took 7.5 ms instead of 6.9, one of 256^3 35.7 instead of 33.7).
+struct KryState {
+  int count, next;   // directions kept, slot of the next one
+  double g[KH][KH];  // (q_i, q_j) by slot
+  double rn[KH];     // 1 / |q_i|
+};
+template <class T>
+struct RShared {
+  RHier<T> H;
+  RCtx c[2];  // the group, CTA 0 alone
+  Op<double> F;
+  unsigned epoch, tn;
+  T red[PT / 32][KDOT];
+  double dots[KDOT], coef[KH];
+  KryState K;
+};
+template <class T>
+__device__ __forceinline__ RShared<T>& rsh() {
+  __shared__ RShared<T> s;
+  return s;
+}
 
 template <class T>
 __device__ __forceinline__ void st4(T* p, const T v[4]) {
@@ -239,32 +281,97 @@ __device__ __forceinline__ void quad_sums(const RLev<T>& L, const QPos& g, QNb<T
     dg[e] = d;
   }
 }
-// The same for a group away from the y and z walls in a full row, in a third
-// of the instructions: the group may touch one x wall, with its first lane
-// (s = 0) or its last one (s = 1), whose diagonal count is `de`.
+// The same in a third of the instructions on levels of two cells or more along
+// each axis: every load goes out at once, what lies outside a y or z wall from
+// the opposite side (which is what the wall's stencil takes, scaled), and the
+// cells at the x walls, lane 0 of a row's first group and lane `hi` of its last
+// one, are put right afterwards.
+struct QEnd {
+  bool lo;
+  int hi;  // 4 or more: none
+};
 template <class T>
-__device__ __forceinline__ bool quad_inner(const RLev<T>& L, const QPos& g) {
-  return L.full && (unsigned)(g.j - 1) < (unsigned)(L.n[1] - 2) && (L.D == 2 || (unsigned)(g.k - 1) < (unsigned)(L.n[2] - 2));
+__device__ __forceinline__ QEnd quad_end(const RLev<T>& L, const QPos& g) {
+  const int last = L.n[0] - 1 - 2 * g.q0 - g.s;  // of both colours' cells, the row's last one lies `last` cells on
+  return QEnd{g.s == 0 && g.q0 == 0, (last & 1) ? 4 : last >> 1};
 }
 template <class T>
-__device__ __forceinline__ void quad_load_in(const RLev<T>& L, const QPos& g, const T* xn, QNb<T>& v, bool& edge) {
+__device__ __forceinline__ void quad_load_in(const RLev<T>& L, const QPos& g, const T* xn, QNb<T>& v) {
   const T* c = xn + 4 * g.t;
-  edge = g.s ? g.q0 + 4 == L.hx : g.q0 == 0;
   ld4(c, v.c);
-  v.xs = c[edge ? 0 : (g.s ? 4 : -1)];
-  ld4(c - L.hx, v.ym);
-  ld4(c + L.hx, v.yp);
+  v.xs = c[g.s ? (g.q0 + 4 < L.hx ? 4 : 0) : (g.q0 ? -1 : 0)];
+  ld4(c + (g.j > 0 ? -L.hx : L.hx), v.ym);
+  ld4(c + (g.j < L.n[1] - 1 ? L.hx : -L.hx), v.yp);
   if (L.D == 3) {
     const int sz = L.hx * L.n[1];
-    ld4(c - sz, v.zm);
-    ld4(c + sz, v.zp);
+    ld4(c + (g.k > 0 ? -sz : sz), v.zm);
+    ld4(c + (g.k < L.n[2] - 1 ? sz : -sz), v.zp);
   } else {
 #pragma unroll
     for (int e = 0; e < 4; ++e) v.zm[e] = v.zp[e] = T(0);
   }
 }
+// scales what was loaded across y and z walls; the diagonal count they add
 template <class T>
-__device__ __forceinline__ void quad_sums_in(const RLev<T>& L, const QPos& g, const QNb<T>& v, bool edge, T sum[4]) {
+__device__ __forceinline__ T quad_walls(const RLev<T>& L, const QPos& g, QNb<T>& v) {
+  T d = T(0);
+  if (g.j == 0) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v.ym[e] *= L.w3[2];
+    d += T(3) * L.wr[2] - T(1);
+  }
+  if (g.j == L.n[1] - 1) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v.yp[e] *= L.w3[3];
+    d += T(3) * L.wr[3] - T(1);
+  }
+  if (L.D == 3) {
+    if (g.k == 0) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v.zm[e] *= L.w3[4];
+      d += T(3) * L.wr[4] - T(1);
+    }
+    if (g.k == L.n[2] - 1) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v.zp[e] *= L.w3[5];
+      d += T(3) * L.wr[5] - T(1);
+    }
+  }
+  return d;
+}
+template <class T>
+__device__ __forceinline__ void quad_sums_in(const RLev<T>& L, const QPos& g, const QEnd& x, const QNb<T>& v, T sum[4]) {
+  const T o = v.xs + (g.s ? v.c[3] : v.c[0]), a = v.c[0] + v.c[1], b = v.c[1] + v.c[2], d = v.c[2] + v.c[3];
+  T h[4] = {g.s ? a : o, g.s ? b : a, g.s ? d : b, g.s ? o : d};
+  if (x.lo) h[0] = v.c[0] + L.w3[0] * v.c[0];
+  if ((unsigned)x.hi < 4u) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const T l = g.s ? v.c[e] : (e ? v.c[e ? e - 1 : 0] : v.xs);
+      if (e == x.hi) h[e] = l + L.w3[1] * l;
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) sum[e] = (h[e] + (v.ym[e] + v.yp[e])) + (v.zm[e] + v.zp[e]);
+}
+// A group away from the y and z walls whose row goes on behind it or ends with
+// its last lane: only lane 0 (s = 0) or lane 3 (s = 1) may lie at an x wall,
+// and nothing has to be scaled.  Nearly every group is one, and takes two
+// thirds of the instructions.
+__host__ __device__ __forceinline__ bool inner_group(int D, int n0, int n1, int n2, const QPos& g) {
+  return (n0 % 8 == 0 || 2 * g.q0 + 8 < n0) && g.j > 0 && g.j < n1 - 1 && (D == 2 || (g.k > 0 && g.k < n2 - 1));
+}
+template <class T>
+__device__ __forceinline__ bool quad_inner(const RLev<T>& L, const QPos& g) {
+  return (L.full || 2 * g.q0 + 8 < L.n[0]) && (unsigned)(g.j - 1) < (unsigned)(L.n[1] - 2) &&
+         (L.D == 2 || (unsigned)(g.k - 1) < (unsigned)(L.n[2] - 2));
+}
+template <class T>
+__device__ __forceinline__ bool quad_edge(const RLev<T>& L, const QPos& g) {
+  return g.s ? g.q0 + 4 == L.hx : g.q0 == 0;
+}
+template <class T>
+__device__ __forceinline__ void quad_sums_inner(const RLev<T>& L, const QPos& g, bool edge, const QNb<T>& v, T sum[4]) {
   const T ce = g.s ? v.c[3] : v.c[0];
   const T xs = edge ? L.w3[g.s] * ce : v.xs;
   const T o = xs + ce, a = v.c[0] + v.c[1], b = v.c[1] + v.c[2], d = v.c[2] + v.c[3];
@@ -272,7 +379,28 @@ __device__ __forceinline__ void quad_sums_in(const RLev<T>& L, const QPos& g, co
 #pragma unroll
   for (int e = 0; e < 4; ++e) sum[e] = (h[e] + (v.ym[e] + v.yp[e])) + (v.zm[e] + v.zp[e]);
 }
-
+// operator values of such a group from its own values xo
+template <class T>
+__device__ __forceinline__ void quad_apply_in(const RLev<T>& L, const QPos& g, int p, QNb<T>& v, const T xo[4], T q[4]) {
+  T sum[4];
+  const T ce = L.ceps[p];
+  if (quad_inner(L, g)) {
+    const bool edge = quad_edge(L, g);
+    quad_sums_inner(L, g, edge, v, sum);
+    const T d = T(2 * L.D) + L.lh[p], de = edge ? L.dge[g.s] + L.lh[p] : d;
+    q[0] = ce * ((g.s ? d : de) * xo[0] - sum[0]);
+    q[1] = ce * (d * xo[1] - sum[1]);
+    q[2] = ce * (d * xo[2] - sum[2]);
+    q[3] = ce * ((g.s ? de : d) * xo[3] - sum[3]);
+    return;
+  }
+  const QEnd x = quad_end(L, g);
+  const T dw = quad_walls(L, g, v);
+  quad_sums_in(L, g, x, v, sum);
+  const T d = T(2 * L.D) + dw + L.lh[p], d0 = x.lo ? L.dge[0] + dw + L.lh[p] : d, d1 = L.dge[1] + dw + L.lh[p];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) q[e] = ce * ((e == x.hi ? d1 : (e ? d : d0)) * xo[e] - sum[e]);
+}
 template <class T>
 __device__ __forceinline__ T quad_inv(const RLev<T>& L, int p, T dg) {
   return dg == T(2 * L.D) ? L.idg[p] : rcp_rn(dg + L.lh[p]);
@@ -290,112 +418,189 @@ __device__ __forceinline__ void quad_store(T* dst, unsigned m, const T v[4]) {
     if ((m >> (8 * e)) & 1u) dst[e] = v[e];
 }
 
-// one group of one phase: relaxed values written
+// The residual (bb) or the operator value (no bb) of any group, out of line:
+// for levels one cell thick and the residual of both colours.  A persistent
+// kernel runs a different phase every few microseconds, and the instructions
+// it has to fetch for one cost more than a small level's arithmetic.
 template <class T>
-__device__ __forceinline__ void quad_relax(const RLev<T>& L, const QPos& g, int p, unsigned m, QNb<T>& v, const T bb[4],
-                                           T* dst) {
-  T sum[4], dg[4], o[4];
+__device__ __noinline__ void quad_slow(const RLev<T>& __restrict__ L, int t, int colour, int p, const T* xn, const T* xo,
+                                       const T* bb, T* o) {
+  const QPos g = quad_pos(L, t, colour);
+  QNb<T> v;
+  T sum[4], dg[4];
+  quad_load(L, g, xn, v);
   quad_sums(L, g, v, sum, dg);
 #pragma unroll
-  for (int e = 0; e < 4; ++e) o[e] = (L.h2e[p] * bb[e] + sum[e]) * quad_inv(L, p, dg[e]);
-  quad_store(dst + 4 * (long long)g.t, m, o);
-}
-
-template <class T>
-__device__ __forceinline__ void quad_relax_in(const RLev<T>& L, const QPos& g, int p, unsigned m, const QNb<T>& v,
-                                              bool edge, const T bb[4], T* dst) {
-  T sum[4], o[4];
-  quad_sums_in(L, g, v, edge, sum);
-  const T inv = L.idg[p], ie = edge ? L.ide[g.s][p] : inv;
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    o[e] = (L.h2e[p] * bb[e] + sum[e]) * (e == 0 ? (g.s ? inv : ie) : (e == 3 ? (g.s ? ie : inv) : inv));
-  quad_store(dst + 4 * (long long)g.t, m, o);
+  for (int e = 0; e < 4; ++e) {
+    const T r = L.ceps[p] * ((dg[e] + L.lh[p]) * xo[4 * (long long)t + e] - sum[e]);
+    o[e] = bb ? bb[4 * (long long)t + e] - r : r;
+  }
 }
 
 // buffers of a level after s sweeps
 __device__ __forceinline__ int rb_red(int s) { return (2 * s) % 3; }
 __device__ __forceinline__ int rb_black(int s) { return (2 * s + 1) % 3; }
 
-// the regular cells of one colour in sweep s (zero: the iterate is zero
-// before the sweep and not read)
+// the diagonals' reciprocals of a group: inside, at lane 0, at lane x.hi
 template <class T>
-__device__ __noinline__ void rb_dense(const RLev<T>& __restrict__ L, int colour, int s, bool zero, const RCtx& c) {
+__device__ __forceinline__ void quad_inverse(const RLev<T>& L, const QEnd& x, int p, T dw, T& in, T& v0, T& v1) {
+  in = L.idg[p];
+  v0 = x.lo ? L.ide[0][p] : in;
+  v1 = L.ide[1][p];
+  if (dw != T(0)) {
+    in = rcp_rn(T(2 * L.D) + dw + L.lh[p]);
+    v0 = x.lo ? rcp_rn(L.dge[0] + dw + L.lh[p]) : in;
+    v1 = rcp_rn(L.dge[1] + dw + L.lh[p]);
+  }
+}
+
+// The regular cells of one colour in sweep s: the inner groups, the phase of
+// each that rb_dense_list does not have.
+template <class T>
+__device__ __noinline__ void rb_dense(int lv, int colour, int s, int cx) {
+  const RLev<T>& L = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
   const int in = colour ? rb_red(s + 1) : rb_black(s);
   const int out = colour ? rb_black(s + 1) : rb_red(s + 1);
   const unsigned* fw = reinterpret_cast<const unsigned*>(L.f[colour]);
-  if (zero && colour == 0) {
-    for (int t = c.i0; t < L.nqt; t += c.st) {
-      const unsigned w = fw[t];
-      for (int p = 0; p < 2; ++p) {
-        const unsigned m = regular_mask(w, p);
-        if (!m) continue;
-        QPos g = quad_pos(L, t, 0);
-        QNb<T> v;
-        T bb[4], sum[4], dg[4], o[4];
-        ld4(L.b[p][0] + 4 * (long long)t, bb);
+  const int st = c.st, nqt = L.nqt;
+  // U groups per thread with all their loads issued first; the flags of the
+  // next ones are loaded one iteration ahead
+  constexpr int U = sizeof(T) == 4 ? 2 : 1;
+  unsigned wn[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) wn[u] = c.i0() + u * st < nqt ? fw[c.i0() + u * st] : 0u;
+#pragma unroll 1
+  for (int t0 = c.i0(); t0 < nqt; t0 += U * st) {
+    unsigned w[U], m[U];
+    int pp[U];
+    QPos g[U];
+    QNb<T> v[U];
+    T bb[U][4];
+    bool ed[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      w[u] = wn[u];
+      const int tn = t0 + (U + u) * st;
+      wn[u] = tn < nqt ? fw[tn] : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      m[u] = regular_mask(w[u], 0);
+      pp[u] = m[u] ? 0 : 1;
+      if (!m[u]) m[u] = regular_mask(w[u], 1);
+      if (!m[u]) continue;
+      g[u] = quad_pos(L, t0 + u * st, colour);
+      if (!quad_inner(L, g[u])) {
+        m[u] = 0u;
+        continue;
+      }
+      const T* x = L.x[pp[u]][in] + 4 * g[u].t;
+      ed[u] = quad_edge(L, g[u]);
+      ld4(x, v[u].c);
+      v[u].xs = x[ed[u] ? 0 : (g[u].s ? 4 : -1)];
+      ld4(x - L.hx, v[u].ym);
+      ld4(x + L.hx, v[u].yp);
+      if (L.D == 3) {
+        const int sz = L.hx * L.n[1];
+        ld4(x - sz, v[u].zm);
+        ld4(x + sz, v[u].zp);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[u].zm[e] = v[u].zp[e] = T(0);
+      }
+      ld4(L.b[pp[u]][colour] + 4 * g[u].t, bb[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (!m[u]) continue;
+      T o[4], sum[4];
+      const int p = pp[u];
+      const T h = L.h2e[p], iv = L.idg[p], ve = ed[u] ? L.ide[g[u].s][p] : iv;
+      quad_sums_inner(L, g[u], ed[u], v[u], sum);
+      o[0] = (h * bb[u][0] + sum[0]) * (g[u].s ? iv : ve);
+      o[1] = (h * bb[u][1] + sum[1]) * iv;
+      o[2] = (h * bb[u][2] + sum[2]) * iv;
+      o[3] = (h * bb[u][3] + sum[3]) * (g[u].s ? ve : iv);
+      quad_store(L.x[p][out] + 4 * g[u].t, m[u], o);
+    }
+  }
+}
+// The other groups, from a list made at set-up: those at a y or z wall or in
+// the last group of a padded row, and the dielectric's cells of a group that
+// holds both phases.  Handled where rb_dense meets them they cost a 1024^2
+// level 1.1 us of a pass and a 256^3 level 6: the general arithmetic is
+// branches and code in the way of every group.  Spread from the middle of the
+// grid on, so that small levels have them on warps of their own.
+template <class T>
+__device__ __noinline__ void rb_dense_list(int lv, int colour, int s, int cx) {
+  const RLev<T>& L = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
+  const int in = colour ? rb_red(s + 1) : rb_black(s);
+  const int out = colour ? rb_black(s + 1) : rb_red(s + 1);
+  const int n = L.ngl[colour], half = c.st / 2;
+  const unsigned* gl = L.gl[colour];
+  const uint8_t* f = L.f[colour];
+  for (int i = c.i0() < half ? c.i0() + half : c.i0() - half; i < n; i += c.st) {
+    const unsigned en = gl[i];
+    const int p = (int)(en >> 31), t = (int)(en & 0x7fffffffu);
+    const unsigned m = regular_mask(reinterpret_cast<const unsigned*>(f)[t], p);
+    const QPos g = quad_pos(L, t, colour);
+    QNb<T> v;
+    T bb[4], sum[4], o[4];
+    ld4(L.b[p][colour] + 4 * t, bb);
+    if (L.wide) {
+      T iv, v0, v1;
+      const QEnd x = quad_end(L, g);
+      quad_load_in(L, g, L.x[p][in], v);
+      const T dw = quad_walls(L, g, v);
+      quad_sums_in(L, g, x, v, sum);
+      quad_inverse(L, x, p, dw, iv, v0, v1);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[e] = (L.h2e[p] * bb[e] + sum[e]) * (e == x.hi ? v1 : (e ? iv : v0));
+    } else {
+      T dg[4];
+      quad_load(L, g, L.x[p][in], v);
+      quad_sums(L, g, v, sum, dg);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[e] = (L.h2e[p] * bb[e] + sum[e]) * quad_inv(L, p, dg[e]);
+    }
+    quad_store(L.x[p][out] + 4 * t, m, o);
+  }
+}
+// all of them in the first red pass over a zero iterate, which is not read
+template <class T>
+__device__ __noinline__ void rb_dense_zero(int lv, int s, int cx) {
+  const RLev<T>& L = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
+  const int out = rb_red(s + 1);
+  const unsigned* fw = reinterpret_cast<const unsigned*>(L.f[0]);
+  for (int t = c.i0(); t < L.nqt; t += c.st) {
+    const unsigned w = fw[t];
+#pragma unroll 1
+    for (int p = 0; p <= L.two; ++p) {
+      const unsigned m = regular_mask(w, p);
+      if (!m) continue;
+      T o[4], bb[4];
+      const QPos g = quad_pos(L, t, 0);
+      QNb<T> v;
+      ld4(L.b[p][0] + 4 * t, bb);
+      if (L.wide) {
+        const QEnd x = quad_end(L, g);
+        T iv, v0, v1;
+        quad_inverse(L, x, p, quad_walls(L, g, v), iv, v0, v1);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[e] = L.h2e[p] * bb[e] * (e == x.hi ? v1 : (e ? iv : v0));
+      } else {
+        T sum[4], dg[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) v.c[e] = v.ym[e] = v.yp[e] = v.zm[e] = v.zp[e] = T(0);
         v.xs = T(0);
         quad_sums(L, g, v, sum, dg);
 #pragma unroll
         for (int e = 0; e < 4; ++e) o[e] = L.h2e[p] * bb[e] * quad_inv(L, p, dg[e]);
-        quad_store(L.x[p][out] + 4 * (long long)t, m, o);
       }
-    }
-    return;
-  }
-  // U groups per thread with all their loads issued first; the flags of the
-  // next ones are loaded one iteration ahead
-  constexpr int U = sizeof(T) == 4 ? 2 : 1;
-  unsigned wn[U];
-#pragma unroll
-  for (int u = 0; u < U; ++u) wn[u] = c.i0 + u * c.st < L.nqt ? fw[c.i0 + u * c.st] : 0u;
-  for (int t0 = c.i0; t0 < L.nqt; t0 += U * c.st) {
-    unsigned w[U], m[U];
-    int pp[U];
-    QPos g[U];
-    QNb<T> v[U];
-    T bb[U][4];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      w[u] = wn[u];
-      const int tn = t0 + (U + u) * c.st;
-      wn[u] = tn < L.nqt ? fw[tn] : 0u;
-    }
-    bool ed[U], in4[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      m[u] = regular_mask(w[u], 0);
-      pp[u] = m[u] ? 0 : 1;
-      if (!m[u]) m[u] = regular_mask(w[u], 1);
-      in4[u] = false;
-      if (!m[u]) continue;
-      g[u] = quad_pos(L, t0 + u * c.st, colour);
-      in4[u] = quad_inner(L, g[u]);
-      if (in4[u]) {
-        quad_load_in(L, g[u], L.x[pp[u]][in], v[u], ed[u]);
-        ld4(L.b[pp[u]][colour] + 4 * g[u].t, bb[u]);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (!m[u]) continue;
-      if (in4[u]) {
-        quad_relax_in(L, g[u], pp[u], m[u], v[u], ed[u], bb[u], L.x[pp[u]][out]);
-      } else {
-        quad_load(L, g[u], L.x[pp[u]][in], v[u]);
-        ld4(L.b[pp[u]][colour] + 4 * (long long)g[u].t, bb[u]);
-        quad_relax(L, g[u], pp[u], m[u], v[u], bb[u], L.x[pp[u]][out]);
-      }
-      if (pp[u] == 0 && m[u] != 0xffffffffu && L.two) {  // lanes of the other phase
-        const unsigned m1 = regular_mask(w[u], 1);
-        if (m1) {
-          quad_load(L, g[u], L.x[1][in], v[u]);
-          ld4(L.b[1][colour] + 4 * (long long)g[u].t, bb[u]);
-          quad_relax(L, g[u], 1, m1, v[u], bb[u], L.x[1][out]);
-        }
-      }
+      quad_store(L.x[p][out] + 4 * t, m, o);
     }
   }
 }
@@ -450,14 +655,14 @@ __device__ __forceinline__ V row_sum1(const RLev<T>& L, int2 re, const Gather<T>
   return s;
 }
 
-// a lane's part (entries g, g + 8, ...) of the sum by a group of 8 lanes, all
-// loads of up to 48 entries of the row in flight at once
-template <class T, class V>
-__device__ __forceinline__ V row_sum8(const unsigned* __restrict__ col, const V* __restrict__ val, int2 re, int g,
+// a lane's part (entries g, g + GL, ...) of the sum by a group of GL lanes, the
+// loads of up to six entries per lane in flight at once
+template <class T, class V, int GL>
+__device__ __forceinline__ V row_sumg(const unsigned* __restrict__ col, const V* __restrict__ val, int2 re, int g,
                                       const Gather<T>& x, unsigned lim) {
   constexpr int RU = 6;
   V s = V(0);
-  for (int e = re.x + g; e < re.y; e += 8 * RU) {
+  for (int e = re.x + g; e < re.y; e += GL * RU) {
     unsigned cl[RU];
     V a[RU];
     T xv[RU];
@@ -465,13 +670,13 @@ __device__ __forceinline__ V row_sum8(const unsigned* __restrict__ col, const V*
     for (int k = 0; k < RU; ++k) {
       cl[k] = 0x7fffffffu;
       a[k] = V(0);
-      if (e + 8 * k < re.y) {
-        cl[k] = col[e + 8 * k];
-        a[k] = val[e + 8 * k];
+      if (e + GL * k < re.y) {
+        cl[k] = col[e + GL * k];
+        a[k] = val[e + GL * k];
       }
     }
 #pragma unroll
-    for (int k = 0; k < RU; ++k) xv[k] = e + 8 * k < re.y && (cl[k] & 0x7fffffffu) < lim ? x(cl[k]) : T(0);
+    for (int k = 0; k < RU; ++k) xv[k] = e + GL * k < re.y && (cl[k] & 0x7fffffffu) < lim ? x(cl[k]) : T(0);
 #pragma unroll
     for (int k = 0; k < RU; ++k) s += a[k] * (V)xv[k];
   }
@@ -486,7 +691,9 @@ __device__ __forceinline__ V row_sum8(const unsigned* __restrict__ col, const V*
 // warps for the two; the sum is in a fixed lane order.  Inside CTA 0 a thread
 // takes a row.
 template <class T, class V>
-__device__ __noinline__ void rb_rows_v(const RLev<T>& __restrict__ L, int colour, int s, bool zero, const RCtx& c) {
+__device__ __noinline__ void rb_rows_v(int lv, int colour, int s, bool zero, int cx) {
+  const RLev<T>& L = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
   const int r0 = colour ? L.nr0 : 0, r1 = colour ? L.nr : L.nr0;
   const int ired = colour ? rb_red(s + 1) : rb_red(s), iblk = rb_black(s);
   const int out = colour ? rb_black(s + 1) : rb_red(s + 1);
@@ -508,7 +715,7 @@ __device__ __noinline__ void rb_rows_v(const RLev<T>& __restrict__ L, int colour
   const unsigned gmask = 0xffu << (threadIdx.x & 24);
   const V* val = (const V*)L.val;
   const int rend = r0 + ((r1 - r0 + c.gst - 1) / c.gst) * c.gst;  // every lane of a warp runs the same trips
-  for (int r = r0 + c.g0; r < rend; r += c.gst) {
+  for (int r = r0 + c.g0(); r < rend; r += c.gst) {
     const bool live = r < r1;
     const int2 re = live ? L.re[r] : make_int2(0, 0);
     const unsigned cl = live ? L.rs[r] : 0u;
@@ -518,7 +725,7 @@ __device__ __noinline__ void rb_rows_v(const RLev<T>& __restrict__ L, int colour
     if (live) {
       const T* b = rb_rhs(L, cl, pos);
       bc = (V)b[pos];
-      if (lim) sum = row_sum8<T, V>(L.col, val, re, g, x, lim);
+      if (lim) sum = row_sumg<T, V, 8>(L.col, val, re, g, x, lim);
     }
     for (int off = 4; off > 0; off >>= 1) sum += __shfl_xor_sync(gmask, sum, off);
     if (live && g == 0) L.x[cl >> 31][out][pos] = (T)((bc - sum) * d);
@@ -527,32 +734,47 @@ __device__ __noinline__ void rb_rows_v(const RLev<T>& __restrict__ L, int colour
 
 // one colour of sweep s
 template <class T>
-__device__ __forceinline__ void rb_pass(const RLev<T>& L, int colour, int s, bool zero, const RCtx& c) {
-  const int n = colour ? L.nr - L.nr0 : L.nr0;
-  if (n) {
-    if (L.staged) rb_rows_v<T, T>(L, colour, s, zero, c);
-    else rb_rows_v<T, double>(L, colour, s, zero, c);
+__device__ __forceinline__ void rb_pass(int lv, int colour, int s, bool zero, int cx) {
+  const RLev<T>& L = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
+  const bool rows = colour ? L.nr > L.nr0 : L.nr0 > 0;
+  // rows and regular cells are independent: every other warp takes the rows
+  // last, so that their chains of dependent loads and the regular cells'
+  // streams share the pass
+  const bool late = L.dense && !c.local && ((threadIdx.x >> 5) & 1), none = zero && colour == 0;
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    if ((h != 0) == late) {
+      if (L.ngl[colour] && !none) rb_dense_list<T>(lv, colour, s, cx);
+      if (!rows) continue;
+      if (L.staged) rb_rows_v<T, T>(lv, colour, s, zero, cx);
+      else rb_rows_v<T, double>(lv, colour, s, zero, cx);
+    } else if (L.dense) {
+      if (none) rb_dense_zero<T>(lv, s, cx);
+      else rb_dense<T>(lv, colour, s, cx);
+    }
   }
-  if (L.dense) rb_dense(L, colour, s, zero, c);
 }
 
 // sweeps s0 .. s1 - 1 of level l; zero: the first one starts from a zero
 // iterate, which is not read
 template <class T>
-__device__ __noinline__ bool rb_smooth(const RLev<T>& L, int s0, int s1, bool zero, const RCtx& c, int l) {
+__device__ __forceinline__ bool rb_smooth(int lv, int s0, int s1, bool zero, int cx, int l) {
   for (int s = s0; s < s1; ++s)
     for (int colour = 0; colour < 2; ++colour) {
-      rb_pass(L, colour, s, zero && s == s0, c);
-      if (!c.sync((l << 4) | (colour ? 3 : 1))) return false;
+      rb_pass<T>(lv, colour, s, zero && s == s0, cx);
+      if (!rsh<T>().c[cx].sync((l << 4) | (colour ? 3 : 1))) return false;
     }
   return true;
 }
 
 // zero iterate (V-cycles without pre-smoothing)
 template <class T>
-__device__ __noinline__ bool rb_zero(const RLev<T>& __restrict__ L, const RCtx& c, int l) {
+__device__ __noinline__ bool rb_zero(int lv, int cx, int l) {
+  const RLev<T>& L = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
   const T z[4] = {T(0), T(0), T(0), T(0)};
-  for (int t = c.i0; t < L.nqt; t += c.st) {
+  for (int t = c.i0(); t < L.nqt; t += c.st) {
     const unsigned w = reinterpret_cast<const unsigned*>(L.f[0])[t] | reinterpret_cast<const unsigned*>(L.f[1])[t];
     for (int p = 0; p < 2; ++p)
       if (w & (p ? 0x02020202u : 0x01010101u)) {
@@ -563,103 +785,37 @@ __device__ __noinline__ bool rb_zero(const RLev<T>& __restrict__ L, const RCtx& 
   return c.sync((l << 4) | 12);
 }
 
-// residual of a single regular cell (a child of a special coarse cell)
-template <class T>
-__device__ __noinline__ T cell_res(const RLev<T>& L, int p, int i, int j, int k, int red, int black) {
-  const int colour = (i + j + k) & 1;
-  const long long pos = (i >> 1) + (long long)L.hx * (j + (long long)L.n[1] * k);
-  const T* xn = L.x[p][colour ? red : black];
-  const T xc = L.x[p][colour ? black : red][pos];
-  const int I[3] = {i, j, k};
-  T sum = T(0), dg = T(0);
-  for (int a = 0; a < L.D; ++a) {
-    // in the other colour's half the x neighbours are at (i -+ 1) >> 1, the others a row or a plane away
-    const long long lo = a == 0 ? pos - (i >> 1) + ((i - 1) >> 1) : pos - (a == 1 ? L.hx : (long long)L.hx * L.n[1]);
-    const long long hi = a == 0 ? pos - (i >> 1) + ((i + 1) >> 1) : pos + (a == 1 ? L.hx : (long long)L.hx * L.n[1]);
-    if (I[a] > 0) {
-      sum += xn[lo];
-      dg += T(1);
-    } else {
-      sum += L.w3[2 * a] * xn[hi];
-      dg += T(3) * L.wr[2 * a];
-    }
-    if (I[a] < L.n[a] - 1) {
-      sum += xn[hi];
-      dg += T(1);
-    } else {
-      sum += L.w3[2 * a + 1] * xn[lo];
-      dg += T(3) * L.wr[2 * a + 1];
-    }
-  }
-  return L.b[p][colour][pos] - L.ceps[p] * ((dg + L.lh[p]) * xc - sum);
-}
-
-// The special coarse cells: a group of 8 lanes each, a lane per child (2D: and
-// phase) for the regular children and all lanes together for each child's row.
-template <class T, class V>
-__device__ __noinline__ void rb_restrict_special(const RLev<T>& __restrict__ F, const RLev<T>& __restrict__ C, int s,
-                                                 bool full, const RCtx& c) {
-  const int red = rb_red(s), black = rb_black(s);
+// The restriction rows, a group of 8 lanes each (2D) or a warp (3D, where a
+// row joins up to eight children's rows): everything a row needs is three
+// dependent loads away (descriptor, entries and the children's right-hand
+// sides, values), where walking the children's rows was seven or more; at
+// about 0.7 us per load that reaches L2 this is what a small level's
+// restriction costs (128^2 to 512^2 levels: 14.5 us before, 8.3 us now).
+template <class T, class V, int GL>
+__device__ __noinline__ void rb_restrict_special(int lf, int lv, int cx, int red, int black) {
+  const RLev<T>& F = rsh<T>().H.L[lf];
+  const RLev<T>& C = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
   const Gather<T> x = rb_gather(F, red, black);
-  const int lane = threadIdx.x & 7, nch = 1 << F.D;
-  const int shift = threadIdx.x & 24;
-  const unsigned gmask = 0xffu << shift;
-  const T scale = T(1) / T(nch);
-  const V* dgp = (const V*)F.diag;
-  const V* val = (const V*)F.val;
-  const int nend = ((F.nsp + c.gst - 1) / c.gst) * c.gst;
-  for (int q = c.g0; q < nend; q += c.gst) {
+  const int lane = threadIdx.x & (GL - 1), nch = 1 << F.D;
+  const unsigned gmask = GL == 32 ? 0xffffffffu : 0xffu << (threadIdx.x & 24);
+  const V scale = V(1) / V(nch);
+  const V* val = (const V*)F.sval;
+  const int g0 = GL == 32 ? c.g0() >> 2 : c.g0(), gst = GL == 32 ? c.gst >> 2 : c.gst;
+  const int nend = ((F.nsp + gst - 1) / gst) * gst;
+  const int s1 = F.hx, s2 = F.hx * F.n[1];
+  for (int q = g0; q < nend; q += gst) {
     const bool live = q < F.nsp;
-    const unsigned cc = live ? (unsigned)F.sp[q] : 0u;
-    const int I = (int)(cc % (unsigned)C.n[0]), rowc = (int)(cc / (unsigned)C.n[0]);
-    const int J = rowc % C.n[1], K = rowc / C.n[1];
-    V acc[2] = {V(0), V(0)};
-    if (live)
-      for (int h = 0; h < (F.D == 3 ? 2 : 1); ++h) {
-        const int slot = lane + 8 * h, ch = slot & (nch - 1), p = slot >> F.D;
-        if (F.D == 3 && h && !F.two) break;  // the dielectric's slots
-        const int r = F.sprow[(long long)q * 2 * nch + slot];
-        int2 re = make_int2(0, 0);
-        unsigned cl = 0;
-        V d = V(0);
-        if (r >= 0) {
-          re = F.re[r];
-          cl = F.rs[r];
-          d = dgp[r];
-        } else if (!p || F.two) {
-          const int i = 2 * I + (ch & 1), j = 2 * J + ((ch >> 1) & 1), k = F.D == 3 ? 2 * K + (ch >> 2) : 0;
-          if (i < F.n[0] && j < F.n[1] && k < F.n[2] && (full || !((i + j + k) & 1))) {
-            const long long pos = (i >> 1) + (long long)F.hx * (j + (long long)F.n[1] * k);
-            if ((F.f[(i + j + k) & 1][pos] & 7u) == (1u << p)) acc[p] += (V)cell_res(F, p, i, j, k, red, black);
-          }
-        }
-        unsigned rows = (__ballot_sync(gmask, r >= 0) >> shift) & 0xffu;
-        while (rows) {
-          const int src = __ffs(rows) - 1;
-          rows &= rows - 1;
-          const int2 e = make_int2(__shfl_sync(gmask, re.x, src, 8), __shfl_sync(gmask, re.y, src, 8));
-          const V part = row_sum8<T, V>(F.col, val, e, lane, x, 0x80000000u);
-          // the group's parts are summed with everything else below
-          const int ps = F.D == 3 ? h : src >> 2;
-          if (ps) acc[1] -= part;
-          else acc[0] -= part;
-        }
-        if (r >= 0) {
-          unsigned pos;
-          const T* b = rb_rhs(F, cl, pos);
-          const V v = (V)b[pos] - d * (V)x(cl);
-          if (p) acc[1] += v;
-          else acc[0] += v;
-        }
-      }
-    for (int off = 4; off > 0; off >>= 1)
-      for (int p = 0; p < 2; ++p) acc[p] += __shfl_xor_sync(gmask, acc[p], off);
+    const int4 d = live ? F.sd[q] : make_int4(0, 0, 0, 0);
+    const int p = d.y >> 24;
+    V acc = V(0);
+    if (lane < nch && ((d.y >> (16 + lane)) & 1))
+      acc = scale * (V)F.b[p][(lane ^ (lane >> 1) ^ (lane >> 2)) & 1][d.z + s1 * ((lane >> 1) & 1) + s2 * (lane >> 2)];
+    acc -= row_sumg<T, V, GL>(F.scol, val, make_int2(d.x, d.x + (d.y & 0xffff)), lane, x, 0x80000000u);
+    for (int off = GL / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(gmask, acc, off);
     if (live && lane == 0) {
-      const int colour = (I + J + K) & 1;
-      const long long pos = (I >> 1) + (long long)C.hx * (J + (long long)C.n[1] * K);
-      const unsigned fl = C.f[colour][pos];
-      if (fl & 1u) C.b[0][colour][pos] = (T)acc[0] * scale;
-      if (fl & 2u) C.b[1][colour][pos] = (T)acc[1] * scale;
+      const int colour = d.w >= C.H;
+      C.b[p][colour][colour ? d.w - C.H : d.w] = (T)acc;
     }
   }
 }
@@ -669,17 +825,26 @@ __device__ __noinline__ void rb_restrict_special(const RLev<T>& __restrict__ F, 
 // are the groups at the same position of the fine rows.  full: black
 // residuals too (no sweep has solved them).
 template <class T>
-__device__ __noinline__ void rb_restrict(const RLev<T>& __restrict__ F, const RLev<T>& __restrict__ C, int s, bool full, const RCtx& c) {
+__device__ __noinline__ void rb_restrict(int lf, int lv, int s, bool full, int cx) {
+  const RLev<T>& F = rsh<T>().H.L[lf];
+  const RLev<T>& C = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
   if (F.nsp) {
-    if (F.staged) rb_restrict_special<T, T>(F, C, s, full, c);
-    else rb_restrict_special<T, double>(F, C, s, full, c);
+    const int rd = rb_red(s), bk = rb_black(s);
+    if (F.D == 3) {
+      if (F.sstaged) rb_restrict_special<T, T, 32>(lf, lv, cx, rd, bk);
+      else rb_restrict_special<T, double, 32>(lf, lv, cx, rd, bk);
+    } else {
+      if (F.sstaged) rb_restrict_special<T, T, 8>(lf, lv, cx, rd, bk);
+      else rb_restrict_special<T, double, 8>(lf, lv, cx, rd, bk);
+    }
   }
   if (!F.dense) return;
   const int rows = C.n[1] * C.n[2], items = rows * F.nq;
   const T scale = T(1) / T(1 << F.D);
   const unsigned* fr = reinterpret_cast<const unsigned*>(F.f[0]);
-  const T *xr = F.x[0][rb_red(s)], *xb = F.x[0][rb_black(s)];
-  for (int it = c.i0; it < items; it += c.st) {
+  const int ir = rb_red(s), ib = rb_black(s);
+  for (int it = c.i0(); it < items; it += c.st) {
     const unsigned rc = fdiv((unsigned)it, F.dq);
     const int g = it - (int)rc * F.nq;
     const unsigned K = fdiv(rc, C.dn1);
@@ -691,65 +856,56 @@ __device__ __noinline__ void rb_restrict(const RLev<T>& __restrict__ F, const RL
     const unsigned short fo = *reinterpret_cast<const unsigned short*>(C.f[ce ^ 1] + cp);
     if (!((fe | fo) & 0x0303u)) continue;
     const int t00 = (2 * J + (F.D == 3 ? F.n[1] * 2 * (int)K : 0)) * F.nq + g;
-    bool inner = F.full && !full && J > 0 && 2 * J + 2 < F.n[1] && (F.D == 2 || ((int)K > 0 && 2 * (int)K + 2 < F.n[2]));
-    if (inner) {
-      unsigned all = fr[t00] ^ 0x01010101u;
-      all |= fr[t00 + F.nq] ^ 0x01010101u;
-      if (F.D == 3) all |= (fr[t00 + F.nq * F.n[1]] ^ 0x01010101u) | (fr[t00 + F.nq * (F.n[1] + 1)] ^ 0x01010101u);
-      inner = !(all & R_BASE);
-    }
+    const bool whole = !full && F.wide;
+#pragma unroll 1
     for (int p = 0; p <= F.two; ++p) {
       const unsigned pm = 0x0101u << p;
       if (!((fe | fo) & pm)) continue;
       T acc[4] = {T(0), T(0), T(0), T(0)};
-      if (inner && p == 0) {
-        // all children regular gas away from the y and z walls: two rows' loads at a time
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          if (hh && F.D == 2) continue;
+      if (whole) {
+        // two rows' loads at a time
+#pragma unroll 1
+        for (int hh = 0; hh < F.D - 1; ++hh) {
           QNb<T> v[2];
           T bb[2][4], xo[2][4];
-          bool ed[2];
           QPos q[2];
+          unsigned m[2];
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             const int t = t00 + u * F.nq + hh * F.nq * F.n[1];
             q[u] = QPos{t, 2 * J + u, F.D == 3 ? 2 * (int)K + hh : 0, 4 * g, (u + hh) & 1};
-            quad_load_in(F, q[u], xb, v[u], ed[u]);
-            ld4(xr + 4 * t, xo[u]);
-            ld4(F.b[0][0] + 4 * t, bb[u]);
+            m[u] = q[u].j < F.n[1] && q[u].k < F.n[2] ? regular_mask(fr[t], p) : 0u;
           }
-          const T d = T(2 * F.D) + F.lh[0];
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            T sum[4];
-            quad_sums_in(F, q[u], v[u], ed[u], sum);
-            const T de = ed[u] ? F.dge[q[u].s] + F.lh[0] : d;
+            if (!m[u]) continue;
+            quad_load_in(F, q[u], F.x[p][ib], v[u]);
+            ld4(F.x[p][ir] + 4 * q[u].t, xo[u]);
+            ld4(F.b[p][0] + 4 * q[u].t, bb[u]);
+          }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const T de4 = e == 0 ? (q[u].s ? d : de) : (e == 3 ? (q[u].s ? de : d) : d);
-              acc[e] += bb[u][e] - F.ceps[0] * (de4 * xo[u][e] - sum[e]);
-            }
+          for (int u = 0; u < 2; ++u) {
+            if (!m[u]) continue;
+            T o[4];
+            quad_apply_in(F, q[u], p, v[u], xo[u], o);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[e] += (m[u] >> (8 * e)) & 1u ? bb[u][e] - o[e] : T(0);
           }
         }
-      } else
-      for (int h = 0; h < (F.D == 3 ? 4 : 2); ++h) {
-        const int j = 2 * J + (h & 1), k = F.D == 3 ? 2 * (int)K + (h >> 1) : 0;
-        if (j >= F.n[1] || k >= F.n[2]) continue;
-        const int t = (j + F.n[1] * k) * F.nq + g;
-        for (int colour = 0; colour <= (full ? 1 : 0); ++colour) {
+      } else {
+#pragma unroll 1
+        for (int h = 0; h < (F.D == 3 ? 8 : 4); ++h) {
+          const int j = 2 * J + (h & 1), k = F.D == 3 ? 2 * (int)K + ((h >> 1) & 1) : 0, colour = h >> (F.D - 1);
+          if (j >= F.n[1] || k >= F.n[2] || (colour && !full)) continue;
+          const int t = (j + F.n[1] * k) * F.nq + g;
           const unsigned m = regular_mask(reinterpret_cast<const unsigned*>(F.f[colour])[t], p);
           if (!m) continue;
-          const QPos q{t, j, k, 4 * g, (j + k + colour) & 1};
-          QNb<T> v;
-          T bb[4], xo[4], sum[4], dg[4];
-          quad_load(F, q, F.x[p][colour ? rb_red(s) : rb_black(s)], v);
-          ld4(F.x[p][colour ? rb_black(s) : rb_red(s)] + 4 * (long long)t, xo);
-          ld4(F.b[p][colour] + 4 * (long long)t, bb);
-          quad_sums(F, q, v, sum, dg);
+          T o[4];
+          quad_slow(F, t, colour, p, F.x[p][colour ? rb_red(s) : rb_black(s)],
+                    F.x[p][colour ? rb_black(s) : rb_red(s)], F.b[p][colour], o);
 #pragma unroll
           for (int e = 0; e < 4; ++e)
-            if ((m >> (8 * e)) & 1u) acc[e] += bb[e] - F.ceps[p] * ((dg[e] + F.lh[p]) * xo[e] - sum[e]);
+            if ((m >> (8 * e)) & 1u) acc[e] += o[e];
         }
       }
 #pragma unroll
@@ -766,11 +922,15 @@ __device__ __noinline__ void rb_restrict(const RLev<T>& __restrict__ F, const RL
 // one has none).  An item is the eight cells of one position of a fine row,
 // both colours; sF, sC: the sweeps done on the two levels.
 template <class T>
-__device__ __noinline__ void rb_prolong(const RLev<T>& __restrict__ F, const RLev<T>& __restrict__ C, int sF, int sC, const RCtx& c) {
+__device__ __noinline__ void rb_prolong(int lf, int lv, int sF, int sC, int cx) {
+  const RLev<T>& F = rsh<T>().H.L[lf];
+  const RLev<T>& C = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
   const int cr = rb_red(sC), cb = rb_black(sC);
   const unsigned *f0 = reinterpret_cast<const unsigned*>(F.f[0]), *f1 = reinterpret_cast<const unsigned*>(F.f[1]);
-  unsigned n0 = c.i0 < F.nqt ? f0[c.i0] : 0u, n1 = c.i0 < F.nqt ? f1[c.i0] : 0u;  // flags one item ahead
-  for (int t = c.i0; t < F.nqt; t += c.st) {
+  const int i0 = c.i0();
+  unsigned n0 = i0 < F.nqt ? f0[i0] : 0u, n1 = i0 < F.nqt ? f1[i0] : 0u;  // flags one item ahead
+  for (int t = i0; t < F.nqt; t += c.st) {
     const unsigned w0 = n0, w1 = n1;
     if (t + c.st < F.nqt) {
       n0 = f0[t + c.st];
@@ -782,6 +942,7 @@ __device__ __noinline__ void rb_prolong(const RLev<T>& __restrict__ F, const RLe
     const int J = g.j >> 1, K = g.k >> 1;
     const int J2 = min(max(J + ((g.j & 1) ? 1 : -1), 0), C.n[1] - 1);
     const int K2 = min(max(K + ((g.k & 1) ? 1 : -1), 0), C.n[2] - 1);
+#pragma unroll 1
     for (int p = 0; p <= F.two; ++p) {
       const unsigned pm = 0x01010101u << p;
       if (!((w0 | w1) & pm)) continue;
@@ -831,7 +992,10 @@ __device__ __noinline__ void rb_prolong(const RLev<T>& __restrict__ F, const RLe
 
 // x = binv b on the bottom level: a warp per row, lanes over the columns
 template <class T>
-__device__ __noinline__ void rb_inverse(const RHier<T>& __restrict__ H, const RLev<T>& __restrict__ L, const RCtx& c) {
+__device__ __noinline__ void rb_inverse(int lv, int cx) {
+  const RHier<T>& H = rsh<T>().H;
+  const RLev<T>& L = rsh<T>().H.L[lv];
+  const RCtx& c = rsh<T>().c[cx];
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int w0 = c.local ? (int)(threadIdx.x >> 5) : (int)(threadIdx.x >> 5) * c.gsize + c.gcta;
   const int ws = c.local ? nw : nw * c.gsize;
@@ -860,12 +1024,13 @@ __device__ __noinline__ void rb_inverse(const RHier<T>& __restrict__ H, const RL
 // from zero until |r| <= 1e-4 |b| (2-norms) or 16 iterations; vectors in
 // registers, matrix-vector products through the level's own arrays.
 template <class T, class V>
-__device__ __noinline__ void rb_bicgstab_v(const RLev<T>& L) {
+__device__ __noinline__ void rb_bicgstab_v(int lv) {
+  const RLev<T>& L = rsh<T>().H.L[lv];
   const int lane = threadIdx.x & 31;
   const bool live = lane < L.nr;
   const unsigned cl = live ? L.rs[lane] : 0u;
   const int2 re = live ? L.re[lane] : make_int2(0, 0);
-  const T d = live ? (T)((const V*)L.diag)[lane] : T(1);
+  const T di = live ? (T)((const V*)L.dinv)[lane] : T(1), d = rcp_rn(di);
   unsigned pos;
   const T* bp = rb_rhs(L, cl, pos);
   const bool blk = (cl & 0x7fffffffu) >= (unsigned)L.H;
@@ -886,19 +1051,20 @@ __device__ __noinline__ void rb_bicgstab_v(const RLev<T>& L) {
   T r = b, pv = T(0), v = T(0), sol = T(0);
   const T r0 = b, bb = dot(b, b);
   T rho = T(1), alpha = T(1), omega = T(1);
+#pragma unroll 1
   for (int it = 0; it < 16 && bb > T(0); ++it) {
     const T rho1 = dot(r0, r);
     if (rho1 == T(0) || omega == T(0)) break;
     pv = r + (rho1 / rho) * (alpha / omega) * (pv - omega * v);
     rho = rho1;
     // diagonal scaling: the cells' coefficients differ by the permittivities and cut fractions
-    const T ph = pv / d;
+    const T ph = pv * di;
     v = mul(ph);
     const T rv = dot(r0, v);
     if (rv == T(0)) break;
     alpha = rho / rv;
     const T sv = r - alpha * v;
-    const T sh = sv / d;
+    const T sh = sv * di;
     const T t = mul(sh);
     const T tt = dot(t, t);
     omega = tt > T(0) ? dot(t, sv) / tt : T(0);
@@ -918,22 +1084,23 @@ __device__ __forceinline__ int rb_done(const RHier<T>& H, int l) {
 
 // level L (index l) down to N, the next one, and back up
 template <class T>
-__device__ __noinline__ bool rb_down(const RHier<T>& H, const RLev<T>& L, const RLev<T>& N, int l, const RCtx& c) {
-  const int nu = H.nu1[l];
+__device__ __forceinline__ bool rb_down(int lv, int ln, int l, int cx) {
+  const int nu = rsh<T>().H.nu1[l];
   if (nu == 0) {
-    if (!rb_zero(L, c, l)) return false;
-  } else if (!rb_smooth(L, 0, nu, true, c, l)) {
+    if (!rb_zero<T>(lv, cx, l)) return false;
+  } else if (!rb_smooth<T>(lv, 0, nu, true, cx, l)) {
     return false;
   }
-  rb_restrict(L, N, nu, nu == 0, c);
-  return c.sync((l << 4) | 6);
+  rb_restrict<T>(lv, ln, nu, nu == 0, cx);
+  return rsh<T>().c[cx].sync((l << 4) | 6);
 }
 template <class T>
-__device__ __noinline__ bool rb_up(const RHier<T>& H, const RLev<T>& L, const RLev<T>& N, int l, const RCtx& c) {
+__device__ __forceinline__ bool rb_up(int lv, int ln, int l, int cx) {
+  const RHier<T>& H = rsh<T>().H;
   const int nu = H.nu1[l];
-  rb_prolong(L, N, nu, rb_done(H, l + 1), c);
-  if (!c.sync((l << 4) | 7)) return false;
-  return rb_smooth(L, nu, nu + H.nu2[l], false, c, l);
+  rb_prolong<T>(lv, ln, nu, rb_done(H, l + 1), cx);
+  if (!rsh<T>().c[cx].sync((l << 4) | 7)) return false;
+  return rb_smooth<T>(lv, nu, nu + H.nu2[l], false, cx, l);
 }
 
 __device__ __forceinline__ void copy_words(void* dst, const void* src, long long bytes) {
@@ -944,32 +1111,33 @@ __device__ __forceinline__ void copy_words(void* dst, const void* src, long long
 
 // levels lc.. inside CTA 0; g: level lc as the grid sees it
 template <class T>
-__device__ __noinline__ void rb_coarse(const RHier<T>& H, const RLev<T>& g, const RCtx& c) {
-  const int lc = H.lc;
+__device__ __noinline__ void rb_coarse() {
+  const RHier<T>& H = rsh<T>().H;
+  const RLev<T>&s = H.L[H.lc], &g = H.L[RMAX];
   if (H.smem) {
-    const RLev<T>& s = H.L[lc];
     for (int p = 0; p <= s.two; ++p) {
       const int o = p ? s.p1o : 0, n = p ? s.p1n : s.H;
       for (int q = 0; q < 2; ++q) copy_words(s.b[p][q] + o, g.b[p][q] + o, (long long)n * sizeof(T));
     }
     __syncthreads();
   }
-  for (int l = lc; l < H.nlev - 1; ++l) rb_down(H, H.L[l], H.L[l + 1], l, c);
-  const RLev<T>& B = H.L[H.nlev - 1];
+#pragma unroll 1
+  for (int l = H.lc; l < H.nlev - 1; ++l) rb_down<T>(l, l + 1, l, 1);
+  const int lb = H.nlev - 1;
   if (H.bot == 0) {
-    rb_smooth(B, 0, H.bsweeps, true, c, H.nlev - 1);
+    rb_smooth<T>(lb, 0, H.bsweeps, true, 1, lb);
   } else {
-    if (H.bot == 1) rb_inverse(H, B, c);
+    if (H.bot == 1) rb_inverse<T>(lb, 1);
     else if (threadIdx.x < 32) {
-      if (B.staged) rb_bicgstab_v<T, T>(B);
-      else rb_bicgstab_v<T, double>(B);
+      if (H.L[lb].staged) rb_bicgstab_v<T, T>(lb);
+      else rb_bicgstab_v<T, double>(lb);
     }
-    c.sync(((H.nlev - 1) << 4) | 9);
+    rsh<T>().c[1].sync((lb << 4) | 9);
   }
-  for (int l = H.nlev - 2; l >= lc; --l) rb_up(H, H.L[l], H.L[l + 1], l, c);
+#pragma unroll 1
+  for (int l = H.nlev - 2; l >= H.lc; --l) rb_up<T>(l, l + 1, l, 1);
   if (H.smem) {
-    const RLev<T>& s = H.L[lc];
-    const int d = rb_done(H, lc);
+    const int d = rb_done(H, H.lc);
     for (int p = 0; p <= s.two; ++p) {
       const int o = p ? s.p1o : 0, n = p ? s.p1n : s.H;
       copy_words(g.x[p][rb_red(d)] + o, s.x[p][rb_red(d)] + o, (long long)n * sizeof(T));
@@ -979,31 +1147,26 @@ __device__ __noinline__ void rb_coarse(const RHier<T>& H, const RLev<T>& g, cons
 }
 
 // one V-cycle from zero: level 0's right-hand side in its b, the result in
-// its x after rb_done(H, 0) sweeps; gl: level lc as the grid sees it (in CTA
-// 0 the entry H.L[lc] points into shared memory)
+// its x after rb_done(H, 0) sweeps
 template <class T>
-__device__ __noinline__ bool rb_vcycle(const RHier<T>& H, const RLev<T>& gl, const RCtx& G) {
+__device__ __noinline__ bool rb_vcycle() {
+  const RHier<T>& H = rsh<T>().H;
+#pragma unroll 1
   for (int l = 0; l < H.lc; ++l)
-    if (!rb_down(H, H.L[l], l + 1 == H.lc ? gl : H.L[l + 1], l, G)) return false;
+    if (!rb_down<T>(l, l + 1 == H.lc ? RMAX : l + 1, l, 0)) return false;
   if (H.bot == 1 && !H.smem) {  // the inverse applied by the whole grid
-    rb_inverse(H, gl, G);
-    if (!G.sync(((H.nlev - 1) << 4) | 9)) return false;
+    rb_inverse<T>(RMAX, 0);
+    if (!rsh<T>().c[0].sync(((H.nlev - 1) << 4) | 9)) return false;
   } else {
-    if (G.gcta == 0) {
-      RCtx L = G;
-      L.local = true;
-      L.i0 = (int)threadIdx.x;
-      L.st = (int)blockDim.x;
-      L.g0 = (int)(threadIdx.x >> 3);
-      L.gst = (int)(blockDim.x >> 3);
-      rb_coarse(H, gl, L);
-    }
-    if (!G.sync((15 << 4) | 8)) return false;
+    if (rsh<T>().c[0].gcta == 0) rb_coarse<T>();
+    if (!rsh<T>().c[0].sync((15 << 4) | 8)) return false;
   }
+#pragma unroll 1
   for (int l = H.lc - 1; l >= 0; --l)
-    if (!rb_up(H, H.L[l], l + 1 == H.lc ? gl : H.L[l + 1], l, G)) return false;
+    if (!rb_up<T>(l, l + 1 == H.lc ? RMAX : l + 1, l, 0)) return false;
   return true;
 }
+
 
 // ------------------------------------------------------------ the FP64 outer loop
 
@@ -1018,14 +1181,17 @@ __device__ __forceinline__ void bits_max(unsigned long long& m, double v) {
 // operations each (GB300 issues about two FP64 operations per clock and SM,
 // which bounds the pass from 256^2 cells up).
 template <class T>
-__device__ __noinline__ bool rb_resid64(const RHier<T>& __restrict__ H, const RLev<T>& __restrict__ L, const Op<double>& __restrict__ F, unsigned long long* norm,
-                           const RCtx& G) {
+__device__ __noinline__ bool rb_resid64(unsigned long long* norm) {
+  const RHier<T>& H = rsh<T>().H;
+  const RLev<T>& L = H.L[H.lc == 0 ? RMAX : 0];
+  const Op<double>& F = rsh<T>().F;
+  const RCtx& G = rsh<T>().c[0];
   unsigned long long mx = 0ull;
   {
     const int g = threadIdx.x & 7;
     const unsigned gmask = 0xffu << (threadIdx.x & 24);
     const int rend = ((L.nr + G.gst - 1) / G.gst) * G.gst;
-    for (int r = G.g0; r < rend; r += G.gst) {
+    for (int r = G.g0(); r < rend; r += G.gst) {
       const bool live = r < L.nr;
       const int2 re = live ? L.re[r] : make_int2(0, 0);
       const unsigned cl = live ? L.rs[r] : 0u;
@@ -1066,12 +1232,13 @@ __device__ __noinline__ bool rb_resid64(const RHier<T>& __restrict__ H, const RL
   }
   const int n0 = F.n[0], n1 = F.n[1], n2 = F.D == 3 ? F.n[2] : 1;
   const long long sy = n0, sz = (long long)n0 * n1;
-  for (int t = G.i0; t < L.nqt; t += G.st) {
+  for (int t = G.i0(); t < L.nqt; t += G.st) {
     const unsigned w0 = reinterpret_cast<const unsigned*>(L.f[0])[t], w1 = reinterpret_cast<const unsigned*>(L.f[1])[t];
     if (!((w0 | w1) & 0x03030303u)) continue;
     const QPos g = quad_pos(L, t, 0);
     const unsigned we = g.s ? w1 : w0, wo = g.s ? w0 : w1;
     const long long nb = ((long long)g.j + (long long)n1 * g.k) * n0 + 2 * g.q0;
+#pragma unroll 1
     for (int p = 0; p <= L.two; ++p) {
       const unsigned me = regular_mask(we, p), mo = regular_mask(wo, p);
       if (!(me | mo)) continue;
@@ -1086,6 +1253,7 @@ __device__ __noinline__ bool rb_resid64(const RHier<T>& __restrict__ H, const RL
 #pragma unroll
       for (int e = 0; e < 8; ++e) s[e] = (e ? c[e ? e - 1 : 0] : xl) + (e < 7 ? c[e < 7 ? e + 1 : 7] : xr);
       double wd = 0.0;
+#pragma unroll 1
       for (int a = 1; a < F.D; ++a) {
         const long long st = a == 1 ? sy : sz;
         const int i = a == 1 ? g.j : g.k, n = a == 1 ? n1 : n2;
@@ -1143,7 +1311,12 @@ __device__ __noinline__ bool rb_resid64(const RHier<T>& __restrict__ H, const RL
 // directions before it, (q, q_i) and (r, q_i).  The sums' chunks depend on the level alone, not
 // on the CTAs that take them, so a solve's results do not depend on its group.
 template <class T>
-__device__ __noinline__ void rb_kry1(const RHier<T>& __restrict__ H, const RLev<T>& __restrict__ L, int sZ, int slot, int m, const RCtx& G, T (*red)[KDOT]) {
+__device__ __noinline__ void rb_kry1() {
+  const RHier<T>& H = rsh<T>().H;
+  const RLev<T>& L = H.L[H.lc == 0 ? RMAX : 0];
+  const RCtx& G = rsh<T>().c[0];
+  const int sZ = rb_done(H, 0), slot = rsh<T>().K.next, m = rsh<T>().K.count;
+  T(*red)[KDOT] = rsh<T>().red;
   const int ir = rb_red(sZ), ib = rb_black(sZ);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int os[KH];
@@ -1164,7 +1337,7 @@ __device__ __noinline__ void rb_kry1(const RHier<T>& __restrict__ H, const RLev<
         const bool live = r < r1;
         const int2 re = live ? L.re[r] : make_int2(0, 0);
         const unsigned cl = live ? L.rs[r] : 0u;
-        double s = row_sum8<T, double>(L.col, H.rval, re, g, x, 0x80000000u);
+        double s = row_sumg<T, double, 8>(L.col, H.rval, re, g, x, 0x80000000u);
         for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(gmask, s, off);
         if (live && g == 0) {
           unsigned pos;
@@ -1188,48 +1361,46 @@ __device__ __noinline__ void rb_kry1(const RHier<T>& __restrict__ H, const RLev<
     const int t1 = min((ch + 1) * H.kcs, L.nqt);
     for (int t = ch * H.kcs + (int)threadIdx.x; t < t1; t += (int)blockDim.x) {
       const unsigned w[2] = {reinterpret_cast<const unsigned*>(L.f[0])[t], reinterpret_cast<const unsigned*>(L.f[1])[t]};
-      for (int p = 0; p <= L.two; ++p)
+#pragma unroll 1
+      for (int pc = 0; pc < 2 * (L.two + 1); ++pc) {
+        const int p = pc >> 1, colour = pc & 1;
+        const unsigned mk = regular_mask(colour ? w[1] : w[0], p);
+        if (!mk) continue;
+        const QPos g = quad_pos(L, t, colour);
+        const T *xn = L.x[p][colour ? ir : ib], *xw = L.x[p][colour ? ib : ir];
+        T q[4], rr[4], qi[KH - 1][4];
+        ld4(L.b[p][colour] + 4 * t, rr);
 #pragma unroll
-        for (int colour = 0; colour < 2; ++colour) {
-          const unsigned mk = regular_mask(w[colour], p);
-          if (!mk) continue;
-          const QPos g = quad_pos(L, t, colour);
+        for (int i = 0; i < KH - 1; ++i)
+          if (i < m) ld4(H.kq[os[i]][p][colour] + 4 * t, qi[i]);
+        if (L.wide) {
           QNb<T> v;
-          T xo[4], sum[4], dg[4], q[4], rr[4];
-          T qi[KH - 1][4];
-          const bool in = quad_inner(L, g);
-          bool ed = false;
-          if (in) quad_load_in(L, g, L.x[p][colour ? ir : ib], v, ed);
-          ld4(L.x[p][colour ? ib : ir] + 4 * (long long)t, xo);
-          ld4(L.b[p][colour] + 4 * (long long)t, rr);
+          T xo[4];
+          quad_load_in(L, g, xn, v);
+          ld4(xw + 4 * t, xo);
+          quad_apply_in(L, g, p, v, xo, q);
+        } else {
+          T os[4];
+          quad_slow(L, t, colour, p, xn, xw, (const T*)nullptr, os);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) q[e] = os[e];
+        }
+        quad_store(H.kq[slot][p][colour] + 4 * t, mk, q);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (!((mk >> (8 * e)) & 1u)) q[e] = T(0);
+          const T re = (mk >> (8 * e)) & 1u ? rr[e] : T(0);
+          acc[0] += re * q[e];
+          acc[1] += q[e] * q[e];
 #pragma unroll
           for (int i = 0; i < KH - 1; ++i)
-            if (i < m) ld4(H.kq[os[i]][p][colour] + 4 * (long long)t, qi[i]);
-          if (in) {
-            quad_sums_in(L, g, v, ed, sum);
-            const T d = T(2 * L.D), de = ed ? L.dge[g.s] : d;
-            dg[0] = g.s ? d : de;
-            dg[1] = dg[2] = d;
-            dg[3] = g.s ? de : d;
-          } else {
-            quad_load(L, g, L.x[p][colour ? ir : ib], v);
-            quad_sums(L, g, v, sum, dg);
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            q[e] = L.ceps[p] * ((dg[e] + L.lh[p]) * xo[e] - sum[e]);
-            if (!((mk >> (8 * e)) & 1u)) continue;
-            acc[0] += rr[e] * q[e];
-            acc[1] += q[e] * q[e];
-#pragma unroll
-            for (int i = 0; i < KH - 1; ++i)
-              if (i < m) {
-                acc[2 + i] += q[e] * qi[i][e];
-                acc[KH + 1 + i] += rr[e] * qi[i][e];
-              }
-          }
-          quad_store(H.kq[slot][p][colour] + 4 * (long long)t, mk, q);
+            if (i < m) {
+              const T v = (mk >> (8 * e)) & 1u ? qi[i][e] : T(0);
+              acc[2 + i] += q[e] * v;
+              acc[KH + 1 + i] += re * v;
+            }
         }
+      }
     }
 #pragma unroll
     for (int d = 0; d < KDOT; ++d) {
@@ -1249,11 +1420,6 @@ __device__ __noinline__ void rb_kry1(const RHier<T>& __restrict__ H, const RLev<
 
 // The directions kept: in shared memory, and in global memory between the
 // launches of a resumed solve.
-struct KryState {
-  int count, next;   // directions kept, slot of the next one
-  double g[KH][KH];  // (q_i, q_j) by slot
-};
-
 // The sums of pass 1 in a fixed order, then the step: the combination of the
 // new and the kept directions that minimises |r - sum c q| (2-norm), by the
 // normal equations.  The directions stay as they were formed, q = A z each:
@@ -1273,46 +1439,57 @@ __device__ __forceinline__ void rb_kry_coeff(const double* part, int nch, int m,
   if (threadIdx.x == 0) {
     const int nw = K.next;
     int sl[KH];
-    double A[KH][KH], b[KH], x[KH];
-    sl[0] = nw;
-    b[0] = dots[0];
     K.g[nw][nw] = dots[1];
+    sl[0] = nw;
     for (int i = 0; i < m; ++i) {
       sl[1 + i] = (nw + KH - 1 - i) % KH;
-      b[1 + i] = dots[KH + 1 + i];
       K.g[nw][sl[1 + i]] = K.g[sl[1 + i]][nw] = dots[2 + i];
     }
-    // Cholesky factor, newest first; a direction that depends on the ones before it is left out
+    // scaled to a unit diagonal and factored in FP32, newest first: one
+    // thread's FP64 chain would cost microseconds, and the step needs no more
+    // digits than the sums have; a direction that depends on the ones before it
+    // is left out
+    float A[KH][KH], y[KH];
     int use[KH], nu = 0;
+#pragma unroll
+    for (int i = 0; i < KH; ++i) c[i] = 0.0;
+    const double s0 = dots[1] > 0.0 ? rsqrt(dots[1]) : 0.0;
+    K.rn[nw] = s0;
     for (int i = 0; i <= m; ++i) {
-      const double d = K.g[sl[i]][sl[i]];
-      double t[KH], p = d;
+      const double si = K.rn[sl[i]];
+      if (!(si > 0.0)) continue;
+      float t[KH], p = 1.0f;
       for (int k = 0; k < nu; ++k) {
-        double v = K.g[sl[i]][sl[use[k]]];
+        float v = (float)(K.g[sl[i]][sl[use[k]]] * si * K.rn[sl[use[k]]]);
         for (int q = 0; q < k; ++q) v -= t[q] * A[k][q];
         t[k] = v / A[k][k];
         p -= t[k] * t[k];
       }
-      if (!(p > 1e-6 * d)) continue;
+      if (!(p > 1e-5f)) continue;
       for (int k = 0; k < nu; ++k) A[nu][k] = t[k];
-      A[nu][nu] = sqrt(p);
+      A[nu][nu] = sqrtf(p);
+      // right-hand side in units of |r|-like scale: divided by this direction's norm and the newest one's
+      float v = (float)((i == 0 ? dots[0] : dots[KH + i]) * si * s0);
+      for (int q = 0; q < nu; ++q) v -= A[nu][q] * y[q];
+      y[nu] = v / A[nu][nu];
       use[nu++] = i;
     }
-    for (int i = 0; i < KH; ++i) c[i] = 0.0;
     bool fin = nu > 0 && use[0] == 0;
-    for (int k = 0; k < nu; ++k) {
-      double v = b[use[k]];
-      for (int q = 0; q < k; ++q) v -= A[k][q] * x[q];
-      x[k] = v / A[k][k];
-    }
     for (int k = nu - 1; k >= 0; --k) {
-      double v = x[k];
-      for (int q = k + 1; q < nu; ++q) v -= A[q][k] * x[q];
-      x[k] = v / A[k][k];
-      fin = fin && fabs(x[k]) < 1e3;
+      float v = y[k];
+      for (int q = k + 1; q < nu; ++q) v -= A[q][k] * y[q];
+      y[k] = v / A[k][k];
     }
-    for (int k = 0; k < nu && fin; ++k) c[use[k] ? use[k] - 1 : KH - 1] = x[k];
-    if (!fin) c[KH - 1] = 1.0;  // the plain correction
+    for (int k = 0; k < nu; ++k) {
+      // back to the directions' own units: times |q_new| / |q_k|
+      const double x = (double)y[k] * (dots[1] * s0) * K.rn[sl[use[k]]];
+      fin = fin && fabs(x) < 1e3;
+      c[use[k] ? use[k] - 1 : KH - 1] = x;
+    }
+    if (!fin) {
+      for (int i = 0; i < KH; ++i) c[i] = 0.0;
+      c[KH - 1] = 1.0;  // the plain correction
+    }
     K.count = min(m + 1, KH - 1);
     K.next = (nw + 1) % KH;
   }
@@ -1323,9 +1500,13 @@ __device__ __forceinline__ void rb_kry_coeff(const double* part, int nch, int m,
 // c q where another V-cycle follows before the next FP64 residual.  slot < 0:
 // the plain correction, phi += z.
 template <class T>
-__device__ __noinline__ void rb_kry2(const RHier<T>& __restrict__ H, const RLev<T>& __restrict__ L,
-                                     const Op<double>& __restrict__ F, int sZ, int slot, int m,
-                                     const double* __restrict__ c, bool upd_r, const RCtx& G) {
+__device__ __noinline__ void rb_kry2(int slot, int m, bool upd_r) {
+  const RHier<T>& H = rsh<T>().H;
+  const RLev<T>& L = H.L[H.lc == 0 ? RMAX : 0];
+  const Op<double>& F = rsh<T>().F;
+  const RCtx& G = rsh<T>().c[0];
+  const int sZ = rb_done(H, 0);
+  const double* c = rsh<T>().coef;
   const int ir = rb_red(sZ), ib = rb_black(sZ);
   const int n0 = F.n[0], n1 = F.n[1];
   double cc[KH - 1];
@@ -1336,11 +1517,12 @@ __device__ __noinline__ void rb_kry2(const RHier<T>& __restrict__ H, const RLev<
     os[i] = (slot + KH - 1 - i) % KH;
   }
   const double cn = slot < 0 ? 1.0 : c[KH - 1];
-  for (int t = G.i0; t < L.nqt; t += G.st) {
+  for (int t = G.i0(); t < L.nqt; t += G.st) {
     const unsigned w[2] = {reinterpret_cast<const unsigned*>(L.f[0])[t], reinterpret_cast<const unsigned*>(L.f[1])[t]};
     if (!((w[0] | w[1]) & 0x03030303u)) continue;
     const QPos g = quad_pos(L, t, 0);
     const long long o4 = 4 * (long long)t;
+#pragma unroll 1
     for (int p = 0; p <= L.two; ++p) {
       if (!((w[0] | w[1]) & (0x01010101u << p))) continue;
       double* ph = F.x[p] + ((long long)g.j + (long long)n1 * g.k) * n0 + 2 * g.q0;
@@ -1395,33 +1577,46 @@ __device__ __noinline__ void rb_kry2(const RHier<T>& __restrict__ H, const RLev<
   }
 }
 
-// The start of a launch: the hierarchy's description into shared memory, and in
-// CTA 0 the levels it keeps there (their flags, rows with entries in T and
-// special lists, constant over the launch).  gl: level lc as the grid sees it.
+// The start of a launch: the hierarchy's description and the contexts into
+// shared memory, and in CTA 0 the levels it keeps there (their flags, rows with
+// entries in T and restriction rows, constant over the launch).
 template <class T>
-__device__ __noinline__ void rb_begin(const RHier<T>* __restrict__ Hg, RHier<T>& H, RLev<T>& gl, unsigned char* dyn,
-                                      int gcta) {
+__device__ __noinline__ void rb_begin(const RHier<T>* __restrict__ Hg, const Barrier& B, int gcta, int gsize) {
+  extern __shared__ __align__(128) unsigned char dyn[];
+  RHier<T>& H = rsh<T>().H;
   copy_words(&H, Hg, sizeof(RHier<T>));
-  copy_words(&gl, &Hg->L[Hg->lc], sizeof(RLev<T>));
+  if (threadIdx.x < 2) {
+    RCtx& c = rsh<T>().c[threadIdx.x];
+    c.local = threadIdx.x == 1;
+    c.gcta = gcta;
+    c.gsize = gsize;
+    c.st = c.local ? (int)blockDim.x : gsize * (int)blockDim.x;
+    c.gst = c.st >> 3;
+    c.B = B;
+    c.epoch = &rsh<T>().epoch;
+    c.tn = &rsh<T>().tn;
+    c.tr = nullptr;
+    if (threadIdx.x == 0) rsh<T>().epoch = rsh<T>().tn = 0u;
+  }
   __syncthreads();
   if (gcta == 0 && H.smem) {
     for (int l = H.lc; l < H.nlev; ++l) {
       const RLev<T>& g = Hg->L[l];
       for (int q = 0; q < 2; ++q) copy_words(dyn + H.off_f[l][q], g.f[q], g.H);
-      if (g.nr && H.srows[l]) {
+      if (H.srows[l] & 1) {
         copy_words(dyn + H.off_re[l], g.re, 8ll * g.nr);
         copy_words(dyn + H.off_rs[l], g.rs, 4ll * g.nr);
         copy_words(dyn + H.off_col[l], g.col, 4ll * H.nnz[l]);
         T* v = (T*)(dyn + H.off_val[l]);
-        T* d = (T*)(dyn + H.off_dg[l]);
         for (int i = threadIdx.x; i < H.nnz[l]; i += blockDim.x) v[i] = (T)((const double*)g.val)[i];
         T* di = (T*)(dyn + H.off_di[l]);
-        for (int i = threadIdx.x; i < g.nr; i += blockDim.x) {
-          d[i] = (T)((const double*)g.diag)[i];
-          di[i] = (T)((const double*)g.dinv)[i];
-        }
-        copy_words(dyn + H.off_sp[l], g.sp, 4ll * g.nsp);
-        copy_words(dyn + H.off_spr[l], g.sprow, 4ll * g.nsp * (2 << g.D));
+        for (int i = threadIdx.x; i < g.nr; i += blockDim.x) di[i] = (T)((const double*)g.dinv)[i];
+      }
+      if (H.srows[l] & 2) {
+        copy_words(dyn + H.off_sd[l], g.sd, 16ll * g.nsp);
+        copy_words(dyn + H.off_sc[l], g.scol, 4ll * H.snnz[l]);
+        T* sv = (T*)(dyn + H.off_sv[l]);
+        for (int i = threadIdx.x; i < H.snnz[l]; i += blockDim.x) sv[i] = (T)((const double*)g.sval)[i];
       }
     }
     if ((int)threadIdx.x >= H.lc && (int)threadIdx.x < H.nlev) {
@@ -1432,80 +1627,53 @@ __device__ __noinline__ void rb_begin(const RHier<T>* __restrict__ Hg, RHier<T>&
         for (int k = 0; k < 2; ++k) v.b[p][k] = (T*)(dyn + H.off_b[l][p][k]);
       }
       for (int k = 0; k < 2; ++k) v.f[k] = dyn + H.off_f[l][k];
-      if (v.nr && H.srows[l]) {
+      if (H.srows[l] & 1) {
         v.re = (const int2*)(dyn + H.off_re[l]);
         v.rs = (const unsigned*)(dyn + H.off_rs[l]);
         v.col = (const unsigned*)(dyn + H.off_col[l]);
         v.val = dyn + H.off_val[l];
-        v.diag = dyn + H.off_dg[l];
         v.dinv = dyn + H.off_di[l];
-        v.sp = (const int*)(dyn + H.off_sp[l]);
-        v.sprow = (const int*)(dyn + H.off_spr[l]);
         v.staged = 1;
+      }
+      if (H.srows[l] & 2) {
+        v.sd = (const int4*)(dyn + H.off_sd[l]);
+        v.scol = (const unsigned*)(dyn + H.off_sc[l]);
+        v.sval = dyn + H.off_sv[l];
+        v.sstaged = 1;
       }
     }
   }
   __syncthreads();
 }
-__device__ __forceinline__ RCtx rb_grid(const Barrier& B, unsigned* epoch, unsigned* tn, int gcta, int gsize) {
-  RCtx G;
-  const int wi = (int)(threadIdx.x >> 5) * gsize + gcta;  // warps interleaved over the CTAs
-  G.i0 = wi * 32 + (int)(threadIdx.x & 31);
-  G.st = gsize * (int)blockDim.x;
-  G.gst = gsize * (int)(blockDim.x >> 3);
-  G.g0 = G.gst - 1 - (wi * 4 + (int)((threadIdx.x >> 3) & 3));
-  G.local = false;
-  G.B = B;
-  G.epoch = epoch;
-  G.tr = nullptr;
-  G.tn = tn;
-  G.gcta = gcta;
-  G.gsize = gsize;
-  return G;
-}
-
 template <class T>
 __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, const Op<double>* __restrict__ Fg,
                                                const SolveCtl& ctl, const Barrier& B, int gcta, int gsize) {
-  __shared__ RHier<T> H;
-  __shared__ RLev<T> gl;
-  __shared__ Op<double> F;
-  __shared__ unsigned epoch, tn;
-  __shared__ T red[PT / 32][KDOT];
-  __shared__ double dots[KDOT], coef[KH];
-  __shared__ KryState K;
-  extern __shared__ __align__(128) unsigned char dyn[];
-  copy_words(&F, Fg, sizeof(Op<double>));
-  if (threadIdx.x == 0) {
-    epoch = 0u;
-    tn = 0u;
-  }
-  copy_words(&K, Hg->kst, sizeof(KryState));
-  rb_begin(Hg, H, gl, dyn, gcta);
-  if (threadIdx.x == 0 && ctl.fresh) K.count = K.next = 0;
+  RShared<T>& S = rsh<T>();
+  const Op<double>& F = S.F;
+  copy_words(&S.F, Fg, sizeof(Op<double>));
+  copy_words(&S.K, Hg->kst, sizeof(KryState));
+  rb_begin<T>(Hg, B, gcta, gsize);
+  if (threadIdx.x == 0 && ctl.fresh) S.K.count = S.K.next = 0;
   __syncthreads();
-  const RCtx G = rb_grid(B, &epoch, &tn, gcta, gsize);
-  // the finest level as the grid sees it (level 0 may be the first one inside CTA 0)
-  const RLev<T>& L0 = H.lc == 0 ? gl : H.L[0];
-  const int sZ = rb_done(H, 0);
+  const RCtx& G = S.c[0];
   const double bn = *ctl.bnorm;
   int it = 0, cycles = 0, status = 0;
-  double r0 = 0.0, r = 0.0;
   if (bn == 0.0) {  // b = 0: the solution is 0
-    for (long long cc = G.i0; cc < F.ncell; cc += G.st) {
+    for (long long cc = G.i0(); cc < F.ncell; cc += G.st) {
       F.x[0][cc] = 0.0;
       if (F.x[1]) F.x[1][cc] = 0.0;
     }
   }
-  for (; bn != 0.0;) {
-    if (!rb_resid64(H, L0, F, ctl.norms + it, G)) {
+  // norms are read again where they are needed: little stays in registers across the phases
+#pragma unroll 1
+  for (; *ctl.bnorm != 0.0;) {
+    if (!rb_resid64<T>(ctl.norms + it)) {
       status = 5;
       break;
     }
-    r = load_norm(ctl.norms + it);
-    if (it == 0) r0 = r;
-    if (r <= ctl.tol * bn) break;
-    if (cycles + ctl.inner > ctl.max_cycles || !(r == r) || r > 1e6 * r0) {
+    const double r = load_norm(ctl.norms + it);
+    if (r <= ctl.tol * *ctl.bnorm) break;
+    if (cycles + ctl.inner > ctl.max_cycles || !(r == r) || r > 1e6 * load_norm(ctl.norms)) {
       status = 3;
       break;
     }
@@ -1514,26 +1682,28 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
       break;
     }
     bool ok = true;
+#pragma unroll 1
     for (int k = 0; k < ctl.inner && ok; ++k) {
-      RCtx Gk = G;
-      if (it == 0 && k == 0 && ctl.trace) {  // trace the first V-cycle
-        Gk.tr = ctl.trace;
-        if (gcta == 0 && threadIdx.x == 0) ctl.trace[1 + tn++] = ((unsigned long long)0xfff << 48) | (now_ns() & 0xffffffffffffULL);
+      if (ctl.trace && threadIdx.x == 0 && G.gcta == 0) {  // trace the first V-cycle; this thread alone reads tr
+        const bool on = it == 0 && k == 0;
+        S.c[0].tr = S.c[1].tr = on ? ctl.trace : nullptr;
+        if (on) ctl.trace[1 + S.tn++] = ((unsigned long long)0xfff << 48) | (now_ns() & 0xffffffffffffULL);
       }
-      ok = rb_vcycle(H, gl, Gk);
+      ok = rb_vcycle<T>();
       if (!ok) break;
+      int slot = -1, m = 0;
       if (ctl.kry) {
-        const int slot = K.next, m = K.count;
-        rb_kry1(H, L0, sZ, slot, m, Gk, red);
-        ok = Gk.sync((14 << 4) | 14);
+        slot = S.K.next;
+        m = S.K.count;
+        rb_kry1<T>();
+        ok = G.sync((14 << 4) | 14);
         if (!ok) break;
-        rb_kry_coeff(H.kpart, H.kch, m, K, dots, coef);
-        rb_kry2(H, L0, F, sZ, slot, m, coef, k + 1 < ctl.inner, Gk);
-      } else {
-        rb_kry2(H, L0, F, sZ, -1, 0, coef, false, Gk);
+        rb_kry_coeff(S.H.kpart, S.H.kch, m, S.K, S.dots, S.coef);
       }
-      ok = Gk.sync((14 << 4) | 12);
+      rb_kry2<T>(slot, m, ctl.kry && k + 1 < ctl.inner);
+      ok = G.sync((14 << 4) | 12);
     }
+    if (threadIdx.x == 0) S.c[0].tr = S.c[1].tr = nullptr;
     if (!ok) {
       status = 5;
       break;
@@ -1542,13 +1712,14 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
     ++it;
   }
   if (gcta == 0 && threadIdx.x == 0) {
-    if (ctl.trace) ctl.trace[0] = tn;
+    if (ctl.trace) ctl.trace[0] = S.tn;
+    const double r = bn == 0.0 ? 0.0 : load_norm(ctl.norms + it);
     ctl.norms[ctl.max_cycles + 1] = (unsigned long long)__double_as_longlong(r);  // final residual max
     ctl.out[0] = status;
     ctl.out[1] = it;
     ctl.out[2] = cycles;
     ctl.out[3] = it;
-    *H.kst = K;
+    *S.H.kst = S.K;
   }
 }
 
@@ -1564,18 +1735,11 @@ template <class T>
 __global__ void __launch_bounds__(PT, 1) k_rb_vcycle(const RHier<T>* __restrict__ Hg, long long ncell,
                                                      const double* __restrict__ b, double* __restrict__ x, int add,
                                                      Barrier B) {
-  __shared__ RHier<T> H;
-  __shared__ RLev<T> gl;
-  __shared__ unsigned epoch, tn;
-  extern __shared__ __align__(128) unsigned char dyn[];
-  if (threadIdx.x == 0) {
-    epoch = 0u;
-    tn = 0u;
-  }
-  rb_begin(Hg, H, gl, dyn, (int)blockIdx.x);
-  const RCtx G = rb_grid(B, &epoch, &tn, (int)blockIdx.x, (int)gridDim.x);
-  const RLev<T>& L = H.lc == 0 ? gl : H.L[0];
-  for (int t = G.i0; t < L.nqt; t += G.st) {
+  rb_begin<T>(Hg, B, (int)blockIdx.x, (int)gridDim.x);
+  const RHier<T>& H = rsh<T>().H;
+  const RCtx& G = rsh<T>().c[0];
+  const RLev<T>& L = H.L[H.lc == 0 ? RMAX : 0];
+  for (int t = G.i0(); t < L.nqt; t += G.st) {
     const unsigned w0 = reinterpret_cast<const unsigned*>(L.f[0])[t], w1 = reinterpret_cast<const unsigned*>(L.f[1])[t];
     const QPos g = quad_pos(L, t, 0);
     for (int p = 0; p <= L.two; ++p) {
@@ -1589,9 +1753,9 @@ __global__ void __launch_bounds__(PT, 1) k_rb_vcycle(const RHier<T>* __restrict_
       st4(L.b[p][g.s ^ 1] + 4 * (long long)t, o);
     }
   }
-  if (!G.sync(0) || !rb_vcycle(H, gl, G)) return;
+  if (!G.sync(0) || !rb_vcycle<T>()) return;
   const int d = rb_done(H, 0), ir = rb_red(d), ib = rb_black(d);
-  for (int t = G.i0; t < L.nqt; t += G.st) {
+  for (int t = G.i0(); t < L.nqt; t += G.st) {
     const unsigned w[2] = {reinterpret_cast<const unsigned*>(L.f[0])[t], reinterpret_cast<const unsigned*>(L.f[1])[t]};
     const QPos g = quad_pos(L, t, 0);
     for (int p = 0; p <= L.two; ++p) {
@@ -1638,13 +1802,20 @@ __global__ void __launch_bounds__(PT, 1) k_rb_batch(const RBatchItem<T>* __restr
 // time them: 0 a colour pass, 1 the residual + restriction, 6 the prolongation
 template <class T>
 __global__ void __launch_bounds__(PT, 1) k_rb_phase(const RHier<T>* __restrict__ Hg, int kernel, int colour) {
-  __shared__ RLev<T> L, N;
-  copy_words(&L, &Hg->L[0], sizeof(RLev<T>));
-  if (Hg->nlev > 1) copy_words(&N, &Hg->L[1], sizeof(RLev<T>));
+  RHier<T>& H = rsh<T>().H;
+  copy_words(&H.L[0], &Hg->L[0], sizeof(RLev<T>));
+  copy_words(&H.L[1], &Hg->L[Hg->nlev > 1 ? 1 : 0], sizeof(RLev<T>));
+  if (threadIdx.x == 0) {
+    RCtx& c = rsh<T>().c[0];
+    c.local = false;
+    c.gcta = (int)blockIdx.x;
+    c.gsize = (int)gridDim.x;
+    c.st = (int)(gridDim.x * blockDim.x);
+    c.gst = c.st >> 3;
+  }
   __syncthreads();
-  const RCtx G = rb_grid(Barrier{}, nullptr, nullptr, (int)blockIdx.x, (int)gridDim.x);
-  if (kernel == 0) rb_dense(L, colour, 1, false, G);
-  else if (kernel == 1) rb_restrict(L, N, 1, false, G);
-  else rb_prolong(L, N, 1, rb_done(*Hg, 1), G);
+  if (kernel == 0) rb_dense<T>(0, colour, 1, 0);
+  else if (kernel == 1) rb_restrict<T>(0, 1, 1, false, 0);
+  else rb_prolong<T>(0, 1, 1, rb_done(*Hg, 1), 0);
 }
 }  // namespace ebp

@@ -980,12 +980,15 @@ static eb_status setup_rb(eb_poisson* P, int smem_cap) {
   // the dielectric's slabs (rows in 2D, planes in 3D): its vectors are stored for these alone
   const int D = G->L[0].g.D;
   int lohi[2] = {0x7fffffff, -1};
-  int* d_cnt = (int*)pool_alloc(P, sizeof(int) * (4 * RMAX + 2), &st);
+  // per level: rows, red rows, restriction rows, has regular cells; then the
+  // restriction rows' entries, the listed groups, and those again as they are written
+  int* d_cnt = (int*)pool_alloc(P, sizeof(int) * (9 * RMAX + 2), &st);
   if (st != EB_OK) return st;
-  cudaMemsetAsync(d_cnt, 0, sizeof(int) * 4 * RMAX, s);
+  cudaMemsetAsync(d_cnt, 0, sizeof(int) * 9 * RMAX, s);
+  int *d_sn = d_cnt + 4 * RMAX, *d_gn = d_cnt + 5 * RMAX;
   const bool two = G->n_phase == 2;
   if (two) {
-    int* d_lohi = d_cnt + 4 * RMAX;
+    int* d_lohi = d_cnt + 9 * RMAX;
     cudaError_t e = cudaMemcpyAsync(d_lohi, lohi, sizeof(lohi), cudaMemcpyHostToDevice, s);
     k_phase1_rows<<<blocks(G->L[0].g.ncell), 256, 0, s>>>(G->L[0].flags, G->L[0].g.ncell, G->L[0].g.n[0], d_lohi);
     if (e == cudaSuccess) e = cudaMemcpyAsync(lohi, d_lohi, sizeof(lohi), cudaMemcpyDeviceToHost, s);
@@ -1035,6 +1038,7 @@ static eb_status setup_rb(eb_poisson* P, int smem_cap) {
     R.dn1 = make_fastdiv((unsigned)R.n[1]);
     R.two = two ? 1 : 0;
     R.full = R.n[0] % 8 == 0;
+    R.wide = R.n[0] > 1 && R.n[1] > 1 && (R.D == 2 || R.n[2] > 1);
     for (int k = 0; k < 2; ++k) {
       R.dge[k] = T(2 * D - 1) + T(3) * o.wr[k];
       for (int p = 0; p < 2; ++p) R.ide[k][p] = T(1) / (R.dge[k] + o.lh[p]);
@@ -1062,12 +1066,18 @@ static eb_status setup_rb(eb_poisson* P, int smem_cap) {
     double* dg = (double*)pool_alloc(P, sizeof(double) * std::max<long long>(nr, 1), &st);
     double* di = (double*)pool_alloc(P, sizeof(double) * std::max<long long>(nr, 1), &st);
     int* rnat = (int*)pool_alloc(P, sizeof(int) * std::max<long long>(nr, 1), &st);
-    int* inv = (int*)pool_alloc(P, sizeof(int) * std::max<long long>(nr, 1), &st);
     unsigned* col = (unsigned*)pool_alloc(P, sizeof(unsigned) * std::max<long long>(nnz, 1), &st);
     const bool last = l == nl - 1;
-    const size_t nsp = last ? 1 : std::max<long long>(L.nirr, 1);
-    int* sp = (int*)pool_alloc(P, sizeof(int) * nsp, &st);
-    int* spr = (int*)pool_alloc(P, sizeof(int) * nsp * (2 << D), &st);
+    // restriction rows: a coarse cell each per cell with a row at most, in
+    // which every row's entries and diagonal occur once and the regular
+    // children's 2 D + 1 terms come on top
+    const size_t nsp = last ? 1 : std::max<long long>(nr, 1);
+    const size_t sne = last ? 1 : (size_t)(nnz + nr) + (size_t)L.nirr * ((1 << D) - 1) * (2 * D + 1);
+    int4* sd = (int4*)pool_alloc(P, sizeof(int4) * nsp, &st);
+    unsigned* scol = (unsigned*)pool_alloc(P, sizeof(unsigned) * sne, &st);
+    double* sval = (double*)pool_alloc(P, sizeof(double) * sne, &st);
+    int2* slist = (int2*)pool_alloc(P, sizeof(int2) * nsp, &st);
+    int* slen = (int*)pool_alloc(P, sizeof(int) * nsp, &st);
     if (st != EB_OK) return st;
     int* cnt = d_cnt + 4 * l;
     cudaMemsetAsync(f, 0, 2 * (size_t)d.H, s);
@@ -1078,13 +1088,26 @@ static eb_status setup_rb(eb_poisson* P, int smem_cap) {
     const int f2 = D == 3 ? fn[2] : 1, c2 = D == 3 ? cn[2] : 1;
     k_split_flags<<<blocks(n), 256, 0, s>>>(D, d, L.flags, Lf ? Lf->flags : nullptr, fn[0], fn[1], f2,
                                             Lc ? Lc->flags : nullptr, cn[0], cn[1], c2, f, cnt + 3);
+    const dim3 gb((unsigned)blocks(R.nqt), 2);
+    k_split_list<<<gb, 256, 0, s>>>(D, d, f, d_gn + 2 * l, nullptr, nullptr);
     if (nr) {
       k_split_rows<<<1, 1024, 0, s>>>(d, L.flags, L.irr_cell, (int)L.nirr, (int)L.nirr_red, L.row_ptr, L.diag, re, rs,
-                                      dg, di, rnat, inv, cnt);
+                                      dg, di, rnat, cnt);
       if (nnz) k_split_cols<<<blocks(nnz), 256, 0, s>>>(d, L.col, nnz, col);
-      if (Lc)
-        k_split_special<<<blocks(Lc->g.ncell), 256, 0, s>>>(D, L.flags, d.n0, d.n1, d.n2, L.irr_of_cell, inv, cn[0],
-                                                            cn[1], c2, sp, spr, cnt);
+      if (Lc) {
+        RestrictView v;
+        v.f = alg_view(L);
+        v.fd = d;
+        v.cd = split_dim(*Lc);
+        v.cf = Lc->flags;
+        v.c0 = cn[0];
+        v.c1 = cn[1];
+        v.c2 = c2;
+        v.all = H.nu1[l] == 0;
+        k_restrict_count<<<blocks(Lc->g.ncell), 256, 0, s>>>(v, slist, slen, cnt);
+        k_restrict_scan<<<1, 1024, 0, s>>>(slen, cnt + 2, d_sn + l);
+        k_restrict_fill<<<blocks((long long)nsp, 64), 64, 0, s>>>(v, slist, slen, cnt + 2, sd, scol, sval);
+      }
     }
     R.f[0] = f;
     R.f[1] = f + d.H;
@@ -1092,10 +1115,10 @@ static eb_status setup_rb(eb_poisson* P, int smem_cap) {
     R.rs = rs;
     R.col = col;
     R.val = L.val;
-    R.diag = dg;
     R.dinv = di;
-    R.sp = sp;
-    R.sprow = spr;
+    R.sd = sd;
+    R.scol = scol;
+    R.sval = sval;
     H.nnz[l] = (int)nnz;
     if (l == 0) {
       H.rnat = rnat;
@@ -1112,9 +1135,10 @@ static eb_status setup_rb(eb_poisson* P, int smem_cap) {
     H.bslot = bs;
   }
   // Krylov directions and the chunks of their sums: chunks of the finest
-  // level's groups alone, about two per CTA of a whole GPU on large levels
+  // level's groups alone, about one per CTA of a whole GPU, two on large levels
   const RLev<T>& R0 = H.L[0];
-  H.kcs = ((R0.nqt + 303) / 304 + PT - 1) / PT * PT;
+  H.kcs = ((R0.nqt + 151) / 152 + PT - 1) / PT * PT;
+  if (H.kcs > 8 * PT) H.kcs = (H.kcs / 2 + PT - 1) / PT * PT;
   H.kch = (R0.nqt + H.kcs - 1) / H.kcs;
   if (P->kry) {
     for (int i = 0; i < KH && st == EB_OK; ++i)
@@ -1128,7 +1152,7 @@ static eb_status setup_rb(eb_poisson* P, int smem_cap) {
   H.kst = (KryState*)pool_alloc(P, sizeof(KryState), &st);
   if (st != EB_OK) return st;
   cudaMemsetAsync(H.kst, 0, sizeof(KryState), s);
-  int cnt[4 * RMAX];
+  int cnt[7 * RMAX];
   cudaError_t e = cudaMemcpyAsync(cnt, d_cnt, sizeof(cnt), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = cudaGetLastError();
@@ -1137,7 +1161,18 @@ static eb_status setup_rb(eb_poisson* P, int smem_cap) {
     H.L[l].nr = cnt[4 * l];
     H.L[l].nr0 = cnt[4 * l + 1];
     H.L[l].nsp = l < nl - 1 ? cnt[4 * l + 2] : 0;
+    H.snnz[l] = cnt[4 * RMAX + l];
     H.L[l].dense = cnt[4 * l + 3];
+    RLev<T>& R = H.L[l];
+    unsigned* gl[2] = {nullptr, nullptr};
+    for (int c = 0; c < 2; ++c) {
+      R.ngl[c] = cnt[5 * RMAX + 2 * l + c];
+      gl[c] = (unsigned*)pool_alloc(P, sizeof(unsigned) * std::max(R.ngl[c], 1), &st);
+      R.gl[c] = gl[c];
+    }
+    if (st != EB_OK) return st;
+    if (R.ngl[0] + R.ngl[1] > 0)
+      k_split_list<<<dim3((unsigned)blocks(R.nqt), 2), 256, 0, s>>>(D, dim[l], R.f[0], d_gn + 2 * RMAX + 2 * l, gl[0], gl[1]);
   }
   H.krows = (H.L[0].nr + H.kch - 1) / H.kch;
   if (H.bot == 2 && H.L[nl - 1].nr > 32) H.bot = 0, H.bsweeps = std::min(H.bsweeps, ALG_BOTTOM_SWEEPS);
@@ -1172,25 +1207,31 @@ static eb_status setup_rb(eb_poisson* P, int smem_cap) {
   long long off = layout(H.lc);
   H.smem = off <= smem_cap && !grid_bottom ? 1 : 0;
   if (H.smem) {
+    // rows first: every pass reads them, the restriction rows once per cycle
+    auto stage = [&](int l, int bit, std::initializer_list<std::pair<int*, long long>> parts) {
+      long long need = 0;
+      for (const auto& q : parts) need += (q.second + 15) / 16 * 16;
+      if (off + need > smem_cap) return;
+      for (const auto& q : parts) {
+        *q.first = (int)off;
+        off += (q.second + 15) / 16 * 16;
+      }
+      H.srows[l] |= bit;
+    };
+    const long long tb = (long long)sizeof(T);
     for (int l = H.lc; l < nl; ++l) {
       const RLev<T>& R = H.L[l];
-      if (!R.nr) continue;
-      auto al = [](long long b) { return (b + 15) / 16 * 16; };
-      const long long b[8] = {al(8ll * R.nr), al(4ll * R.nr), al(4ll * H.nnz[l]), al((long long)sizeof(T) * H.nnz[l]),
-                              al((long long)sizeof(T) * R.nr), al((long long)sizeof(T) * R.nr), al(4ll * R.nsp),
-                              al(4ll * R.nsp * (2 << D))};
-      long long need = 0;
-      for (long long v : b) need += v;
-      if (off + need > smem_cap) continue;
-      int* dst[8] = {&H.off_re[l], &H.off_rs[l], &H.off_col[l], &H.off_val[l],
-                     &H.off_dg[l], &H.off_di[l], &H.off_sp[l],  &H.off_spr[l]};
-      for (int k = 0; k < 8; ++k) {
-        *dst[k] = (int)off;
-        off += b[k];
-      }
-      H.srows[l] = 1;
+      if (R.nr)
+        stage(l, 1, {{&H.off_re[l], 8ll * R.nr}, {&H.off_rs[l], 4ll * R.nr}, {&H.off_col[l], 4ll * H.nnz[l]},
+                     {&H.off_val[l], tb * H.nnz[l]}, {&H.off_di[l], tb * R.nr}});
+    }
+    for (int l = H.lc; l < nl; ++l) {
+      const RLev<T>& R = H.L[l];
+      if (R.nsp)
+        stage(l, 2, {{&H.off_sd[l], 16ll * R.nsp}, {&H.off_sc[l], 4ll * H.snnz[l]}, {&H.off_sv[l], tb * H.snnz[l]}});
     }
   }
+  H.L[RMAX] = H.L[H.lc];
   P->smem_bytes = H.smem ? (int)off : 0;
   P->bm = H.bm;
   P->d_hier = pool_alloc(P, sizeof(RHier<T>), &st);
