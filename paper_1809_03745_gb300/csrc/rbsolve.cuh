@@ -21,10 +21,11 @@
 // modes that the coarse grids represent badly (a pin thinner than a coarse
 // cell, a rough interface) no longer set the rate, so three sweeps per leg do
 // in 3D what six did.  Measured on a GB300, solves to 1e-13 of max|b|, against
-// the plain layout without any of this: pin-plane 256^3 134 -> 40 ms (24
-// V-cycles of 6+6 sweeps -> 16 of 3+3), 384^3 334 -> 95 ms; rod-plane 1024^2
-// 10.2 -> 8.4 ms; 632 x 488, whose 79 x 61 bottom was BiCGStab over the grid
-// and is now algebraic levels, 62 -> 7.5 ms; 512^2 in FP64 20.7 -> 12.5 ms.
+// the plain layout without any of this: pin-plane 256^3 134 -> 34 ms (24
+// V-cycles of 6+6 sweeps -> 16 of 3+3), 384^3 334 -> 89 ms; rod-plane 128^2
+// 3.5 -> 2.7 ms, 1024^2 10.3 -> 7.0 ms; 632 x 488, whose 79 x 61 bottom was
+// BiCGStab over the grid and is now algebraic levels, 62.6 -> 6.3 ms; 512^2 in
+// FP64 20.7 -> 9.3 ms.
 // The phases are functions out of line: inlined into one kernel, ptxas spilled
 // 4.8 KB of them and took minutes.  The grid barrier, the bounded waits and the
 // trace are those of persistent.cuh.
