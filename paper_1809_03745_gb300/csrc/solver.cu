@@ -1494,9 +1494,10 @@ static eb_status read_norms(eb_poisson* P, double* r, double* b) {
 // r = sgn (b - A x) on the finest level in the plain layout (b null: b = 0), in
 // two independent kernels: the regular cells, eight of an x row per thread
 // with seven FP64 operations each (GB300's FP64 pipe bounds it), and the
-// sparse rows, a group of 8 lanes each.  256^3: 0.30 ms, against 0.75 ms for
-// a thread per cell and a row pass before it.  zero: entries without an
-// unknown are written as 0, else left alone.
+// sparse rows, a group of 8 lanes each.  256^3: 0.34 + 0.02 ms (a thread per
+// cell: 0.36 + 0.02); it replaces a composite level's masked copies and
+// separate zeroing too.  zero: entries without an unknown are written as 0,
+// else left alone.
 // AL: x, b and r are 16-byte aligned (a caller's pointers need not be).
 template <bool AL>
 __device__ __forceinline__ void ldd4(const double* p, double v[4]) {

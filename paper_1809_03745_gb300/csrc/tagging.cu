@@ -15,7 +15,8 @@
 // the square root is monotone, so its root is max |E|).  The second evaluates
 // the tests in FP32 with a bound on their error, and where a threshold lies
 // within it, or a value outside FP32's range, in FP64 from E as above.
-// 256^3: 0.25 ms, against 1.9 ms for three passes in FP64.
+// 256^3 on a random field: 0.30 + 0.41 ms, against 0.55 + 0.25 + 1.23 ms for
+// three passes in FP64.
 #include <cuda_runtime.h>
 
 #include <climits>
