@@ -554,20 +554,23 @@ __global__ void k_field_irregular(LevelGeom L, const double* phi, const double* 
   }
 }
 
+// Normal derivatives at the EB facets, a thread per facet and phase (by
+// blockIdx.y): the least-squares fit behind one is a long FP64 chain, so the
+// two sides of a dielectric facet run next to each other, and warps are spread
+// thinly.  256^3: 0.22 ms, against 0.35 ms for both phases in one thread.
 __global__ void k_field_eb(LevelGeom L, const int* eb_q, long long n_eb, const double* phi, const double* sigma,
                            double* En) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int p = (int)blockIdx.y;
   if (i >= n_eb) return;
-  long long q = eb_q[i];
-  long long cell = L.R.cell[q];
+  const long long q = eb_q[i];
+  const long long cell = L.R.cell[q];
   int I[3];
   cell_ijk(L.g, cell, I);
-  uint8_t f = L.flags[cell];
-  for (int p = 0; p < 2; ++p) {
-    double v = 0.0;
-    if (((f >> p) & 1) && L.R.ebk[q] != EBK_NONE) v = -eval_dn(L, q, I, p, phi, sigma, cell);
-    En[2 * i + p] = v;
-  }
+  const uint8_t f = L.flags[cell];
+  double v = 0.0;
+  if (((f >> p) & 1) && L.R.ebk[q] != EBK_NONE) v = -eval_dn(L, q, I, p, phi, sigma, cell);
+  En[2 * i + p] = v;
 }
 
 __global__ void k_export_kappa(LevelGeom L, double* kappa) {
@@ -1005,7 +1008,7 @@ eb_status launch_field(const eb_geom* G, const double* phi, const double* sigma,
       k_field_regular<false><<<nb, TB, 0, s>>>(v, phi, E, h2, 1.0 / h2, 1.0 / h, pow2);
     if (L.nirr) k_field_irregular<<<nblk(L.nirr, 64), 64, 0, s>>>(v, phi, sigma, E);
   }
-  if (En && L.n_eb) k_field_eb<<<nblk(L.n_eb, 64), 64, 0, s>>>(v, L.eb_q, L.n_eb, phi, sigma, En);
+  if (En && L.n_eb) k_field_eb<<<dim3((unsigned)nblk(L.n_eb, 32), 2), 32, 0, s>>>(v, L.eb_q, L.n_eb, phi, sigma, En);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? EB_OK : cuda_fail(e, "field");
 }
