@@ -141,16 +141,19 @@ struct RCtx {
   }
 };
 
+// The directions kept: in shared memory, and in global memory between the
+// launches of a resumed solve.
+struct KryState {
+  int count, next;   // directions kept, slot of the next one
+  int es;            // the V-cycles' right-hand side is the residual / 2^es (see unit_of)
+  double g[KH][KH];  // (q_i, q_j) by slot
+  double rn[KH];     // 1 / |q_i|
+};
 // The state of a launch.  The phases are functions out of line that find it
 // here and take a few integers: ptxas gives a function the registers that its
 // callers leave, and with descriptions, contexts and loop state held in the
 // callers' registers the phases spilled in their loops (a tenth of all
 // instructions; a solve of 1024^2 took 7.5 ms instead of 6.9, one of 256^3 35.7 instead of 33.7).
-struct KryState {
-  int count, next;   // directions kept, slot of the next one
-  double g[KH][KH];  // (q_i, q_j) by slot
-  double rn[KH];     // 1 / |q_i|
-};
 template <class T>
 struct RShared {
   RHier<T> H;
@@ -1177,11 +1180,34 @@ __device__ __forceinline__ void bits_max(unsigned long long& m, double v) {
   if (b > m && b <= 0x7ff0000000000000ull) m = b;
 }
 
-// FP64 residual of the finest level into level 0's right-hand side (rounded
-// to T) and its max norm; eight cells of an x row per item, seven FP64
+// The unit of the FP32 V-cycles.  The Krylov sums multiply FP32 residuals: below
+// about 1e-20 these products vanish, above 1e17 they overflow, and data in SI
+// units reach both.  Where max|b| is outside 2^-10 .. 2^50 the residual is
+// therefore divided by 2^es, the power of two under max|b|, when it is rounded to
+// FP32, and the correction is multiplied by it when it is added to phi; both are
+// exact, so a solve takes the same steps in every unit.  Inside that range, where
+// a residual 13 digits under max|b| still has its square in FP32's range, es is 0.
+// Where max|r| leaves 2^-56 .. 2^50 units (a guess far from the solution), es is
+// chosen anew from it; the directions kept stay in the unit they were formed in,
+// since z and A z scale alike.  FP64 V-cycles have the range as they are.
+constexpr int ES_LO = -56, ES_MIN = -10, ES_HI = 50;
+__device__ __forceinline__ int exponent_of(double v) {
+  const int e = ((__double2hiint(v) >> 20) & 0x7ff) - 1023;
+  return max(-1000, min(1000, e));
+}
+__device__ __forceinline__ int unit_of(double v) {
+  const int e = exponent_of(v);
+  return e >= ES_MIN && e <= ES_HI ? 0 : e;
+}
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// FP64 residual of the finest level into level 0's right-hand side (in its
+// unit, rounded to T) and its max norm; eight cells of an x row per item, seven FP64
 // operations each (GB300 issues about two FP64 operations per clock and SM,
-// which bounds the pass from 256^2 cells up).
-template <class T>
+// which bounds the pass from 256^2 cells up).  US: in units of 2^es; a build of
+// its own, since even a branch or an FP32 product per cell cost the one without
+// 30 us at 256^3 (the whole solve 0.5 to 2.3%).
+template <class T, bool US>
 __device__ __noinline__ bool rb_resid64(unsigned long long* norm) {
   const RHier<T>& H = rsh<T>().H;
   const RLev<T>& L = H.L[H.lc == 0 ? RMAX : 0];
@@ -1226,7 +1252,7 @@ __device__ __noinline__ bool rb_resid64(unsigned long long* norm) {
         const double v = (bc - s) - d * xc;
         unsigned pos;
         T* b = rb_rhs(L, cl, pos);
-        b[pos] = (T)v;
+        b[pos] = (T)(US ? v * pow2(-rsh<T>().K.es) : v);
         bits_max(mx, v);
       }
     }
@@ -1287,12 +1313,13 @@ __device__ __noinline__ bool rb_resid64(unsigned long long* norm) {
       ld4(F.b[p] + nb, bb);
       ld4(F.b[p] + nb + 4, bb + 4);
       T oe[4], oo[4];
+      const double unit = US ? pow2(-rsh<T>().K.es) : 1.0;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const double dg = e == 0 ? dl : (e == 7 ? dr : d0);
         const double r = bb[e] - F.ceps[p] * (dg * c[e] - s[e]);
-        if (e & 1) oo[e >> 1] = (T)r;
-        else oe[e >> 1] = (T)r;
+        if (e & 1) oo[e >> 1] = (T)(US ? r * unit : r);
+        else oe[e >> 1] = (T)(US ? r * unit : r);
         if (((e & 1) ? mo : me) >> (8 * (e >> 1)) & 1u) bits_max(mx, r);
       }
       quad_store(L.b[p][g.s] + 4 * (long long)t, me, oe);
@@ -1419,8 +1446,6 @@ __device__ __noinline__ void rb_kry1() {
   }
 }
 
-// The directions kept: in shared memory, and in global memory between the
-// launches of a resumed solve.
 // The sums of pass 1 in a fixed order, then the step: the combination of the
 // new and the kept directions that minimises |r - sum c q| (2-norm), by the
 // normal equations.  The directions stay as they were formed, q = A z each:
@@ -1499,7 +1524,7 @@ __device__ __forceinline__ void rb_kry_coeff(const double* part, int nch, int m,
 
 // Krylov pass 2: phi += sum c z in FP64, z kept in slot `slot`, and r -= sum
 // c q where another V-cycle follows before the next FP64 residual.  slot < 0:
-// the plain correction, phi += z.
+// the plain correction, phi += z.  z and r are in the V-cycles' unit, phi is not.
 template <class T>
 __device__ __noinline__ void rb_kry2(int slot, int m, bool upd_r) {
   const RHier<T>& H = rsh<T>().H;
@@ -1517,7 +1542,7 @@ __device__ __noinline__ void rb_kry2(int slot, int m, bool upd_r) {
     cc[i] = i < m ? c[i] : 0.0;
     os[i] = (slot + KH - 1 - i) % KH;
   }
-  const double cn = slot < 0 ? 1.0 : c[KH - 1];
+  const double cn = slot < 0 ? 1.0 : c[KH - 1], unit = pow2(rsh<T>().K.es);
   for (int t = G.i0(); t < L.nqt; t += G.st) {
     const unsigned w[2] = {reinterpret_cast<const unsigned*>(L.f[0])[t], reinterpret_cast<const unsigned*>(L.f[1])[t]};
     if (!((w[0] | w[1]) & 0x03030303u)) continue;
@@ -1568,8 +1593,8 @@ __device__ __noinline__ void rb_kry2(int slot, int m, bool upd_r) {
         const int odd = g.s ^ colour;  // red cells are the even ones where s = 0
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          if (odd) f[2 * e + 1] += (double)s[e];
-          else f[2 * e] += (double)s[e];
+          if (odd) f[2 * e + 1] = fma((double)s[e], unit, f[2 * e + 1]);
+          else f[2 * e] = fma((double)s[e], unit, f[2 * e]);
         }
       }
       st4(ph, f);
@@ -1647,6 +1672,11 @@ __device__ __noinline__ void rb_begin(const RHier<T>* __restrict__ Hg, const Bar
   __syncthreads();
 }
 template <class T>
+__device__ __forceinline__ bool rb_residual(unsigned long long* norm) {
+  if (sizeof(T) == 4 && rsh<T>().K.es) return rb_resid64<T, sizeof(T) == 4>(norm);
+  return rb_resid64<T, false>(norm);
+}
+template <class T>
 __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, const Op<double>* __restrict__ Fg,
                                                const SolveCtl& ctl, const Barrier& B, int gcta, int gsize) {
   RShared<T>& S = rsh<T>();
@@ -1654,7 +1684,10 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
   copy_words(&S.F, Fg, sizeof(Op<double>));
   copy_words(&S.K, Hg->kst, sizeof(KryState));
   rb_begin<T>(Hg, B, gcta, gsize);
-  if (threadIdx.x == 0 && ctl.fresh) S.K.count = S.K.next = 0;
+  if (threadIdx.x == 0 && ctl.fresh) {
+    S.K.count = S.K.next = 0;
+    S.K.es = sizeof(T) == 4 ? unit_of(*ctl.bnorm) : 0;
+  }
   __syncthreads();
   const RCtx& G = S.c[0];
   const double bn = *ctl.bnorm;
@@ -1668,7 +1701,7 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
   // norms are read again where they are needed: little stays in registers across the phases
 #pragma unroll 1
   for (; *ctl.bnorm != 0.0;) {
-    if (!rb_resid64<T>(ctl.norms + it)) {
+    if (!rb_residual<T>(ctl.norms + it)) {
       status = 5;
       break;
     }
@@ -1683,6 +1716,18 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
       break;
     }
     bool ok = true;
+    if (sizeof(T) == 4) {
+      const int off = exponent_of(r) - S.K.es;  // the same in every CTA
+      if (off < ES_LO || off > ES_HI) {
+        __syncthreads();
+        if (threadIdx.x == 0) S.K.es = unit_of(r);
+        __syncthreads();
+        if (!rb_residual<T>(ctl.norms + it)) {  // again in the new unit
+          status = 5;
+          break;
+        }
+      }
+    }
 #pragma unroll 1
     for (int k = 0; k < ctl.inner && ok; ++k) {
       if (ctl.trace && threadIdx.x == 0 && G.gcta == 0) {  // trace the first V-cycle; this thread alone reads tr
