@@ -176,8 +176,9 @@ typedef struct {
   double tol;        /* stop when max|r| <= tol * max|b| (Sec. 3.3.2), default 1e-10 */
   int max_cycles;    /* cap on V-cycles in total, default 100 */
   int nu1, nu2;      /* red-black Gauss-Seidel sweeps before / after the coarse correction;
-                        -1 (the default) = by dimension: 2 in 2D, 3 in 3D, the fastest
-                        on the rod-plane and pin-plane workloads */
+                        -1 (the default) = 2 in 2D; in 3D 3 on the default path, whose V-cycles join
+                        a Krylov space, and 6 without it (launch modes 1 and 2, tile-streamed
+                        levels): the fastest on the rod-plane and pin-plane workloads */
   int precision;     /* EB_PREC_FP64: FP64 V-cycles; EB_PREC_MIXED: FP32 V-cycles inside FP64 defect correction */
   int inner_cycles;  /* FP32 V-cycles per FP64 outer iteration (mixed), default 2 */
   int bottom_sweeps; /* relaxation sweeps on the coarsest level, default 64 */

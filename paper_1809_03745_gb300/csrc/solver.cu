@@ -1389,16 +1389,23 @@ eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, int use, e
   if (opts) P->o = *opts;
   else eb_solver_opts_default(&P->o);
   eb_solver_opts& o = P->o;
-  const int nu_auto = G->L[0].g.D == 3 ? 3 : 2;
-  if (o.nu1 == -1) o.nu1 = nu_auto;
-  if (o.nu2 == -1) o.nu2 = nu_auto;
-  if (!(o.tol > 0.0) || o.max_cycles < 1 || o.nu1 < 0 || o.nu2 < 0 || o.inner_cycles < 1 || o.bottom_sweeps < 1 ||
+  if (!(o.tol > 0.0) || o.max_cycles < 1 || o.nu1 < -1 || o.nu2 < -1 || o.inner_cycles < 1 || o.bottom_sweeps < 1 ||
       (o.precision != EB_PREC_FP64 && o.precision != EB_PREC_MIXED) || o.launch_mode < 0 || o.launch_mode > 2) {
     delete P;
     set_error("invalid solver options");
     return EB_ERR_INVALID;
   }
   P->nlev = (int)G->L.size();
+  int coop = 0;
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, G->device);
+  P->rb = coop && o.launch_mode == 0 && (use != PS_SOLVE || !sweeps_requested(P));
+  P->kry = use == PS_SOLVE;
+  // Sweeps by default: 2 in 2D; in 3D 3 where the V-cycles join a Krylov space
+  // and 6 where they do not (256^3: 16 V-cycles either way, 36 with 3 and no
+  // Krylov step).
+  const int nu_auto = G->L[0].g.D == 2 ? 2 : (P->rb && P->kry ? 3 : 6);
+  if (o.nu1 == -1) o.nu1 = nu_auto;
+  if (o.nu2 == -1) o.nu2 = nu_auto;
   eb_status st = EB_OK;
   int np = G->n_phase;
   const DevLevel& F = G->L[0];
@@ -1412,10 +1419,6 @@ eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, int use, e
   }
   // finest FP64 operator over the solver's own phi and b
   P->op64.push_back(make_op<double>(F, P->allocs, &P->bytes, &st, np, P->phi64, P->b64, P->phi64 + n0, P->b64 + n0));
-  int coop = 0;
-  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, G->device);
-  P->rb = coop && o.launch_mode == 0 && (use != PS_SOLVE || !sweeps_requested(P));
-  P->kry = use == PS_SOLVE;
   if (P->rb || use == PS_OPERATOR) {
     // the colour-split hierarchy has vectors of its own
   } else if (o.precision == EB_PREC_FP64) {
