@@ -55,18 +55,27 @@ struct Done {
   eb_solve_info info{};
 };
 
-// Upper estimate of the device bytes of one instance before it is built: per
-// cell the FP64 solution and right-hand side of both phases (32 B), the
-// caller-side fields (40 B), the inner-precision hierarchy (<= 32 B x 8/7..4/3),
-// geometry arrays per level (~12 B) and the FP64 level copies of the
-// multi-launch path (<= 43 B); cut cells and sparse rows stay well inside the
-// slack; plus the node labels, a fixed part for the small buffers and the
-// dense bottom inverse: coarsening halves even sizes down to 8 cells but may
-// stop earlier on the geometry, so any bottom of at most 1024 unknowns is
-// possible unless the finest grid alone is already larger at the deepest
-// level it could reach.  (Set-up scratch of the inverse is transient.)
-long long estimate_bytes(const eb_geom_desc& d) {
-  long long n = 1, nodes = 1, deepest = 2;
+// Upper estimate of the device bytes of one instance before it is built.
+//   Per cell: the FP64 solution and right-hand side of both phases (32 B) and
+//   the caller-side fields (40 B); per phase, in words of the V-cycles' type, 3
+//   halves of x and 2 of b for each colour on every level (2.5 words, levels sum
+//   to 4/3 in 2D and 8/7 in 3D) and the finest level's four Krylov pairs (8
+//   words); flags twice and two index maps per level (11 B).  A dielectric may
+//   fill the grid, so its vectors count in full.
+//   Per cut cell: its records, and its sparse rows in three forms with the
+//   restriction rows of the coarse cells above, on every level.  Measured with a
+//   dielectric over 0.8 of the grid (232508 cells with rows at 256^3): 4.2-6.7 KB
+//   a cell.  How many there are is not known before the build; each of the two
+//   kinds of surface may be as large as the grid's faces on one side of every axis:
+//   7 KB per face cell for a dielectric's, whose cells have rows of both phases,
+//   and 4 KB for the electrodes'.
+//   Node labels, a fixed part for the small buffers, and the dense bottom inverse:
+//   coarsening halves even sizes down to 8 cells but may stop earlier on the
+//   geometry, so any bottom of at most 1024 unknowns is possible unless the finest
+//   grid alone is already larger at the deepest level it could reach.  (Set-up
+//   scratch of the inverse is transient.)
+long long estimate_bytes(const eb_geom_desc& d, int precision) {
+  long long n = 1, nodes = 1, deepest = 2, faces = 0;
   for (int k = 0; k < d.dim; ++k) {
     n *= d.n[k];
     nodes *= d.n[k] + 1;
@@ -74,8 +83,13 @@ long long estimate_bytes(const eb_geom_desc& d) {
     while (m % 2 == 0 && m / 2 >= 8) m /= 2;
     deepest *= m;
   }
+  for (int k = 0; k < d.dim; ++k) faces += n / std::max(d.n[k], 1);
+  const double levels = d.dim == 2 ? 4.0 / 3.0 : 8.0 / 7.0, word = precision == EB_PREC_MIXED ? 4.0 : 8.0;
+  const int phases = d.dielectric_root >= 0 ? 2 : 1;
+  const double cell = 72.0 + phases * word * (2.5 * levels + 8.0) + 11.0 * levels;
+  const long long cut = faces * ((d.dielectric_root >= 0 ? 7168 : 0) + (d.electrode_root >= 0 ? 4096 : 0));
   long long inv = deepest > 1024 ? 0 : 1024ll * 1024ll * 8ll;
-  return n * 200 + nodes + (8ll << 20) + inv;
+  return (long long)(cell * (double)n) + cut + nodes + (8ll << 20) + inv;
 }
 
 }  // namespace
@@ -270,7 +284,8 @@ void eb_server::run() {
   }
 }
 
-static eb_status copy_request(const eb_geom_desc* d, const double* h_rhs, const double* h_sigma, Request& r) {
+static eb_status copy_request(const eb_geom_desc* d, const double* h_rhs, const double* h_sigma, int precision,
+                              Request& r) {
   if (!d || !h_rhs || d->dim < 2 || d->dim > 3 || d->n_prims < 0 || d->n_prims > EB_MAX_PRIMS || d->n_nodes < 0 ||
       d->n_nodes > EB_MAX_NODES || (d->n_prims && !d->prims) || (d->n_nodes && !d->nodes)) {
     set_error("invalid request");
@@ -292,7 +307,7 @@ static eb_status copy_request(const eb_geom_desc* d, const double* h_rhs, const 
   r.ncell = n;
   r.rhs.assign(h_rhs, h_rhs + 2 * n);
   if (h_sigma) r.sigma.assign(h_sigma, h_sigma + n);
-  r.estimate = estimate_bytes(*d);
+  r.estimate = estimate_bytes(*d, precision);
   return EB_OK;
 }
 
@@ -334,7 +349,7 @@ extern "C" eb_status eb_server_submit(eb_server* S, const eb_geom_desc* desc, co
     return EB_ERR_INVALID;
   }
   auto r = std::make_unique<Request>();
-  eb_status st = copy_request(desc, h_rhs, h_sigma, *r);
+  eb_status st = copy_request(desc, h_rhs, h_sigma, S->o.solver.precision, *r);
   if (st != EB_OK) return st;
   std::lock_guard<std::mutex> lk(S->m);
   if (S->stop) {
