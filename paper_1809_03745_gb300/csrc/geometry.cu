@@ -425,14 +425,17 @@ __device__ double eval_dn(const LevelGeom& L, long long q, const int I[3], int p
 // x / b for a fixed divisor b > 0 with rb = 1 / b correctly rounded: the
 // quotient's rounding is corrected by one fused step (Markstein, IBM J. Res.
 // Dev. 34, 1990), so it equals the division in three FP64 operations; GB300
-// issues about two of them per clock and SM, and a division is ten.  pow2: b
-// is a power of two and the product alone is exact.
+// issues about two of them per clock and SM, and a division is ten.  The step
+// is right while the remainder is exact: where x or the quotient lies within
+// 2^64 of either end of FP64's range (by the exponent bits) it is divided, and
+// zeros keep their sign.  pow2: b is a power of two and the product alone is exact.
+__device__ __noinline__ double div_ends(double x, double b) { return x / b; }
 __device__ __forceinline__ double div_fixed(double x, double b, double rb, bool pow2) {
   const double q = __dmul_rn(x, rb);
   if (pow2) return q;
-  const double r = __fma_rn(-q, b, x);
-  const double v = __fma_rn(r, rb, q);
-  return r == r ? v : q;  // infinite or not a number
+  const unsigned eq = ((unsigned)__double2hiint(q) >> 20) & 0x7ffu, ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  if (eq - 64u < 1920u && ex - 64u < 1920u) return __fma_rn(__fma_rn(-q, b, x), rb, q);
+  return x == 0.0 ? q : div_ends(x, b);
 }
 
 // E at regular cells, four of an x row per thread: every face neighbour in
