@@ -405,7 +405,8 @@ eb_status eb_amr_residual(eb_amr* A, const double* d_rhs_c, const double* d_sig_
  * correction on the box with zero Dirichlet data on its CF sides, each one V-cycle
  * of the persistent multigrid solve (3+3 sweeps, a relaxed bottom at most 32
  * sweeps).  d_phi_c / d_phi_f hold the guess on
- * entry; on return d_phi_c under the box holds the fine means.  info:
+ * entry (entries without an unknown are not read); on return d_phi_c under
+ * the box holds the fine means and entries without an unknown hold 0.  info:
  * outer_iters = FGMRES iterations, vcycles = V-cycles of the corrections.
  * The work space (27 composite vectors) is allocated at the first call. */
 eb_status eb_amr_solve(eb_amr* A, const double* d_rhs_c, const double* d_sig_c, const double* d_rhs_f,
@@ -458,8 +459,9 @@ eb_status eb_amr_residual_levels(eb_amr* A, const double* const* d_rhs, const do
  * finer level a correction of what remains there with zero Dirichlet data on
  * its CF sides), each correction one V-cycle of the persistent multigrid
  * solve (3+3 sweeps, a relaxed bottom at most 32 sweeps).  d_phi holds the
- * guess on entry; on return every level's values
- * under the next finer box hold the finer means.  info as eb_amr_solve. */
+ * guess on entry (entries without an unknown are not read); on return every
+ * level's values under the next finer box hold the finer means and entries
+ * without an unknown hold 0.  info as eb_amr_solve. */
 eb_status eb_amr_solve_levels(eb_amr* A, const double* const* d_rhs, const double* const* d_sig,
                               double* const* d_phi, eb_solve_info* info, void* stream);
 /* E = -grad phi on level `level`'s grid alone (as eb_field_eval; the level's CF

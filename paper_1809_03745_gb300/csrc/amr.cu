@@ -387,6 +387,15 @@ __global__ void k_cv_update(const uint8_t* __restrict__ flags, long long n, int 
   }
 }
 
+// entries without an unknown of the caller's array = 0
+__global__ void k_zero_absent(const uint8_t* __restrict__ flags, long long n, double* __restrict__ x) {
+  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n) return;
+  const unsigned f = flags[c];
+  if (!(f & 1u)) x[c] = 0.0;
+  if (!(f & 2u)) x[n + c] = 0.0;
+}
+
 }  // namespace
 
 constexpr int AMR_MAXL = EB_AMR_MAX_LEVELS;
@@ -1091,8 +1100,14 @@ extern "C" eb_status eb_amr_solve_levels(eb_amr* A, const double* const* d_rhs, 
       note_launch();
     }
   }
-  // report every level's phi under the next finer box as the finer means (finest first)
+  // report every level's phi under the next finer box as the finer means
+  // (finest first), and 0 where there is no unknown: what the guess held in those
+  // entries was neither read nor written so far
   if (st == EB_OK || st == EB_ERR_NOT_CONVERGED) {
+    for (int l = 0; l < L; ++l) {
+      k_zero_absent<<<nb(A->lv[l].n), TBA, 0, s>>>(A->lv[l].flags, A->lv[l].n, d_phi[l]);
+      note_launch();
+    }
     for (int l = L - 2; l >= 0; --l) {
       const AmrLevel &c = A->lv[l], &f = A->lv[l + 1];
       k_avg_down<<<nb(box_cells(A->pr[l + 1].B)), TBA, 0, s>>>(A->pr[l + 1].B, c.flags, f.flags, f.kap,
