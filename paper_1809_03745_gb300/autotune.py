@@ -3,7 +3,7 @@
 The paper fixes no sweep counts (Sec. 3.3.2 only names red-black
 Gauss-Seidel V-cycles), and the best choice depends on the dimension and on
 the cut-cell content: on two-phase rod-plane grids 2+2 sweeps are fastest,
-on 3D pin-plane grids 6+6 sweeps need a sixth of the V-cycles.  The tuner
+on 3D pin-plane grids 3+3 (6+6 without the Krylov step of the default path).  The tuner
 times complete solves (device time of the persistent solve kernel, from
 CUDA events) for a small set of candidate schedules on a sample problem of a
 size class, keeps the fastest that converges, and caches it in a JSON file
@@ -25,9 +25,10 @@ import threading
 CANDIDATES = [(2, 2, 2), (2, 2, 3), (3, 3, 2), (4, 4, 2), (4, 4, 3), (6, 6, 2), (8, 8, 2)]
 
 
-def default_schedule(dim: int):
-    """The library's own choice when nothing is cached (nu1 = nu2 = -1)."""
-    return (6, 6, 2) if dim == 3 else (2, 2, 2)
+def default_schedule(dim: int, accelerated: bool = False):
+    """The library's own choice when nothing is cached (nu1 = nu2 = -1): where
+    the V-cycles join a Krylov space (the default launch mode) or do not."""
+    return (2, 2, 2) if dim == 2 else (3, 3, 2) if accelerated else (6, 6, 2)
 
 
 def size_class(dim: int, ncell: int, n_phase: int, precision: str) -> str:
@@ -101,10 +102,12 @@ class Autotuner:
 
     def schedule(self, geom, precision="mixed"):
         key = size_class(geom.dim, geom.ncell, int(geom.info["n_phase"]), precision)
-        return self.lookup(key) or default_schedule(geom.dim)
+        return self.lookup(key) or default_schedule(geom.dim, accelerated=True)
 
     def solver(self, geom, *, precision="mixed", **kw):
-        """A Poisson solver with the cached (else default) schedule of the class."""
+        """A Poisson solver with the cached schedule of the class, else the
+        library's own choice for the path that it takes."""
         from . import ebpoisson as E
-        nu1, nu2, inner = self.schedule(geom, precision)
+        key = size_class(geom.dim, geom.ncell, int(geom.info["n_phase"]), precision)
+        nu1, nu2, inner = self.lookup(key) or (-1, -1, 2)
         return E.Poisson(geom, precision=precision, nu1=nu1, nu2=nu2, inner_cycles=inner, **kw)
