@@ -349,8 +349,11 @@ eb_status eb_poisson_profile(eb_poisson* P, int kernel, int reps, double* ms_per
  * the bounded-wait self-test: two CTAs wait at a grid barrier sized for
  * three, so the wait ends only by its clock bound (about 2 s); the call then
  * returns EB_ERR_TIMEOUT with ms_per_launch the kernel's duration, and the
- * context stays usable.  Kernels 4 and 5 need a finest level relaxed by
- * tile-streamed sweeps (EB_ERR_UNSUPPORTED otherwise): 4 is one such sweep,
+ * context stays usable.  Kernels 4 and 5 are the tile-streamed passes over the
+ * finest level (EB_ERR_UNSUPPORTED where it does not take them: FP32 3D levels of
+ * at least 2^25 cells or as EBP_SWEEP_MIN_CELLS says, extents as under
+ * sweep_levels; a handle that solves without them is set up a second time for
+ * the call, so it needs that much free memory): 4 is one such sweep,
  * both colours in one pass (bytes: read x, b, flags, write x per cell), 5 the
  * tile-streamed residual + restriction (read x, b, flags per fine cell, write
  * coarse b and x); a wait of theirs that gives up returns EB_ERR_TIMEOUT. */

@@ -130,8 +130,9 @@ eb_status batch_step(eb_poisson* const* P, int n, const double* const* rhs, cons
                      double* const* phi, bool fresh, bool copy_out, int max_iters, cudaStream_t s,
                      double* kernel_ms);
 // what a handle is for: solves, V-cycles that precondition an outer Krylov
-// method (no acceleration of their own), or applying the operator alone
-enum { PS_SOLVE = 0, PS_PLAIN = 1, PS_OPERATOR = 2 };
+// method (no acceleration of their own), applying the operator alone, or
+// tile-streamed levels unasked
+enum { PS_SOLVE = 0, PS_PLAIN = 1, PS_OPERATOR = 2, PS_STREAMED = 3 };
 eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, int use, eb_poisson** out);
 void batch_info(eb_poisson* Q, eb_solve_info* inf);
 eb_status batch_copy_out(eb_poisson* P, double* phi, cudaStream_t s);

@@ -537,9 +537,10 @@ static bool tmap3(CUtensorMap* m, CUtensorMapDataType type, int esize, const voi
 }
 
 // Tile-streamed sweeps run on request alone (EBP_SWEEP_MIN_CELLS=n: levels of
-// at least n cells).  Measured on a GB300 at 384^3 a streamed sweep of the plain
-// layout takes 0.39 ms; two passes over the colour-split layout of rbsolve.cuh
-// take 0.18 ms.
+// at least n cells), and where eb_poisson_profile times them, from SW_MIN_CELLS
+// on: there a streamed sweep of the plain layout (0.39 ms at 384^3 on a GB300)
+// beats the plain layout's two colour passes (0.53 ms).  Two passes over the
+// colour-split layout of rbsolve.cuh take 0.18 ms, so no solve streams by itself.
 static constexpr long long SW_MIN_CELLS = 1LL << 25;
 
 // Items of a level cut into z-chunks of zc planes: tile t = it % ntiles,
@@ -585,7 +586,7 @@ static int sweep_chunk(const int n[3], int workers, const std::vector<uint8_t>* 
   return zc_best;
 }
 
-// Marks the FP32 3D grid levels of at least SW_MIN_CELLS cells (each extent
+// Marks the FP32 3D grid levels of at least SW_MIN_CELLS (or the requested) cells (each extent
 // a multiple of 4, x a multiple of 16) for tile-streamed passes: a second x
 // buffer per phase, tensor maps of x, the second buffer, b and the flags with
 // two-plane boxes, and the list of items that hold dielectric unknowns.
@@ -1362,16 +1363,18 @@ static eb_status solve_persistent(eb_poisson* P, double* r, int* iters, int* cyc
   return EB_OK;
 }
 
-// Whether the environment asks for tile-streamed sweeps (EBP_SWEEP_MIN_CELLS=n)
-// and the finest level takes them.
-static bool sweeps_requested(const eb_poisson* P) {
-  const char* env = std::getenv("EBP_SWEEP_MIN_CELLS");
-  if (!env || P->o.precision != EB_PREC_MIXED || P->nlev < 2) return false;
+// Whether the finest level takes tile-streamed sweeps from min_cells cells on.
+static bool takes_sweeps(const eb_poisson* P, long long min_cells) {
+  if (P->o.precision != EB_PREC_MIXED || P->nlev < 2) return false;
   if (const char* off = std::getenv("EBP_SWEEP"))
     if (std::atoi(off) == 0) return false;
   const Grid& g = P->G->L[0].g;
-  return g.D == 3 && g.ncell >= std::max(1LL, std::atoll(env)) && g.ncell > 4096 && g.n[0] % 16 == 0 && g.n[1] % 4 == 0 &&
-         g.n[2] % 4 == 0;
+  return g.D == 3 && g.ncell >= min_cells && g.ncell > 4096 && g.n[0] % 16 == 0 && g.n[1] % 4 == 0 && g.n[2] % 4 == 0;
+}
+// Whether the environment asks for them (EBP_SWEEP_MIN_CELLS=n).
+static bool sweeps_requested(const eb_poisson* P) {
+  const char* env = std::getenv("EBP_SWEEP_MIN_CELLS");
+  return env && takes_sweeps(P, std::max(1LL, std::atoll(env)));
 }
 
 extern "C" eb_status eb_poisson_setup(const eb_geom* G, const eb_solver_opts* opts, void* stream, eb_poisson** out) {
@@ -1398,7 +1401,7 @@ eb_status poisson_setup(const eb_geom* G, const eb_solver_opts* opts, int use, e
   P->nlev = (int)G->L.size();
   int coop = 0;
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, G->device);
-  P->rb = coop && o.launch_mode == 0 && (use != PS_SOLVE || !sweeps_requested(P));
+  P->rb = coop && o.launch_mode == 0 && use != PS_STREAMED && (use != PS_SOLVE || !sweeps_requested(P));
   P->kry = use == PS_SOLVE;
   // Sweeps by default: 2 in 2D; in 3D 3 where the V-cycles join a Krylov space
   // and 6 where they do not (256^3: 16 V-cycles either way, 36 with 3 and no
@@ -2123,6 +2126,48 @@ extern "C" eb_status eb_field_eval(eb_poisson* P, const double* d_phi, const dou
   return e == cudaSuccess ? EB_OK : cuda_fail(e, "field");
 }
 
+// kernel 4: one tile-streamed sweep (both colours) of the finest level on its
+// own; kernel 5: the streamed residual + restriction of that level
+static eb_status profile_streamed(eb_poisson* P, int kernel, int reps, double* ms, double* bytes, cudaStream_t s) {
+  if (!P->persistent || P->o.precision != EB_PREC_MIXED || P->sweep_first != 0 || P->nlev < 2) {
+    set_error("the finest level has no tile-streamed sweep");
+    return EB_ERR_UNSUPPORTED;
+  }
+  cudaMemsetAsync(P->d_bar, 0, 4 * sizeof(unsigned), s);
+  int* err = (int*)(P->d_bar + 2);
+  const Hier<float>* H = (const Hier<float>*)P->d_hier;
+  const size_t dyn = (size_t)P->sweep_bytes;
+  cudaEvent_t e0, e1;
+  cudaEventCreate(&e0);
+  cudaEventCreate(&e1);
+  auto go = [&]() {
+    if (kernel == 4) k_sweep_phase<float><<<P->grid, PT, dyn, s>>>(H, 0, err);
+    else k_restrict3d_phase<float><<<P->grid, PT, dyn, s>>>(H, 0, err);
+  };
+  go();
+  cudaEventRecord(e0, s);
+  for (int i = 0; i < reps; ++i) go();
+  cudaEventRecord(e1, s);
+  cudaError_t e = cudaEventSynchronize(e1);
+  float t = 0.0f;
+  if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  unsigned bar[3] = {0, 0, 0};
+  if (e == cudaSuccess) e = cudaMemcpy(bar, P->d_bar, sizeof(bar), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return cuda_fail(e, "sweep profile");
+  if (bar[2]) {
+    sweep_reset(P, s);
+    set_error("a sweep wait gave up");
+    return EB_ERR_TIMEOUT;
+  }
+  *ms = (double)t / reps;
+  // sweep: read x and b, write x (4 bytes each), read the flag byte, per cell;
+  // restriction: read x and b, the flag byte, write coarse b and x (8 / 8 bytes)
+  *bytes = (double)P->G->L[0].g.ncell * (kernel == 4 ? 13.0 : 10.0);
+  return EB_OK;
+}
+
 extern "C" eb_status eb_poisson_profile(eb_poisson* P, int kernel, int reps, double* ms, double* bytes, void* stream) {
   if (P && kernel == 2 && reps >= 1 && ms && bytes) {
     if (!P->persistent) {
@@ -2178,46 +2223,15 @@ extern "C" eb_status eb_poisson_profile(eb_poisson* P, int kernel, int reps, dou
     return EB_OK;
   }
   if (P && (kernel == 4 || kernel == 5) && reps >= 1 && ms && bytes) {
-    // kernel 4: one tile-streamed sweep (both colours) of the finest level on
-    // its own; kernel 5: the streamed residual + restriction of that level
-    if (!P->persistent || P->o.precision != EB_PREC_MIXED || P->sweep_first != 0 || P->nlev < 2) {
-      set_error("the finest level has no tile-streamed sweep");
-      return EB_ERR_UNSUPPORTED;
-    }
     cudaStream_t s = (cudaStream_t)stream;
-    cudaMemsetAsync(P->d_bar, 0, 4 * sizeof(unsigned), s);
-    int* err = (int*)(P->d_bar + 2);
-    const Hier<float>* H = (const Hier<float>*)P->d_hier;
-    const size_t dyn = (size_t)P->sweep_bytes;
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    auto go = [&]() {
-      if (kernel == 4) k_sweep_phase<float><<<P->grid, PT, dyn, s>>>(H, 0, err);
-      else k_restrict3d_phase<float><<<P->grid, PT, dyn, s>>>(H, 0, err);
-    };
-    go();
-    cudaEventRecord(e0, s);
-    for (int i = 0; i < reps; ++i) go();
-    cudaEventRecord(e1, s);
-    cudaError_t e = cudaEventSynchronize(e1);
-    float t = 0.0f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    unsigned bar[3] = {0, 0, 0};
-    if (e == cudaSuccess) e = cudaMemcpy(bar, P->d_bar, sizeof(bar), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "sweep profile");
-    if (bar[2]) {
-      sweep_reset(P, s);
-      set_error("a sweep wait gave up");
-      return EB_ERR_TIMEOUT;
-    }
-    *ms = (double)t / reps;
-    // sweep: read x and b, write x (4 bytes each), read the flag byte, per cell;
-    // restriction: read x and b, the flag byte, write coarse b and x (8 / 8 bytes)
-    *bytes = (double)P->G->L[0].g.ncell * (kernel == 4 ? 13.0 : 10.0);
-    return EB_OK;
+    if (!P->rb || !P->persistent || !takes_sweeps(P, SW_MIN_CELLS)) return profile_streamed(P, kernel, reps, ms, bytes, s);
+    // a solve does not stream this level any more: a handle that does, for this call
+    eb_poisson* Q = nullptr;
+    eb_status st = poisson_setup(P->G, &P->o, PS_STREAMED, &Q);
+    if (st != EB_OK) return st;
+    st = profile_streamed(Q, kernel, reps, ms, bytes, s);
+    eb_poisson_destroy(Q);
+    return st;
   }
   if (!P || reps < 1 || (kernel != 0 && kernel != 1 && kernel != 6) || !ms || !bytes) {
     set_error("invalid argument");
