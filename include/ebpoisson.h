@@ -334,14 +334,18 @@ void eb_tga_destroy(eb_tga* T);
  * finest multigrid level `reps` times on `stream` between CUDA events and
  * reports the mean duration per launch and the algorithmic bytes one launch
  * must move.  It relaxes the solver's own work arrays (left as the last solve
- * left them); the caller's fields are not touched.  Both run the persistent
+ * left them); the caller's fields are not touched.  They run the persistent
  * solve kernel's own phase code in its grid shape.  kernel 0: one colour of
- * the red-black Gauss-Seidel sweep (regular cells) of the inner-precision finest level
- * (bytes: half of read x, read b, write x, read flags per cell); kernel 1: the
- * fused residual + restriction of that level (read x, b, flags per fine cell,
- * write coarse b and x); kernel 6: the prolongation of the next level's
- * correction onto it (read and write x, read the flags per fine cell, read
- * the coarse x and flags). */
+ * the red-black Gauss-Seidel sweep of the inner-precision finest level, its
+ * sparse rows included on the default path, whose pass does both (bytes: half
+ * of read x, read b, write x, read flags per cell; the rows' are not counted);
+ * kernel 1: the fused residual + restriction of that level (default path: read
+ * x and half of b and of the flags per fine cell, since the black residuals are
+ * 0 after a sweep, read the flags and write b per coarse cell; launch modes 1
+ * and 2: read x, b, flags per fine cell, write coarse b and x); kernel 6: the
+ * prolongation of the next level's correction onto it (read and write x, read
+ * the flags per fine cell, read the coarse x, on the launch modes 1 and 2 the
+ * coarse flags too). */
 eb_status eb_poisson_profile(eb_poisson* P, int kernel, int reps, double* ms_per_launch, double* bytes_per_launch,
                              void* stream);
 /* kernel 2 of eb_poisson_profile times `reps` grid barriers of the persistent

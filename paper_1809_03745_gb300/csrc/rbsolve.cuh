@@ -1845,7 +1845,8 @@ __global__ void __launch_bounds__(PT, 1) k_rb_batch(const RBatchItem<T>* __restr
 }
 
 // single phases of the finest level in the persistent kernel's grid shape, to
-// time them: 0 a colour pass, 1 the residual + restriction, 6 the prolongation
+// time them: 0 a colour pass (its regular cells, listed groups and sparse rows),
+// 1 the residual + restriction, 6 the prolongation
 template <class T>
 __global__ void __launch_bounds__(PT, 1) k_rb_phase(const RHier<T>* __restrict__ Hg, int kernel, int colour) {
   RHier<T>& H = rsh<T>().H;
@@ -1860,7 +1861,7 @@ __global__ void __launch_bounds__(PT, 1) k_rb_phase(const RHier<T>* __restrict__
     c.gst = c.st >> 3;
   }
   __syncthreads();
-  if (kernel == 0) rb_dense<T>(0, colour, 1, 0);
+  if (kernel == 0) rb_pass<T>(0, colour, 1, false, 0);
   else if (kernel == 1) rb_restrict<T>(0, 1, 1, false, 0);
   else rb_prolong<T>(0, 1, 1, rb_done(*Hg, 1), 0);
 }

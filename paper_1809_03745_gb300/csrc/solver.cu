@@ -2279,7 +2279,10 @@ extern "C" eb_status eb_poisson_profile(eb_poisson* P, int kernel, int reps, dou
   cudaEventDestroy(e1);
   if (e != cudaSuccess) return cuda_fail(e, "profile");
   *ms = (double)t / reps;
+  const double coarse = (double)n / (double)(1 << D);
   if (kernel == 0) *bytes = (double)n * (3.0 * tb + 1.0) / 2.0;
+  else if (P->rb && kernel == 1) *bytes = (double)n * (1.5 * tb + 0.5) + coarse * (tb + 1.0);  // red b and flags alone
+  else if (P->rb) *bytes = (double)n * (2.0 * tb + 1.0) + coarse * tb;
   else if (kernel == 1) *bytes = (double)n * (2.0 * tb + 1.0) + (double)n / (double)(1 << D) * 2.0 * tb;
   else *bytes = (double)n * (2.0 * tb + 1.0) + (double)n / (double)(1 << D) * (tb + 1.0);
   return EB_OK;
