@@ -197,8 +197,8 @@ def run_reference(args):
 
 
 def vcycle_bytes(dim, wb, sweeps):
-    """Algorithmic bytes per finest-level cell of one V-cycle with `sweeps`
-    red-black sweeps per level (nu1 + nu2) in precision wb (bytes): per sweep
+    """Algorithmic bytes per finest-level cell of one V-cycle in the plain layout
+    with `sweeps` red-black sweeps per level (nu1 + nu2) in precision wb (bytes): per sweep
     read x, read b, write x and read the flag byte; residual + restriction
     read x, b and the flags and write the coarse b and x (2 wb / 2^D);
     prolongation reads the coarse correction (wb / 2^D), reads and writes x
@@ -209,12 +209,31 @@ def vcycle_bytes(dim, wb, sweeps):
 
 
 def solve_bytes(ncell, dim, mixed, vcycles, outer, sweeps=4, launches=1):
-    """Algorithmic bytes of persistent solves over ncell finest cells: the
+    """Algorithmic bytes of persistent plain-layout solves over ncell finest cells: the
     V-cycles, 44 B per FP64 outer iteration (the FP64 residual: read phi, b,
     write r, 24 B; the update: read phi, the FP32 correction, write phi, 20 B)
     and the initial FP64 residual (24 B) of each launch."""
     wb = 4 if mixed else 8
     return ncell * (vcycles * vcycle_bytes(dim, wb, sweeps) + outer * 44.0 + 24.0 * launches)
+
+
+def split_vcycle_bytes(dim, wb, sweeps):
+    """The same of one V-cycle from zero on the colour-split levels: the first
+    colour pass reads no x, the residual + restriction after a sweep reads x, the
+    red half of b and of the flags and per coarse cell reads the flags and writes
+    b, the prolongation reads per coarse cell x alone."""
+    c = 2 ** dim
+    per = sweeps * (3 * wb + 1) - wb / 2 + (1.5 * wb + 0.5 + (wb + 1) / c) + (2 * wb + 1 + wb / c)
+    return per * (4.0 / 3.0 if dim == 2 else 8.0 / 7.0)
+
+
+def precond_bytes(ncell, dim, mixed, launches, sweeps):
+    """Algorithmic bytes of V-cycles applied as a preconditioner, one per launch:
+    around each, b is read in FP64 and level 0's written with its flags read, and
+    x is read with the flags and added to the FP64 result (read and written).
+    There is no FP64 residual or update."""
+    wb = 4 if mixed else 8
+    return ncell * launches * (split_vcycle_bytes(dim, wb, sweeps) + (8 + wb + 1) + (wb + 1 + 16))
 
 
 def kernels_at_scale(dev, E, W, n=384):
@@ -232,7 +251,8 @@ def kernels_at_scale(dev, E, W, n=384):
     out = {"workload": f"3D pin-plane {n}^3 with dielectric disk, FP32 finest level", "cells": n ** 3,
            "smooth_colour_ms": sms, "smooth_colour_bytes": sb, "smooth_colour_gbs": sb / sms / 1e6,
            "smooth_frac": sb / sms / 1e6 / hbm,
-           "smooth_note": "one colour on the colour-split level: read the other colour, b, flags, write the colour",
+           "smooth_note": "one colour pass of the colour-split level, cut-cell rows included in the time: read the "
+                          "other colour, b, flags, write the colour",
            "resid_restrict_ms": rms, "resid_restrict_bytes": rb, "resid_restrict_gbs": rb / rms / 1e6,
            "resid_restrict_frac": rb / rms / 1e6 / hbm,
            "prolong_ms": pms, "prolong_bytes": pb, "prolong_gbs": pb / pms / 1e6,
@@ -390,10 +410,8 @@ def run_gpu(args):
     k_ms = statistics.mean(r[1]["coarse"]["kernel_ms"] + r[1]["fine"]["kernel_ms"] for r in res)
     k_launch = kst["coarse"]["launches"] + kst["fine"]["launches"]
     sweeps = 6  # the corrections' V-cycles use 3 + 3 sweeps
-    k_bytes = (solve_bytes(G.n_coarse, 3, True, kst["coarse"]["vcycles"], kst["coarse"]["outer"], sweeps,
-                           kst["coarse"]["launches"]) +
-               solve_bytes(G.n_fine, 3, True, kst["fine"]["vcycles"], kst["fine"]["outer"], sweeps,
-                           kst["fine"]["launches"]))
+    k_bytes = (precond_bytes(G.n_coarse, 3, True, kst["coarse"]["launches"], sweeps) +
+               precond_bytes(G.n_fine, 3, True, kst["fine"]["launches"], sweeps))
     scale = kernels_at_scale(dev, E, W, args.scale_n) if (rank == 0 and not args.no_scale) else None
 
     # end to end through the public API with host buffers
@@ -473,8 +491,8 @@ def run_gpu(args):
                      "traffic": traffic, "peak_source": "measured" if peaks else "fallback",
                      "ms_per_launch": k_ms / max(k_launch, 1), "bytes_per_launch": k_bytes / max(k_launch, 1),
                      "launches_per_step": k_launch, "kernel_ms_per_step": k_ms,
-                     "bytes_model": "per finest cell and launch: V-cycles x (6 sweeps x 13 B + residual/restriction "
-                                    "10 B + prolongation 9.5 B) x 8/7 + 44 B per FP64 outer iteration + 24 B"},
+                     "bytes_model": "per finest cell and launch: (6 sweeps x 13 B - 2 B from zero + residual/restriction "
+                                    "7.125 B + prolongation 9.5 B) x 8/7 + 13 B (FP64 b in) + 21 B (FP64 x added)"},
         "kernels_at_scale": scale,
         "extra_configs": extra,
         "cpu_baseline": cpu,
