@@ -1629,6 +1629,12 @@ __device__ __noinline__ void rb_begin(const RHier<T>* __restrict__ Hg, const Bar
     for (int l = H.lc; l < H.nlev; ++l) {
       const RLev<T>& g = Hg->L[l];
       for (int q = 0; q < 2; ++q) copy_words(dyn + H.off_f[l][q], g.f[q], g.H);
+      // zeros, as the vectors in global memory start with
+      for (int p = 0; p <= g.two; ++p)
+        for (int k = 0; k < 5; ++k) {
+          T* v = (T*)(dyn + (k < 3 ? H.off_x[l][p][k] : H.off_b[l][p][k - 3]));
+          for (int i = threadIdx.x; i < g.H; i += blockDim.x) v[i] = T(0);
+        }
       if (H.srows[l] & 1) {
         copy_words(dyn + H.off_re[l], g.re, 8ll * g.nr);
         copy_words(dyn + H.off_rs[l], g.rs, 4ll * g.nr);
