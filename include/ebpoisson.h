@@ -486,17 +486,19 @@ eb_status eb_amr_field_eval(eb_amr* A, int level, const double* d_phi, const dou
  * grad T by differences over the axis neighbours that carry T: centred
  * ((T+ - T-)/2 in index units, dx cancels), one-sided where one neighbour
  * does, 0 where none does; the ratio is 0 where T and the gradient are 0 and
- * infinite where only T is 0.  Covered cells get no tag.  All arithmetic is
- * FP64 without contraction, so the tags are a function of d_E alone.
+ * infinite where only T is 0.  Covered cells get no tag.  The tags are those of
+ * FP64 without contraction, a function of d_E alone (FP32 decides where its
+ * error cannot change them).
  * d_E: [D][2][n_cells] as eb_field_eval writes it.  keep_lo / keep_hi (both
  * or neither NULL): the current finer box on this grid; its cells that carry
  * T and are not tagged for coarsening are marked as well (a refined region is
  * kept until the coarsening test releases it).  d_tags (may be NULL):
  * [n_cells] tag bytes.  On return bbox_lo / bbox_hi (host, 3 ints; hi
  * exclusive) bound the marked cells (refine-tagged or kept), *n_marked counts
- * them (0: bbox undefined) and *e_max is max |E|.  The call allocates a
- * scratch of n_cells doubles (T) for its duration and synchronises the
- * stream.  EB_ERR_INVALID for a NULL argument, an eps that is not finite, or
+ * them (0: bbox undefined) and *e_max is max |E|.  The geometry keeps a
+ * scratch of n_cells floats from the first call on (counted in device_bytes;
+ * a call that finds another thread using it takes one of its own).  The call
+ * synchronises the stream.  EB_ERR_INVALID for a NULL argument, an eps that is not finite, or
  * a current device other than the geometry's (checked before any launch). */
 eb_status eb_tag_cells(const eb_geom* G, const double* d_E, const double eps[4], const int* keep_lo,
                        const int* keep_hi, unsigned char* d_tags, int bbox_lo[3], int bbox_hi[3],

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -53,6 +54,7 @@ struct eb_geom {
   // scratch of eb_tag_cells, taken at its first call and kept
   mutable std::mutex scratch_lock;
   mutable void* scratch = nullptr;
+  mutable std::atomic<long long> scratch_bytes{0};
 };
 
 namespace ebp {

@@ -264,7 +264,7 @@ extern "C" eb_status eb_geom_query(const eb_geom* G, eb_geom_info* out) {
   for (size_t l = 0; l < G->L.size(); ++l)
     for (int k = 0; k < 3; ++k) out->level_n[l][k] = G->L[l].g.n[k];
   for (int k = 0; k < 3; ++k) out->stencil_order[k] = G->stencil_counts[k];
-  out->device_bytes = G->bytes;
+  out->device_bytes = G->bytes + G->scratch_bytes;
   return EB_OK;
 }
 

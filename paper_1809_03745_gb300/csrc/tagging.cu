@@ -224,9 +224,13 @@ extern "C" eb_status eb_tag_cells(const eb_geom* G, const double* d_E, const dou
   const bool kept = lock.owns_lock();
   char* d_buf = kept ? (char*)G->scratch : nullptr;
   cudaError_t e = cudaSuccess;
-  if (!d_buf) e = cudaMalloc(&d_buf, head + sizeof(float) * (size_t)v.ncell);
+  const size_t size = head + sizeof(float) * (size_t)v.ncell;
+  if (!d_buf) e = cudaMalloc(&d_buf, size);
   if (e != cudaSuccess) return cuda_fail(e, "tag scratch");
-  if (kept) G->scratch = d_buf;
+  if (kept) {
+    G->scratch = d_buf;
+    G->scratch_bytes = (long long)size;
+  }
   TagOut* d_out = (TagOut*)d_buf;
   float* d_M = (float*)(d_buf + head);
   e = cudaMemcpyAsync(d_out, &init, sizeof(init), cudaMemcpyHostToDevice, s);
