@@ -371,12 +371,12 @@ eb_status eb_device_fma_rates(int device, double* fp64_tflops, double* fp32_tflo
 
 /* Diagnostics (no counterpart in the paper): the phases of the first V-cycle
  * of the last persistent solve.  out[0] = number of phases m; then for each
- * phase i, out[1+2i] = its code ((level << 4) | kind; kinds 1 red regular
- * cells, 3 black regular cells (each also writes the sparse-row values of
- * its colour), 2 sparse rows computed, 5 sparse residual rows, 6 residual +
- * restriction, 7 prolongation,
- * 8 end of the one-CTA levels, 9 bottom solve) and
- * out[2+2i] its duration in ms.  n is the capacity of out. */
+ * phase i, out[1+2i] = its code ((level << 4) | kind; kinds 1 red cells, 3
+ * black cells (regular ones and sparse rows), 6 residual + restriction, 7
+ * prolongation, 8 end of the one-CTA levels, 9 bottom solve, 12 a zero iterate
+ * or, as level 14, the update of phi, 14 as level 14 the Krylov sums; on
+ * tile-streamed hierarchies 2 sparse rows computed, 5 sparse residual rows and
+ * 13 a streamed sweep too) and out[2+2i] its duration in ms.  n is the capacity of out. */
 eb_status eb_poisson_trace(eb_poisson* P, double* out, int n);
 
 /* ---------------------------------------------------------------- composite grid

@@ -197,7 +197,7 @@ def kernels_once(n, reps):
     for k in (4, 0, 5, 1, 6):
         try:
             ms, by = P.profile(k, reps=reps)
-        except E.EBError as exc:  # streamed levels are built on request only
+        except E.EBError as exc:  # streamed levels start at 2^25 cells
             print(json.dumps({"kernel": names[k], "n": n, "skipped": str(exc)}), flush=True)
             continue
         print(json.dumps({"kernel": names[k], "n": n, "ms": ms, "gbs": by / ms / 1e6}), flush=True)

@@ -374,11 +374,6 @@ __global__ void k_split_cols(SplitDim d, const int* col, long long nnz, unsigned
   const unsigned cl = (unsigned)col[e];
   out[e] = ((cl >> 30) << 31) | split_index(d, cl & 0x3fffffffu);
 }
-// Restriction rows: for every unknown of the coarse grid whose cell has a
-// child with a sparse row, the mean of its children's residuals as one row
-// over the fine level, the children's rows one after the other.  all: black
-// regular children too (without a sweep their residuals are not zero).  The
-// order of the rows does not matter (each writes its own unknown).
 // The groups that a pass takes from a list (rb_dense_list): counted into
 // n[colour], and written to out[colour] where that is given.
 __global__ void k_split_list(int D, SplitDim d, const uint8_t* f, int* n, unsigned* out0, unsigned* out1) {
@@ -401,6 +396,11 @@ __global__ void k_split_list(int D, SplitDim d, const uint8_t* f, int* n, unsign
     if (out) out[i] = (unsigned)t | p << 31;
   }
 }
+// Restriction rows: for every unknown of the coarse grid whose cell has a
+// child with a sparse row, the mean of its children's residuals as one row
+// over the fine level, the children's rows one after the other.  all: black
+// regular children too (without a sweep their residuals are not zero).  The
+// order of the rows does not matter (each writes its own unknown).
 struct RestrictView {
   AlgView f;
   SplitDim fd, cd;

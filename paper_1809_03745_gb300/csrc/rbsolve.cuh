@@ -1205,8 +1205,8 @@ __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + 
 // unit, rounded to T) and its max norm; eight cells of an x row per item, seven FP64
 // operations each (GB300 issues about two FP64 operations per clock and SM,
 // which bounds the pass from 256^2 cells up).  US: in units of 2^es; a build of
-// its own, since even a branch or an FP32 product per cell cost the one without
-// 30 us at 256^3 (the whole solve 0.5 to 2.3%).
+// its own, since a shift of the exponent bits, or a branch and an FP32 product,
+// in every cell cost this one 20 to 100 us at 256^3 (a whole solve 0.5 to 2.3%).
 template <class T, bool US>
 __device__ __noinline__ bool rb_resid64(unsigned long long* norm) {
   const RHier<T>& H = rsh<T>().H;
