@@ -426,16 +426,44 @@ __device__ double eval_dn(const LevelGeom& L, long long q, const int I[3], int p
 // quotient's rounding is corrected by one fused step (Markstein, IBM J. Res.
 // Dev. 34, 1990), so it equals the division in three FP64 operations; GB300
 // issues about two of them per clock and SM, and a division is ten.  The step
-// is right while the remainder is exact: where x or the quotient lies within
-// 2^64 of either end of FP64's range (by the exponent bits) it is divided, and
-// zeros keep their sign.  pow2: b is a power of two and the product alone is exact.
-__device__ __noinline__ double div_ends(double x, double b) { return x / b; }
-__device__ __forceinline__ double div_fixed(double x, double b, double rb, bool pow2) {
+// is right while the remainder is exact: `bad` is set where x or the quotient
+// lies within 2^64 of either end of FP64's range (high word of |quotient| outside
+// lo .. lo + n) and is not zero.  pow2: b is a power of two and the product alone
+// is exact.
+struct DivRange {
+  unsigned lo, n;
+};
+__device__ __forceinline__ double div_fixed(double x, double b, double rb, bool pow2, const DivRange& R, bool& bad) {
   const double q = __dmul_rn(x, rb);
   if (pow2) return q;
-  const unsigned eq = ((unsigned)__double2hiint(q) >> 20) & 0x7ffu, ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
-  if (eq - 64u < 1920u && ex - 64u < 1920u) return __fma_rn(__fma_rn(-q, b, x), rb, q);
-  return x == 0.0 ? q : div_ends(x, b);
+  const unsigned h = (unsigned)__double2hiint(q) & 0x7fffffffu;
+  bad = bad || (h - R.lo >= R.n && (h | (unsigned)__double2loint(q)) != 0u);
+  return copysign(__fma_rn(__fma_rn(-q, b, x), rb, q), q);  // the sign of a zero
+}
+// The regular cells of a group with a `bad` quotient, by divisions, once the
+// group is done: out of line and from memory, since a division beside each
+// quotient takes the pass from 47 to 70 registers a thread (256^3: 3% of field
+// and tags).
+__device__ __noinline__ void field_redo(const double* ph, double* E, unsigned w, const int I0, int I1, int I2, int n0,
+                                        int n1, int n2, int D, double h) {
+  const int I[3] = {I0, I1, I2}, n[3] = {n0, n1, n2};
+  const long long ncell = (long long)n0 * n1 * n2;
+  for (int e = 0; e < 4; ++e) {
+    const unsigned f = (w >> (8 * e)) & 7u;
+    if (f & F_IRR) continue;
+    for (int p = 0; p < 2; ++p) {
+      if (!((f >> p) & 1u)) continue;
+      const double* c = ph + p * ncell + e;
+      long long st = 1;
+      for (int a = 0; a < D; ++a) {
+        const int i = a ? I[a] : I[0] + e;
+        const bool l = i > 0, u = i < n[a] - 1;
+        E[((long long)a * 2 + p) * ncell + e] = l && u ? -(c[st] - c[-st]) / (2.0 * h)
+                                                : u ? -(c[st] - c[0]) / h : l ? -(c[0] - c[-st]) / h : 0.0;
+        st *= n[a];
+      }
+    }
+  }
 }
 
 // E at regular cells, four of an x row per thread: every face neighbour in
@@ -447,7 +475,8 @@ __device__ __forceinline__ double div_fixed(double x, double b, double rb, bool 
 // 3.9 ms for a thread per cell with the face records looked up.
 template <bool AL>
 __global__ void __launch_bounds__(256) k_field_regular(LevelGeom L, const double* __restrict__ phi,
-                                                       double* __restrict__ E, double h2, double rh2, double rh, int pow2) {
+                                                       double* __restrict__ E, double h2, double rh2, double rh, int pow2,
+                                                       DivRange R) {
   const Grid& g = L.g;
   const long long c0 = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
   if (c0 >= g.ncell) return;
@@ -473,6 +502,7 @@ __global__ void __launch_bounds__(256) k_field_regular(LevelGeom L, const double
         if (!((irr >> (8 * e)) & 4u)) p[e] = v[e];
     }
   };
+  bool bad = false;
   for (int p = 0; p < 2; ++p) {
     const bool any = (w & ~((irr >> 2) * 255u) & (0x01010101u << p)) != 0;  // a regular lane of the phase
     const double* ph = phi + (long long)p * g.ncell + c0;
@@ -506,14 +536,15 @@ __global__ void __launch_bounds__(256) k_field_regular(LevelGeom L, const double
         for (int e = 0; e < 4; ++e) {
           if (!((w >> (8 * e + p)) & 1u)) continue;
           const bool l = a == 0 ? (e > 0 || l1) : l1, h = a == 0 ? (e < 3 || h1) : h1;
-          if (l && h) v[e] = div_fixed(-(hi[e] - lo[e]), h2, rh2, pow2);
-          else if (h) v[e] = div_fixed(-(hi[e] - c[e]), g.h, rh, pow2);
-          else if (l) v[e] = div_fixed(-(c[e] - lo[e]), g.h, rh, pow2);
+          if (l && h) v[e] = div_fixed(-(hi[e] - lo[e]), h2, rh2, pow2, R, bad);
+          else if (h) v[e] = div_fixed(-(hi[e] - c[e]), g.h, rh, pow2, R, bad);
+          else if (l) v[e] = div_fixed(-(c[e] - lo[e]), g.h, rh, pow2, R, bad);
         }
       }
       put(E + ((long long)a * 2 + p) * g.ncell + c0, v);
     }
   }
+  if (bad) field_redo(phi + c0, E + c0, w, I[0], I[1], I[2], g.n[0], g.n[1], g.n[2], g.D, g.h);
 }
 
 __global__ void k_field_irregular(LevelGeom L, const double* phi, const double* sigma, double* E) {
@@ -1005,10 +1036,14 @@ eb_status launch_field(const eb_geom* G, const double* phi, const double* sigma,
     int ex = 0;
     const int pow2 = std::frexp(h, &ex) == 0.5;
     const int nb = nblk(L.g.ncell / 4);
+    // exponent bits of a quotient by h or 2 h that, like its dividend, keeps
+    // 2^64 away from the ends of FP64's range
+    const int lo = std::max(64, 66 - ex), hi = std::min(1983, 1981 - ex);
+    const DivRange R{(unsigned)lo << 20, hi > lo ? (unsigned)(hi - lo) << 20 : 0u};
     if (!(((unsigned long long)phi | (unsigned long long)E) & 15ull))
-      k_field_regular<true><<<nb, TB, 0, s>>>(v, phi, E, h2, 1.0 / h2, 1.0 / h, pow2);
+      k_field_regular<true><<<nb, TB, 0, s>>>(v, phi, E, h2, 1.0 / h2, 1.0 / h, pow2, R);
     else
-      k_field_regular<false><<<nb, TB, 0, s>>>(v, phi, E, h2, 1.0 / h2, 1.0 / h, pow2);
+      k_field_regular<false><<<nb, TB, 0, s>>>(v, phi, E, h2, 1.0 / h2, 1.0 / h, pow2, R);
     if (L.nirr) k_field_irregular<<<nblk(L.nirr, 64), 64, 0, s>>>(v, phi, sigma, E);
   }
   if (En && L.n_eb) k_field_eb<<<dim3((unsigned)nblk(L.n_eb, 32), 2), 32, 0, s>>>(v, L.eb_q, L.n_eb, phi, sigma, En);
