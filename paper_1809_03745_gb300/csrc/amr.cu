@@ -651,12 +651,12 @@ extern "C" eb_status eb_amr_setup_levels(const eb_geom_desc* desc, int n_levels,
     st = eb_geom_export(A->lv[l].G, &ga, stream);
   }
   if (st != EB_OK) return amr_fail(A, st);
-  // a correction inside the preconditioner is one V-cycle of 3+3 sweeps: one
-  // inner V-cycle per defect-correction step and a loose tolerance (on the
-  // 256^3 + 128^3 pin-plane grid: 21 FGMRES iterations and 285 ms, against 19
-  // and 447 ms with two 6+6 V-cycles to 1e-2; 2+2 sweeps needed 23 iterations).
-  // A relaxed bottom takes at most 32 sweeps there: the same 21 iterations in
-  // 243 ms against 252 ms with 64; 16 sweeps needed 23 iterations (261 ms).
+  // a correction inside the preconditioner is one V-cycle of 3+3 sweeps (on the
+  // 256^3 + 128^3 pin-plane grid, before the levels were split by colour: 21
+  // FGMRES iterations and 285 ms, against 19 and 447 ms with two 6+6 V-cycles to
+  // 1e-2; 2+2 sweeps needed 23 iterations; now 84 ms).  A relaxed bottom grid
+  // takes at most 32 sweeps (then 243 ms against 252 ms with 64; 16 sweeps needed
+  // 23 iterations).
   eb_solver_opts oc = A->o;
   oc.inner_cycles = 1;
   oc.nu1 = oc.nu2 = 3;
