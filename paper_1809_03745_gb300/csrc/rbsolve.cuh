@@ -145,7 +145,7 @@ struct RCtx {
 // launches of a resumed solve.
 struct KryState {
   int count, next;   // directions kept, slot of the next one
-  int es;            // the V-cycles' right-hand side is the residual / 2^es (see unit_of)
+  int es;            // the solve's unit is 2^es (see unit_of)
   double g[KH][KH];  // (q_i, q_j) by slot
   double rn[KH];     // 1 / |q_i|
 };
@@ -160,6 +160,7 @@ struct RShared {
   RCtx c[2];  // the group, CTA 0 alone
   Op<double> F;
   unsigned epoch, tn;
+  int cur;  // phi and b are in units of 2^cur
   T red[PT / 32][KDOT];
   double dots[KDOT], coef[KH];
   KryState K;
@@ -1180,20 +1181,21 @@ __device__ __forceinline__ void bits_max(unsigned long long& m, double v) {
   if (b > m && b <= 0x7ff0000000000000ull) m = b;
 }
 
-// The unit of the FP32 V-cycles.  The Krylov sums multiply FP32 residuals: below
-// about 1e-20 these products vanish, above 1e17 they overflow, and data in SI
-// units reach both.  Where max|b| is outside 2^-10 .. 2^50 the residual is
-// therefore divided by 2^es, the power of two under max|b|, when it is rounded to
-// FP32, and the correction is multiplied by it when it is added to phi; both are
-// exact, so a solve takes the same steps in every unit.  Inside that range, where
-// a residual 13 digits under max|b| still has its square in FP32's range, es is 0.
-// Where max|r| leaves 2^-56 .. 2^50 units (a guess far from the solution), es is
-// chosen anew from it; the directions kept stay in the unit they were formed in,
-// since z and A z scale alike.  FP64 V-cycles have the range as they are.
+// The unit of a mixed solve.  The Krylov sums multiply FP32 residuals: below about
+// 1e-20 these products vanish, above 1e17 they overflow, and data in SI units
+// reach both.  Where max|b| is outside 2^-10 .. 2^50, phi and b are therefore
+// divided by 2^es, the power of two under max|b|, for the solve; that is exact, so
+// it takes the same steps in every unit.  Inside that range, where a residual 13
+// digits under max|b| still has its square in FP32's range, es is 0.  Where max|r|
+// leaves 2^-56 .. 2^50 units (a guess far from the solution), es is chosen anew
+// from it; the directions kept stay in the unit they were formed in, since z and A
+// z scale alike.  FP64 V-cycles have the range as they are.  (A unit in the phases
+// themselves, a factor on every residual and correction, cost every solve 0.5 to 2%,
+// and as builds of their own the phases beside them 1% at 384^3.)
 constexpr int ES_LO = -56, ES_MIN = -10, ES_HI = 50;
 __device__ __forceinline__ int exponent_of(double v) {
   const int e = ((__double2hiint(v) >> 20) & 0x7ff) - 1023;
-  return max(-1000, min(1000, e));
+  return max(-900, min(900, e));
 }
 __device__ __forceinline__ int unit_of(double v) {
   const int e = exponent_of(v);
@@ -1201,13 +1203,27 @@ __device__ __forceinline__ int unit_of(double v) {
 }
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
-// FP64 residual of the finest level into level 0's right-hand side (in its
-// unit, rounded to T) and its max norm; eight cells of an x row per item, seven FP64
-// operations each (GB300 issues about two FP64 operations per clock and SM,
-// which bounds the pass from 256^2 cells up).  US: in units of 2^es; a build of
-// its own, since a shift of the exponent bits, or a branch and an FP32 product,
-// in every cell cost this one 20 to 100 us at 256^3 (a whole solve 0.5 to 2.3%).
-template <class T, bool US>
+// phi and b times 2^e
+template <class T>
+__device__ __noinline__ bool rb_rescale(int e) {
+  const Op<double>& F = rsh<T>().F;
+  const RCtx& G = rsh<T>().c[0];
+  const double u = pow2(e / 2), v = pow2(e - e / 2);  // e may be twice what an exponent holds
+  for (int p = 0; p < 2; ++p) {
+    if (!F.x[p]) continue;
+    for (long long c = G.i0(); c < F.ncell; c += G.st) {
+      F.x[p][c] = F.x[p][c] * u * v;
+      F.b[p][c] = F.b[p][c] * u * v;
+    }
+  }
+  return G.sync((14 << 4) | 10);
+}
+
+// FP64 residual of the finest level into level 0's right-hand side (rounded
+// to T) and its max norm (in the caller's unit); eight cells of an x row per item,
+// seven FP64 operations each (GB300 issues about two FP64 operations per clock and
+// SM, which bounds the pass from 256^2 cells up).
+template <class T>
 __device__ __noinline__ bool rb_resid64(unsigned long long* norm) {
   const RHier<T>& H = rsh<T>().H;
   const RLev<T>& L = H.L[H.lc == 0 ? RMAX : 0];
@@ -1252,7 +1268,7 @@ __device__ __noinline__ bool rb_resid64(unsigned long long* norm) {
         const double v = (bc - s) - d * xc;
         unsigned pos;
         T* b = rb_rhs(L, cl, pos);
-        b[pos] = (T)(US ? v * pow2(-rsh<T>().K.es) : v);
+        b[pos] = (T)v;
         bits_max(mx, v);
       }
     }
@@ -1313,13 +1329,12 @@ __device__ __noinline__ bool rb_resid64(unsigned long long* norm) {
       ld4(F.b[p] + nb, bb);
       ld4(F.b[p] + nb + 4, bb + 4);
       T oe[4], oo[4];
-      const double unit = US ? pow2(-rsh<T>().K.es) : 1.0;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const double dg = e == 0 ? dl : (e == 7 ? dr : d0);
         const double r = bb[e] - F.ceps[p] * (dg * c[e] - s[e]);
-        if (e & 1) oo[e >> 1] = (T)(US ? r * unit : r);
-        else oe[e >> 1] = (T)(US ? r * unit : r);
+        if (e & 1) oo[e >> 1] = (T)r;
+        else oe[e >> 1] = (T)r;
         if (((e & 1) ? mo : me) >> (8 * (e >> 1)) & 1u) bits_max(mx, r);
       }
       quad_store(L.b[p][g.s] + 4 * (long long)t, me, oe);
@@ -1330,7 +1345,10 @@ __device__ __noinline__ bool rb_resid64(unsigned long long* norm) {
     const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
     mx = o > mx ? o : mx;
   }
-  if ((threadIdx.x & 31) == 0 && mx) atomicMax(norm, mx);
+  if ((threadIdx.x & 31) == 0 && mx) {
+    if (rsh<T>().cur) mx = (unsigned long long)__double_as_longlong(__longlong_as_double((long long)mx) * pow2(rsh<T>().cur));
+    atomicMax(norm, mx);
+  }
   return G.sync((14 << 4) | 11);
 }
 
@@ -1524,10 +1542,8 @@ __device__ __forceinline__ void rb_kry_coeff(const double* part, int nch, int m,
 
 // Krylov pass 2: phi += sum c z in FP64, z kept in slot `slot`, and r -= sum
 // c q where another V-cycle follows before the next FP64 residual.  slot < 0:
-// the plain correction, phi += z.  US: z and r are in units of 2^es, phi is not (a
-// build of its own, as of rb_resid64: with the product in this one a solve of
-// 1024^2 took 0.6% longer).
-template <class T, bool US>
+// the plain correction, phi += z.
+template <class T>
 __device__ __noinline__ void rb_kry2(int slot, int m, bool upd_r) {
   const RHier<T>& H = rsh<T>().H;
   const RLev<T>& L = H.L[H.lc == 0 ? RMAX : 0];
@@ -1595,9 +1611,8 @@ __device__ __noinline__ void rb_kry2(int slot, int m, bool upd_r) {
         const int odd = g.s ^ colour;  // red cells are the even ones where s = 0
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const double d = US ? (double)s[e] * pow2(rsh<T>().K.es) : (double)s[e];
-          if (odd) f[2 * e + 1] += d;
-          else f[2 * e] += d;
+          if (odd) f[2 * e + 1] += (double)s[e];
+          else f[2 * e] += (double)s[e];
         }
       }
       st4(ph, f);
@@ -1681,11 +1696,6 @@ __device__ __noinline__ void rb_begin(const RHier<T>* __restrict__ Hg, const Bar
   __syncthreads();
 }
 template <class T>
-__device__ __forceinline__ bool rb_residual(unsigned long long* norm) {
-  if (sizeof(T) == 4 && rsh<T>().K.es) return rb_resid64<T, sizeof(T) == 4>(norm);
-  return rb_resid64<T, false>(norm);
-}
-template <class T>
 __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, const Op<double>* __restrict__ Fg,
                                                const SolveCtl& ctl, const Barrier& B, int gcta, int gsize) {
   RShared<T>& S = rsh<T>();
@@ -1693,9 +1703,12 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
   copy_words(&S.F, Fg, sizeof(Op<double>));
   copy_words(&S.K, Hg->kst, sizeof(KryState));
   rb_begin<T>(Hg, B, gcta, gsize);
-  if (threadIdx.x == 0 && ctl.fresh) {
-    S.K.count = S.K.next = 0;
-    S.K.es = sizeof(T) == 4 ? unit_of(*ctl.bnorm) : 0;
+  if (threadIdx.x == 0) {
+    S.cur = 0;
+    if (ctl.fresh) {
+      S.K.count = S.K.next = 0;
+      S.K.es = sizeof(T) == 4 ? unit_of(*ctl.bnorm) : 0;
+    }
   }
   __syncthreads();
   const RCtx& G = S.c[0];
@@ -1710,7 +1723,7 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
   // norms are read again where they are needed: little stays in registers across the phases
 #pragma unroll 1
   for (; *ctl.bnorm != 0.0;) {
-    if (!rb_residual<T>(ctl.norms + it)) {
+    if (!rb_resid64<T>(ctl.norms + it)) {
       status = 5;
       break;
     }
@@ -1726,12 +1739,18 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
     }
     bool ok = true;
     if (sizeof(T) == 4) {
-      const int off = exponent_of(r) - S.K.es;  // the same in every CTA
-      if (off < ES_LO || off > ES_HI) {  // again in the unit of r, which holds it
+      int want = S.K.es;  // the same in every CTA
+      const int off = exponent_of(r) - want;
+      if (off < ES_LO || off > ES_HI) want = unit_of(r);
+      if (want != S.cur) {
+        if (!rb_rescale<T>(S.cur - want)) {
+          status = 5;
+          break;
+        }
         __syncthreads();
-        if (threadIdx.x == 0) S.K.es = unit_of(r);
+        if (threadIdx.x == 0) S.cur = S.K.es = want;
         __syncthreads();
-        continue;
+        continue;  // the residual in the new unit
       }
     }
 #pragma unroll 1
@@ -1752,8 +1771,7 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
         if (!ok) break;
         rb_kry_coeff(S.H.kpart, S.H.kch, m, S.K, S.dots, S.coef);
       }
-      if (sizeof(T) == 4 && S.K.es) rb_kry2<T, sizeof(T) == 4>(slot, m, ctl.kry && k + 1 < ctl.inner);
-      else rb_kry2<T, false>(slot, m, ctl.kry && k + 1 < ctl.inner);
+      rb_kry2<T>(slot, m, ctl.kry && k + 1 < ctl.inner);
       ok = G.sync((14 << 4) | 12);
     }
     if (threadIdx.x == 0) S.c[0].tr = S.c[1].tr = nullptr;
@@ -1764,6 +1782,7 @@ __device__ __forceinline__ void rb_solve_group(const RHier<T>* __restrict__ Hg, 
     cycles += ctl.inner;
     ++it;
   }
+  if (sizeof(T) == 4 && S.cur && status != 5) rb_rescale<T>(S.cur);
   if (gcta == 0 && threadIdx.x == 0) {
     if (ctl.trace) ctl.trace[0] = S.tn;
     const double r = bn == 0.0 ? 0.0 : load_norm(ctl.norms + it);
